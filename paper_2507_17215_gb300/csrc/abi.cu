@@ -512,13 +512,13 @@ struct LoadPairs {
     uint64_t* table;
     int lg;
     uint32_t* slotw;
-    int* over;
+    int* flags;
 };
 
 template <bool INSERT>
 __device__ __forceinline__ uint32_t load_slot_word(const LoadPairs& lp, int32_t x, int32_t y, int32_t n) {
     if (!INSERT || x < 0 || x >= n || y < 0 || y >= n) return PAIR_LOOP;
-    return pair_slot_word(lp.table, lp.lg, x, y, n, lp.over);
+    return pair_slot_word(lp.table, lp.lg, x, y, n, lp.flags);
 }
 
 // The same checks fused with the copy of the input into the graph's own arrays: one
@@ -543,6 +543,7 @@ __global__ void k_load_copy(const int32_t* __restrict__ src, const int32_t* __re
         const bool act = j < m4;
         int4 x{}, y{};
         longlong2 t01{}, t23{};
+        const bool over = INSERT && pair_table_over(lp.flags);  // the table serves no more
         if (act) {
             x = __ldcs(reinterpret_cast<const int4*>(src) + j);
             y = __ldcs(reinterpret_cast<const int4*>(dst) + j);
@@ -561,7 +562,7 @@ __global__ void k_load_copy(const int32_t* __restrict__ src, const int32_t* __re
             st.edge(i + 1, x.y, y.y, t01.y, t01.x, n);
             st.edge(i + 2, x.z, y.z, t23.x, t01.y, n);
             st.edge(i + 3, x.w, y.w, t23.y, t23.x, n);
-            if (INSERT) {
+            if (INSERT && !over) {
                 // the four edges' first probes issued together (most find their pair, or
                 // an empty slot, there); the rest of a probe sequence one edge at a time
                 const int32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
@@ -592,7 +593,7 @@ __global__ void k_load_copy(const int32_t* __restrict__ src, const int32_t* __re
         odst[i] = y;
         ot[i] = ti;
         st.edge(i, x, y, ti, i > 0 ? t[i - 1] : 0, n);
-        if (INSERT) lp.slotw[i] = load_slot_word<INSERT>(lp, x, y, n);
+        if (INSERT && !pair_table_over(lp.flags)) lp.slotw[i] = load_slot_word<INSERT>(lp, x, y, n);
     }
     st.flush(stat);
 }
@@ -649,7 +650,7 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
         g->pre_lg = lp.lg;
         g->pre_table = graph_alloc<uint64_t>(g, 1ll << lp.lg, s);
         g->pre_slotw = graph_alloc<uint32_t>(g, m, s);
-        g->pre_flags = graph_alloc<int>(g, 2, s);
+        g->pre_flags = graph_alloc<int>(g, PAIR_FLAGS, s);
         if (!a16(g->pre_slotw)) {  // a caller's allocator may not align it for 16-byte stores
             graph_release(g, g->pre_table, s);
             graph_release(g, g->pre_slotw, s);
@@ -660,7 +661,7 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
             insert = false;
         } else {
             FOLTY_CUDA(cudaMemsetAsync(g->pre_table, 0, sizeof(uint64_t) * ((size_t)1 << lp.lg), s));
-            FOLTY_CUDA(cudaMemsetAsync(g->pre_flags, 0, 2 * sizeof(int), s));
+            FOLTY_CUDA(cudaMemsetAsync(g->pre_flags, 0, PAIR_FLAGS * sizeof(int), s));
             lp = LoadPairs{g->pre_table, lp.lg, g->pre_slotw, g->pre_flags};
         }
     }

@@ -154,12 +154,15 @@ constexpr int PAIR_COMPACT_ITEMS = 16;            // table slots per thread and 
 
 // Every non-loop edge's pair goes into the table (value rank + 1, 0 = empty), and edge i
 // keeps its slot and direction in slotw[i] (PAIR_LOOP for a self-loop). A probe sequence
-// that runs out sets *over.
+// that runs out, or too many distinct pairs, abandon the table, and the insert stops.
 __global__ void k_pair_insert(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m, int32_t n,
                               uint64_t* __restrict__ table, int lg, uint32_t* __restrict__ slotw,
-                              int* __restrict__ over) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        __stcs(slotw + i, pair_slot_word(table, lg, src[i], dst[i], n, over));
+                              int* flags) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t x = src[i], y = dst[i];
+        if (pair_table_over(flags)) return;
+        __stcs(slotw + i, pair_slot_word(table, lg, x, y, n, flags));
+    }
 }
 
 // The occupied slots as (rank, slot) lists, in no particular order: each block takes
@@ -2659,10 +2662,9 @@ static bool pair_ids_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
     uint64_t* table = nullptr;
     uint64_t* urank = nullptr;
     uint32_t* uslot = nullptr;
-    // the first try's table, slot words and flags ([0] a probe ran out, [1] distinct
-    // pairs) may already be filled by the load
+    // the first try's table, slot words and flags may already be filled by the load
     const bool pre = g->pre_table != nullptr && g->pre_lg == lg;
-    int* flags = pre ? g->pre_flags : sc.get<int>(2);
+    int* flags = pre ? g->pre_flags : sc.get<int>(PAIR_FLAGS);
     uint32_t* slotw = pre ? g->pre_slotw : sc.get<uint32_t>(m);
     bool first = true;
     while (true) {
@@ -2673,7 +2675,7 @@ static bool pair_ids_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
         } else {
             table = sc.get<uint64_t>(tb);
             FOLTY_CUDA(cudaMemsetAsync(table, 0, sizeof(uint64_t) * (size_t)tb, s));
-            FOLTY_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), s));
+            FOLTY_CUDA(cudaMemsetAsync(flags, 0, PAIR_FLAGS * sizeof(int), s));
             FOLTY_LAUNCH(k_pair_insert, grid_for(m, T), T, 0, s, g->in_src, g->in_dst, m, n, table, lg, slotw, flags);
         }
         first = false;

@@ -1,0 +1,67 @@
+"""The sizes at which the library changes from one kernel or table size to another, against
+the CPU oracle (bit-exact: all arithmetic is integer)."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+from _support import pairs_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2507_17215_gb300 as F
+    return F
+
+
+def _check(F, g, queries, device=False):
+    if device:
+        import torch
+        arrays = [torch.from_numpy(x).cuda() for x in (g.src, g.dst, g.t)]
+    else:
+        arrays = [g.src, g.dst, g.t]
+    with F.TemporalGraph(g.n, *arrays) as G, oracle.OracleGraph.of(g) as og:
+        for q in queries:
+            got, want = G.query(q), og.query(q)
+            if q.want_edge_counts:
+                np.testing.assert_array_equal(got["edge_count"], want["edge_count"], err_msg=str(q))
+            assert pairs_of(got) == pairs_of(want), str(q)
+            assert got["n_cert_edges"] == want["n_cert_edges"], str(q)
+        return G.info()
+
+
+def _distinct_pairs_graph(pairs, repeats, seed):
+    """A time-ordered graph of exactly `pairs` distinct pairs, `repeats` of them twice: a
+    block of 120 vertices with every pair (triangles), the rest random pairs."""
+    rng = np.random.default_rng(seed)
+    n, b = 400_000, 120
+    i, j = np.triu_indices(b, 1)
+    keys = i.astype(np.int64) * n + j
+    while keys.shape[0] < pairs:
+        x, y = rng.integers(b, n, (2, pairs))
+        more = np.unique(np.minimum(x, y) * n + np.maximum(x, y))
+        more = more[more // n != more % n]
+        keys = np.unique(np.concatenate([keys, rng.permutation(more)[: pairs - keys.shape[0]]]))
+    keys = np.concatenate([keys, keys[:repeats]])
+    a, c = keys // n, keys % n
+    flip = rng.random(keys.shape[0]) < 0.5
+    t = rng.integers(0, 1000, keys.shape[0])
+    o = np.argsort(t, kind="stable")
+    return W.TemporalGraph(n, np.where(flip, c, a)[o].astype(np.int32), np.where(flip, a, c)[o].astype(np.int32),
+                           t[o].astype(np.int64))
+
+
+# the first table of 524,289 to 12.5M edges has 2^20 slots: it serves up to 2^19 pairs, is
+# retried when it turns out fuller, and is abandoned on the way past 9/16 of its slots
+@pytest.mark.parametrize("pairs", [(1 << 19) - 1, 1 << 19, (1 << 19) + 1, 560_000, 590_000, 700_000, 1_100_000])
+@pytest.mark.parametrize("device", [False, True])
+def test_pair_table_sizes(F, pairs, device):
+    g = _distinct_pairs_graph(pairs, 30_000, pairs)
+    info = _check(F, g, [W.Query(300, 1, 4, W.Q_FORALL_T, W.DIR_EITHER, W.U_COMMON, True)], device)
+    assert info["static_edges"] == pairs
