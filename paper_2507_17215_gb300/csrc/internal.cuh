@@ -192,6 +192,7 @@ struct folty_graph {
     int32_t* core;    // [n] core numbers of G_S
     int32_t* common;  // [S] |N(a) cap N(b)| = triangles on the static edge
     int32_t* by_b;    // [S] static edge ids ordered by (b, a)
+    int32_t* binv;    // [S] place of each static edge in by_b
     int32_t* prank;   // [2S] rank of directed pair 2s + d in (u, v) order (batched queries; made on first use)
     int64_t ntri;
     int4* tri;        // [ntri] {s_uv, s_uw, s_vw, id-order bits}, u < v < w in degeneracy rank
@@ -360,8 +361,8 @@ void launch_probe(folty_graph* g, int64_t delta, int dir, int32_t* cnt, cudaStre
 // edge-major rows of kstride bins (bin j of sorted edge e at e * kstride + j), as int32 or,
 // with bins16 (bins null), as 16-bit counts (counts must stay below 2^16).
 // rflag (mode 0, may be null): byte 6 * triangle + role set to 1 when the role has a hit.
-// touched (mode 1, may be null): bit g of word g / 32 set when one of sorted edges
-// [32 g, 32 g + 32) received a binned hit (the caller clears the words first).
+// touched (may be null): bit g of word g / 32 set when one of sorted edges
+// [32 g, 32 g + 32) received a hit (the caller clears the words first).
 void launch_probe_live(folty_graph* g, int64_t delta, int dir, int mode, int32_t* cnt, int32_t* bins, int k,
                        int kstride, const void* deltas, cudaStream_t s, uint8_t* rflag = nullptr,
                        uint16_t* bins16 = nullptr, uint32_t* touched = nullptr);
@@ -403,18 +404,19 @@ struct ProbeBuffers {
     int64_t* totals;  // kept triangles, slots
     int64_t* ltile;
     int64_t max_tiles;
-    int32_t* wcnt;    // per selection warp: kept triangles, then their exclusive prefix
-    int64_t* wcost;   // per selection warp: their slots, then the exclusive prefix
-    int64_t nw;
+    int ush;                  // log2 of the slots per unit of the selection's counter
+    unsigned long long* ctl;  // the selection's counters, zero between selections
 };
 // The same buffers owned by the graph (held by its query plans).
 ProbeBuffers probe_buffers(folty_graph* g, cudaStream_t s);
-// Selection and probes of one query into counters (cnt or cnt16, zeroed), the window
-// taken from the device parameter block qp (slot 0: 64-bit, slot 1: the 32-bit store's
-// clamped value): no host value in any launch, so a captured sequence replays for any
-// window.
+// Selection and probes of one query into counters (cnt or cnt16, zeroed) and the bits of
+// the 32-edge groups with a hit (touched, zeroed), the window taken from the device
+// parameter block qp (slot 0: 64-bit, slot 1: the 32-bit store's clamped value): no host
+// value in any launch, so a captured sequence replays for any window.
 void enqueue_probe_pass(folty_graph* g, const int64_t* qp, int dir, const ProbeBuffers& pb, int32_t* cnt,
-                        uint16_t* cnt16, cudaStream_t s);
+                        uint16_t* cnt16, uint32_t* touched, cudaStream_t s);
+// A cleared device counter of model bytes while profiling is on, else null.
+unsigned long long* prof_counter(folty_graph* g, cudaStream_t s);
 // Kept roles, probes and model bytes of one query's selection (live.cu; synchronises).
 void probe_stats(folty_graph* g, int64_t delta, int dir, folty_probe_stats* out, cudaStream_t s);
 // The same pass with the counters in a file-scope device array (noalloc.cu).

@@ -134,39 +134,47 @@ __device__ __forceinline__ int kept_roles_of(const int4 tr, const RunEnds<TS>* _
 }
 
 // Kept roles of every triangle for one query: kept triangle j = L[j] with its role mask
-// lmask[j] and its first probe slot loff[j] (prefix of the kept triangles' costs = kept
-// probes + LIVE_IDLE idle slots); totals[0] = kept triangles, totals[1] = slots,
-// loff[totals[0]] = totals[1]; and the probe tiles' map: ltile[b] = kept triangle holding
-// slot min(b * ptile, slots - 1) for b <= the number of probe tiles (each kept triangle
-// writes the tile starts inside its slots).
+// lmask[j] and its first probe slot loff[j] (the kept triangles' costs = kept probes +
+// LIVE_IDLE idle slots, laid out one after another); totals[0] = kept triangles, totals[1]
+// = slots, loff[totals[0]] = totals[1]; and the probe tiles' map: ltile[b] = kept triangle
+// holding slot min(b * ptile, slots - 1) for b <= the number of probe tiles (each kept
+// triangle writes the tile starts inside its slots).
 //
-// Three passes without a look-back: every warp takes LS_WARP consecutive triangles (a
-// lane LS_ITEMS of them, read as 16-byte chunks of their liveness bytes: the smallest
-// bucket of each triangle's roles for this direction variant); k_live_sums writes the
-// warp's number of kept triangles and their cost, k_live_offsets turns those into
-// exclusive prefixes (one block), and k_live_write writes the kept triangles at them.
-// Only the triangles whose byte admits delta read their record and run ends: they are
-// few, but cluster, so a warp deals its candidates round-robin over its lanes (candidate
-// k of the warp, in triangle order, goes to lane k mod 32), and the write pass orders
-// their costs by a warp scan per round of 32.
-constexpr int LS_ITEMS = 64;
-constexpr int LS_WARP = 32 * LS_ITEMS;  // 2048 triangles per warp
+// One pass. A warp takes 32 * ITEMS consecutive triangles (a lane ITEMS of them, read as
+// 16-byte chunks of their liveness bytes: the smallest bucket of each triangle's roles for
+// this direction variant). Only the triangles whose byte admits delta read their record
+// and run ends: they are few, but cluster, so a warp deals its candidates over its lanes,
+// LS_EACH per lane and step, orders their costs by a warp scan and reserves the step's
+// list entries and slots together with one 64-bit addition (the counter ls_count_shift
+// packs). The list is therefore in the order of the reservations, not of the triangles:
+// the probes only add to counters, so no result depends on it. The last block to finish
+// writes the totals and clears the counter for the next selection.
+//
+// It replaced a counting pass, a one-block scan of the warps' sums and a writing pass that
+// read every kept triangle again: 122 -> 29 us for 76M triangles of which 42K are kept
+// (the one-block scan alone took 71), 75 -> 9 us for 68K triangles, where warps of 2048
+// triangles left all but a few SMs idle. 64 triangles a lane (four 16-byte loads in flight)
+// from LS_LARGE triangles on, where the pass streams the bytes; below, 16 a lane, for more
+// warps with fewer candidates each.
 constexpr int LS_THREADS = 256;
-constexpr int LS_BLOCK = (LS_THREADS / 32) * LS_WARP;
+constexpr int LS_EACH = 4;                        // candidates per lane and step
+constexpr int64_t LS_LARGE = int64_t(1) << 24;
+constexpr int LS_UNIT_BITS = 33;                  // packed counter: kept triangles << 33 | slots in units
 
-// Bit i of the result: triangle t0 + i (i < LS_ITEMS) is kept at delta (rows are padded
+// Bit i of the result: triangle t0 + i (i < ITEMS) is kept at delta (rows are padded
 // with DMIN_NEVER to whole 16-byte chunks). A byte b admits delta exactly when
 // b <= B = bit length of delta (b = 0 always, b >= 1 when delta >= 2^(b-1); DMIN_NEVER
 // never, as B <= 63): four bytes at a time, (0x80 + B) - (b & 0x7f) keeps bit 7 set
 // exactly for b <= B (bytes never borrow from one another, and 255 & 0x7f = 127 > B), and
 // one multiplication gathers the four bit-7s.
+template <int ITEMS>
 __device__ __forceinline__ uint64_t live_mask(const uint8_t* __restrict__ tlive, int64_t t0, int64_t ntri,
                                               int64_t delta) {
     const uint32_t B = delta > 0 ? (uint32_t)(64 - __clzll((unsigned long long)delta)) : 0u;
     const uint32_t bias = 0x80808080u | (B * 0x01010101u);
     uint64_t lm = 0;
 #pragma unroll
-    for (int h = 0; h < LS_ITEMS / 16; h++) {
+    for (int h = 0; h < ITEMS / 16; h++) {
         uint4 w = make_uint4(~0u, ~0u, ~0u, ~0u);
         if (t0 + 16 * h < ntri) w = __ldcs(reinterpret_cast<const uint4*>(tlive + t0 + 16 * h));
         const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
@@ -198,6 +206,7 @@ __device__ __forceinline__ int warp_candidates(uint64_t lm, int& pre) {
 // Position within the warp's range of candidate k (< the warp's total): the lane l with
 // pre[l] <= k < pre[l + 1], and the (k - pre[l])-th set bit of its mask. The whole warp
 // must call it.
+template <int ITEMS>
 __device__ __forceinline__ int candidate_at(int k, uint64_t lm, int pre) {
     int l = 0;
 #pragma unroll
@@ -206,156 +215,106 @@ __device__ __forceinline__ int candidate_at(int k, uint64_t lm, int pre) {
         if (pc <= k) l += step;
     }
     const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)lm, l);
-    const uint32_t hi = __shfl_sync(0xffffffffu, (uint32_t)(lm >> 32), l);
+    const uint32_t hi = ITEMS > 32 ? __shfl_sync(0xffffffffu, (uint32_t)(lm >> 32), l) : 0u;
     const int n = k - __shfl_sync(0xffffffffu, pre, l);  // 0-based rank among l's candidates
     const int plo = __popc(lo);
     const int bit = n < plo ? __fns(lo, 0, n + 1) : 32 + __fns(hi, 0, n - plo + 1);
-    return l * LS_ITEMS + bit;
+    return l * ITEMS + bit;
 }
 
-// Per warp: its kept triangles and their total cost.
-template <typename TS, int DIR>
-__global__ void __launch_bounds__(LS_THREADS) k_live_sums(const uint8_t* __restrict__ tlive,
-                                                          const int4* __restrict__ tri,
-                                                          const RunEnds<TS>* __restrict__ ends, int64_t ntri,
-                                                          int64_t delta, const int64_t* __restrict__ qp,
-                                                          int32_t* __restrict__ wcnt, int64_t* __restrict__ wcost) {
-    if (qp) delta = qp[0];  // the window from a device parameter block (replayed query plans)
+struct SelectArgs {
+    const uint8_t* tlive;
+    const int4* tri;
+    int64_t ntri;
+    int64_t delta;
+    const int64_t* qp;  // may be null: device parameter block whose slot 0 holds the window
+    int ush;            // log2 of the slots per unit of the packed counter
+    unsigned long long* ctl;  // [0] packed counter, [1] blocks done; both zero before and after
+    int32_t* L;
+    int64_t* loff;
+    uint8_t* lmask;
+    int64_t* ltile;
+    int64_t max_tiles, ptile;
+    int64_t* totals;
+    unsigned long long* prof;  // may be null
+};
+
+template <typename TS, int DIR, int ITEMS>
+__global__ void __launch_bounds__(LS_THREADS) k_live_select(const SelectArgs a, const RunEnds<TS>* __restrict__ ends) {
+    const int64_t delta = a.qp ? a.qp[0] : a.delta;
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * LS_THREADS + threadIdx.x) >> 5;
-    const int64_t tw = w * LS_WARP;
-    const uint64_t lm = live_mask(tlive, tw + (int64_t)lane * LS_ITEMS, ntri, delta);
+    const int64_t tw = w * (32 * ITEMS);
+    const uint64_t lm = live_mask<ITEMS>(a.tlive, tw + (int64_t)lane * ITEMS, a.ntri, delta);
     int pre;
     const int total = warp_candidates(lm, pre);
-    int64_t cost = 0;
-    for (int k0 = 0; k0 < total; k0 += 32) {
-        const int k = k0 + lane;
-        const int at = candidate_at(min(k, total - 1), lm, pre);
-        if (k < total) {
-            int64_t pr;
-            kept_roles_of<TS, DIR>(tri[tw + at], ends, delta, pr);
-            cost += pr + LIVE_IDLE;
+    for (int k0 = 0; k0 < total; k0 += 32 * LS_EACH) {
+        const int kl = k0 + lane * LS_EACH;  // this lane's candidates kl ... kl + LS_EACH - 1
+        int at[LS_EACH];
+        int4 tr[LS_EACH];
+#pragma unroll
+        for (int r = 0; r < LS_EACH; r++) {
+            at[r] = candidate_at<ITEMS>(min(kl + r, total - 1), lm, pre);
+            if (kl + r < total) tr[r] = a.tri[tw + at[r]];
         }
-    }
+        int m[LS_EACH];
+        int64_t v[LS_EACH], sum = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cost += __shfl_xor_sync(0xffffffffu, cost, o);
-    if (lane == 0) {
-        wcnt[w] = total;
-        wcost[w] = cost;
-    }
-}
-
-// One block: the warps' counts and costs become exclusive prefixes in place; the totals,
-// the end of loff and of the tile map, and the kept triangles' model bytes.
-template <typename TS>
-__global__ void __launch_bounds__(1024) k_live_offsets(int32_t* __restrict__ wcnt, int64_t* __restrict__ wcost,
-                                                       int64_t nw, int64_t* __restrict__ totals,
-                                                       int64_t* __restrict__ loff, int64_t* __restrict__ ltile,
-                                                       int64_t max_tiles, int64_t ptile,
-                                                       unsigned long long* __restrict__ prof) {
-    __shared__ int64_t sc[32], sp[32];
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const int64_t per = (nw + 1023) / 1024;
-    const int64_t b = (int64_t)threadIdx.x * per, e = min(b + per, nw);
-    int64_t c = 0, p = 0;
-    for (int64_t i = b; i < e; i++) {
-        c += wcnt[i];
-        p += wcost[i];
-    }
-    int64_t ic = c, ip = p;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t yc = __shfl_up_sync(0xffffffffu, ic, o), yp = __shfl_up_sync(0xffffffffu, ip, o);
-        if (lane >= o) {
-            ic += yc;
-            ip += yp;
-        }
-    }
-    if (lane == 31) {
-        sc[wi] = ic;
-        sp[wi] = ip;
-    }
-    __syncthreads();
-    if (wi == 0) {
-        int64_t xc = sc[lane], xp = sp[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t yc = __shfl_up_sync(0xffffffffu, xc, o), yp = __shfl_up_sync(0xffffffffu, xp, o);
-            if (lane >= o) {
-                xc += yc;
-                xp += yp;
+        for (int r = 0; r < LS_EACH; r++) {
+            m[r] = 0;
+            v[r] = 0;
+            if (kl + r < total) {
+                int64_t pr;
+                m[r] = kept_roles_of<TS, DIR>(tr[r], ends, delta, pr);
+                v[r] = pr + LIVE_IDLE;
             }
+            sum += v[r];
         }
-        sc[lane] = xc;  // inclusive over warps
-        sp[lane] = xp;
-    }
-    __syncthreads();
-    int64_t oc = ic - c + (wi ? sc[wi - 1] : 0), op = ip - p + (wi ? sp[wi - 1] : 0);
-    for (int64_t i = b; i < e; i++) {
-        const int32_t x = wcnt[i];
-        const int64_t y = wcost[i];
-        wcnt[i] = (int32_t)oc;
-        wcost[i] = op;
-        oc += x;
-        op += y;
-    }
-    if (threadIdx.x == 0) {
-        const int64_t nl = sc[31], P = sp[31];
-        totals[0] = nl;
-        totals[1] = P;
-        loff[nl] = P;
-        const int64_t tiles = (P + ptile - 1) / ptile;
-        if (P > 0 && tiles <= max_tiles) ltile[tiles] = nl - 1;
-        if (prof) atomicAdd(prof, (unsigned long long)((16 + 3 * sizeof(RunEnds<TS>) + 13) * nl));
-    }
-}
-
-// Per warp: its kept triangles at their prefixes, with their masks, first slots and tile
-// starts.
-template <typename TS, int DIR>
-__global__ void __launch_bounds__(LS_THREADS) k_live_write(const uint8_t* __restrict__ tlive,
-                                                           const int4* __restrict__ tri,
-                                                           const RunEnds<TS>* __restrict__ ends, int64_t ntri,
-                                                           int64_t delta, const int64_t* __restrict__ qp,
-                                                           const int32_t* __restrict__ woffc,
-                                                           const int64_t* __restrict__ woffp, int32_t* __restrict__ L,
-                                                           int64_t* __restrict__ loff, uint8_t* __restrict__ lmask,
-                                                           int64_t* __restrict__ ltile, int64_t max_tiles,
-                                                           int64_t ptile) {
-    if (qp) delta = qp[0];
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * LS_THREADS + threadIdx.x) >> 5;
-    const int64_t tw = w * LS_WARP;
-    const uint64_t lm = live_mask(tlive, tw + (int64_t)lane * LS_ITEMS, ntri, delta);
-    int pre;
-    const int total = warp_candidates(lm, pre);
-    if (total == 0) return;  // warp-uniform
-    const int64_t bc = woffc[w];
-    int64_t run = woffp[w];
-    for (int k0 = 0; k0 < total; k0 += 32) {
-        const int k = k0 + lane;
-        const int at = candidate_at(min(k, total - 1), lm, pre);
-        int m = 0;
-        int64_t v = 0;
-        if (k < total) {
-            int64_t pr;
-            m = kept_roles_of<TS, DIR>(tri[tw + at], ends, delta, pr);
-            v = pr + LIVE_IDLE;
-        }
-        int64_t inc = v;
+        int64_t inc = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += y;
         }
-        if (k < total) {
-            const int64_t jc = bc + k, jp = run + inc - v;
-            L[jc] = (int32_t)(tw + at);
-            loff[jc] = jp;
-            lmask[jc] = (uint8_t)m;
-            for (int64_t b = (jp + ptile - 1) / ptile; b * ptile < jp + v && b <= max_tiles; b++) ltile[b] = jc;
+        const int64_t all = __shfl_sync(0xffffffffu, inc, 31);
+        const int64_t units = (all + ((int64_t)1 << a.ush) - 1) >> a.ush;
+        const int n = min(total - k0, 32 * LS_EACH);
+        unsigned long long base = 0;
+        if (lane == 0)
+            base = atomicAdd(a.ctl, ((unsigned long long)n << LS_UNIT_BITS) | (unsigned long long)units);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        const int64_t bc = (int64_t)(base >> LS_UNIT_BITS);
+        int64_t jp = ((int64_t)(base & ((1ull << LS_UNIT_BITS) - 1)) << a.ush) + inc - sum;
+#pragma unroll
+        for (int r = 0; r < LS_EACH; r++) {
+            if (kl + r >= total) break;
+            const int64_t jc = bc + lane * LS_EACH + r;
+            // the step's last triangle also holds the slots that round the step up to whole units
+            const int64_t end = jp + v[r] + (lane * LS_EACH + r == n - 1 ? (units << a.ush) - all : 0);
+            a.L[jc] = (int32_t)(tw + at[r]);
+            a.loff[jc] = jp;
+            a.lmask[jc] = (uint8_t)m[r];
+            for (int64_t b = (jp + a.ptile - 1) / a.ptile; b * a.ptile < end && b <= a.max_tiles; b++) a.ltile[b] = jc;
+            jp = end;
         }
-        run += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.ctl + 1, 1ull) == gridDim.x - 1) {
+            __threadfence();
+            const unsigned long long c = *(volatile unsigned long long*)a.ctl;
+            const int64_t nl = (int64_t)(c >> LS_UNIT_BITS);
+            const int64_t P = (int64_t)(c & ((1ull << LS_UNIT_BITS) - 1)) << a.ush;
+            a.totals[0] = nl;
+            a.totals[1] = P;
+            a.loff[nl] = P;
+            const int64_t tiles = (P + a.ptile - 1) / a.ptile;
+            if (P > 0 && tiles <= a.max_tiles) a.ltile[tiles] = nl - 1;
+            if (a.prof) atomicAdd(a.prof, (unsigned long long)((16 + 3 * sizeof(RunEnds<TS>) + 13) * nl));
+            a.ctl[0] = 0;
+            a.ctl[1] = 0;
+        }
     }
 }
 
@@ -398,8 +357,8 @@ struct LiveArgs {
     uint8_t* rflag;    // MODE 0, may be null: 6 * triangle + role flags of roles with a hit
     const int64_t* qp; // may be null: a device block whose slot 0 (64-bit store) or 1 (32-bit
                        // store) holds the window, read instead of the delta argument
-    uint32_t* touched; // MODE 1, may be null: bit g set when a sorted edge of group g (edges
-                       // [32 g, 32 g + 32)) received a binned hit
+    uint32_t* touched; // may be null: bit g set when a sorted edge of group g (edges
+                       // [32 g, 32 g + 32)) received a hit
 };
 
 // MODE 0: cnt[pos] += hit at window delta. MODE 1: bin the gap t3 - t (<= delta, the
@@ -481,7 +440,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
                 if (o < s1) break;
                 o -= s1;
             }
-            if (r == 6) continue;  // cannot happen: o < the kept roles' total
+            if (r == 6) continue;  // a slot that rounds a step of the selection up to whole units
             const int32_t pos = off[3 * (r >> 1) + (r & 1)] + o;
             const int code = (int)((st.desc[j] >> (6 * r)) & 63);
             const TS t = T[pos];
@@ -498,11 +457,11 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
                 const int64_t x = (int64_t)pos * a.kstride + jb;  // edge-major: an edge's bins are contiguous
                 if (a.bins16) atomicAdd(&a.bins16[x >> 1], 1u << (16 * (int)(x & 1)));
                 else atomicAdd(&a.bins[x], 1);
-                if (a.touched) {
-                    // a plain read first: most hits find their group's bit already set
-                    const uint32_t bit = 1u << ((pos >> 5) & 31);
-                    if (!(a.touched[pos >> 10] & bit)) atomicOr(&a.touched[pos >> 10], bit);
-                }
+            }
+            if (a.touched) {
+                // a plain read first: most hits find their group's bit already set
+                const uint32_t bit = 1u << ((pos >> 5) & 31);
+                if (!(a.touched[pos >> 10] & bit)) atomicOr(&a.touched[pos >> 10], bit);
             }
         }
     }
@@ -620,32 +579,27 @@ static void launch_live_t(const folty_graph* g, int dir, const LiveArgs& la, TS 
     else launch_live_shape<TS, MODE, 8>(g, dir, la, g->tune.probe_blocks, delta, deltas, s);
 }
 
+template <typename TS, int ITEMS>
+static void launch_select_items(int dir, const SelectArgs& a, const RunEnds<TS>* ends, cudaStream_t s) {
+    const int64_t per_block = (int64_t)LS_THREADS * ITEMS;
+    const unsigned blocks = (unsigned)((a.ntri + per_block - 1) / per_block);
+    if (dir == FOLTY_DIR_OUT)
+        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_OUT, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
+    else if (dir == FOLTY_DIR_IN)
+        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_IN, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
+    else
+        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_EITHER, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
+}
+
 template <typename TS>
 static void launch_select_t(const folty_graph* g, int dir, const uint8_t* tl, int64_t delta, const ProbeBuffers& ls,
                             unsigned long long* prof, const int64_t* qp, cudaStream_t s) {
     const RunEnds<TS>* ends = static_cast<const RunEnds<TS>*>(g->run_ends);
-    const int64_t ntri = g->ntri;
     const int64_t tile = (int64_t)PB_THREADS * g->tune.probe_items;
-    const unsigned blocks = (unsigned)((ntri + LS_BLOCK - 1) / LS_BLOCK);
-#define FOLTY_SUMS_ARGS tl, g->tri, ends, ntri, delta, qp, ls.wcnt, ls.wcost
-#define FOLTY_WRITE_ARGS \
-    tl, g->tri, ends, ntri, delta, qp, ls.wcnt, ls.wcost, ls.L, ls.loff, ls.lmask, ls.ltile, ls.max_tiles, tile
-    if (dir == FOLTY_DIR_OUT)
-        FOLTY_LAUNCH((k_live_sums<TS, FOLTY_DIR_OUT>), blocks, LS_THREADS, 0, s, FOLTY_SUMS_ARGS);
-    else if (dir == FOLTY_DIR_IN)
-        FOLTY_LAUNCH((k_live_sums<TS, FOLTY_DIR_IN>), blocks, LS_THREADS, 0, s, FOLTY_SUMS_ARGS);
-    else
-        FOLTY_LAUNCH((k_live_sums<TS, FOLTY_DIR_EITHER>), blocks, LS_THREADS, 0, s, FOLTY_SUMS_ARGS);
-    FOLTY_LAUNCH(k_live_offsets<TS>, 1, 1024, 0, s, ls.wcnt, ls.wcost, ls.nw, ls.totals, ls.loff, ls.ltile,
-                 ls.max_tiles, tile, prof);
-    if (dir == FOLTY_DIR_OUT)
-        FOLTY_LAUNCH((k_live_write<TS, FOLTY_DIR_OUT>), blocks, LS_THREADS, 0, s, FOLTY_WRITE_ARGS);
-    else if (dir == FOLTY_DIR_IN)
-        FOLTY_LAUNCH((k_live_write<TS, FOLTY_DIR_IN>), blocks, LS_THREADS, 0, s, FOLTY_WRITE_ARGS);
-    else
-        FOLTY_LAUNCH((k_live_write<TS, FOLTY_DIR_EITHER>), blocks, LS_THREADS, 0, s, FOLTY_WRITE_ARGS);
-#undef FOLTY_SUMS_ARGS
-#undef FOLTY_WRITE_ARGS
+    const SelectArgs a{tl,       g->tri,  g->ntri,      delta, qp,        ls.ush, ls.ctl, ls.L,
+                       ls.loff,  ls.lmask, ls.ltile, ls.max_tiles, tile, ls.totals, prof};
+    if (g->ntri >= LS_LARGE) launch_select_items<TS, 64>(dir, a, ends, s);
+    else launch_select_items<TS, 16>(dir, a, ends, s);
 }
 
 // Buffers of one selection: from a call's scratch, or owned by the graph. The tile map
@@ -653,32 +607,44 @@ static void launch_select_t(const folty_graph* g, int dir, const uint8_t* tl, in
 constexpr int PB_TILE_MIN = PB_THREADS * 4;
 
 template <typename A>
-static ProbeBuffers make_probe_buffers(const folty_graph* g, A&& get) {
+static ProbeBuffers make_probe_buffers(const folty_graph* g, cudaStream_t s, A&& get) {
     const int64_t ntri = g->ntri;
     ProbeBuffers ls;
     ls.L = get((int32_t*)nullptr, ntri + 1);
     ls.loff = get((int64_t*)nullptr, ntri + 1);
     ls.lmask = get((uint8_t*)nullptr, ntri + 1);
     ls.totals = get((int64_t*)nullptr, 2);
-    ls.max_tiles = (g->info.probes + LIVE_IDLE * ntri + PB_TILE_MIN - 1) / PB_TILE_MIN;
+    // slots are reserved in units of 2^ush, so that all of them fit the packed counter (one
+    // slot per unit up to 2^32 slots); a selection has at most one partial unit per step,
+    // and steps hold a triangle or more
+    const int64_t slots = g->info.probes + LIVE_IDLE * ntri;
+    ls.ush = 0;
+    while ((slots >> ls.ush) + ntri >= ((int64_t)1 << LS_UNIT_BITS)) ls.ush++;
+    const int64_t padded = slots + (ls.ush > 0 ? ntri << ls.ush : 0);
+    ls.max_tiles = (padded + PB_TILE_MIN - 1) / PB_TILE_MIN;
     ls.ltile = get((int64_t*)nullptr, ls.max_tiles + 2);
-    ls.nw = (ntri + LS_BLOCK - 1) / LS_BLOCK * (LS_THREADS / 32);  // the selection's warps
-    ls.wcnt = get((int32_t*)nullptr, ls.nw + 1);
-    ls.wcost = get((int64_t*)nullptr, ls.nw + 1);
+    ls.ctl = get((unsigned long long*)nullptr, 2);
+    FOLTY_CUDA(cudaMemsetAsync(ls.ctl, 0, 2 * sizeof(unsigned long long), s));
     return ls;
 }
 
 ProbeBuffers probe_buffers(folty_graph* g, cudaStream_t s) {
-    return make_probe_buffers(g, [&](auto* tag, int64_t n) {
+    return make_probe_buffers(g, s, [&](auto* tag, int64_t n) {
         return graph_alloc<std::remove_pointer_t<decltype(tag)>>(g, n, s);
     });
 }
 
+unsigned long long* prof_counter(folty_graph* g, cudaStream_t s) {
+    if (!profiling_on()) return nullptr;
+    unsigned long long* p = g->prof_bytes + (g->prof_next++ % PROF_SLOTS);
+    FOLTY_CUDA(cudaMemsetAsync(p, 0, sizeof(unsigned long long), s));
+    return p;
+}
+
 // Selects the roles kept for delta (or the window in qp) into ls. prof_sel (may be null)
 // receives the selection's model bytes beyond its one byte per triangle.
-static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& ls, int* err,
+static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& ls,
                            unsigned long long* prof_sel, const int64_t* qp, cudaStream_t s) {
-    (void)err;  // no waits: the selection cannot run out of time
     StageSpan span(ST_SELECT, s, g->ntri, prof_sel);
     const uint8_t* tl = g->tlive + (int64_t)dir * g->tlive_stride;
     if (g->ts32) launch_select_t<uint32_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
@@ -687,11 +653,11 @@ static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBu
 
 static ProbeBuffers select_live(folty_graph* g, int64_t delta, int dir, Scratch& sc, cudaStream_t s,
                                 unsigned long long* prof_sel) {
-    const ProbeBuffers ls = make_probe_buffers(g, [&](auto* tag, int64_t n) {
+    const ProbeBuffers ls = make_probe_buffers(g, s, [&](auto* tag, int64_t n) {
         return sc.get<std::remove_pointer_t<decltype(tag)>>(n);
     });
     ensure_liveness(g, dir, s);
-    enqueue_select(g, delta, dir, ls, sc.err(), prof_sel, nullptr, s);
+    enqueue_select(g, delta, dir, ls, prof_sel, nullptr, s);
     return ls;
 }
 
@@ -707,14 +673,8 @@ void launch_probe_live(folty_graph* g, int64_t delta, int dir, int mode, int32_t
     // model bytes counted on the device: the selection reads one liveness byte per
     // triangle, and per kept one its record and run ends, and writes 13 B; the probes'
     // bytes per staged triangle and kept role are summed by the probe kernel
-    unsigned long long* prof_sel = nullptr;
-    unsigned long long* prof = nullptr;
-    if (profiling_on()) {
-        prof_sel = g->prof_bytes + (g->prof_next++ % PROF_SLOTS);
-        prof = g->prof_bytes + (g->prof_next++ % PROF_SLOTS);
-        FOLTY_CUDA(cudaMemsetAsync(prof_sel, 0, sizeof(unsigned long long), s));
-        FOLTY_CUDA(cudaMemsetAsync(prof, 0, sizeof(unsigned long long), s));
-    }
+    unsigned long long* prof_sel = prof_counter(g, s);
+    unsigned long long* prof = prof_counter(g, s);
     const ProbeBuffers ls = select_live(g, delta, dir, sc, s, prof_sel);
     StageSpan span(ST_PROBE, s, 0, prof);
     LiveArgs la{g->tri, g->seg, ls.L, ls.loff, ls.lmask, ls.ltile, ls.totals + 1, cnt, bins, (uint32_t*)bins16,
@@ -730,11 +690,13 @@ void launch_probe_live(folty_graph* g, int64_t delta, int dir, int mode, int32_t
 }
 
 void enqueue_probe_pass(folty_graph* g, const int64_t* qp, int dir, const ProbeBuffers& pb, int32_t* cnt,
-                        uint16_t* cnt16, cudaStream_t s) {
+                        uint16_t* cnt16, uint32_t* touched, cudaStream_t s) {
     if (g->ntri == 0 || g->info.probes == 0) return;
-    enqueue_select(g, 0, dir, pb, g->dev_err, nullptr, qp, s);
+    enqueue_select(g, 0, dir, pb, prof_counter(g, s), qp, s);
+    unsigned long long* prof = prof_counter(g, s);
+    StageSpan span(ST_PROBE, s, 0, prof);
     LiveArgs la{g->tri, g->seg, pb.L, pb.loff, pb.lmask, pb.ltile, pb.totals + 1, cnt, nullptr, (uint32_t*)cnt16,
-                g->m_kept, 0, 0, nullptr, nullptr, qp};
+                g->m_kept, 0, 0, prof, nullptr, qp, touched};
     if (g->ts32) launch_live_t<uint32_t, 0>(g, dir, la, 0u, nullptr, s);
     else launch_live_t<int64_t, 0>(g, dir, la, 0, nullptr, s);
 }

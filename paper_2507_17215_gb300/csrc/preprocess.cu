@@ -500,7 +500,8 @@ __global__ void k_fill_adj(const int32_t* __restrict__ ea, const int32_t* __rest
                            const int32_t* __restrict__ rowptr, const int32_t* __restrict__ deg_lo,
                            const int32_t* __restrict__ hi_start, const int32_t* __restrict__ lo_start,
                            const uint32_t* __restrict__ by_b, int32_t* __restrict__ adj,
-                           int32_t* __restrict__ adj_eid, int32_t* __restrict__ adj_src) {
+                           int32_t* __restrict__ adj_eid, int32_t* __restrict__ adj_src,
+                           int32_t* __restrict__ binv) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < S;
          j += (int64_t)gridDim.x * blockDim.x) {
         // upper part: static edges are sorted by (a, b)
@@ -512,6 +513,7 @@ __global__ void k_fill_adj(const int32_t* __restrict__ ea, const int32_t* __rest
         adj_src[p] = a;
         // lower part: by_b lists static edges by (b, a)
         int32_t s2 = (int32_t)by_b[j];
+        binv[s2] = (int32_t)j;
         int32_t b = eb[s2];
         int64_t q = (int64_t)rowptr[b] + ((int32_t)j - lo_start[b]);
         adj[q] = ea[s2];
@@ -2894,6 +2896,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         sort_check(g, s);
     }
     g->by_b = graph_alloc<int32_t>(g, S, s);
+    g->binv = graph_alloc<int32_t>(g, S, s);
     if (S > 0) FOLTY_CUDA(cudaMemcpyAsync(g->by_b, by_b, sizeof(int32_t) * (size_t)S, cudaMemcpyDeviceToDevice, s));
     int32_t* runs = sc.get<int32_t>(4 * ((int64_t)n + 1));  // hi_first, hi_last, lo_first, lo_last
     int32_t* hi_first = runs;
@@ -2917,7 +2920,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     int32_t* adj_src = sc.get<int32_t>(n2);
     if (S > 0)
         FOLTY_LAUNCH(k_fill_adj, grid_for(S, T), T, 0, s, g->ea, g->eb, S, rowptr, deg_lo, hi_first, lo_first,
-                     by_b, adj, adj_eid, adj_src);
+                     by_b, adj, adj_eid, adj_src, g->binv);
 
     // ---------------- A3: peeling
     int* peel_ctl = nullptr;

@@ -69,7 +69,6 @@ struct ThresholdArgs {
     const int32_t* perm;  // with cert_in: certificate flag of input edge perm[i]
     int32_t* cert_in;     // [m] or null
     const uint16_t* cnt16;  // 16-bit counts instead of cnt (batched queries), or null
-    const int64_t* qp;      // may be null: a device block whose slots 2, 3 hold num, den
 };
 
 // Certificate test of Definition 1.1 with rho = num / den, exact in int64.
@@ -92,7 +91,7 @@ __global__ void __launch_bounds__(TH_THREADS) k_threshold(ThresholdArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t num = a.qp ? a.qp[2] : a.num, den = a.qp ? a.qp[3] : a.den;
+    const int64_t num = a.num, den = a.den;
     unsigned long long my_cert = 0;
     for (int64_t b0 = gw * 32 * TH_BATCH; b0 < a.mk; b0 += nw * 32 * TH_BATCH) {
         const int32_t* sd = a.sd + b0;
@@ -166,6 +165,213 @@ static void launch_threshold(const ThresholdArgs& a, unsigned grid, cudaStream_t
     if (a.universe == FOLTY_U_HEAD) launch_threshold_u<FOLTY_U_HEAD>(a, cert, grid, s);
     else if (a.universe == FOLTY_U_TAIL) launch_threshold_u<FOLTY_U_TAIL>(a, cert, grid, s);
     else launch_threshold_u<FOLTY_U_COMMON>(a, cert, grid, s);
+}
+
+// The same test for a plain query (pairs and totals only), over the edges the probes hit.
+//
+// The probe pass marks the 32-edge groups of the store that received a hit, and the counts
+// of every other group are zero: a block takes `words` words of that bit array, lists
+// their marked groups and deals them to its warps, TH_HITS groups in flight per warp. The
+// counters, the group bits and the pair bits live with the graph's query plans and are zero
+// between queries: the pass clears the counts and bits it has read, so a query neither
+// clears nor reads a counter per temporal edge. An edge's count certifies or not together
+// with the pair's largest one (all edges of a directed pair share the universe), so only
+// runs with a certificate add to their pair, and the pair's bit goes into the output's
+// order: bit s for ea -> eb of static edge s, bit 32 wa + binv[s] for eb -> ea (binv: the
+// edge's place in (b, a) order).
+//
+// On the paper-scale graph (70M edges) the dense pass read 420 MB of keys and counts (94
+// us) after a memset of 140 MB of counters (29 us); this one takes 7 us. On 20M edges 41 ->
+// 6 us. Blocks of few words while that gives every SM blocks, so that a small graph, all of
+// whose groups may be hit, still uses the chip (100,000 edges: 24 -> 6 us).
+struct HitArgs {
+    uint16_t* cnt16;  // 16-bit counts, or
+    int32_t* cnt;     // 32-bit ones
+    uint32_t* touched;  // bit g: a sorted edge of [32 g, 32 g + 32) was hit
+    int64_t nwords;
+    int words;  // words per block, at most HIT_WORDS
+    int64_t mk;
+    const int32_t* sd;
+    const int32_t* ea;
+    const int32_t* eb;
+    const int32_t* deg;
+    const int32_t* common;
+    const int32_t* binv;
+    const int64_t* qp;  // slots 2, 3: num, den
+    int32_t* seg_max;
+    int32_t* seg_ncert;
+    uint32_t* pbits;
+    int64_t wa;
+    unsigned long long* n_cert;
+    unsigned long long* ctl;  // words [0, nctl) of the output pass's look-back, cleared here
+    int64_t nctl;
+    unsigned long long* prof;  // may be null: model bytes
+};
+
+constexpr int HIT_WORDS = 64;
+constexpr int TH_HITS = 4;
+
+template <int UNI, int QUANT>
+__global__ void __launch_bounds__(TH_THREADS) k_threshold_hits(const HitArgs a) {
+    __shared__ uint16_t groups[HIT_WORDS * 32];
+    __shared__ int n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) n = 0;
+    for (int64_t i = blockIdx.x * (int64_t)TH_THREADS + threadIdx.x; i < a.nctl; i += (int64_t)gridDim.x * TH_THREADS)
+        a.ctl[i] = 0;
+    __syncthreads();
+    const int64_t w0 = (int64_t)blockIdx.x * a.words;
+    if ((int)threadIdx.x < a.words && w0 + threadIdx.x < a.nwords) {
+        uint32_t word = a.touched[w0 + threadIdx.x];
+        if (word) {
+            a.touched[w0 + threadIdx.x] = 0;
+            int at = atomicAdd(&n, __popc(word));
+            while (word) {
+                groups[at++] = (uint16_t)(threadIdx.x * 32 + __ffs(word) - 1);
+                word &= word - 1;
+            }
+        }
+    }
+    __syncthreads();
+    const int64_t num = a.qp[2], den = a.qp[3];
+    unsigned long long my_cert = 0;
+    for (int i0 = warp * TH_HITS; i0 < n; i0 += (TH_THREADS / 32) * TH_HITS) {
+        int64_t e[TH_HITS];
+        int32_t kb[TH_HITS], cb[TH_HITS], ub[TH_HITS];
+#pragma unroll
+        for (int k = 0; k < TH_HITS; k++) {
+            e[k] = i0 + k < n ? ((w0 << 5) + groups[i0 + k]) * 32 + lane : a.mk;
+            const bool in = e[k] < a.mk;
+            kb[k] = in ? a.sd[e[k]] : -1;
+            cb[k] = in ? (a.cnt16 ? (int32_t)a.cnt16[e[k]] : a.cnt[e[k]]) : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < TH_HITS; k++) {
+            ub[k] = 0;
+            if (cb[k] >= 1) {
+                if (a.cnt16) a.cnt16[e[k]] = 0;
+                else a.cnt[e[k]] = 0;
+            }
+            if (QUANT != FOLTY_Q_EXISTS && cb[k] >= 1) {
+                const int32_t s = kb[k] >> 1;
+                if (UNI == FOLTY_U_COMMON) ub[k] = a.common[s];
+                else ub[k] = ((UNI == FOLTY_U_HEAD) != (bool)(kb[k] & 1)) ? a.ea[s] : a.eb[s];
+            }
+        }
+        if (QUANT != FOLTY_Q_EXISTS && UNI != FOLTY_U_COMMON) {
+#pragma unroll
+            for (int k = 0; k < TH_HITS; k++)
+                if (cb[k] >= 1) ub[k] = a.deg[ub[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < TH_HITS; k++) {
+            const int32_t key = kb[k], c = cb[k];
+            const bool sat = c >= 1 && (QUANT == FOLTY_Q_EXISTS || (int64_t)c * den >= num * (int64_t)ub[k]);
+            if (!__any_sync(0xffffffffu, sat)) continue;
+            const int prev = __shfl_up_sync(0xffffffffu, key, 1);
+            const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || key != prev);
+            const unsigned above = heads & ~((2u << lane) - 1u);
+            const int start = 31 - __clz(heads & ((2u << lane) - 1u));
+            const unsigned peers = (above ? (above & (0u - above)) - 1u : 0xffffffffu) & ~((1u << start) - 1u);
+            const int run_max = __reduce_max_sync(peers, c);
+            const int run_sat = __reduce_add_sync(peers, sat ? 1 : 0);
+            if (run_sat > 0 && lane == start) {
+                atomicMax(&a.seg_max[key], run_max);
+                atomicAdd(&a.seg_ncert[key], run_sat);
+                const int32_t s = key >> 1;
+                const int64_t bit = (key & 1) ? 32 * a.wa + a.binv[s] : (int64_t)s;
+                const uint32_t mask = 1u << (bit & 31);
+                if (!(a.pbits[bit >> 5] & mask)) atomicOr(&a.pbits[bit >> 5], mask);
+            }
+            my_cert += sat ? 1ull : 0ull;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) my_cert += __shfl_xor_sync(0xffffffffu, my_cert, o);
+    if (lane == 0 && my_cert) atomicAdd(a.n_cert, my_cert);
+    if (a.prof && threadIdx.x == 0) atomicAdd(a.prof, (unsigned long long)n * 32 * (a.cnt16 ? 6 : 8));
+}
+
+template <int UNI>
+static void launch_hits_u(const HitArgs& a, int quant, unsigned grid, cudaStream_t s) {
+    if (quant == FOLTY_Q_EXISTS) FOLTY_LAUNCH((k_threshold_hits<UNI, FOLTY_Q_EXISTS>), grid, TH_THREADS, 0, s, a);
+    else FOLTY_LAUNCH((k_threshold_hits<UNI, FOLTY_Q_FORALL_T>), grid, TH_THREADS, 0, s, a);
+}
+
+static void launch_hits(HitArgs a, int quant, int universe, cudaStream_t s) {
+    const int64_t per = (a.nwords + 8 * num_sms() - 1) / (8 * num_sms());  // eight blocks an SM
+    a.words = (int)std::min<int64_t>(std::max<int64_t>(per, 1), HIT_WORDS);
+    const unsigned grid = (unsigned)std::max<int64_t>((a.nwords + a.words - 1) / a.words, 1);
+    if (universe == FOLTY_U_HEAD) launch_hits_u<FOLTY_U_HEAD>(a, quant, grid, s);
+    else if (universe == FOLTY_U_TAIL) launch_hits_u<FOLTY_U_TAIL>(a, quant, grid, s);
+    else launch_hits_u<FOLTY_U_COMMON>(a, quant, grid, s);
+}
+
+// The solution pairs of a plain query from its pair bits, in the order of the bits (pairs x
+// < y by (a, b), then pairs x > y by (b, a)): tiles of SCAN_THREADS words in block start
+// order, a decoupled look-back by warp 0 while the other warps list the tile's set bits,
+// then one thread per pair. Clears the bits and the pairs' entries for the next query.
+// tot[0] = pairs x < y, tot[1] = all pairs.
+struct EmitArgs {
+    uint32_t* pbits;  // [wa + wb] words, both halves whole 16-word lines
+    int64_t wa, wt;
+    const int32_t* ea;
+    const int32_t* eb;
+    const int32_t* by_b;
+    int32_t* seg_max;
+    int32_t* seg_ncert;
+    unsigned long long* ctl;  // [0] tile counter, then the look-back; zero before
+    int* err;
+    uint64_t* key;
+    int32_t* cnt_c;
+    int32_t* nc_c;
+    int64_t* tot;
+};
+
+__global__ void __launch_bounds__(SCAN_THREADS) k_pair_emit(const EmitArgs a) {
+    __shared__ uint16_t bits[SCAN_THREADS * 32];
+    __shared__ int32_t wc[SCAN_THREADS / 32];
+    __shared__ int32_t totc;
+    __shared__ unsigned long long s_exc;
+    __shared__ int64_t s_tile;
+    if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd((unsigned int*)a.ctl, 1u);
+    __syncthreads();
+    const int64_t tile = s_tile;
+    const int64_t w = tile * SCAN_THREADS + threadIdx.x;
+    uint32_t word = w < a.wt ? a.pbits[w] : 0u;
+    const int32_t off = block_exclusive_sum<int32_t>(__popc(word), wc, &totc);
+    if (threadIdx.x < 32) {
+        volatile unsigned long long* v = a.ctl + 1;
+        const unsigned long long tc = (unsigned long long)totc;
+        if (tile == 0) {
+            if (threadIdx.x == 0) {
+                v[0] = SC_PREFIX | tc;
+                s_exc = 0;
+            }
+        } else {
+            if (threadIdx.x == 0) v[tile] = SC_AGG | tc;
+            const unsigned long long ex = warp_lookback(v, tile, tc, a.err);
+            if (threadIdx.x == 0) s_exc = ex;
+        }
+    }
+    if (word) a.pbits[w] = 0;
+    for (int at = off; word; word &= word - 1) bits[at++] = (uint16_t)(threadIdx.x * 32 + __ffs(word) - 1);
+    __syncthreads();
+    if (w == a.wa) a.tot[0] = (int64_t)s_exc + off;
+    if (tile * SCAN_THREADS + SCAN_THREADS >= a.wt && threadIdx.x == 0) a.tot[1] = (int64_t)s_exc + totc;
+    for (int i = threadIdx.x; i < totc; i += SCAN_THREADS) {
+        const int64_t bit = tile * SCAN_THREADS * 32 + bits[i];
+        const bool up = bit < 32 * a.wa;
+        const int32_t s = up ? (int32_t)bit : a.by_b[bit - 32 * a.wa];
+        const int64_t sdir = 2 * (int64_t)s + (up ? 0 : 1);
+        const uint64_t x = (uint64_t)(up ? a.ea[s] : a.eb[s]), y = (uint64_t)(up ? a.eb[s] : a.ea[s]);
+        const int64_t p = (int64_t)s_exc + i;
+        a.key[p] = (x << 32) | y;
+        a.cnt_c[p] = a.seg_max[sdir];
+        a.nc_c[p] = a.seg_ncert[sdir];
+        a.seg_max[sdir] = 0;
+        a.seg_ncert[sdir] = 0;
+    }
 }
 
 // Solution pairs come in two lists that are already sorted by (x, y): pairs x < y in
@@ -295,6 +501,32 @@ __global__ void k_pair_merge_stage(const uint64_t* __restrict__ key, const int32
     if (np > cap) return;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np;
          p += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[p];
+        const int64_t f = (p < nA) ? p + lower_bound_u64(key + nA, np - nA, k) : (p - nA) + lower_bound_u64(key, nA, k);
+        out[f] = (int32_t)(k >> 32);
+        out[np + f] = (int32_t)(k & 0xffffffffull);
+        out[2 * np + f] = cnt_c[p];
+        out[3 * np + f] = nc_c[p];
+    }
+}
+
+// The same for a plain query's lists (tot[0] = nA, tot[1] = np), with its read-back: block 0
+// writes nA, np, the certificates and the device error word to the pinned stage, and clears
+// the certificate total for the next query.
+__global__ void k_plain_output(const uint64_t* __restrict__ key, const int32_t* __restrict__ cnt_c,
+                               const int32_t* __restrict__ nc_c, const int64_t* __restrict__ tot, int64_t cap,
+                               int32_t* __restrict__ out, unsigned long long* n_cert, const int* dev_err,
+                               int64_t* __restrict__ stage, int32_t* __restrict__ stage_err) {
+    const int64_t nA = tot[0], np = tot[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        stage[0] = nA;
+        stage[1] = np;
+        stage[2] = (int64_t)*n_cert;
+        *stage_err = *dev_err;
+        *n_cert = 0;
+    }
+    if (np > cap) return;
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t k = key[p];
         const int64_t f = (p < nA) ? p + lower_bound_u64(key + nA, np - nA, k) : (p - nA) + lower_bound_u64(key, nA, k);
         out[f] = (int32_t)(k >> 32);
@@ -434,7 +666,7 @@ static PairStage pair_stage(Scratch& sc, const folty_graph* g, const folty_query
 
 // Certificate test, per-pair reduction, flags, positions, compaction (no host sync).
 static void pairs_device(folty_graph* g, const folty_query_params& q, const CountView& cnt, const PairStage& p,
-                         Scratch* sc, cudaStream_t s, const int64_t* qp = nullptr) {
+                         Scratch* sc, cudaStream_t s) {
     const int T = 256;
     const int64_t mk = g->m_kept;
     const int64_t S = g->S, n2 = 2 * S;
@@ -445,7 +677,7 @@ static void pairs_device(folty_graph* g, const folty_query_params& q, const Coun
         if (p.cert_flag) ensure_perm(g, s);  // certificates are listed by input index
         ThresholdArgs a{cnt.c32, g->sd, mk, g->ea, g->eb, g->deg, g->common, (int)q.quant, (int)q.universe,
                         (int64_t)q.rho_num, (int64_t)q.rho_den, p.seg_max, p.seg_ncert, p.n_cert,
-                        p.cert_flag ? g->perm : nullptr, p.cert_flag, cnt.c16, qp};
+                        p.cert_flag ? g->perm : nullptr, p.cert_flag, cnt.c16};
         StageSpan span(ST_THRESHOLD, s, 8 * mk);  // pair key + count per edge
         launch_threshold(a, grid_for((mk + TH_BATCH - 1) / TH_BATCH, TH_THREADS), s);
     }
@@ -650,20 +882,33 @@ static void triples_result(folty_graph* g, const uint8_t* rflag, folty_result* o
 
 // A plain query (no per-edge counts, certificates, vertex or triple outputs) replays a
 // CUDA graph captured once per graph and query shape (direction variant, quantifier,
-// universe). Its window and rho reach the kernels through a device parameter block that
-// the graph's first node copies from the graph's pinned stage, so no launch argument
-// changes between queries: a query costs one graph launch and one synchronisation
-// instead of about fifteen launches, memsets and allocations. The buffers the graphs
-// work in are allocated once and owned by the graph.
+// universe): the parameter block's copy and five kernels (selection, probes, threshold over
+// the hit groups, pairs, output). Its window and rho reach the kernels through a device
+// parameter block that the graph's first node copies from the graph's pinned stage, so no
+// launch argument changes between queries. The buffers the graphs work in are allocated
+// once and owned by the graph; counters and bits are zero between queries (each pass clears
+// what it read), and are cleared in full before the first query and after one that failed.
 constexpr int QP_SLOT = 448;  // pinned stage slots [QP_SLOT, QP_SLOT + 4): delta, delta32, num, den
 static_assert(QP_SLOT > ERR_SLOT && QP_SLOT + 4 <= HOST_STAGE, "the parameter block has its own stage slots");
 
 struct QueryPlans {
-    CountView cnt;
     int32_t* cnt32 = nullptr;
     uint16_t* cnt16 = nullptr;
+    uint32_t* touched = nullptr;  // a bit per 32 sorted edges
+    int64_t nwords = 0;
     ProbeBuffers pb{};
-    PairStage ps{};
+    int32_t* seg_max = nullptr;    // [2S], then seg_ncert [2S]
+    int32_t* seg_ncert = nullptr;
+    uint32_t* pbits = nullptr;     // [wa + wb] solution pair bits
+    int64_t wa = 0, wt = 0;
+    unsigned long long* ctl = nullptr;  // look-back of k_pair_emit
+    int64_t nctl = 0;
+    uint64_t* key = nullptr;       // [2S] the pairs
+    int32_t* cnt_c = nullptr;
+    int32_t* nc_c = nullptr;
+    int64_t* tot = nullptr;        // pairs x < y, all pairs, certificates
+    unsigned long long* n_cert = nullptr;
+    bool clean = false;            // counters and bits are zero
     int64_t* qp = nullptr;  // device parameter block [4]
     cudaStream_t cs = nullptr;  // capture stream
     cudaGraphExec_t exec[3][2][3] = {};
@@ -686,45 +931,61 @@ static QueryPlans* plans_of(folty_graph* g, cudaStream_t s) {
     if (g->plans) return g->plans;
     QueryPlans* p = new QueryPlans();
     g->plans = p;  // the buffers below are graph-owned; destroy_plans releases the rest
-    const int64_t mk = g->m_kept, n2 = 2 * (int64_t)g->S;
+    const int64_t mk = g->m_kept, S = g->S, n2 = 2 * S;
     if (g->info.max_degree < 65535) p->cnt16 = graph_alloc<uint16_t>(g, mk + 2, s);
     else p->cnt32 = graph_alloc<int32_t>(g, mk, s);
-    p->cnt = CountView{p->cnt32, p->cnt16};
+    p->nwords = (mk + 1023) / 1024;
+    p->touched = graph_alloc<uint32_t>(g, p->nwords, s);
     p->pb = probe_buffers(g, s);
-    PairStage& ps = p->ps;
-    std::memset(&ps, 0, sizeof(ps));
-    ps.seg_max = graph_alloc<int32_t>(g, 2 * n2 + 2, s);
-    ps.seg_ncert = ps.seg_max + n2 + 1;
-    ps.flag = graph_alloc<int32_t>(g, 2 * n2 + 2, s);
-    ps.pos = ps.flag + n2 + 1;
-    ps.key = graph_alloc<uint64_t>(g, n2, s);
-    ps.cnt_c = graph_alloc<int32_t>(g, 2 * n2 + 2, s);
-    ps.nc_c = ps.cnt_c + n2 + 1;
-    ps.n_cert = graph_alloc<unsigned long long>(g, 1, s);
-    ps.ctl = graph_alloc<unsigned long long>(g, (n2 + PS_TILE - 1) / PS_TILE + 1, s);
+    p->seg_max = graph_alloc<int32_t>(g, 2 * n2, s);
+    p->seg_ncert = p->seg_max + n2;
+    p->wa = (S + 31) / 32;
+    p->wt = 2 * p->wa;
+    p->pbits = graph_alloc<uint32_t>(g, p->wt, s);
+    p->nctl = (p->wt + SCAN_THREADS - 1) / SCAN_THREADS + 1;
+    p->ctl = graph_alloc<unsigned long long>(g, p->nctl, s);
+    p->key = graph_alloc<uint64_t>(g, n2, s);
+    p->cnt_c = graph_alloc<int32_t>(g, 2 * n2, s);
+    p->nc_c = p->cnt_c + n2;
+    p->tot = graph_alloc<int64_t>(g, 3, s);
+    p->n_cert = (unsigned long long*)(p->tot + 2);
     p->qp = graph_alloc<int64_t>(g, 4, s);
     FOLTY_CUDA(cudaStreamCreateWithFlags(&p->cs, cudaStreamNonBlocking));
     return p;
 }
 
+// Everything a plain query expects to be zero.
+static void clear_plan(folty_graph* g, QueryPlans* p, cudaStream_t s) {
+    const size_t mk = (size_t)g->m_kept, n2 = 2 * (size_t)g->S;
+    if (p->cnt16) FOLTY_CUDA(cudaMemsetAsync(p->cnt16, 0, sizeof(uint16_t) * (mk + 2), s));
+    if (p->cnt32) FOLTY_CUDA(cudaMemsetAsync(p->cnt32, 0, sizeof(int32_t) * mk, s));
+    FOLTY_CUDA(cudaMemsetAsync(p->touched, 0, sizeof(uint32_t) * (size_t)p->nwords, s));
+    FOLTY_CUDA(cudaMemsetAsync(p->seg_max, 0, sizeof(int32_t) * 2 * n2, s));
+    FOLTY_CUDA(cudaMemsetAsync(p->pbits, 0, sizeof(uint32_t) * (size_t)p->wt, s));
+    FOLTY_CUDA(cudaMemsetAsync(p->tot, 0, sizeof(int64_t) * 3, s));
+    FOLTY_CUDA(cudaMemsetAsync(p->pb.ctl, 0, sizeof(unsigned long long) * 2, s));
+}
+
 // The launch sequence of one plain query of shape (dir, quant, universe) on stream cs.
 static void enqueue_plain_query(folty_graph* g, QueryPlans* p, int dir, int quant, int universe, cudaStream_t cs) {
-    const int64_t mk = g->m_kept, S = g->S;
     FOLTY_CUDA(cudaMemcpyAsync(p->qp, g->host_stage + QP_SLOT, 4 * sizeof(int64_t), cudaMemcpyHostToDevice, cs));
-    if (mk > 0 && p->cnt16) FOLTY_CUDA(cudaMemsetAsync(p->cnt16, 0, sizeof(uint16_t) * (size_t)(mk + 2), cs));
-    if (mk > 0 && p->cnt32) FOLTY_CUDA(cudaMemsetAsync(p->cnt32, 0, sizeof(int32_t) * (size_t)mk, cs));
-    enqueue_probe_pass(g, p->qp, dir, p->pb, p->cnt32, p->cnt16, cs);
-    folty_query_params q{};
-    q.dir = (uint8_t)dir;
-    q.quant = (uint8_t)quant;
-    q.universe = (uint8_t)universe;
-    q.rho_den = 1;
-    pairs_device(g, q, p->cnt, p->ps, nullptr, cs, p->qp);
-    FOLTY_LAUNCH(k_pair_merge_stage, grid_for(PAIR_STAGE, 256, 1), 256, 0, cs, p->ps.key, p->ps.cnt_c, p->ps.nc_c,
-                 p->ps.pos, S, PAIR_STAGE, g->pair_stage);
-    const void* ptrs[3] = {p->ps.pos + S, p->ps.pos + 2 * S, p->ps.n_cert};
-    const int sizes[3] = {4, 4, 8};
-    enqueue_read_back(g, ptrs, sizes, 3, cs);
+    enqueue_probe_pass(g, p->qp, dir, p->pb, p->cnt32, p->cnt16, p->touched, cs);
+    {
+        // the group bits; per marked group (counted on the device) its keys and counts
+        unsigned long long* prof = prof_counter(g, cs);
+        StageSpan span(ST_THRESHOLD, cs, 4 * p->nwords, prof);
+        const HitArgs h{p->cnt16,  p->cnt32,    p->touched, p->nwords, 1,         g->m_kept, g->sd,  g->ea,   g->eb, g->deg,
+                        g->common, g->binv,     p->qp,      p->seg_max, p->seg_ncert, p->pbits, p->wa, p->n_cert, p->ctl,
+                        p->nctl,   prof};
+        launch_hits(h, quant, universe, cs);
+    }
+    if (p->wt > 0) {
+        const EmitArgs e{p->pbits, p->wa,     p->wt,  g->ea,     g->eb,    g->by_b, p->seg_max,
+                         p->seg_ncert, p->ctl, g->dev_err, p->key, p->cnt_c, p->nc_c, p->tot};
+        FOLTY_LAUNCH(k_pair_emit, (unsigned)(p->nctl - 1), SCAN_THREADS, 0, cs, e);
+    }
+    FOLTY_LAUNCH(k_plain_output, grid_for(PAIR_STAGE, 256, 1), 256, 0, cs, p->key, p->cnt_c, p->nc_c, p->tot, PAIR_STAGE,
+                 g->pair_stage, p->n_cert, g->dev_err, g->stage_dev, (int32_t*)(g->stage_dev + ERR_SLOT));
 }
 
 static cudaGraphExec_t plan_exec(folty_graph* g, QueryPlans* p, int dir, int quant, int universe) {
@@ -770,22 +1031,30 @@ static bool plans_enabled() {
 
 static bool run_query_plan(folty_graph* g, const folty_query_params& q, folty_result* out, cudaStream_t s) {
     if (q.want_edge_counts || q.want_certificates || q.outer || q.want_triples) return false;
-    if (profiling_on() || !plans_enabled()) return false;  // stage events are recorded by the launch path
     tune_probe(g, q.delta, q.dir, s);  // the captured sequence takes the tuned probe shape
     ensure_liveness(g, q.dir, s);      // the replay on s reads the variant's liveness row
     QueryPlans* p = plans_of(g, s);
-    const cudaGraphExec_t e = plan_exec(g, p, q.dir, q.quant, q.universe);
+    // stage events are recorded by the launch path
+    const bool replay = !profiling_on() && plans_enabled();
+    const cudaGraphExec_t e = replay ? plan_exec(g, p, q.dir, q.quant, q.universe) : nullptr;
     int64_t* hp = g->host_stage + QP_SLOT;
     hp[0] = q.delta;
     hp[1] = q.delta >= 0xfffffffell ? 0xfffffffell - 1 : q.delta;  // gaps of the 32-bit store stay below 2^32 - 1
     hp[2] = q.rho_num;
     hp[3] = q.rho_den;
     g->stage_busy = 1;
-    FOLTY_CUDA(cudaGraphLaunch(e, s));
-    g_launches.fetch_add((uint64_t)p->kernels[q.dir][q.quant][q.universe], std::memory_order_relaxed);
+    if (!p->clean) clear_plan(g, p, s);
+    p->clean = false;
+    if (replay) {
+        FOLTY_CUDA(cudaGraphLaunch(e, s));
+        g_launches.fetch_add((uint64_t)p->kernels[q.dir][q.quant][q.universe], std::memory_order_relaxed);
+    } else {
+        enqueue_plain_query(g, p, q.dir, q.quant, q.universe, s);
+    }
     FOLTY_CUDA(cudaStreamSynchronize(s));
     int64_t rb[3];
     collect_read_back(g, 3, rb, s);
+    p->clean = true;
     const int64_t nA = rb[0], np = rb[1], nc = rb[2];
     fill_result_host(out, np, g->m, false, 0, false, nc, false);
     out->n_cert_edges = nc;
@@ -795,7 +1064,7 @@ static bool run_query_plan(folty_graph* g, const folty_query_params& q, folty_re
         try {
             Scratch sc(g->alloc, s, g->dev_err);
             int32_t* packed = sc.get<int32_t>(4 * np);
-            FOLTY_LAUNCH(k_pair_merge, grid_for(np, 256), 256, 0, s, p->ps.key, p->ps.cnt_c, p->ps.nc_c, nA, np, packed);
+            FOLTY_LAUNCH(k_pair_merge, grid_for(np, 256), 256, 0, s, p->key, p->cnt_c, p->nc_c, nA, np, packed);
             FOLTY_CUDA(cudaMemcpyAsync(out->u, packed, sizeof(int32_t) * 4 * (size_t)np, cudaMemcpyDeviceToHost, s));
             FOLTY_CUDA(cudaStreamSynchronize(s));
         } catch (...) {

@@ -65,3 +65,34 @@ def test_pair_table_sizes(F, pairs, device):
     g = _distinct_pairs_graph(pairs, 30_000, pairs)
     info = _check(F, g, [W.Query(300, 1, 4, W.Q_FORALL_T, W.DIR_EITHER, W.U_COMMON, True)], device)
     assert info["static_edges"] == pairs
+
+
+def _plain(deltas):
+    return [W.Query(d, num, 4, quant, dr, uni, False) for d in deltas
+            for num, quant, dr, uni in ((1, W.Q_FORALL_T, W.DIR_OUT, W.U_HEAD), (1, W.Q_EXISTS, W.DIR_EITHER, W.U_TAIL),
+                                        (3, W.Q_FORALL_T, W.DIR_IN, W.U_COMMON))]
+
+
+# one group of 32 edges, one word of 32 groups, and their edges; a plain query leaves its
+# counters and bits zero for the next one, so every query runs twice, in both orders
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 1023, 1024, 1025, 33_000])
+def test_plain_queries_leave_their_workspace_clear(F, m):
+    g = W.random_small_graph(np.random.default_rng(m), 12 if m < 2000 else 90, m, 500)
+    qs = _plain((0, 20, 500))
+    _check(F, g, qs + qs[::-1])
+
+
+def test_plain_query_with_32_bit_counters_and_hit_groups_everywhere(F):
+    """A hub of degree past 16 bits (32-bit counters) in a graph whose hits spread over more
+    32-edge groups than one block lists."""
+    rng = np.random.default_rng(3)
+    n, extra = 66_000, 200_000
+    leaves = np.arange(1, n, dtype=np.int32)
+    a = rng.integers(1, n, extra).astype(np.int32)
+    b = np.minimum(a + rng.integers(1, 4, extra), n - 1).astype(np.int32)
+    src = np.concatenate([np.zeros(2 * (n - 1), np.int32), a])
+    dst = np.concatenate([leaves, leaves, b])
+    t = rng.integers(0, 1000, src.shape[0]).astype(np.int64)
+    qs = _plain((100, 900))
+    info = _check(F, W.TemporalGraph(n, src, dst, t), qs + qs[:3])
+    assert info["max_degree"] >= 65_535
