@@ -398,6 +398,7 @@ void ensure_perm(folty_graph* g, cudaStream_t s);
 // Device buffers of one query's probe stage (kept triangles, probe tiles, look-back
 // control).
 struct ProbeBuffers {
+    int32_t* cand;  // triangles whose liveness byte admits the window
     int32_t* L;
     int64_t* loff;
     uint8_t* lmask;

@@ -113,11 +113,11 @@ __device__ __forceinline__ bool bucket_live(uint8_t b, int64_t delta) {
     return b != DMIN_NEVER && (b == 0 || delta >= ((int64_t)1 << (b - 1)));
 }
 
-// Role mask (stored role order: bit 2e + d = direction d of stored edge e) and kept
-// probes of triangle tr at window delta for direction variant DIR.
+// Role mask (stored role order: bit 2e + d = direction d of stored edge e) and probe slots
+// of the kept roles of triangle tr at window delta for direction variant DIR.
 template <typename TS, int DIR>
 __device__ __forceinline__ int kept_roles_of(const int4 tr, const RunEnds<TS>* __restrict__ ends, int64_t delta,
-                                             int64_t& probes) {
+                                             int64_t& slots) {
     FrameRuns<TS> fr;
     frame_runs<TS>(tr, ends, fr);
     int m = 0;
@@ -126,110 +126,119 @@ __device__ __forceinline__ int kept_roles_of(const int4 tr, const RunEnds<TS>* _
     for (int r = 0; r < 6; r++) {
         if (bucket_live(frame_bucket<DIR, TS>(fr, r), delta)) {  // never for an empty run
             m |= 1 << (2 * fr.oe[r >> 1] + (r & 1));
-            c += fr.n[r];
+            int32_t n = fr.n[r];
+            if (n >= ROLE_LONG) {
+                int s2, s3;
+                role_segments(7, r >> 1, r & 1, DIR, s2, s3);
+                const int32_t n2 = DIR == FOLTY_DIR_EITHER ? fr.n[s2] + fr.n[s2 + 1] : fr.n[s2];
+                const int32_t n3 = DIR == FOLTY_DIR_EITHER ? fr.n[s3] + fr.n[s3 + 1] : fr.n[s3];
+                n = long_role_plan(n, n2, n3).slots;
+            }
+            c += n;
         }
     }
-    probes = c;
+    slots = c;
     return m;
 }
 
 // Kept roles of every triangle for one query: kept triangle j = L[j] with its role mask
-// lmask[j] and its first probe slot loff[j] (the kept triangles' costs = kept probes +
-// LIVE_IDLE idle slots, laid out one after another); totals[0] = kept triangles, totals[1]
-// = slots, loff[totals[0]] = totals[1]; and the probe tiles' map: ltile[b] = kept triangle
-// holding slot min(b * ptile, slots - 1) for b <= the number of probe tiles (each kept
-// triangle writes the tile starts inside its slots).
+// lmask[j] and its first probe slot loff[j] (the kept triangles' costs = the kept roles'
+// slots (probe.cuh) + LIVE_IDLE idle ones, laid out one after another); totals[0] = kept triangles, totals[1]
+// = slots, loff[totals[0]] = totals[1]; and the map of the probe groups (PB_GROUP slots):
+// ltile[b] = kept triangle holding slot min(b * ptile, slots - 1) for b <= the number of
+// groups (each kept triangle writes the group starts inside its slots).
 //
-// One pass. A warp takes 32 * ITEMS consecutive triangles (a lane ITEMS of them, read as
-// 16-byte chunks of their liveness bytes: the smallest bucket of each triangle's roles for
-// this direction variant). Only the triangles whose byte admits delta read their record
-// and run ends: they are few, but cluster, so a warp deals its candidates over its lanes,
-// LS_EACH per lane and step, orders their costs by a warp scan and reserves the step's
-// list entries and slots together with one 64-bit addition (the counter ls_count_shift
-// packs). The list is therefore in the order of the reservations, not of the triangles:
-// the probes only add to counters, so no result depends on it. The last block to finish
-// writes the totals and clears the counter for the next selection.
+// Two passes. k_live_candidates streams the row of liveness bytes (the smallest bucket of
+// each triangle's roles for this direction variant; a thread 32 of them per step, the next
+// step's 16-byte loads in flight) and lists the triangles whose byte admits delta, one
+// addition per block and step. They are few, but cluster; k_live_select takes them from the
+// list, one thread each, so the work is even whatever their places: it reads their records
+// and run ends, orders the costs of a warp's 32 by a scan and reserves their entries and
+// slots together with one 64-bit addition (kept triangles << LS_UNIT_BITS | slots). The list
+// is therefore in the order of the reservations, not of the triangles: the probes only add
+// to counters, so no result depends on it. The last block to finish writes the totals and
+// clears the counters for the next selection.
 //
 // It replaced a counting pass, a one-block scan of the warps' sums and a writing pass that
-// read every kept triangle again: 122 -> 29 us for 76M triangles of which 42K are kept
-// (the one-block scan alone took 71), 75 -> 9 us for 68K triangles, where warps of 2048
-// triangles left all but a few SMs idle. 64 triangles a lane (four 16-byte loads in flight)
-// from LS_LARGE triangles on, where the pass streams the bytes; below, 16 a lane, for more
-// warps with fewer candidates each.
+// read every kept triangle again: 122 us for 76M triangles of which 42K are kept, 75 us for
+// 68K triangles (warps of 2048 triangles left all but a few SMs idle); now 28 and 9 us. One
+// kernel whose warps or blocks worked off their own candidates took 50 to 75 us at 76M:
+// thousands of neighbouring triangles may all be candidates.
 constexpr int LS_THREADS = 256;
-constexpr int LS_EACH = 4;                        // candidates per lane and step
-constexpr int64_t LS_LARGE = int64_t(1) << 24;
-constexpr int LS_UNIT_BITS = 33;                  // packed counter: kept triangles << 33 | slots in units
+constexpr int LS_ITEMS = 32;
+constexpr int LS_PER_SM = 8;      // blocks per SM of both passes
+constexpr int LS_UNIT_BITS = 33;  // packed counter: kept triangles << 33 | slots in units
 
-// Bit i of the result: triangle t0 + i (i < ITEMS) is kept at delta (rows are padded
+// Bit i of the result: byte i of the ITEMS liveness bytes in w admits delta (rows are padded
 // with DMIN_NEVER to whole 16-byte chunks). A byte b admits delta exactly when
 // b <= B = bit length of delta (b = 0 always, b >= 1 when delta >= 2^(b-1); DMIN_NEVER
 // never, as B <= 63): four bytes at a time, (0x80 + B) - (b & 0x7f) keeps bit 7 set
 // exactly for b <= B (bytes never borrow from one another, and 255 & 0x7f = 127 > B), and
-// one multiplication gathers the four bit-7s.
+// one multiplication gathers the four bit-7s. bias = 0x80 + B in every byte.
 template <int ITEMS>
-__device__ __forceinline__ uint64_t live_mask(const uint8_t* __restrict__ tlive, int64_t t0, int64_t ntri,
-                                              int64_t delta) {
-    const uint32_t B = delta > 0 ? (uint32_t)(64 - __clzll((unsigned long long)delta)) : 0u;
-    const uint32_t bias = 0x80808080u | (B * 0x01010101u);
-    uint64_t lm = 0;
+__device__ __forceinline__ uint32_t live_mask(const uint4 (&w)[ITEMS / 16], uint32_t bias) {
+    uint32_t lm = 0;
 #pragma unroll
     for (int h = 0; h < ITEMS / 16; h++) {
-        uint4 w = make_uint4(~0u, ~0u, ~0u, ~0u);
-        if (t0 + 16 * h < ntri) w = __ldcs(reinterpret_cast<const uint4*>(tlive + t0 + 16 * h));
-        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+        const uint32_t ws[4] = {w[h].x, w[h].y, w[h].z, w[h].w};
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             const uint32_t hit = (bias - (ws[q] & 0x7f7f7f7fu)) & 0x80808080u;
             const uint32_t nib = ((hit >> 7) * 0x10204080u) >> 28;  // bit j = byte j admits delta
-            lm |= (uint64_t)nib << (16 * h + 4 * q);
+            lm |= nib << (16 * h + 4 * q);
         }
     }
     return lm;
 }
 
-// The warp's candidates: this lane's mask lm, the number of candidates of the lanes
-// before it (pre) and of the warp (returned).
-__device__ __forceinline__ int warp_candidates(uint64_t lm, int& pre) {
-    const int lane = threadIdx.x & 31;
-    const int own = __popcll(lm);
-    int inc = own;
+template <int ITEMS>
+__device__ __forceinline__ void live_load(const uint8_t* __restrict__ tlive, int64_t t0, int64_t ntri,
+                                          uint4 (&w)[ITEMS / 16]) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
+    for (int h = 0; h < ITEMS / 16; h++) {
+        w[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        if (t0 + 16 * h < ntri) w[h] = __ldcs(reinterpret_cast<const uint4*>(tlive + t0 + 16 * h));
     }
-    pre = inc - own;
-    return __shfl_sync(0xffffffffu, inc, 31);
 }
 
-// Position within the warp's range of candidate k (< the warp's total): the lane l with
-// pre[l] <= k < pre[l + 1], and the (k - pre[l])-th set bit of its mask. The whole warp
-// must call it.
+// The selection's counters, zero between selections.
+struct SelectCtl {
+    unsigned long long packed;  // kept triangles << LS_UNIT_BITS | slots in units
+    unsigned int cand, done;    // candidates, blocks of k_live_select done
+};
+
+// The triangles whose byte admits delta, in no particular order, into cand.
 template <int ITEMS>
-__device__ __forceinline__ int candidate_at(int k, uint64_t lm, int pre) {
-    int l = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-        const int pc = __shfl_sync(0xffffffffu, pre, l + step);
-        if (pc <= k) l += step;
+__global__ void __launch_bounds__(LS_THREADS) k_live_candidates(const uint8_t* __restrict__ tlive, int64_t ntri,
+                                                                int64_t delta, const int64_t* __restrict__ qp,
+                                                                SelectCtl* ctl, int32_t* __restrict__ cand) {
+    __shared__ int warp_tot[LS_THREADS / 32];
+    __shared__ int total;
+    __shared__ unsigned int base;
+    if (qp) delta = qp[0];  // the window from a device parameter block (replayed query plans)
+    const uint32_t bias = 0x80808080u | ((delta > 0 ? (uint32_t)(64 - __clzll((unsigned long long)delta)) : 0u) * 0x01010101u);
+    const int64_t stride = (int64_t)gridDim.x * (LS_THREADS * ITEMS);
+    int64_t t0 = ((int64_t)blockIdx.x * LS_THREADS + threadIdx.x) * ITEMS;
+    uint4 next[ITEMS / 16];
+    live_load<ITEMS>(tlive, t0, ntri, next);
+    for (int64_t b0 = (int64_t)blockIdx.x * (LS_THREADS * ITEMS); b0 < ntri; b0 += stride, t0 += stride) {
+        uint32_t lm = live_mask<ITEMS>(next, bias);
+        live_load<ITEMS>(tlive, t0 + stride, ntri, next);
+        if (!__syncthreads_or(lm != 0)) continue;
+        int at = block_exclusive_sum<int>(__popc(lm), warp_tot, &total);
+        if (threadIdx.x == 0) base = atomicAdd(&ctl->cand, (unsigned int)total);
+        __syncthreads();
+        for (at += (int)base; lm; lm &= lm - 1) cand[at++] = (int32_t)(t0 + __ffs((int)lm) - 1);
     }
-    const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)lm, l);
-    const uint32_t hi = ITEMS > 32 ? __shfl_sync(0xffffffffu, (uint32_t)(lm >> 32), l) : 0u;
-    const int n = k - __shfl_sync(0xffffffffu, pre, l);  // 0-based rank among l's candidates
-    const int plo = __popc(lo);
-    const int bit = n < plo ? __fns(lo, 0, n + 1) : 32 + __fns(hi, 0, n - plo + 1);
-    return l * ITEMS + bit;
 }
 
 struct SelectArgs {
-    const uint8_t* tlive;
     const int4* tri;
-    int64_t ntri;
+    const int32_t* cand;
     int64_t delta;
     const int64_t* qp;  // may be null: device parameter block whose slot 0 holds the window
     int ush;            // log2 of the slots per unit of the packed counter
-    unsigned long long* ctl;  // [0] packed counter, [1] blocks done; both zero before and after
+    SelectCtl* ctl;
     int32_t* L;
     int64_t* loff;
     uint8_t* lmask;
@@ -239,38 +248,23 @@ struct SelectArgs {
     unsigned long long* prof;  // may be null
 };
 
-template <typename TS, int DIR, int ITEMS>
+template <typename TS, int DIR>
 __global__ void __launch_bounds__(LS_THREADS) k_live_select(const SelectArgs a, const RunEnds<TS>* __restrict__ ends) {
     const int64_t delta = a.qp ? a.qp[0] : a.delta;
     const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * LS_THREADS + threadIdx.x) >> 5;
-    const int64_t tw = w * (32 * ITEMS);
-    const uint64_t lm = live_mask<ITEMS>(a.tlive, tw + (int64_t)lane * ITEMS, a.ntri, delta);
-    int pre;
-    const int total = warp_candidates(lm, pre);
-    for (int k0 = 0; k0 < total; k0 += 32 * LS_EACH) {
-        const int kl = k0 + lane * LS_EACH;  // this lane's candidates kl ... kl + LS_EACH - 1
-        int at[LS_EACH];
-        int4 tr[LS_EACH];
-#pragma unroll
-        for (int r = 0; r < LS_EACH; r++) {
-            at[r] = candidate_at<ITEMS>(min(kl + r, total - 1), lm, pre);
-            if (kl + r < total) tr[r] = a.tri[tw + at[r]];
+    const int64_t total = (int64_t)*(volatile unsigned int*)&a.ctl->cand;
+    const int64_t stride = (int64_t)gridDim.x * LS_THREADS;
+    for (int64_t k0 = (int64_t)blockIdx.x * LS_THREADS + (threadIdx.x & ~31); k0 < total; k0 += stride) {
+        const bool on = k0 + lane < total;
+        int32_t t = 0;
+        int m = 0;
+        int64_t v = 0;
+        if (on) {
+            t = a.cand[k0 + lane];
+            m = kept_roles_of<TS, DIR>(a.tri[t], ends, delta, v);
+            v += LIVE_IDLE;
         }
-        int m[LS_EACH];
-        int64_t v[LS_EACH], sum = 0;
-#pragma unroll
-        for (int r = 0; r < LS_EACH; r++) {
-            m[r] = 0;
-            v[r] = 0;
-            if (kl + r < total) {
-                int64_t pr;
-                m[r] = kept_roles_of<TS, DIR>(tr[r], ends, delta, pr);
-                v[r] = pr + LIVE_IDLE;
-            }
-            sum += v[r];
-        }
-        int64_t inc = sum;
+        int64_t inc = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
@@ -278,32 +272,28 @@ __global__ void __launch_bounds__(LS_THREADS) k_live_select(const SelectArgs a, 
         }
         const int64_t all = __shfl_sync(0xffffffffu, inc, 31);
         const int64_t units = (all + ((int64_t)1 << a.ush) - 1) >> a.ush;
-        const int n = min(total - k0, 32 * LS_EACH);
+        const int n = (int)min(total - k0, (int64_t)32);
         unsigned long long base = 0;
         if (lane == 0)
-            base = atomicAdd(a.ctl, ((unsigned long long)n << LS_UNIT_BITS) | (unsigned long long)units);
+            base = atomicAdd(&a.ctl->packed, ((unsigned long long)n << LS_UNIT_BITS) | (unsigned long long)units);
         base = __shfl_sync(0xffffffffu, base, 0);
-        const int64_t bc = (int64_t)(base >> LS_UNIT_BITS);
-        int64_t jp = ((int64_t)(base & ((1ull << LS_UNIT_BITS) - 1)) << a.ush) + inc - sum;
-#pragma unroll
-        for (int r = 0; r < LS_EACH; r++) {
-            if (kl + r >= total) break;
-            const int64_t jc = bc + lane * LS_EACH + r;
+        if (on) {
+            const int64_t jc = (int64_t)(base >> LS_UNIT_BITS) + lane;
+            const int64_t jp = ((int64_t)(base & ((1ull << LS_UNIT_BITS) - 1)) << a.ush) + inc - v;
             // the step's last triangle also holds the slots that round the step up to whole units
-            const int64_t end = jp + v[r] + (lane * LS_EACH + r == n - 1 ? (units << a.ush) - all : 0);
-            a.L[jc] = (int32_t)(tw + at[r]);
+            const int64_t end = jp + v + (lane == n - 1 ? (units << a.ush) - all : 0);
+            a.L[jc] = t;
             a.loff[jc] = jp;
-            a.lmask[jc] = (uint8_t)m[r];
+            a.lmask[jc] = (uint8_t)m;
             for (int64_t b = (jp + a.ptile - 1) / a.ptile; b * a.ptile < end && b <= a.max_tiles; b++) a.ltile[b] = jc;
-            jp = end;
         }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(a.ctl + 1, 1ull) == gridDim.x - 1) {
+        if (atomicAdd(&a.ctl->done, 1u) == gridDim.x - 1) {
             __threadfence();
-            const unsigned long long c = *(volatile unsigned long long*)a.ctl;
+            const unsigned long long c = *(volatile unsigned long long*)&a.ctl->packed;
             const int64_t nl = (int64_t)(c >> LS_UNIT_BITS);
             const int64_t P = (int64_t)(c & ((1ull << LS_UNIT_BITS) - 1)) << a.ush;
             a.totals[0] = nl;
@@ -311,30 +301,31 @@ __global__ void __launch_bounds__(LS_THREADS) k_live_select(const SelectArgs a, 
             a.loff[nl] = P;
             const int64_t tiles = (P + a.ptile - 1) / a.ptile;
             if (P > 0 && tiles <= a.max_tiles) a.ltile[tiles] = nl - 1;
-            if (a.prof) atomicAdd(a.prof, (unsigned long long)((16 + 3 * sizeof(RunEnds<TS>) + 13) * nl));
-            a.ctl[0] = 0;
-            a.ctl[1] = 0;
+            if (a.prof) atomicAdd(a.prof, (unsigned long long)((16 + 3 * sizeof(RunEnds<TS>) + 13 + 8) * nl));
+            *a.ctl = SelectCtl{0, 0, 0};
         }
     }
 }
 
 // Model bytes of a staged triangle's kept roles (its first slot lies in this tile):
-// staging 61 B, and per role w sigma1 + w min(sigma2, sigma1 ceil(log2(sigma2 + 1))) + the
-// same for L3 + 8 sigma1, w = bytes per timestamp.
+// staging 61 B, and per role, driven by a list of nd entries: w nd + w min(n, nd
+// ceil(log2(n + 1))) for each of the two other lists of n entries, w = bytes per timestamp.
 template <typename TS, int DIR>
 __device__ __forceinline__ unsigned long long kept_role_bytes(const int32_t* off, int m, uint64_t desc) {
     const int64_t w = sizeof(TS);
     unsigned long long b = 61;
     for (int r = 0; r < 6; r++) {
         if (!((m >> r) & 1)) continue;
-        const int64_t s1 = off[3 * (r >> 1) + (r & 1) + 1] - off[3 * (r >> 1) + (r & 1)];
         const int code = (int)((desc >> (6 * r)) & 63);
-        const int c2 = code & 7, c3 = code >> 3;
+        const int o1 = 3 * (r >> 1) + (r & 1), c2 = code & 7, c3 = code >> 3;
         const int o2 = 3 * (c2 >> 1) + (c2 & 1), o3 = 3 * (c3 >> 1) + (c3 & 1);
-        const int64_t s2 = DIR == FOLTY_DIR_EITHER ? off[o2 + 2] - off[o2] : off[o2 + 1] - off[o2];
-        const int64_t s3 = DIR == FOLTY_DIR_EITHER ? off[o3 + 2] - off[o3] : off[o3 + 1] - off[o3];
-        const int64_t l2 = 64 - __clzll((unsigned long long)s2), l3 = 64 - __clzll((unsigned long long)s3);
-        b += (unsigned long long)(w * s1 + w * min(s2, s1 * l2) + w * min(s3, s1 * l3) + 8 * s1);
+        constexpr int W = DIR == FOLTY_DIR_EITHER ? 2 : 1;
+        const int64_t n[3] = {off[o1 + 1] - off[o1], off[o2 + W] - off[o2], off[o3 + W] - off[o3]};
+        const int d = staged_role_plan<DIR>(off, r, code).drv - 1;
+        b += (unsigned long long)(w * n[d]);
+#pragma unroll
+        for (int l = 0; l < 3; l++)
+            if (l != d) b += (unsigned long long)(w * min(n[l], n[d] * (64 - __clzll((unsigned long long)n[l]))));
     }
     return b;
 }
@@ -361,14 +352,42 @@ struct LiveArgs {
                        // [32 g, 32 g + 32)) received a hit
 };
 
+constexpr int PROBE_LANE_HITS = 4;
+
+__device__ __forceinline__ uint32_t shfl_ts(uint32_t v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ int64_t shfl_ts(int64_t v, int src) {
+    return (int64_t)__shfl_sync(0xffffffffu, (long long)v, src);
+}
+
+// Records the hit of the sorted edge at pos with window end t3: its counter (MODE 0) or
+// the bin of its gap (MODE 1), and its group's bit.
+template <typename TS, int MODE>
+__device__ __forceinline__ void record_hit(const LiveArgs& a, const TS* __restrict__ T, const TS* sD, int32_t pos,
+                                           TS t3) {
+    if (MODE == 0) {
+        if (a.bins16) atomicAdd(&a.bins16[pos >> 1], 1u << (16 * (pos & 1)));
+        else atomicAdd(&a.cnt[pos], 1);
+    } else {
+        const int jb = lower_bound_ts<TS>(sD, 0, a.k, (TS)(t3 - T[pos]));
+        const int64_t x = (int64_t)pos * a.kstride + jb;  // edge-major: an edge's bins are contiguous
+        if (a.bins16) atomicAdd(&a.bins16[x >> 1], 1u << (16 * (int)(x & 1)));
+        else atomicAdd(&a.bins[x], 1);
+    }
+    if (a.touched) {
+        // a plain read first: most hits find their group's bit already set
+        const uint32_t bit = 1u << ((pos >> 5) & 31);
+        if (!(a.touched[pos >> 10] & bit)) atomicOr(&a.touched[pos >> 10], bit);
+    }
+}
+
 // MODE 0: cnt[pos] += hit at window delta. MODE 1: bin the gap t3 - t (<= delta, the
-// largest bin bound) against the sorted bounds deltas[0..k). A block takes probe tiles of
-// PB_THREADS * ITEMS slots (the tile size the autotuner picks).
+// largest bin bound) against the sorted bounds deltas[0..k). A block takes probe tiles of up
+// to PB_GROUP * ITEMS slots (the tile size the autotuner picks); a thread takes a slot: one
+// entry of a kept role's driving list (probe.cuh).
 template <typename TS, int DIR, int MODE, int ITEMS>
 __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS* __restrict__ T, TS delta,
                                                            const TS* __restrict__ deltas) {
-    constexpr int TILE = PB_THREADS * ITEMS;
-    constexpr int MAXTRI = TILE / 3 + 4;  // every kept triangle holds >= 3 slots
+    constexpr int MAXTRI = PB_GROUP * ITEMS / 3 + 4;  // every kept triangle holds >= 3 slots
     __shared__ TriStageT<MAXTRI> st;
     __shared__ uint8_t smask[MAXTRI];
     __shared__ TS sD[1024];
@@ -376,12 +395,15 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
     if (MODE == 1)
         for (int i = threadIdx.x; i < a.k; i += blockDim.x) sD[i] = deltas[i];
     const int64_t P = *a.P;
-    const int64_t tiles = (P + TILE - 1) / TILE;
-    for (int64_t b = blockIdx.x; b < tiles; b += gridDim.x) {
+    const int64_t groups = (P + PB_GROUP - 1) / PB_GROUP;
+    // a slot is a chain of searches: fewer groups per tile while that gives more blocks work
+    const int64_t each = min(max(groups / gridDim.x, (int64_t)1), (int64_t)ITEMS);
+    for (int64_t b = (int64_t)blockIdx.x * each; b < groups; b += (int64_t)gridDim.x * each) {
         __syncthreads();  // the previous tile's stage is no longer read
+        const int64_t be = min(b + each, groups);
         const int64_t t0 = a.ltile[b];
-        const int nt = (int)(a.ltile[b + 1] - t0 + 1);
-        const int64_t p0 = b * (int64_t)TILE;
+        const int nt = (int)(a.ltile[be] - t0 + 1);
+        const int64_t p0 = b * (int64_t)PB_GROUP;
         unsigned long long pbytes = 0;
         for (int j = threadIdx.x; j < nt; j += blockDim.x) {
             const int4 tr = a.tri[a.L[t0 + j]];
@@ -407,16 +429,16 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
             st.base[nt] = INT_MAX;
         }
         __syncthreads();
-        const int32_t count = (int32_t)min((int64_t)TILE, P - p0);
+        const int32_t count = (int32_t)min((be - b) * PB_GROUP, P - p0);
 #pragma unroll 1
-        for (int it = 0; it < ITEMS; it++) {
+        for (int it = 0; it < (int)(be - b); it++) {
             const int32_t local = it * PB_THREADS + (int32_t)threadIdx.x;
             if ((local & ~31) >= count) break;  // warp-uniform
-            bool active = local < count;
+            const bool active = local < count;
             // triangle of the slot: one lane bisects for the warp, lanes walk forward
             const int lane = threadIdx.x & 31;
             const int32_t first = __shfl_sync(0xffffffffu, local, 0);
-            int j0 = 0;
+            int j = 0;
             if (lane == 0) {
                 int lo = 0, hi = st.nt - 1;
                 while (lo < hi) {
@@ -424,44 +446,56 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
                     if (st.base[mid] <= first) lo = mid;
                     else hi = mid - 1;
                 }
-                j0 = lo;
+                j = lo;
             }
-            int j = __shfl_sync(0xffffffffu, j0, 0);
-            if (!active) continue;
-            while (st.base[j + 1] <= local) j++;
-            int32_t o = local - st.base[j] - LIVE_IDLE;
-            if (o < 0) continue;  // idle slot
-            const int32_t* off = st.off[j];
-            const int m = smask[j];
-            int r = 0;
-            for (; r < 6; r++) {
-                if (!((m >> r) & 1)) continue;
-                const int32_t s1 = off[3 * (r >> 1) + (r & 1) + 1] - off[3 * (r >> 1) + (r & 1)];
-                if (o < s1) break;
-                o -= s1;
+            j = __shfl_sync(0xffffffffu, j, 0);
+            // this slot's hits: positions [lo, hi) of L1, all with the same t3
+            int32_t lo = 0, hi = 0;
+            TS t3 = 0;
+            if (active) {
+                while (st.base[j + 1] <= local) j++;
+                const int32_t* off = st.off[j];
+                int32_t o = local - st.base[j] - LIVE_IDLE;
+                int m = o >= 0 ? smask[j] : 0;
+                while (m) {
+                    const int r = __ffs(m) - 1;
+                    m &= m - 1;
+                    const int code = (int)((st.desc[j] >> (6 * r)) & 63);
+                    const RolePlan rp = staged_role_plan<DIR>(off, r, code);
+                    if (o >= rp.slots) {
+                        o -= rp.slots;
+                        continue;
+                    }
+                    if (rp.drv == 1) {
+                        lo = off[3 * (r >> 1) + (r & 1)] + o;
+                        const TS t = T[lo];
+                        t3 = probe_window<TS, DIR>(T, off, code & 7, code >> 3, t, delta);
+                        hi = t3 != TsNone<TS>::value && (TS)(t3 - t) <= delta ? lo + 1 : lo;
+                    } else {
+                        const int c = rp.drv == 2 ? code & 7 : code >> 3;
+                        const int32_t* ld = off + 3 * (c >> 1) + (c & 1);
+                        const int32_t n1 = off[3 * (r >> 1) + (r & 1) + 1] - off[3 * (r >> 1) + (r & 1)];
+                        const int32_t real = (ld[DIR == FOLTY_DIR_EITHER ? 2 : 1] - ld[0]) *
+                                             (int32_t)(((int64_t)n1 + (1 << ROLE_CHUNK_LG) - 1) >> ROLE_CHUNK_LG);
+                        int sh = __clz(real) - __clz(rp.slots);  // the largest with real << sh <= slots
+                        if (((int64_t)real << sh) > rp.slots) sh--;
+                        if ((o & ((1 << sh) - 1)) == 0 && (o >> sh) < real)
+                            driven_range<TS, DIR>(T, off, r, code, rp.drv, o >> sh, delta, lo, hi, t3);
+                    }
+                    if (MODE == 0 && hi > lo && a.rflag) a.rflag[6 * (int64_t)a.L[t0 + j] + r] = 1;
+                    break;
+                }
             }
-            if (r == 6) continue;  // a slot that rounds a step of the selection up to whole units
-            const int32_t pos = off[3 * (r >> 1) + (r & 1)] + o;
-            const int code = (int)((st.desc[j] >> (6 * r)) & 63);
-            const TS t = T[pos];
-            const TS t3 = probe_window<TS, DIR>(T, off, code & 7, code >> 3, t, delta);
-            if (t3 == TsNone<TS>::value) continue;
-            const TS gap = (TS)(t3 - t);
-            if (gap > delta) continue;
-            if (MODE == 0) {
-                if (a.bins16) atomicAdd(&a.bins16[pos >> 1], 1u << (16 * (pos & 1)));
-                else atomicAdd(&a.cnt[pos], 1);
-                if (a.rflag) a.rflag[6 * (int64_t)a.L[t0 + j] + r] = 1;
-            } else {
-                const int jb = lower_bound_ts<TS>(sD, 0, a.k, gap);
-                const int64_t x = (int64_t)pos * a.kstride + jb;  // edge-major: an edge's bins are contiguous
-                if (a.bins16) atomicAdd(&a.bins16[x >> 1], 1u << (16 * (int)(x & 1)));
-                else atomicAdd(&a.bins[x], 1);
-            }
-            if (a.touched) {
-                // a plain read first: most hits find their group's bit already set
-                const uint32_t bit = 1u << ((pos >> 5) & 31);
-                if (!(a.touched[pos >> 10] & bit)) atomicOr(&a.touched[pos >> 10], bit);
+            // short ranges by their lane, the others by the whole warp
+            if (hi - lo <= PROBE_LANE_HITS)
+                for (int32_t pos = lo; pos < hi; pos++) record_hit<TS, MODE>(a, T, sD, pos, t3);
+            unsigned wide = __ballot_sync(0xffffffffu, hi - lo > PROBE_LANE_HITS);
+            while (wide) {
+                const int src = __ffs(wide) - 1;
+                wide &= wide - 1;
+                const int32_t p0r = __shfl_sync(0xffffffffu, lo, src), p1r = __shfl_sync(0xffffffffu, hi, src);
+                const TS x = shfl_ts(t3, src);
+                for (int32_t pos = p0r + lane; pos < p1r; pos += 32) record_hit<TS, MODE>(a, T, sD, pos, x);
             }
         }
     }
@@ -553,7 +587,7 @@ void triangle_liveness(folty_graph* g, cudaStream_t s, const TriLayout* from) {
     g->live_ready[FOLTY_DIR_OUT] = 1;
 }
 
-// The probe kernel of the graph's tuned shape: tile of PB_THREADS * items slots,
+// The probe kernel of the graph's tuned shape: tiles of up to PB_GROUP * items slots,
 // blocks per SM as many as fit or the tuned count.
 template <typename TS, int MODE, int ITEMS>
 static void launch_live_shape(const folty_graph* g, int dir, const LiveArgs& la, int blocks, TS delta,
@@ -579,37 +613,27 @@ static void launch_live_t(const folty_graph* g, int dir, const LiveArgs& la, TS 
     else launch_live_shape<TS, MODE, 8>(g, dir, la, g->tune.probe_blocks, delta, deltas, s);
 }
 
-template <typename TS, int ITEMS>
-static void launch_select_items(int dir, const SelectArgs& a, const RunEnds<TS>* ends, cudaStream_t s) {
-    const int64_t per_block = (int64_t)LS_THREADS * ITEMS;
-    const unsigned blocks = (unsigned)((a.ntri + per_block - 1) / per_block);
-    if (dir == FOLTY_DIR_OUT)
-        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_OUT, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
-    else if (dir == FOLTY_DIR_IN)
-        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_IN, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
-    else
-        FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_EITHER, ITEMS>), blocks, LS_THREADS, 0, s, a, ends);
-}
-
 template <typename TS>
 static void launch_select_t(const folty_graph* g, int dir, const uint8_t* tl, int64_t delta, const ProbeBuffers& ls,
                             unsigned long long* prof, const int64_t* qp, cudaStream_t s) {
     const RunEnds<TS>* ends = static_cast<const RunEnds<TS>*>(g->run_ends);
-    const int64_t tile = (int64_t)PB_THREADS * g->tune.probe_items;
-    const SelectArgs a{tl,       g->tri,  g->ntri,      delta, qp,        ls.ush, ls.ctl, ls.L,
-                       ls.loff,  ls.lmask, ls.ltile, ls.max_tiles, tile, ls.totals, prof};
-    if (g->ntri >= LS_LARGE) launch_select_items<TS, 64>(dir, a, ends, s);
-    else launch_select_items<TS, 16>(dir, a, ends, s);
+    SelectCtl* ctl = reinterpret_cast<SelectCtl*>(ls.ctl);
+    const SelectArgs a{g->tri,  ls.cand, delta,    qp,           ls.ush,   ctl,       ls.L,
+                       ls.loff, ls.lmask, ls.ltile, ls.max_tiles, PB_GROUP, ls.totals, prof};
+    FOLTY_LAUNCH(k_live_candidates<LS_ITEMS>, grid_for((g->ntri + LS_ITEMS - 1) / LS_ITEMS, LS_THREADS, LS_PER_SM), LS_THREADS,
+                 0, s, tl, g->ntri, delta, qp, ctl, ls.cand);
+    const unsigned grid = grid_for(g->ntri, LS_THREADS, LS_PER_SM);
+    if (dir == FOLTY_DIR_OUT) FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_OUT>), grid, LS_THREADS, 0, s, a, ends);
+    else if (dir == FOLTY_DIR_IN) FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_IN>), grid, LS_THREADS, 0, s, a, ends);
+    else FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_EITHER>), grid, LS_THREADS, 0, s, a, ends);
 }
 
-// Buffers of one selection: from a call's scratch, or owned by the graph. The tile map
-// has room for the smallest probe tile the tuner may pick.
-constexpr int PB_TILE_MIN = PB_THREADS * 4;
-
+// Buffers of one selection: from a call's scratch, or owned by the graph.
 template <typename A>
 static ProbeBuffers make_probe_buffers(const folty_graph* g, cudaStream_t s, A&& get) {
     const int64_t ntri = g->ntri;
     ProbeBuffers ls;
+    ls.cand = get((int32_t*)nullptr, ntri);
     ls.L = get((int32_t*)nullptr, ntri + 1);
     ls.loff = get((int64_t*)nullptr, ntri + 1);
     ls.lmask = get((uint8_t*)nullptr, ntri + 1);
@@ -621,7 +645,7 @@ static ProbeBuffers make_probe_buffers(const folty_graph* g, cudaStream_t s, A&&
     ls.ush = 0;
     while ((slots >> ls.ush) + ntri >= ((int64_t)1 << LS_UNIT_BITS)) ls.ush++;
     const int64_t padded = slots + (ls.ush > 0 ? ntri << ls.ush : 0);
-    ls.max_tiles = (padded + PB_TILE_MIN - 1) / PB_TILE_MIN;
+    ls.max_tiles = (padded + PB_GROUP - 1) / PB_GROUP;
     ls.ltile = get((int64_t*)nullptr, ls.max_tiles + 2);
     ls.ctl = get((unsigned long long*)nullptr, 2);
     FOLTY_CUDA(cudaMemsetAsync(ls.ctl, 0, 2 * sizeof(unsigned long long), s));
@@ -727,8 +751,7 @@ void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s) {
         for (int c = 0; c < TUNE_TRIALS; c++) {
             g->tune.probe_items = PROBE_CAND[c][0];
             g->tune.probe_blocks = PROBE_CAND[c][1];
-            // the selection's tile map depends on the tile, so each trial selects again
-            // (outside its timed span)
+            // each trial selects anew (outside its timed span)
             const ProbeBuffers ls = select_live(g, delta, dir, sc, s, nullptr);
             if (cnt16) FOLTY_CUDA(cudaMemsetAsync(cnt16, 0, sizeof(uint16_t) * (size_t)(mk + 2), s));
             else FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)mk, s));
@@ -843,7 +866,7 @@ void probe_stats(folty_graph* g, int64_t delta, int dir, folty_probe_stats* out,
     out->kept_roles = v[1];
     out->kept_probes = v[2];
     out->probe_bytes = v[3];
-    out->select_bytes += (int64_t)(16 + 3 * (g->ts32 ? sizeof(RunEnds<uint32_t>) : sizeof(RunEnds<int64_t>)) + 13) * v[0];
+    out->select_bytes += (int64_t)(16 + 3 * (g->ts32 ? sizeof(RunEnds<uint32_t>) : sizeof(RunEnds<int64_t>)) + 13 + 8) * v[0];
 }
 
 }  // namespace folty

@@ -182,8 +182,10 @@ static void launch_threshold(const ThresholdArgs& a, unsigned grid, cudaStream_t
 //
 // On the paper-scale graph (70M edges) the dense pass read 420 MB of keys and counts (94
 // us) after a memset of 140 MB of counters (29 us); this one takes 7 us. On 20M edges 41 ->
-// 6 us. Blocks of few words while that gives every SM blocks, so that a small graph, all of
-// whose groups may be hit, still uses the chip (100,000 edges: 24 -> 6 us).
+// 6 us. Hits cluster (at the hubs' edges), so blocks are short, one word each up to 32
+// blocks an SM: with 8 blocks an SM the pass over 6M edges took 57 us, its first blocks
+// holding nearly all marked groups; a small graph, all of whose groups may be hit, still
+// uses the chip (100,000 edges: 24 -> 6 us).
 struct HitArgs {
     uint16_t* cnt16;  // 16-bit counts, or
     int32_t* cnt;     // 32-bit ones
@@ -267,17 +269,25 @@ __global__ void __launch_bounds__(TH_THREADS) k_threshold_hits(const HitArgs a) 
         for (int k = 0; k < TH_HITS; k++) {
             const int32_t key = kb[k], c = cb[k];
             const bool sat = c >= 1 && (QUANT == FOLTY_Q_EXISTS || (int64_t)c * den >= num * (int64_t)ub[k]);
-            if (!__any_sync(0xffffffffu, sat)) continue;
+            const unsigned sats = __ballot_sync(0xffffffffu, sat);
+            if (!sats) continue;
             const int prev = __shfl_up_sync(0xffffffffu, key, 1);
             const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || key != prev);
-            const unsigned above = heads & ~((2u << lane) - 1u);
-            const int start = 31 - __clz(heads & ((2u << lane) - 1u));
-            const unsigned peers = (above ? (above & (0u - above)) - 1u : 0xffffffffu) & ~((1u << start) - 1u);
-            const int run_max = __reduce_max_sync(peers, c);
-            const int run_sat = __reduce_add_sync(peers, sat ? 1 : 0);
-            if (run_sat > 0 && lane == start) {
-                atomicMax(&a.seg_max[key], run_max);
-                atomicAdd(&a.seg_ncert[key], run_sat);
+            bool add = sat;
+            int add_max = c, add_n = 1;
+            // a reduction is issued once per run of the group: only where few runs hold many
+            // of the certificates
+            if (__popc(heads) <= 4 && __popc(sats) > 4) {
+                const unsigned above = heads & ~((2u << lane) - 1u);
+                const int start = 31 - __clz(heads & ((2u << lane) - 1u));
+                const unsigned peers = (above ? (above & (0u - above)) - 1u : 0xffffffffu) & ~((1u << start) - 1u);
+                add_max = __reduce_max_sync(peers, c);
+                add_n = __reduce_add_sync(peers, sat ? 1 : 0);
+                add = lane == start && add_n > 0;
+            }
+            if (add) {
+                atomicMax(&a.seg_max[key], add_max);
+                atomicAdd(&a.seg_ncert[key], add_n);
                 const int32_t s = key >> 1;
                 const int64_t bit = (key & 1) ? 32 * a.wa + a.binv[s] : (int64_t)s;
                 const uint32_t mask = 1u << (bit & 31);
@@ -299,7 +309,7 @@ static void launch_hits_u(const HitArgs& a, int quant, unsigned grid, cudaStream
 }
 
 static void launch_hits(HitArgs a, int quant, int universe, cudaStream_t s) {
-    const int64_t per = (a.nwords + 8 * num_sms() - 1) / (8 * num_sms());  // eight blocks an SM
+    const int64_t per = (a.nwords + 32 * num_sms() - 1) / (32 * num_sms());  // hits cluster: many short blocks
     a.words = (int)std::min<int64_t>(std::max<int64_t>(per, 1), HIT_WORDS);
     const unsigned grid = (unsigned)std::max<int64_t>((a.nwords + a.words - 1) / a.words, 1);
     if (universe == FOLTY_U_HEAD) launch_hits_u<FOLTY_U_HEAD>(a, quant, grid, s);

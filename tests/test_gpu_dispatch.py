@@ -96,3 +96,40 @@ def test_plain_query_with_32_bit_counters_and_hit_groups_everywhere(F):
     qs = _plain((100, 900))
     info = _check(F, W.TemporalGraph(n, src, dst, t), qs + qs[:3])
     assert info["max_degree"] >= 65_535
+
+
+def _triangles_of_sizes(sizes, t_max, seed, scale=1):
+    """One triangle per ordered choice of three sizes: each side holds that many edges, about
+    a third of them against the side's direction."""
+    import itertools
+    rng = np.random.default_rng(seed)
+    src, dst = [], []
+    n = 0
+    for combo in sorted(set(itertools.permutations(sizes, 3))):
+        v = rng.permutation(3) + n
+        n += 3
+        for (a, b), c in zip(((0, 1), (0, 2), (1, 2)), combo):
+            flip = rng.random(c) < 0.33
+            src.append(np.where(flip, v[b], v[a]))
+            dst.append(np.where(flip, v[a], v[b]))
+    src, dst = np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+    t = rng.integers(0, t_max, src.shape[0]).astype(np.int64) * scale
+    o = np.argsort(t, kind="stable")
+    return W.TemporalGraph(n, src[o], dst[o], t[o])
+
+
+# the probes of a role are driven by its shortest list: lists around the sizes at which L2 or
+# L3 takes over from L1 (half the slots, 64 entries of L1 per slot) and at which L1 is cut
+# into chunks (16384); many equal times, all of them, few; 32- and 64-bit stores
+@pytest.mark.parametrize("sizes", [(1, 1, 2, 3, 4, 5), (1, 2, 63, 64, 65, 129), (3, 40, 500, 520), (2, 300, 16_384, 16_385),
+                                   (5, 1, 60_000)])
+@pytest.mark.parametrize("t_max,scale", [(1, 1), (30, 1), (5000, 1), (10 ** 6, 1), (10 ** 6, 10 ** 7)])
+def test_probes_from_every_list(F, sizes, t_max, scale):
+    g = _triangles_of_sizes(sizes, t_max, sum(sizes) + t_max, scale)
+    qs = [W.Query(d * scale, 1, 2, W.Q_EXISTS, dr, W.U_HEAD, True) for d in (0, 1, max(t_max // 50, 2), t_max)
+          for dr in (W.DIR_OUT, W.DIR_IN, W.DIR_EITHER)]
+    _check(F, g, qs)
+    batch = [W.Query(q.delta, 1, 2, W.Q_EXISTS, q.dir, W.U_HEAD, False) for q in qs]
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G, oracle.OracleGraph.of(g) as og:
+        for q, r in zip(batch, G.query_batch(batch)):
+            assert pairs_of(r) == pairs_of(og.query(q)), str(q)
