@@ -355,17 +355,11 @@ bool profiling_on();
 
 // Window-probe pass of one query into counters cnt[m_kept] (sorted order, zeroed).
 void launch_probe(folty_graph* g, int64_t delta, int dir, int32_t* cnt, cudaStream_t s);
-// Window probes of the roles that can hit (live.cu): mode 0 counts hits at delta into
-// cnt or, with bins16 (cnt null), into 16-bit counters two to a word; mode 1 bins gaps
-// <= delta against the k sorted bounds `deltas` (in the timestamp store's type) into
-// edge-major rows of kstride bins (bin j of sorted edge e at e * kstride + j), as int32 or,
-// with bins16 (bins null), as 16-bit counts (counts must stay below 2^16).
-// rflag (mode 0, may be null): byte 6 * triangle + role set to 1 when the role has a hit.
-// touched (may be null): bit g of word g / 32 set when one of sorted edges
-// [32 g, 32 g + 32) received a hit (the caller clears the words first).
-void launch_probe_live(folty_graph* g, int64_t delta, int dir, int mode, int32_t* cnt, int32_t* bins, int k,
-                       int kstride, const void* deltas, cudaStream_t s, uint8_t* rflag = nullptr,
-                       uint16_t* bins16 = nullptr, uint32_t* touched = nullptr);
+// Window probes of the roles that can hit (live.cu): hits at delta into cnt or, with cnt16
+// (cnt null), into 16-bit counters. rflag (may be null): byte 6 * triangle + role set to 1
+// when the role has a hit.
+void launch_probe_live(folty_graph* g, int64_t delta, int dir, int32_t* cnt, uint16_t* cnt16, uint8_t* rflag,
+                       cudaStream_t s);
 // Autotuner (tune.cu). Parameters are cached process-wide by graph statistics (a key of
 // int64 values); forced parameters (folty_tuning_force) take precedence over both.
 bool tune_lookup(const std::vector<int64_t>& key, TuneParams* p, bool probe);
@@ -416,6 +410,16 @@ ProbeBuffers probe_buffers(folty_graph* g, cudaStream_t s);
 // value in any launch, so a captured sequence replays for any window.
 void enqueue_probe_pass(folty_graph* g, const int64_t* qp, int dir, const ProbeBuffers& pb, int32_t* cnt,
                         uint16_t* cnt16, uint32_t* touched, cudaStream_t s);
+// A batch's probes of one direction variant: the selection at its largest window; the bits
+// of the sorted edges with a hit (ebits, zeroed); and the hits with gap <= delta binned
+// against the k sorted bounds `deltas` (in the timestamp store's type) into the marked
+// edges' rows of kstride bins (row_of), as int32 or, with bins16 (bins null), as 16-bit
+// counts (counts must stay below 2^16).
+ProbeBuffers select_probes(folty_graph* g, int64_t delta, int dir, Scratch& sc, cudaStream_t s);
+void launch_marks(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& pb, uint32_t* ebits, cudaStream_t s);
+void launch_bins(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& pb, const uint32_t* ebits,
+                 const int32_t* wpref, int32_t* bins, uint16_t* bins16, int k, int kstride, const void* deltas,
+                 cudaStream_t s);
 // A cleared device counter of model bytes while profiling is on, else null.
 unsigned long long* prof_counter(folty_graph* g, cudaStream_t s);
 // Kept roles, probes and model bytes of one query's selection (live.cu; synchronises).
@@ -442,6 +446,11 @@ void fill_result_triples(folty_result* out, int64_t n);
 void release_result(folty_result* r);
 
 // ------------------------------------------------------------------ device helpers
+
+// Marked edges (bits of ebits, wpref = marked edges before each word) before sorted position x.
+__device__ __forceinline__ int32_t row_of(const uint32_t* __restrict__ ebits, const int32_t* __restrict__ wpref, int32_t x) {
+    return wpref[x >> 5] + __popc(ebits[x >> 5] & ((1u << (x & 31)) - 1u));
+}
 
 // First index in [lo, hi) with a[i] >= key (hi if none).
 __device__ __forceinline__ int lower_bound_i64(const int64_t* __restrict__ a, int lo, int hi,

@@ -330,6 +330,9 @@ __device__ __forceinline__ unsigned long long kept_role_bytes(const int32_t* off
     return b;
 }
 
+// What a hit does: count, bin or mark its edge.
+enum { PROBE_COUNT = 0, PROBE_BIN = 1, PROBE_MARK = 2 };
+
 struct LiveArgs {
     const int4* tri;
     const int32_t* seg;
@@ -338,18 +341,16 @@ struct LiveArgs {
     const uint8_t* lmask;
     const int64_t* ltile;
     const int64_t* P;  // device: total slots
-    int32_t* cnt;      // MODE 0
-    int32_t* bins;     // MODE 1, or
-    uint32_t* bins16;  // MODE 1: 16-bit counts, two to a word
-    int64_t mk;
-    int k;             // MODE 1: number of bins
-    int kstride;       // MODE 1: bins per edge row (k rounded up to whole 16-byte rows)
+    int32_t* cnt;      // PROBE_COUNT counters or PROBE_BIN bins, as int32, or
+    uint32_t* cnt16;   // 16-bit ones, two to a word
+    uint32_t* bits;    // PROBE_COUNT, may be null: bit g set when a sorted edge of [32 g, 32 g + 32) was hit;
+                       // PROBE_MARK: bit e set when sorted edge e was hit; PROBE_BIN: the marks
+    const int32_t* wpref;      // PROBE_BIN: marked edges before each word of the marks
+    int k, kstride;            // PROBE_BIN: number of bins, bins per row
     unsigned long long* prof;  // model bytes of the kept roles (may be null)
-    uint8_t* rflag;    // MODE 0, may be null: 6 * triangle + role flags of roles with a hit
+    uint8_t* rflag;    // PROBE_COUNT, may be null: 6 * triangle + role flags of roles with a hit
     const int64_t* qp; // may be null: a device block whose slot 0 (64-bit store) or 1 (32-bit
                        // store) holds the window, read instead of the delta argument
-    uint32_t* touched; // may be null: bit g set when a sorted edge of group g (edges
-                       // [32 g, 32 g + 32)) received a hit
 };
 
 constexpr int PROBE_LANE_HITS = 4;
@@ -359,40 +360,41 @@ __device__ __forceinline__ int64_t shfl_ts(int64_t v, int src) {
     return (int64_t)__shfl_sync(0xffffffffu, (long long)v, src);
 }
 
-// Records the hit of the sorted edge at pos with window end t3: its counter (MODE 0) or
-// the bin of its gap (MODE 1), and its group's bit.
+__device__ __forceinline__ void set_bit(uint32_t* bits, int32_t i) {
+    // a plain read first: most hits find the bit already set
+    const uint32_t bit = 1u << (i & 31);
+    if (!(bits[i >> 5] & bit)) atomicOr(&bits[i >> 5], bit);
+}
+
+// Records the hit of the sorted edge at pos with window end t3.
 template <typename TS, int MODE>
 __device__ __forceinline__ void record_hit(const LiveArgs& a, const TS* __restrict__ T, const TS* sD, int32_t pos,
                                            TS t3) {
-    if (MODE == 0) {
-        if (a.bins16) atomicAdd(&a.bins16[pos >> 1], 1u << (16 * (pos & 1)));
-        else atomicAdd(&a.cnt[pos], 1);
-    } else {
-        const int jb = lower_bound_ts<TS>(sD, 0, a.k, (TS)(t3 - T[pos]));
-        const int64_t x = (int64_t)pos * a.kstride + jb;  // edge-major: an edge's bins are contiguous
-        if (a.bins16) atomicAdd(&a.bins16[x >> 1], 1u << (16 * (int)(x & 1)));
-        else atomicAdd(&a.bins[x], 1);
+    if (MODE == PROBE_MARK) {
+        set_bit(a.bits, pos);
+        return;
     }
-    if (a.touched) {
-        // a plain read first: most hits find their group's bit already set
-        const uint32_t bit = 1u << ((pos >> 5) & 31);
-        if (!(a.touched[pos >> 10] & bit)) atomicOr(&a.touched[pos >> 10], bit);
-    }
+    int64_t x = pos;
+    if (MODE == PROBE_BIN)
+        x = (int64_t)row_of(a.bits, a.wpref, pos) * a.kstride + lower_bound_ts<TS>(sD, 0, a.k, (TS)(t3 - T[pos]));
+    if (a.cnt16) atomicAdd(&a.cnt16[x >> 1], 1u << (16 * (int)(x & 1)));
+    else atomicAdd(&a.cnt[x], 1);
+    if (MODE == PROBE_COUNT && a.bits) set_bit(a.bits, pos >> 5);
 }
 
-// MODE 0: cnt[pos] += hit at window delta. MODE 1: bin the gap t3 - t (<= delta, the
-// largest bin bound) against the sorted bounds deltas[0..k). A block takes probe tiles of up
-// to PB_GROUP * ITEMS slots (the tile size the autotuner picks); a thread takes a slot: one
-// entry of a kept role's driving list (probe.cuh).
+// PROBE_COUNT: cnt[pos] += hit at window delta. PROBE_BIN: bin the gap t3 - t (<= delta, the
+// largest bin bound) against the sorted bounds deltas[0..k). PROBE_MARK: mark pos. A block
+// takes probe tiles of up to PB_GROUP * ITEMS slots (the tile size the autotuner picks); a
+// thread takes a slot: one entry of a kept role's driving list (probe.cuh).
 template <typename TS, int DIR, int MODE, int ITEMS>
 __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS* __restrict__ T, TS delta,
                                                            const TS* __restrict__ deltas) {
     constexpr int MAXTRI = PB_GROUP * ITEMS / 3 + 4;  // every kept triangle holds >= 3 slots
     __shared__ TriStageT<MAXTRI> st;
     __shared__ uint8_t smask[MAXTRI];
-    __shared__ TS sD[1024];
+    __shared__ TS sD[MODE == PROBE_BIN ? 1024 : 1];
     if (a.qp) delta = (TS)a.qp[sizeof(TS) == 4 ? 1 : 0];
-    if (MODE == 1)
+    if (MODE == PROBE_BIN)
         for (int i = threadIdx.x; i < a.k; i += blockDim.x) sD[i] = deltas[i];
     const int64_t P = *a.P;
     const int64_t groups = (P + PB_GROUP - 1) / PB_GROUP;
@@ -482,7 +484,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_probe_live(LiveArgs a, const TS*
                         if ((o & ((1 << sh) - 1)) == 0 && (o >> sh) < real)
                             driven_range<TS, DIR>(T, off, r, code, rp.drv, o >> sh, delta, lo, hi, t3);
                     }
-                    if (MODE == 0 && hi > lo && a.rflag) a.rflag[6 * (int64_t)a.L[t0 + j] + r] = 1;
+                    if (MODE == PROBE_COUNT && hi > lo && a.rflag) a.rflag[6 * (int64_t)a.L[t0 + j] + r] = 1;
                     break;
                 }
             }
@@ -685,44 +687,83 @@ static ProbeBuffers select_live(folty_graph* g, int64_t delta, int dir, Scratch&
     return ls;
 }
 
-// Kept roles for delta (the largest window of the pass), then the probe kernel.
-// mode 0: counts into cnt; mode 1: bins (deltas = k sorted bounds in the store's type).
-void launch_probe_live(folty_graph* g, int64_t delta, int dir, int mode, int32_t* cnt, int32_t* bins, int k,
-                       int kstride, const void* deltas, cudaStream_t s, uint8_t* rflag, uint16_t* bins16,
-                       uint32_t* touched) {
-    const int64_t ntri = g->ntri;
-    if (ntri == 0 || g->info.probes == 0) return;
-    tune_probe(g, delta, dir, s);
+template <int MODE>
+static void launch_live(const folty_graph* g, int dir, const LiveArgs& la, int64_t delta, const void* deltas, cudaStream_t s) {
+    const uint32_t d32 = delta >= 0xfffffffell ? 0xfffffffeu : (uint32_t)delta;
+    if (g->ts32) launch_live_t<uint32_t, MODE>(g, dir, la, d32, (const uint32_t*)deltas, s);
+    else launch_live_t<int64_t, MODE>(g, dir, la, delta, (const int64_t*)deltas, s);
+}
+
+static LiveArgs live_args(const folty_graph* g, const ProbeBuffers& pb) {
+    LiveArgs la{};
+    la.tri = g->tri;
+    la.seg = g->seg;
+    la.L = pb.L;
+    la.loff = pb.loff;
+    la.lmask = pb.lmask;
+    la.ltile = pb.ltile;
+    la.P = pb.totals + 1;
+    return la;
+}
+
+// Kept roles for delta, then the probes.
+void launch_probe_live(folty_graph* g, int64_t delta, int dir, int32_t* cnt, uint16_t* cnt16, uint8_t* rflag,
+                       cudaStream_t s) {
+    if (g->ntri == 0 || g->info.probes == 0) return;
     Scratch sc(g->alloc, s, g->dev_err);
+    const ProbeBuffers ls = select_probes(g, delta, dir, sc, s);
+    LiveArgs la = live_args(g, ls);
+    la.cnt = cnt;
+    la.cnt16 = (uint32_t*)cnt16;
+    la.rflag = rflag;
+    la.prof = prof_counter(g, s);
+    StageSpan span(ST_PROBE, s, 0, la.prof);
+    launch_live<PROBE_COUNT>(g, dir, la, delta, nullptr, s);
+}
+
+ProbeBuffers select_probes(folty_graph* g, int64_t delta, int dir, Scratch& sc, cudaStream_t s) {
+    tune_probe(g, delta, dir, s);
     // model bytes counted on the device: the selection reads one liveness byte per
     // triangle, and per kept one its record and run ends, and writes 13 B; the probes'
     // bytes per staged triangle and kept role are summed by the probe kernel
-    unsigned long long* prof_sel = prof_counter(g, s);
-    unsigned long long* prof = prof_counter(g, s);
-    const ProbeBuffers ls = select_live(g, delta, dir, sc, s, prof_sel);
-    StageSpan span(ST_PROBE, s, 0, prof);
-    LiveArgs la{g->tri, g->seg, ls.L, ls.loff, ls.lmask, ls.ltile, ls.totals + 1, cnt, bins, (uint32_t*)bins16,
-                g->m_kept, k, kstride, prof, rflag, nullptr, touched};
-    if (g->ts32) {
-        const uint32_t d32 = delta >= 0xfffffffell ? 0xfffffffeu : (uint32_t)delta;
-        if (mode == 0) launch_live_t<uint32_t, 0>(g, dir, la, d32, nullptr, s);
-        else launch_live_t<uint32_t, 1>(g, dir, la, d32, (const uint32_t*)deltas, s);
-    } else {
-        if (mode == 0) launch_live_t<int64_t, 0>(g, dir, la, delta, nullptr, s);
-        else launch_live_t<int64_t, 1>(g, dir, la, delta, (const int64_t*)deltas, s);
-    }
+    return select_live(g, delta, dir, sc, s, prof_counter(g, s));
+}
+
+void launch_marks(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& pb, uint32_t* ebits, cudaStream_t s) {
+    LiveArgs la = live_args(g, pb);
+    la.bits = ebits;
+    la.prof = prof_counter(g, s);
+    StageSpan span(ST_PROBE, s, 0, la.prof);
+    launch_live<PROBE_MARK>(g, dir, la, delta, nullptr, s);
+}
+
+void launch_bins(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& pb, const uint32_t* ebits,
+                 const int32_t* wpref, int32_t* bins, uint16_t* bins16, int k, int kstride, const void* deltas,
+                 cudaStream_t s) {
+    LiveArgs la = live_args(g, pb);
+    la.cnt = bins;
+    la.cnt16 = (uint32_t*)bins16;
+    la.bits = const_cast<uint32_t*>(ebits);
+    la.wpref = wpref;
+    la.k = k;
+    la.kstride = kstride;
+    la.prof = prof_counter(g, s);
+    StageSpan span(ST_PROBE, s, 0, la.prof);
+    launch_live<PROBE_BIN>(g, dir, la, delta, deltas, s);
 }
 
 void enqueue_probe_pass(folty_graph* g, const int64_t* qp, int dir, const ProbeBuffers& pb, int32_t* cnt,
                         uint16_t* cnt16, uint32_t* touched, cudaStream_t s) {
     if (g->ntri == 0 || g->info.probes == 0) return;
     enqueue_select(g, 0, dir, pb, prof_counter(g, s), qp, s);
-    unsigned long long* prof = prof_counter(g, s);
-    StageSpan span(ST_PROBE, s, 0, prof);
-    LiveArgs la{g->tri, g->seg, pb.L, pb.loff, pb.lmask, pb.ltile, pb.totals + 1, cnt, nullptr, (uint32_t*)cnt16,
-                g->m_kept, 0, 0, prof, nullptr, qp, touched};
-    if (g->ts32) launch_live_t<uint32_t, 0>(g, dir, la, 0u, nullptr, s);
-    else launch_live_t<int64_t, 0>(g, dir, la, 0, nullptr, s);
+    LiveArgs la = live_args(g, pb);
+    la.cnt = cnt;
+    la.cnt16 = (uint32_t*)cnt16;
+    la.bits = touched;
+    la.qp = qp;
+    la.prof = prof_counter(g, s);
+    StageSpan span(ST_PROBE, s, 0, la.prof);
+    launch_live<PROBE_COUNT>(g, dir, la, 0, nullptr, s);
 }
 
 // ------------------------------------------------------------------ autotuning
@@ -755,15 +796,11 @@ void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s) {
             const ProbeBuffers ls = select_live(g, delta, dir, sc, s, nullptr);
             if (cnt16) FOLTY_CUDA(cudaMemsetAsync(cnt16, 0, sizeof(uint16_t) * (size_t)(mk + 2), s));
             else FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)mk, s));
-            LiveArgs la{g->tri, g->seg, ls.L, ls.loff, ls.lmask, ls.ltile, ls.totals + 1, cnt, nullptr,
-                        (uint32_t*)cnt16, mk, 0, 0, nullptr, nullptr, nullptr};
+            LiveArgs la = live_args(g, ls);
+            la.cnt = cnt;
+            la.cnt16 = (uint32_t*)cnt16;
             FOLTY_CUDA(cudaEventRecord(ev[0], s));
-            if (g->ts32) {
-                const uint32_t d32 = delta >= 0xfffffffell ? 0xfffffffeu : (uint32_t)delta;
-                launch_live_t<uint32_t, 0>(g, dir, la, d32, nullptr, s);
-            } else {
-                launch_live_t<int64_t, 0>(g, dir, la, delta, nullptr, s);
-            }
+            launch_live<PROBE_COUNT>(g, dir, la, delta, nullptr, s);
             FOLTY_CUDA(cudaEventRecord(ev[c + 1], s));
             FOLTY_CUDA(cudaEventSynchronize(ev[c + 1]));
             float ms = 0.f;

@@ -1101,7 +1101,7 @@ void run_query(folty_graph* g, const folty_query_params& q, folty_result* out, c
         rflag = sc.get<uint8_t>(6 * g->ntri + 1);
         FOLTY_CUDA(cudaMemsetAsync(rflag, 0, (size_t)(6 * g->ntri + 1), s));
     }
-    launch_probe_live(g, q.delta, q.dir, 0, cnt, nullptr, 0, 0, nullptr, s, rflag, cnt16);
+    launch_probe_live(g, q.delta, q.dir, cnt, cnt16, rflag, s);
     const folty_query_params* qp = &q;
     const CountView cv{cnt, cnt16};
     finish_queries(g, &qp, &cv, 1, &out, s);  // synchronises the stream
