@@ -361,7 +361,7 @@ void fill_result_host(folty_result* out, int64_t n_pairs, int64_t m, bool want_e
     }
     bool ok = true;
     if (want_edges) {
-        out->edge_count = (int32_t*)std::calloc((size_t)(m > 0 ? m : 1), sizeof(int32_t));
+        out->edge_count = (int32_t*)std::malloc(sizeof(int32_t) * (size_t)(m > 0 ? m : 1));  // all m are copied in
         ok = ok && out->edge_count;
     }
     if (want_vertices) {
