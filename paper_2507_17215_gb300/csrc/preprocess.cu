@@ -3,8 +3,7 @@
 //   A1  drop self-loops; sort temporal edges by (static pair, direction, t) so that
 //       every E_{x,y} is a contiguous ascending run of the timestamp store T;
 //   A2  static graph G_S as CSR, neighbours ascending, with static-edge ids;
-//   A3  core numbers and a degeneracy order by parallel peeling (Definition 2.1 and
-//       the Matula-Beck removal of Section 2, done a frontier at a time);
+//   A3  core numbers and a degeneracy order (core.cu);
 //   A4  orientation G->pi: u -> v iff (round(u), u) < (round(v), v); out-degree <= alpha;
 //   A5  every triangle of G_S exactly once: (u, v) in G->, w in N+(u) cap N+(v)
 //       (Algorithm 3's enumeration skeleton), with its per-triangle probe count.
@@ -14,11 +13,9 @@
 #include <cstring>
 #include <optional>
 
+#include "core.cuh"
 #include "internal.cuh"
 #include "pairs.cuh"
-
-#include <cooperative_groups.h>
-namespace cg = cooperative_groups;
 #include "probe.cuh"
 
 namespace folty {
@@ -552,1559 +549,6 @@ __global__ void k_out_sigma(const int32_t* __restrict__ sigma, const int32_t* __
     if ((threadIdx.x & 31) == 0) atomicMax(out, best);
 }
 
-// ================================================================== A3
-
-enum {
-    C_BAR = 0,
-    C_GEN = 1,
-    C_ERR = 2,
-    C_ACNT = 3,   // 2 slots
-    C_MIN = 5,    // 2 slots
-    C_FCNT = 7,   // 3 slots: light frontier sizes
-    C_HCNT = 10,  // 3 slots: heavy frontier sizes
-    C_ROUNDS = 13,
-    C_ALPHA = 14,
-    C_TAIL = 15,    // 1 when the grid kernel stopped early for the single-block tail
-    C_TAIL_K = 16,  // state handed to the tail: level, round, alive buffer, alive count
-    C_TAIL_R = 17,
-    C_TAIL_AC = 18,
-    C_TAIL_N = 19,
-    C_RM = 20,  // 2 slots by level parity: vertices removed after the level's compaction
-    C_SOLO = 22,    // 1 when the cluster tail stopped early for the single-CTA phase
-    C_SOLO_K = 23,  // level and round handed to the single-CTA phase
-    C_SOLO_R = 24,
-    C_SLOTS = 28
-};
-
-struct PeelArgs {
-    const int32_t* rowptr;
-    const int32_t* adj;
-    int32_t n;
-    int32_t* deg;   // working copy of the degrees
-    int32_t* rnd;   // removal round, -1 while alive
-    int32_t* core;  // core number
-    int32_t* alive[2];
-    int32_t* fr[2];  // light frontier (degree <= PEEL_HEAVY): one warp per vertex
-    int64_t* hr[2];  // heavy frontier as (vertex, piece) entries: piece << 32 | vertex
-    int32_t hcap;    // capacity of hr[0], hr[1]: n + 2S / PEEL_PIECE + 1
-    int* ctl;
-    long long timeout_ns;
-    int32_t tail_n;  // stop when at most this many vertices may still be alive
-};
-
-__device__ __forceinline__ long long global_ns() {
-    long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Grid-wide barrier for a cooperative launch (all blocks co-resident). The wait is
-// bounded: after timeout_ns the block records an error and every block returns.
-__device__ bool grid_barrier(int* ctl, long long timeout_ns) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile int* vgen = (volatile int*)&ctl[C_GEN];
-        volatile int* verr = (volatile int*)&ctl[C_ERR];
-        int gen = *vgen;
-        __threadfence();
-        int arrived = atomicAdd(&ctl[C_BAR], 1);
-        if (arrived == (int)gridDim.x - 1) {
-            atomicExch(&ctl[C_BAR], 0);
-            __threadfence();
-            atomicAdd(&ctl[C_GEN], 1);
-        } else {
-            long long t0 = global_ns();
-            while (*vgen == gen) {
-                if (*verr) break;
-                if (global_ns() - t0 > timeout_ns) {
-                    atomicExch(&ctl[C_ERR], 1);
-                    break;
-                }
-                __nanosleep(20);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return *(volatile int*)&ctl[C_ERR] == 0;
-}
-
-// Appends v for every lane with pred set; the whole warp must call it. A list never
-// holds more than cap entries (each vertex joins at most one frontier and one alive
-// list); an append beyond cap is dropped and recorded in *err instead of written.
-__device__ __forceinline__ void warp_append(bool pred, int32_t v, int32_t* out, int* counter, int cap,
-                                            int* err) {
-    unsigned mask = __ballot_sync(0xffffffffu, pred);
-    if (!mask) return;
-    int lane = threadIdx.x & 31;
-    int leader = __ffs(mask) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(counter, __popc(mask));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (pred) {
-        int idx = base + __popc(mask & ((1u << lane) - 1u));
-        if (idx < cap) out[idx] = v;
-        else atomicExch(err, 2);
-    }
-}
-
-// Adds the number of lanes with pred set to *counter (one atomic per warp). The whole
-// warp must call it.
-__device__ __forceinline__ void warp_count(bool pred, int* counter) {
-    const unsigned m = __ballot_sync(0xffffffffu, pred);
-    if (m && (threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(counter, __popc(m));
-}
-
-constexpr int PEEL_THREADS = 1024;
-constexpr int PEEL_SHORT = 32;      // rows up to this length are walked by one thread,
-constexpr int PEEL_CHUNK = 8;       // PEEL_CHUNK entries at a time
-constexpr int PEEL_HEAVY = 128;     // vertices above this degree go to the heavy frontier
-constexpr int PEEL_PIECE = PEEL_THREADS;  // adjacency entries per heavy piece
-constexpr int PEEL_BUF = 4096;            // entries of each block-local append buffer
-
-// Block-local staging of list appends: warps append into shared memory (one shared-memory
-// atomic per warp) and peel_flush moves a phase's entries to the global list with one
-// global atomic per block, instead of one contended global atomic per warp. Entries
-// beyond PEEL_BUF go to the global list directly.
-struct PeelBuf {
-    int32_t* fr;  // light-frontier entries
-    int32_t* al;  // alive-list entries
-    int* n;       // n[0], n[1]: entries staged in fr, al; n[2]: removals counted; n[3], n[4]: bases
-};
-
-// Appends v for every lane with pred set to the block's buffer sbuf (count *scnt), or past
-// its capacity to the global list (out, counter, cap). The whole warp must call it.
-__device__ __forceinline__ void buf_append(bool pred, int32_t v, int32_t* sbuf, int* scnt, int32_t* out,
-                                           int* counter, int cap, int* err) {
-    const unsigned m = __ballot_sync(0xffffffffu, pred);
-    if (!m) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(scnt, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    const int idx = base + __popc(m & ((1u << lane) - 1u));
-    if (pred && idx < PEEL_BUF) sbuf[idx] = v;
-    warp_append(pred && idx >= PEEL_BUF, v, out, counter, cap, err);
-}
-
-// Moves the block's staged entries to the global lists and its removal count to rm_cnt
-// (null when the phase counts none); every thread of the block calls it after its last
-// append of the phase. A list never holds more than cap entries: an entry beyond is
-// dropped and recorded in *err.
-__device__ __forceinline__ void peel_flush(PeelBuf pb, int32_t* fr_out, int* fr_cnt, int32_t* al_out, int* al_cnt,
-                                           int* rm_cnt, int cap, int* err) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nf = min(pb.n[0], PEEL_BUF), na = min(pb.n[1], PEEL_BUF);
-        pb.n[3] = nf ? atomicAdd(fr_cnt, nf) : 0;
-        pb.n[4] = na ? atomicAdd(al_cnt, na) : 0;
-        if (pb.n[2]) atomicAdd(rm_cnt, pb.n[2]);
-    }
-    __syncthreads();
-    const int nf = min(pb.n[0], PEEL_BUF), na = min(pb.n[1], PEEL_BUF);
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) {
-        const int idx = pb.n[3] + i;
-        if (idx < cap) fr_out[idx] = pb.fr[i];
-        else atomicExch(err, 2);
-    }
-    for (int i = threadIdx.x; i < na; i += blockDim.x) {
-        const int idx = pb.n[4] + i;
-        if (idx < cap) al_out[idx] = pb.al[i];
-        else atomicExch(err, 2);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) pb.n[0] = pb.n[1] = pb.n[2] = 0;
-}
-
-// Files vertex v (removed at round rr) in the frontier of round rr: light vertices as
-// themselves (staged in the block's buffer), heavy ones as their PEEL_PIECE-entry pieces
-// of adjacency. The whole warp must call it; b, e = v's row bounds.
-__device__ __forceinline__ void frontier_append(const PeelArgs& a, const PeelBuf& pb, bool in, int32_t v, int32_t b,
-                                                int32_t e, int rr) {
-    const bool heavy = in && (e - b > PEEL_HEAVY);
-    buf_append(in && !heavy, v, pb.fr, &pb.n[0], (rr & 1) ? a.fr[1] : a.fr[0], &a.ctl[C_FCNT + rr % 3], a.n,
-               &a.ctl[C_ERR]);
-    if (heavy) {
-        const int np = (e - b + PEEL_PIECE - 1) / PEEL_PIECE;
-        const int base = atomicAdd(&a.ctl[C_HCNT + rr % 3], np);
-        if (base + np <= a.hcap) {
-            int64_t* hr = (rr & 1) ? a.hr[1] : a.hr[0];
-            for (int q = 0; q < np; q++) hr[base + q] = ((int64_t)q << 32) | (uint32_t)v;
-        } else {
-            atomicExch(&a.ctl[C_ERR], 2);
-        }
-    }
-}
-
-// Neighbour j of a vertex leaving in round r: its degree drops, and a vertex whose degree
-// crosses k + 1 -> k joins round r + 1. A vertex that already left never crosses again
-// (its degree was <= k when it left and only falls), so no liveness test is needed.
-// The whole warp must call it.
-__device__ __forceinline__ void peel_neighbour(const PeelArgs& a, const PeelBuf& pb, bool valid, int32_t j, int k,
-                                               int r) {
-    bool cross = false;
-    int32_t v = 0, b = 0, e = 0;
-    if (valid) {
-        v = a.adj[j];
-        int old = atomicSub(&a.deg[v], 1);
-        if (old == k + 1) {
-            cross = true;
-            a.rnd[v] = r + 1;
-            a.core[v] = k;
-            b = a.rowptr[v];
-            e = a.rowptr[v + 1];
-        }
-    }
-    warp_count(cross, &pb.n[2]);
-    frontier_append(a, pb, cross, v, b, e, r + 1);
-}
-
-// Vertex v (valid when cross) crossed k + 1 -> k in round r: it leaves in round r + 1.
-// The whole warp must call it.
-__device__ __forceinline__ void peel_crossing(const PeelArgs& a, const PeelBuf& pb, bool cross, int32_t v, int k,
-                                              int r) {
-    warp_count(cross, &pb.n[2]);
-    int32_t rb = 0, re = 0;
-    if (cross) {
-        a.rnd[v] = r + 1;
-        a.core[v] = k;
-        rb = a.rowptr[v];
-        re = a.rowptr[v + 1];
-    }
-    frontier_append(a, pb, cross, v, rb, re, r + 1);
-}
-
-// Parallel Matula-Beck peeling. Level k = smallest remaining degree; within a level,
-// round after round, every remaining vertex of current degree <= k is removed at once
-// and its neighbours' degrees drop. A vertex enters the next round exactly when its
-// degree crosses k + 1 -> k. Each vertex gets core = k and the round it left in.
-//
-// One block per SM; every phase ends with one grid barrier. A level starts with one
-// phase that compacts the alive list and, at the same time, takes the vertices of
-// degree <= k + 1 as the next frontier (levels are usually consecutive); only when that
-// frontier is empty does a second phase jump to the minimum degree. A round hands light
-// frontier vertices to single warps; heavy ones (hubs) are filed as PEEL_PIECE-entry
-// pieces of their adjacency, one block per piece, so no warp walks a hub alone.
-//
-// Counter discipline: a phase only appends to counters that no block reads before the
-// phase's closing barrier, and only reads counters completed before its opening
-// barrier. Frontier counters rotate over three slots by round number; every new
-// frontier (level start, jump, next round) is filed under round r + 1, so the slot a
-// slow block may still be reading (round r) is never written in the same phase.
-__global__ void __launch_bounds__(PEEL_THREADS, 1) k_peel(PeelArgs a) {
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t gsize = (int64_t)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    const int64_t gwarp = gtid >> 5, nwarps = gsize >> 5;
-    int* ctl = a.ctl;
-    __shared__ int s_wmin[PEEL_THREADS / 32];
-    __shared__ int32_t s_fr[PEEL_BUF], s_al[PEEL_BUF];
-    __shared__ int s_n[5];
-    const PeelBuf pb{s_fr, s_al, s_n};
-    if (threadIdx.x < 5) s_n[threadIdx.x] = 0;
-    __syncthreads();
-    int k = -1, r = 0, lvl = 0, ac = 0, rounds = 0;
-    int nalive = a.n;
-    while (true) {
-        // few vertices left: hand the rest to the cluster tail (all blocks agree: nalive
-        // and the removals since the last compaction were read after the same barrier)
-        const int removed = lvl > 0 ? *(volatile int*)&ctl[C_RM + ((lvl - 1) & 1)] : 0;
-        if (nalive - removed <= a.tail_n) {
-            if (gtid == 0) {
-                ctl[C_TAIL] = 1;
-                ctl[C_TAIL_K] = k;
-                ctl[C_TAIL_R] = r;
-                ctl[C_TAIL_AC] = ac;
-                ctl[C_TAIL_N] = nalive;
-                ctl[C_ROUNDS] = rounds;
-            }
-            return;
-        }
-        // ---- level start: compaction + frontier at k + 1, filed as round r + 1
-        const int kk = k + 1;
-        if (gtid == 0) {
-            ctl[C_MIN + ((lvl + 1) & 1)] = INT_MAX;
-            ctl[C_ACNT + ((lvl + 1) & 1)] = 0;
-            ctl[C_RM + (lvl & 1)] = 0;
-            ctl[C_FCNT + (r + 2) % 3] = 0;
-            ctl[C_HCNT + (r + 2) % 3] = 0;
-        }
-        int lmin = INT_MAX;
-        {
-            const int32_t* acur = ac ? a.alive[1] : a.alive[0];
-            int32_t* anxt = ac ? a.alive[0] : a.alive[1];
-            for (int64_t base = gwarp * 32; base < nalive; base += nwarps * 32) {
-                int64_t i = base + lane;
-                bool keep = false, in = false;
-                int32_t v = 0;
-                int32_t rb = 0, re = 0;
-                if (i < nalive) {
-                    v = __ldcg(&acur[i]);
-                    const int rv = __ldcg(&a.rnd[v]);
-                    const int d = __ldcg(&a.deg[v]);
-                    rb = a.rowptr[v];
-                    re = a.rowptr[v + 1];
-                    if (rv < 0) {
-                        if (d <= kk) {
-                            in = true;
-                            a.rnd[v] = r + 1;
-                            a.core[v] = kk;
-                        } else {
-                            keep = true;
-                            lmin = min(lmin, d);
-                        }
-                    }
-                }
-                frontier_append(a, pb, in, v, rb, re, r + 1);
-                buf_append(keep, v, pb.al, &pb.n[1], anxt, &ctl[C_ACNT + (lvl & 1)], a.n, &ctl[C_ERR]);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
-        if (lane == 0) s_wmin[threadIdx.x >> 5] = lmin;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int bm = INT_MAX;
-            for (int w = 0; w < PEEL_THREADS / 32; w++) bm = min(bm, s_wmin[w]);
-            if (bm != INT_MAX) atomicMin(&ctl[C_MIN + (lvl & 1)], bm);
-        }
-        peel_flush(pb, ((r + 1) & 1) ? a.fr[1] : a.fr[0], &ctl[C_FCNT + (r + 1) % 3], ac ? a.alive[0] : a.alive[1],
-                   &ctl[C_ACNT + (lvl & 1)], nullptr, a.n, &ctl[C_ERR]);
-        if (!grid_barrier(ctl, a.timeout_ns)) return;
-        r += 1;
-        ac ^= 1;
-        nalive = *(volatile int*)&ctl[C_ACNT + (lvl & 1)];
-        const int fs = *(volatile int*)&ctl[C_FCNT + r % 3] + *(volatile int*)&ctl[C_HCNT + r % 3];
-        if (fs == 0) {
-            if (nalive == 0) break;
-            // no vertex of degree k + 1: jump to the smallest remaining degree, round r + 1
-            const int kj = *(volatile int*)&ctl[C_MIN + (lvl & 1)];
-            const int32_t* al = ac ? a.alive[1] : a.alive[0];
-            for (int64_t base = gwarp * 32; base < nalive; base += nwarps * 32) {
-                int64_t i = base + lane;
-                bool in = false;
-                int32_t v = 0;
-                int32_t rb = 0, re = 0;
-                if (i < nalive) {
-                    v = __ldcg(&al[i]);
-                    const int d = __ldcg(&a.deg[v]);
-                    rb = a.rowptr[v];
-                    re = a.rowptr[v + 1];
-                    if (d <= kj) {
-                        in = true;
-                        a.rnd[v] = r + 1;
-                        a.core[v] = kj;
-                    }
-                }
-                warp_count(in, &pb.n[2]);
-                frontier_append(a, pb, in, v, rb, re, r + 1);
-            }
-            k = kj;
-            peel_flush(pb, ((r + 1) & 1) ? a.fr[1] : a.fr[0], &ctl[C_FCNT + (r + 1) % 3], nullptr, nullptr,
-                       &ctl[C_RM + (lvl & 1)], a.n, &ctl[C_ERR]);
-            if (!grid_barrier(ctl, a.timeout_ns)) return;
-            r += 1;
-        } else {
-            k = kk;
-        }
-        // ---- rounds at level k (the first one has a non-empty frontier)
-        while (true) {
-            const int fsz = *(volatile int*)&ctl[C_FCNT + r % 3];
-            const int hsz = *(volatile int*)&ctl[C_HCNT + r % 3];
-            if (fsz + hsz == 0) break;
-            if (gtid == 0) {
-                ctl[C_FCNT + (r + 2) % 3] = 0;
-                ctl[C_HCNT + (r + 2) % 3] = 0;
-            }
-            // light vertices: a row of at most PEEL_SHORT entries is walked by one thread,
-            // PEEL_CHUNK entries at a time, a longer one (up to PEEL_HEAVY) by the whole warp
-            // in turn; every load of a chunk is issued, then every decrement, before a result
-            // is used
-            const int32_t* F = (r & 1) ? a.fr[1] : a.fr[0];
-            for (int64_t i0 = gwarp * 32; i0 < fsz; i0 += nwarps * 32) {
-                const int64_t i = i0 + lane;
-                const bool have = i < fsz;
-                const int32_t u = have ? __ldcg(&F[i]) : 0;
-                const int32_t b = have ? a.rowptr[u] : 0, e = have ? a.rowptr[u + 1] : 0;
-                const bool shortrow = have && e - b <= PEEL_SHORT;
-                const int chunks = __reduce_max_sync(0xffffffffu, shortrow ? (e - b + PEEL_CHUNK - 1) / PEEL_CHUNK : 0);
-                for (int c = 0; c < chunks; c++) {  // warp-uniform trip count
-                    const int32_t j0 = b + c * PEEL_CHUNK;
-                    int32_t v[PEEL_CHUNK];
-                    int old[PEEL_CHUNK];
-#pragma unroll
-                    for (int t = 0; t < PEEL_CHUNK; t++) v[t] = (shortrow && j0 + t < e) ? a.adj[j0 + t] : -1;
-#pragma unroll
-                    for (int t = 0; t < PEEL_CHUNK; t++) old[t] = (v[t] >= 0) ? atomicSub(&a.deg[v[t]], 1) : 0;
-#pragma unroll
-                    for (int t = 0; t < PEEL_CHUNK; t++)
-                        peel_crossing(a, pb, v[t] >= 0 && old[t] == k + 1, v[t], k, r);
-                }
-                unsigned mm = __ballot_sync(0xffffffffu, have && !shortrow);
-                while (mm) {
-                    const int src = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const int32_t bb = __shfl_sync(0xffffffffu, b, src), ee = __shfl_sync(0xffffffffu, e, src);
-                    constexpr int Q = PEEL_HEAVY / 32;
-                    int32_t v[Q];
-                    int old[Q];
-#pragma unroll
-                    for (int q = 0; q < Q; q++) {
-                        const int32_t j = bb + q * 32 + lane;
-                        v[q] = (j < ee) ? a.adj[j] : -1;
-                    }
-#pragma unroll
-                    for (int q = 0; q < Q; q++) old[q] = (v[q] >= 0) ? atomicSub(&a.deg[v[q]], 1) : 0;
-#pragma unroll
-                    for (int q = 0; q < Q; q++) peel_crossing(a, pb, v[q] >= 0 && old[q] == k + 1, v[q], k, r);
-                }
-            }
-            // heavy vertices: one block per piece of PEEL_PIECE adjacency entries
-            const int64_t* H = (r & 1) ? a.hr[1] : a.hr[0];
-            for (int pc = blockIdx.x; pc < hsz; pc += gridDim.x) {
-                const int64_t hp = __ldcg(&H[pc]);
-                const int32_t u = (int32_t)(hp & 0xffffffffll);
-                const int32_t q = (int32_t)(hp >> 32);
-                const int32_t j = a.rowptr[u] + q * PEEL_PIECE + (int32_t)threadIdx.x;
-                peel_neighbour(a, pb, j < a.rowptr[u + 1], j, k, r);
-            }
-            peel_flush(pb, ((r + 1) & 1) ? a.fr[1] : a.fr[0], &ctl[C_FCNT + (r + 1) % 3], nullptr, nullptr,
-                       &ctl[C_RM + (lvl & 1)], a.n, &ctl[C_ERR]);
-            if (!grid_barrier(ctl, a.timeout_ns)) return;
-            r++;
-            rounds++;
-        }
-        lvl++;
-    }
-    if (gtid == 0) {
-        ctl[C_ROUNDS] = rounds;
-        ctl[C_ALPHA] = k;
-    }
-}
-
-// ================================================================== A3 tail
-
-// The last levels run on one thread-block cluster, on the subgraph induced by the vertices
-// still alive, renumbered 0..NL-1 ("local" ids): degrees, row bounds and frontiers live
-// in the CTAs' shared memory (each CTA owns the local ids congruent to its rank) and a
-// round ends with one cluster barrier instead of a grid barrier.
-constexpr int TAIL_THREADS = 1024;
-constexpr int SOLO_DEG_CAP = 1 << 18;  // degree sum (remaining decrements) the single CTA takes over
-constexpr int TAIL_OWN = 10240;  // local vertices owned per CTA: a C-CTA tail takes up to 10240 C
-
-// Local ids for the vertices of the grid kernel's alive list that are still alive (at
-// most cap; more would be an internal error, recorded in *err instead of written).
-// Nothing to do when the grid kernel finished the peeling itself (ctl[C_TAIL] == 0).
-__global__ void k_tail_select(const int32_t* __restrict__ alive0, const int32_t* __restrict__ alive1,
-                              const int* __restrict__ ctl, const int32_t* __restrict__ rnd, int cap,
-                              int32_t* __restrict__ L, int32_t* __restrict__ gmap, int* __restrict__ nl,
-                              int* __restrict__ err) {
-    if (ctl[C_TAIL] != 1) return;
-    const int nalive = ctl[C_TAIL_N];
-    const int32_t* __restrict__ alive = ctl[C_TAIL_AC] ? alive1 : alive0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nalive;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t v = alive[i];
-        if (rnd[v] < 0) {
-            int li = atomicAdd(nl, 1);
-            if (li < cap) {
-                L[li] = v;
-                gmap[v] = li;
-            } else {
-                atomicExch(err, 2);
-            }
-        }
-    }
-}
-
-// Local degree (alive neighbours = current degree) and full row length per local id.
-__global__ void k_tail_degrees(const int32_t* __restrict__ L, const int* __restrict__ nl,
-                               const int32_t* __restrict__ deg, const int32_t* __restrict__ rowptr, int tn,
-                               int32_t* __restrict__ ld, int32_t* __restrict__ d0) {
-    const int n = *nl;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < tn; i += gridDim.x * blockDim.x) {
-        if (i < n) {
-            int32_t v = L[i];
-            ld[i] = deg[v];
-            d0[i] = rowptr[v + 1] - rowptr[v];
-        } else {
-            ld[i] = 0;
-            d0[i] = 0;
-        }
-    }
-}
-
-// Entry e of the concatenated full rows of the local vertices (eoff = prefix of d0):
-// alive neighbours go to the owner's local row (order within a row is irrelevant).
-constexpr int FILL_RUN = 8;  // consecutive entries per thread in the subgraph fills
-
-__global__ void k_tail_fill(const int32_t* __restrict__ L, const int32_t* __restrict__ eoff, int tn,
-                            const int32_t* __restrict__ rowptr, const int32_t* __restrict__ adj,
-                            const int32_t* __restrict__ rnd, const int32_t* __restrict__ gmap,
-                            const int32_t* __restrict__ lrow, const int32_t* __restrict__ ld,
-                            int32_t* __restrict__ fillc, uint32_t* __restrict__ ladj, int* __restrict__ err) {
-    const int64_t total = eoff[tn];
-    // a thread takes FILL_RUN consecutive entries: one search for the first one's owner,
-    // then the owner moves forward (rows average a few entries), and the alive entries of
-    // each owner's part of the run take their places with one atomic (a hub's counter
-    // would serialise one atomic per entry)
-    const int64_t step = (int64_t)gridDim.x * blockDim.x * FILL_RUN;
-    for (int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * FILL_RUN; e0 < total; e0 += step) {
-        int lo = 0, hi = tn - 1;  // last owner with eoff[owner] <= e0
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (eoff[mid] <= e0) lo = mid;
-            else hi = mid - 1;
-        }
-        const int64_t e1 = min(e0 + FILL_RUN, total);
-        int64_t e = e0;
-        while (e < e1) {
-            while (lo + 1 < tn && eoff[lo + 1] <= e) lo++;
-            const int64_t end = (lo + 1 < tn) ? min(e1, (int64_t)eoff[lo + 1]) : e1;  // this owner's part
-            uint32_t keep[FILL_RUN];
-            int nk = 0;
-            const int32_t rb = rowptr[L[lo]];
-            for (; e < end; e++) {
-                const int32_t v = adj[rb + (int32_t)(e - eoff[lo])];
-                if (rnd[v] < 0) keep[nk++] = (uint32_t)gmap[v];
-            }
-            if (nk) {
-                const int p = atomicAdd(&fillc[lo], nk);
-                if (p + nk <= ld[lo]) {
-                    for (int q = 0; q < nk; q++) ladj[lrow[lo] + p + q] = keep[q];
-                } else {
-                    atomicExch(err, 3);  // more alive neighbours than the degree says
-                }
-            }
-        }
-    }
-}
-
-struct TailArgs {
-    const int* nl;
-    const int32_t* L;
-    const int32_t* ld;
-    const int32_t* lrow;
-    const uint32_t* ladj;
-    int32_t* rnd;
-    int32_t* core;
-    int* ctl;
-    // hand-off to the single-CTA phase once at most solo_cap vertices are left: their
-    // local ids (slist), current degrees (sdeg), and map2[local id] = position in slist
-    int solo_cap;
-    int* ns;
-    int32_t* slist;
-    int32_t* sdeg;
-    int32_t* map2;
-    // decrements of a heavy round, by owner and slot (owner * TAIL_OWN + slot), zero
-    // between rounds
-    int32_t* dec;
-};
-
-constexpr int TAIL_AGG_MIN = 128;  // frontier size from which a round's decrements go through L2
-constexpr int TAIL_SHORT = 32;   // rows up to this length: one thread, TAIL_CHUNK loads at a time
-constexpr int TAIL_CHUNK = 8;
-constexpr int TAIL_LIGHT = 256;  // rows up to this length: one warp, all loads in flight at once
-constexpr int TAIL_HCAP = 512;   // heavy vertices per CTA and round (more wait for the next pass)
-
-// Shared memory of one tail CTA of a C-CTA cluster. Local vertex v is owned by CTA v % C
-// at slot q = v / C; the owner keeps its degree, row bounds and global id, and the
-// frontier lists hold owned slots: a thread that drives a vertex's degree across k + 1 -> k
-// files it directly in the owner's next frontier through distributed shared memory.
-template <int C>
-struct TailShared {
-    static constexpr int OWN = TAIL_OWN;
-    int32_t odeg[OWN];
-    int32_t orb[OWN], ore[OWN];  // row [orb, ore) of ladj
-    int32_t oL[OWN];             // global id
-    uint16_t FL[2][OWN];         // frontier by round parity (owned slots)
-    uint16_t FH[TAIL_HCAP];      // heavy rows of the current round
-    int cntL[3], cntH[2], smin[2];
-    int acnt[2];                 // owned vertices alive at the level start, by level parity
-    int adeg[2];                 // their degree sum (twice the edges left), by level parity
-    int made[2];                 // crossings this CTA filed (anywhere) in a round, by round parity
-    int slots[2][C][4];          // every CTA's values of one cluster barrier, by barrier parity
-};
-
-// Neighbours vv[0..N) (negative: none) lose one degree each in round r at level k: all N
-// decrements are issued before any result is used, then every k + 1 -> k crossing files
-// its vertex in the owner's frontier of round r + 1.
-template <int C, int N>
-__device__ __forceinline__ void tail_decrement(TailShared<C>& sh, cg::cluster_group& cl, const int (&vv)[N], int k,
-                                               int r, int32_t* __restrict__ dec) {
-    if (dec) {
-        // a heavy round: many frontier rows share their targets, and one shared-memory
-        // atomic of the target's owner per decrement would queue at that SM; the
-        // decrements add up in L2 instead, and each owner applies its own after the
-        // round's barrier
-#pragma unroll
-        for (int t = 0; t < N; t++)
-            if (vv[t] >= 0) atomicAdd(&dec[(vv[t] % C) * TAIL_OWN + vv[t] / C], 1);
-        return;
-    }
-    int old[N];
-#pragma unroll
-    for (int t = 0; t < N; t++)
-        old[t] = (vv[t] >= 0) ? atomicSub(&cl.map_shared_rank(sh.odeg, vv[t] % C)[vv[t] / C], 1) : 0;
-#pragma unroll
-    for (int t = 0; t < N; t++) {
-        if (vv[t] >= 0 && old[t] == k + 1) {
-            TailShared<C>* p = cl.map_shared_rank(&sh, vv[t] % C);
-            const int at = atomicAdd(&p->cntL[(r + 1) % 3], 1);
-            p->FL[(r + 1) & 1][at] = (uint16_t)(vv[t] / C);
-            atomicAdd(&sh.made[r & 1], 1);
-        }
-    }
-}
-
-// Publishes this CTA's values v of the next cluster barrier (number s) in every CTA's
-// slot s & 1 (threads 0..C-1 each write one CTA's copy); after the barrier, tail_totals
-// combines the C copies from this CTA's own shared memory, without a remote read after
-// the barrier. A slot is rewritten two barriers later, after every CTA has read it. The
-// values must be final (the caller's __syncthreads) before the call.
-template <int C>
-__device__ __forceinline__ void tail_publish(TailShared<C>& sh, cg::cluster_group& cl, int s, int4 v) {
-    if (threadIdx.x < C) {
-        TailShared<C>* q = cl.map_shared_rank(&sh, (int)threadIdx.x);
-        int* d = q->slots[s & 1][cl.block_rank()];
-        d[0] = v.x;
-        d[1] = v.y;
-        d[2] = v.z;
-        d[3] = v.w;
-    }
-}
-
-// After the barrier: the sums of the C copies' x, z, w and the minimum of their y (each
-// warp reduces them for itself).
-template <int C>
-__device__ __forceinline__ int4 tail_totals(const TailShared<C>& sh, int s) {
-    const int lane = threadIdx.x & 31;
-    int x = 0, y = INT_MAX, z = 0, w = 0;
-    if (lane < C) {
-        const int* d = sh.slots[s & 1][lane];
-        x = d[0];
-        y = d[1];
-        z = d[2];
-        w = d[3];
-    }
-    return make_int4(__reduce_add_sync(0xffffffffu, x), __reduce_min_sync(0xffffffffu, y),
-                     __reduce_add_sync(0xffffffffu, z), __reduce_add_sync(0xffffffffu, w));
-}
-
-// The same peeling as k_peel (levels, rounds, k + 1 -> k crossings), on the local
-// subgraph, continuing the level k and round r where the grid kernel stopped.
-//
-// A vertex is alive at a level start exactly when its degree exceeds the finished level
-// k (a removed vertex had degree <= k when it left, and degrees only fall). Frontier
-// counters rotate over three rounds (round r reads slot r % 3 of every CTA, crossings
-// append to (r + 1) % 3, and each CTA clears its own (r + 2) % 3, which no CTA touches in
-// round r); the level minima alternate by level parity. Every decision that ends a loop
-// is taken by all CTAs from the same values read between the same two cluster barriers,
-// so the CTAs always meet at the same barrier. In a round, the owner of each frontier
-// vertex writes its round and core number and walks its row: its own thread for a short
-// row, its warp for a medium one, the whole CTA for a heavy one, every load of a walk in
-// flight before its first decrement.
-template <int C>
-__global__ void __launch_bounds__(TAIL_THREADS, 1) k_peel_tail(TailArgs a) {
-    using Sh = TailShared<C>;
-    constexpr int OWN = Sh::OWN;
-    cg::cluster_group cl = cg::this_cluster();
-    extern __shared__ __align__(16) unsigned char smem[];
-    Sh& sh = *reinterpret_cast<Sh*>(smem);
-    if (a.ctl[C_TAIL] != 1) return;  // the grid kernel finished (every CTA reads the same value)
-    const int rank = (int)cl.block_rank();
-    const int nl = *a.nl;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int q = tid; q < OWN; q += TAIL_THREADS) {
-        const int v = q * C + rank;
-        const bool in = v < nl;
-        sh.odeg[q] = in ? a.ld[v] : 0;
-        sh.orb[q] = in ? a.lrow[v] : 0;
-        sh.ore[q] = in ? a.lrow[v + 1] : 0;
-        sh.oL[q] = in ? a.L[v] : 0;
-    }
-    if (tid < 3) sh.cntL[tid] = 0;
-    if (tid < 2) {
-        sh.cntH[tid] = 0;
-        sh.smin[tid] = INT_MAX;
-        sh.acnt[tid] = 0;
-        sh.adeg[tid] = 0;
-        sh.made[tid] = 0;
-    }
-    int k = a.ctl[C_TAIL_K], r = a.ctl[C_TAIL_R], rounds = a.ctl[C_ROUNDS], lvl = 0, gs = 0;
-    bool handed = false;
-    cl.sync();
-    while (true) {
-        // ---- level start: owned vertices of degree k + 1 join round r + 1
-        if (tid == 0) {
-            sh.cntL[(r + 2) % 3] = 0;
-            sh.cntH[(r + 1) & 1] = 0;
-            sh.made[0] = sh.made[1] = 0;  // no crossings are filed before the next round
-            sh.smin[(lvl + 1) & 1] = INT_MAX;
-            sh.acnt[(lvl + 1) & 1] = 0;
-            sh.adeg[(lvl + 1) & 1] = 0;
-        }
-        int kk = k + 1;
-        int lmin = INT_MAX;
-        for (int q0 = 0; q0 < OWN; q0 += TAIL_THREADS) {
-            const int q = q0 + tid;
-            bool rem = false, alive = false;
-            if (q < OWN && q * C + rank < nl) {
-                const int d = sh.odeg[q];
-                if (d > k) {
-                    alive = true;
-                    if (d <= kk) rem = true;
-                    else lmin = min(lmin, d);
-                }
-            }
-            warp_count(alive, &sh.acnt[lvl & 1]);
-            const int dsum = __reduce_add_sync(0xffffffffu, alive ? sh.odeg[q] : 0);
-            if (lane == 0 && dsum) atomicAdd(&sh.adeg[lvl & 1], dsum);
-            const unsigned m = __ballot_sync(0xffffffffu, rem);
-            if (m) {
-                const int leader = __ffs(m) - 1;
-                int base = 0;
-                if (lane == leader) base = atomicAdd(&sh.cntL[(r + 1) % 3], __popc(m));
-                base = __shfl_sync(0xffffffffu, base, leader);
-                if (rem) sh.FL[(r + 1) & 1][base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)q;
-            }
-        }
-        lmin = __reduce_min_sync(0xffffffffu, lmin);
-        if (lane == 0 && lmin != INT_MAX) atomicMin(&sh.smin[lvl & 1], lmin);
-        __syncthreads();  // the level start's own filings, minimum and sums are final
-        tail_publish(sh, cl, gs,
-                     make_int4(sh.cntL[(r + 1) % 3], sh.smin[lvl & 1], sh.acnt[lvl & 1], sh.adeg[lvl & 1]));
-        cl.sync();
-        const int4 g = tail_totals(sh, gs++);
-        // the single CTA takes over once few vertices and few edges are left (dense
-        // remainders, such as planted communities, keep the cluster's sixteen SMs)
-        if (g.z > 0 && g.z <= a.solo_cap && g.w <= SOLO_DEG_CAP) {
-            // few vertices left: export them (local id, current degree) to the single-CTA
-            // phase, which starts this level again; the frontier filed above is dropped
-            for (int q0 = 0; q0 < OWN; q0 += TAIL_THREADS) {
-                const int q = q0 + tid;
-                const int v = q * C + rank;
-                const bool alive = q < OWN && v < nl && sh.odeg[q] > k;
-                const unsigned m = __ballot_sync(0xffffffffu, alive);
-                if (m) {
-                    const int leader = __ffs(m) - 1;
-                    int base = 0;
-                    if (lane == leader) base = atomicAdd(a.ns, __popc(m));
-                    base = __shfl_sync(0xffffffffu, base, leader);
-                    if (alive) {
-                        const int i = base + __popc(m & ((1u << lane) - 1u));
-                        if (i < a.solo_cap) {
-                            a.slist[i] = v;
-                            a.sdeg[i] = sh.odeg[q];
-                            a.map2[v] = i;
-                        } else {
-                            atomicExch(&a.ctl[C_ERR], 2);
-                        }
-                    }
-                }
-            }
-            if (rank == 0 && tid == 0) {
-                a.ctl[C_SOLO] = 1;
-                a.ctl[C_SOLO_K] = k;
-                a.ctl[C_SOLO_R] = r;
-                a.ctl[C_ROUNDS] = rounds;
-            }
-            handed = true;
-            break;
-        }
-        int total = g.x;
-        if (total == 0) {
-            if (g.y == INT_MAX) break;  // nothing left anywhere
-            kk = g.y;                   // jump to the smallest remaining degree
-            cl.sync();  // every CTA has read the empty totals before appends resume
-            for (int q0 = 0; q0 < OWN; q0 += TAIL_THREADS) {
-                const int q = q0 + tid;
-                bool rem = false;
-                if (q < OWN && q * C + rank < nl) {
-                    const int d = sh.odeg[q];
-                    rem = d > k && d <= kk;
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, rem);
-                if (m) {
-                    const int leader = __ffs(m) - 1;
-                    int base = 0;
-                    if (lane == leader) base = atomicAdd(&sh.cntL[(r + 1) % 3], __popc(m));
-                    base = __shfl_sync(0xffffffffu, base, leader);
-                    if (rem) sh.FL[(r + 1) & 1][base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)q;
-                }
-            }
-            cl.sync();
-            total = 1;  // some vertex has the minimum degree: the jump frontier is not empty
-        }
-        k = kk;
-        r += 1;
-        // ---- rounds at level k
-        while (total > 0) {
-            const int nL = sh.cntL[r % 3];
-            int32_t* const rdec = total >= TAIL_AGG_MIN ? a.dec : nullptr;  // the same in every CTA
-            if (tid == 0) {
-                sh.cntL[(r + 2) % 3] = 0;
-                sh.cntH[(r + 1) & 1] = 0;  // read in round r + 1, after this round's barriers
-                sh.made[(r + 1) & 1] = 0;
-            }
-            // one pass, up to 32 frontier vertices per warp, dealt round-robin over the warps
-            // (a small frontier spreads one vertex per warp): round and core number; a short
-            // row is walked by its own lane, a medium one by the whole warp in turn, and a
-            // heavy one is left to the whole CTA below
-            const uint16_t* fl = sh.FL[r & 1];
-            constexpr int NW = TAIL_THREADS / 32;
-            for (int i0 = warp; i0 - warp < nL; i0 += TAIL_THREADS) {
-                const int i = i0 + lane * NW;
-                const bool have = i < nL;
-                const int q = have ? fl[i] : 0;
-                const int b = have ? sh.orb[q] : 0, e = have ? sh.ore[q] : 0;
-                if (have) {
-                    a.rnd[sh.oL[q]] = r;
-                    a.core[sh.oL[q]] = k;
-                }
-                // a short row is walked by its own lane (TAIL_CHUNK loads at a time) when the
-                // frontier gives every warp several rows, or when it takes one step anyway;
-                // in a small frontier the whole warp walks it in one step
-                const bool lanewalk = nL > 4 * NW || e - b <= TAIL_CHUNK;
-                const bool shortrow = have && e - b <= TAIL_SHORT && lanewalk;
-                bool medium = have && !shortrow;
-                if (have && e - b > TAIL_LIGHT) {
-                    const int h = atomicAdd(&sh.cntH[r & 1], 1);
-                    if (h < TAIL_HCAP) {
-                        sh.FH[h] = (uint16_t)q;
-                        medium = false;
-                    }
-                }
-                if (shortrow) {
-                    for (int j0 = b; j0 < e; j0 += TAIL_CHUNK) {
-                        int vv[TAIL_CHUNK];
-#pragma unroll
-                        for (int t = 0; t < TAIL_CHUNK; t++) vv[t] = (j0 + t < e) ? (int)a.ladj[j0 + t] : -1;
-                        tail_decrement<C>(sh, cl, vv, k, r, rdec);
-                    }
-                }
-                unsigned mm = __ballot_sync(0xffffffffu, medium);
-                while (mm) {
-                    const int src = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const int bb = __shfl_sync(0xffffffffu, b, src), ee = __shfl_sync(0xffffffffu, e, src);
-                    for (int j0 = bb; j0 < ee; j0 += TAIL_LIGHT) {
-                        int vv[TAIL_LIGHT / 32];
-#pragma unroll
-                        for (int t = 0; t < TAIL_LIGHT / 32; t++) {
-                            const int j = j0 + t * 32 + lane;
-                            vv[t] = (j < ee) ? (int)a.ladj[j] : -1;
-                        }
-                        tail_decrement<C>(sh, cl, vv, k, r, rdec);
-                    }
-                }
-            }
-            __syncthreads();  // this round's heavy list is complete
-            // the whole CTA per heavy row
-            const int nH = min(sh.cntH[r & 1], TAIL_HCAP);
-            for (int h = 0; h < nH; h++) {
-                const int q = sh.FH[h];
-                const int b = sh.orb[q], e = sh.ore[q];
-                for (int j0 = b; j0 < e; j0 += 4 * TAIL_THREADS) {
-                    int vv[4];
-#pragma unroll
-                    for (int t = 0; t < 4; t++) {
-                        const int j = j0 + t * TAIL_THREADS + tid;
-                        vv[t] = (j < e) ? (int)a.ladj[j] : -1;
-                    }
-                    tail_decrement<C>(sh, cl, vv, k, r, rdec);
-                }
-            }
-            if (rdec) {
-                // every CTA's decrements are in L2: each owner applies its own, and files the
-                // vertices that crossed k + 1 -> k (the sum may cross in one step)
-                cl.sync();
-                for (int q0 = 0; q0 < OWN; q0 += TAIL_THREADS) {
-                    const int q = q0 + tid;
-                    bool cross = false;
-                    if (q < OWN && q * C + rank < nl) {
-                        int32_t* dp = rdec + rank * TAIL_OWN + q;
-                        const int d = __ldcg(dp);
-                        if (d) {
-                            *dp = 0;
-                            const int old = sh.odeg[q];
-                            sh.odeg[q] = old - d;
-                            cross = old > k && old - d <= k;
-                        }
-                    }
-                    const unsigned m = __ballot_sync(0xffffffffu, cross);
-                    if (m) {
-                        const int leader = __ffs(m) - 1;
-                        int base = 0;
-                        if (lane == leader) {
-                            base = atomicAdd(&sh.cntL[(r + 1) % 3], __popc(m));
-                            atomicAdd(&sh.made[r & 1], __popc(m));
-                        }
-                        base = __shfl_sync(0xffffffffu, base, leader);
-                        if (cross) sh.FL[(r + 1) & 1][base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)q;
-                    }
-                }
-            }
-            __syncthreads();  // this CTA's crossings of the round are counted
-            tail_publish(sh, cl, gs, make_int4(sh.made[r & 1], INT_MAX, 0, 0));
-            cl.sync();
-            r++;
-            rounds++;
-            total = tail_totals(sh, gs++).x;
-        }
-        lvl++;
-    }
-    if (rank == 0 && tid == 0 && !handed) {
-        a.ctl[C_ROUNDS] = rounds;
-        a.ctl[C_ALPHA] = k;
-    }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
-}
-
-// Launch configuration of the tail on one cluster of C CTAs.
-template <int C>
-static cudaLaunchConfig_t tail_config(cudaLaunchAttribute* attr, cudaStream_t s) {
-    const size_t smem = sizeof(TailShared<C>);
-    FOLTY_CUDA(cudaFuncSetAttribute(k_peel_tail<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (C > 8) FOLTY_CUDA(cudaFuncSetAttribute(k_peel_tail<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(TAIL_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
-}
-
-// CTAs of the tail's cluster: 16 when the device places such a cluster, else 8.
-static int tail_cluster_size(cudaStream_t s) {
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = tail_config<16>(attr, s);
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, k_peel_tail<16>, &cfg) == cudaSuccess && clusters >= 1) return 16;
-    cudaGetLastError();
-    cfg = tail_config<8>(attr, s);
-    if (cudaOccupancyMaxActiveClusters(&clusters, k_peel_tail<8>, &cfg) == cudaSuccess && clusters >= 1) return 8;
-    cudaGetLastError();
-    fail(FOLTY_ECUDA, "peeling: the device cannot place the tail's thread-block cluster");
-}
-
-template <int C>
-static void launch_tail(const TailArgs& ta, cudaStream_t s) {
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = tail_config<C>(attr, s);
-    FOLTY_CUDA(cudaLaunchKernelEx(&cfg, k_peel_tail<C>, ta));
-    after_launch("k_peel_tail");
-}
-
-// ================================================================== A3 last levels
-
-// Once at most SOLO_CAP vertices are left, a single CTA finishes the peeling: degrees, row
-// starts and frontiers of the remaining subgraph fit in its shared memory, so a round ends
-// with __syncthreads instead of a cluster barrier. Vertices are renumbered 0..ns-1 again
-// ("solo" ids, 16-bit) in the order the cluster exported them.
-constexpr int SOLO_THREADS = 1024;
-constexpr int SOLO_CAP = 12288;  // vertices of the single-CTA phase
-constexpr int SOLO_PASS = 2048;  // frontier vertices laid out per pass (2 per thread)
-constexpr int SOLO_CHUNK = 8;    // adjacency entries per thread in flight together (large frontiers)
-constexpr int SOLO_CHUNK_S = 2;
-constexpr int SOLO_COARSE = 1024;  // coarse owner table of a large frontier's flat entries  // the same for small frontiers (W <= 2048 in one step; less code)
-
-// Cluster row length and global id of each exported vertex (0 past the exported count).
-__global__ void k_solo_rows(const int* __restrict__ ctl, const int* __restrict__ ns_p,
-                            const int32_t* __restrict__ slist, const int32_t* __restrict__ lrow,
-                            const int32_t* __restrict__ L, int32_t* __restrict__ dl, int32_t* __restrict__ sgid) {
-    if (ctl[C_SOLO] != 1) return;
-    const int ns = *ns_p;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < SOLO_CAP; i += gridDim.x * blockDim.x) {
-        if (i < ns) {
-            const int32_t v = slist[i];
-            dl[i] = lrow[v + 1] - lrow[v];
-            sgid[i] = L[v];
-        } else {
-            dl[i] = 0;
-        }
-    }
-}
-
-// Entry e of the concatenated cluster rows of the exported vertices (eo = prefix of dl):
-// an alive neighbour (map2 >= 0) goes to its owner's row of the remaining subgraph, in
-// solo ids (order within a row is irrelevant). Every row must come out with exactly the
-// degree the cluster exported (its alive neighbours): fc counts them, and the
-// single-CTA kernel checks the count; an entry beyond it is recorded in *err (4).
-// L2 residency of the single-CTA phase's rows: written and read with an "evict last"
-// policy, so that the streaming kernels of the temporal store, which run beside the
-// peeling, evict their own lines first; set back to normal when the phase ends.
-__device__ __forceinline__ uint64_t l2_keep_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-__device__ __forceinline__ int ld_keep_u16(const uint16_t* p, uint64_t pol) {
-    unsigned short v;
-    asm("ld.global.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(p), "l"(pol));
-    return (int)v;
-}
-
-__device__ __forceinline__ void st_keep_u16(uint16_t* p, uint16_t v, uint64_t pol) {
-    asm volatile("st.global.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(p), "h"(v), "l"(pol) : "memory");
-}
-
-__device__ __forceinline__ void l2_release_line(const void* p) {
-    asm volatile("applypriority.global.L2::evict_normal [%0], 128;" ::"l"(p) : "memory");
-}
-
-__global__ void k_solo_fill(const int* __restrict__ ctl, const int32_t* __restrict__ eo,
-                            const int32_t* __restrict__ slist, const int32_t* __restrict__ sdeg,
-                            const int32_t* __restrict__ srow, const int32_t* __restrict__ lrow,
-                            const uint32_t* __restrict__ ladj, const int32_t* __restrict__ map2,
-                            int32_t* __restrict__ fc, uint16_t* __restrict__ sadj, int* __restrict__ err) {
-    if (ctl[C_SOLO] != 1 || ctl[C_ERR] != 0) return;
-    const uint64_t keep = l2_keep_policy();
-    const int64_t total = eo[SOLO_CAP];
-    const int64_t step = (int64_t)gridDim.x * blockDim.x * FILL_RUN;
-    for (int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * FILL_RUN; e0 < total; e0 += step) {
-        int lo = 0, hi = SOLO_CAP - 1;  // last owner with eo[owner] <= e0
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (eo[mid] <= e0) lo = mid;
-            else hi = mid - 1;
-        }
-        const int64_t e1 = min(e0 + FILL_RUN, total);
-        for (int64_t e = e0; e < e1; e++) {
-            while (lo + 1 < SOLO_CAP && eo[lo + 1] <= e) lo++;
-            const int32_t m = map2[ladj[lrow[slist[lo]] + (int32_t)(e - eo[lo])]];
-            if (m >= 0) {
-                const int p = atomicAdd(&fc[lo], 1);
-                if (p < sdeg[lo]) st_keep_u16(&sadj[srow[lo] + p], (uint16_t)m, keep);
-                else atomicExch(err, 4);
-            }
-        }
-    }
-}
-
-struct SoloArgs {
-    const int* ns;
-    const int32_t* sdeg;
-    const int32_t* fc;    // entries k_solo_fill wrote per row (must equal sdeg)
-    const int32_t* srow;  // exclusive prefix of sdeg: row i = sadj[srow[i], srow[i + 1])
-    const uint16_t* sadj;
-    const int32_t* sgid;  // global vertex id
-    int32_t* rnd;
-    int32_t* core;
-    int* ctl;
-};
-
-// Once at most BM_CAP vertices are left, their induced subgraph moves into shared memory
-// as a bit matrix (row v, bit u: edge v-u), so that a round reads no global memory.
-constexpr int BM_CAP = 960;
-constexpr int BM_W = BM_CAP / 32;  // words per row
-
-struct SoloShared {
-    int cnt[3];                // frontier sizes, rotating over three rounds
-    int smin[2];               // smallest degree above the level, by level parity
-    int acnt[2];               // vertices alive at the level start, by level parity
-    int wsum[SOLO_THREADS / 32];
-    int sx[32], sb[32];        // small frontier: exclusive prefix of row lengths, row start - prefix
-    int sW;                    // small frontier: total row length
-    uint16_t coarse[SOLO_COARSE];  // large frontier: row holding flat entry b << cs
-    int32_t rs[SOLO_CAP + 1];
-    uint16_t FL[2][SOLO_CAP];  // frontier by round parity; FL[0] / FL[1] hold the bit-matrix phase's
-                               // id map / its small arrays
-    int32_t P[SOLO_PASS + 1];  // prefix of the row lengths of one pass of a large frontier
-    int32_t D[SOLO_PASS];      // row start - P: adjacency index of flat entry x is D[o] + x
-    union {
-        int32_t deg[SOLO_CAP];
-        uint32_t bm[BM_CAP * BM_W];  // bit-matrix phase (replaces deg)
-    } u;
-};
-static_assert(sizeof(SoloShared) <= 232448, "single-CTA phase exceeds the shared memory of a CTA");
-static_assert(4 * BM_CAP * 2 + 2 * BM_CAP * 3 <= 2 * SOLO_CAP, "bit-matrix phase arrays fit one frontier list");
-
-constexpr int SOLO_SLOTS = SOLO_CAP / SOLO_THREADS;  // vertices each thread checks at level starts
-static_assert(SOLO_CAP % SOLO_THREADS == 0 && SOLO_SLOTS <= 32, "level-start slots fit one mask word");
-
-// Appends solo id v to the frontier list for every lane with pred set (one shared-memory
-// atomic per warp). A list never holds more than SOLO_CAP entries (a vertex joins one
-// frontier); an append beyond that is dropped and the count, above SOLO_CAP, reports it.
-// The whole warp must call it.
-__device__ __forceinline__ void solo_append(bool pred, int v, uint16_t* fl, int* cnt) {
-    const unsigned m = __ballot_sync(0xffffffffu, pred);
-    if (!m) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(cnt, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    const int at = base + __popc(m & ((1u << lane) - 1u));
-    if (pred && at < SOLO_CAP) fl[at] = (uint16_t)v;
-}
-
-// The same append for one thread alone (no warp-wide step), into a list of cap entries.
-__device__ __forceinline__ void solo_push(int v, uint16_t* fl, int* cnt, int cap = SOLO_CAP) {
-    const int at = atomicAdd(cnt, 1);
-    if (at < cap) fl[at] = (uint16_t)v;
-}
-
-// Row entries at or past ns cannot come from rows that k_solo_fill checked; such an
-// entry is dropped and flags an internal error. Checked after all N loads were issued,
-// so that the loads overlap.
-template <int N>
-__device__ __forceinline__ void solo_check_rows(int (&vv)[N], int ns, int* ctl) {
-#pragma unroll
-    for (int c = 0; c < N; c++) {
-        if (vv[c] >= ns) {
-            atomicExch(&ctl[C_ERR], 5);
-            vv[c] = -1;
-        }
-    }
-}
-
-// Neighbours vv[0..N) (negative: none) lose one degree each at level k; a k + 1 -> k
-// crossing files the vertex in the next frontier. Only the first nch items can hold
-// neighbours; nch must be the same across the warp, which must call it whole.
-template <int N>
-__device__ __forceinline__ void solo_decrement(SoloShared& sh, const int (&vv)[N], int nch, int k, uint16_t* fn,
-                                               int* cn, const uint16_t* sadj) {
-    int old[N];
-#pragma unroll
-    for (int c = 0; c < N; c++) old[c] = vv[c] >= 0 ? atomicSub(&sh.u.deg[vv[c]], 1) : 0;
-#pragma unroll
-    for (int c = 0; c < N; c++) {
-        if (c < nch) {
-            const bool joins = vv[c] >= 0 && old[c] == k + 1;
-            solo_append(joins, vv[c], fn, cn);
-            // the next round reads this vertex's row: start its first line on the way to L1
-            if (joins) asm volatile("prefetch.global.L1 [%0];" ::"l"(sadj + sh.rs[vv[c]]));
-        }
-    }
-}
-
-// The last levels on the bit matrix. At entry every thread's mask lists its alive slots
-// (degree > k) at the start of level k + 1, n3 <= BM_CAP of them in all; the level starts
-// again here. New ids 0..n3-1 follow the slots in thread order; FL[0] maps slot -> new
-// id while the matrix is built, FL[1] holds the new ids' degrees, global ids, frontier
-// lists and slots. A round hands each frontier vertex to one warp, whose lanes each take
-// one 32-bit word of its row and decrement the degree of every neighbour in it.
-__device__ __forceinline__ void bm_phase(SoloShared& sh, const SoloArgs& a, int ns, int n3, unsigned mine, int& k,
-                                         int& r, int& rounds, int& lvl, int& steps, bool& bad) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint64_t keep = l2_keep_policy();
-    constexpr uint16_t NONE = 0xffff;
-    uint16_t* map = sh.FL[0];
-    int32_t* deg3 = reinterpret_cast<int32_t*>(sh.FL[1]);
-    int32_t* gid3 = deg3 + BM_CAP;
-    uint16_t* fl3 = reinterpret_cast<uint16_t*>(gid3 + BM_CAP);  // two lists of BM_CAP
-    uint16_t* n2o = fl3 + 2 * BM_CAP;
-    // ---- new ids: block-wide exclusive prefix of the alive slot counts
-    for (int i = tid; i < SOLO_CAP; i += SOLO_THREADS) map[i] = NONE;
-    const int mc = __popc(mine);
-    int inc = mc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    __syncthreads();  // the level start's reads of wsum and the frontier counts are done
-    if (lane == 31) sh.wsum[warp] = inc;
-    if (tid == 0) {
-        sh.cnt[(r + 1) % 3] = 0;  // the frontier filed by the level start is dropped
-        sh.smin[lvl & 1] = INT_MAX;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const int w = sh.wsum[lane];
-        int wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        sh.wsum[lane] = wi - w;
-    }
-    __syncthreads();
-    int id = sh.wsum[warp] + inc - mc;
-    for (unsigned m = mine; m; m &= m - 1) {
-        const int i = tid + (__ffs(m) - 1) * SOLO_THREADS;
-        if (id < BM_CAP) {
-            map[i] = (uint16_t)id;
-            n2o[id] = (uint16_t)i;
-            deg3[id] = sh.u.deg[i];
-            gid3[id] = a.sgid[i];
-        }
-        id++;
-    }
-    __syncthreads();
-    // ---- the matrix (it overlays the degrees just copied)
-    for (int w = tid; w < BM_CAP * BM_W; w += SOLO_THREADS) sh.u.bm[w] = 0;
-    __syncthreads();
-    for (int v = warp; v < n3; v += SOLO_THREADS / 32) {
-        const int o = n2o[v];
-        const int b = sh.rs[o], e = sh.rs[o + 1];
-        for (int j0 = b; j0 < e; j0 += 8 * 32) {
-            int nb[8];
-#pragma unroll
-            for (int t = 0; t < 8; t++) {
-                const int j = j0 + t * 32 + lane;
-                nb[t] = j < e ? ld_keep_u16(&a.sadj[j], keep) : -1;
-            }
-#pragma unroll
-            for (int t = 0; t < 8; t++) {
-                if (nb[t] < 0 || nb[t] >= ns) continue;
-                const int u = map[nb[t]];
-                if (u != NONE) atomicOr(&sh.u.bm[v * BM_W + (u >> 5)], 1u << (u & 31));
-            }
-        }
-    }
-    // ---- levels and rounds on the matrix
-    while (true) {
-        __syncthreads();
-        uint16_t* fs = fl3 + ((r + 1) & 1) * BM_CAP;
-        int* cs = &sh.cnt[(r + 1) % 3];
-        int kk = k + 1, lmin = INT_MAX;
-        if (tid < n3) {
-            const int d = deg3[tid];
-            if (d > k) {
-                if (d <= kk) solo_push(tid, fs, cs, BM_CAP);
-                else lmin = d;
-            }
-        }
-        lmin = __reduce_min_sync(0xffffffffu, lmin);
-        if (lane == 0 && lmin != INT_MAX) atomicMin(&sh.smin[lvl & 1], lmin);
-        __syncthreads();
-        const int c0 = *cs, m0 = sh.smin[lvl & 1];
-        if (tid == 0) sh.smin[(lvl + 1) & 1] = INT_MAX;
-        if (++steps > 2 * ns + 2 || c0 > BM_CAP) {
-            bad = true;
-            return;
-        }
-        if (c0 == 0) {
-            if (m0 == INT_MAX) return;  // nothing left
-            kk = m0;
-            __syncthreads();  // every thread has read c0 before the jump appends
-            if (tid < n3) {
-                const int d = deg3[tid];
-                if (d > k && d <= kk) solo_push(tid, fs, cs, BM_CAP);
-            }
-        }
-        k = kk;
-        r += 1;
-        lvl++;
-        while (true) {
-            __syncthreads();  // the round's frontier is complete
-            const int nL = sh.cnt[r % 3];
-            if (tid == 0) sh.cnt[(r + 2) % 3] = 0;
-            if (nL == 0) break;
-            if (++steps > 2 * ns + 2 || nL > BM_CAP) {
-                bad = true;
-                return;
-            }
-            const uint16_t* fl = fl3 + (r & 1) * BM_CAP;
-            uint16_t* fn = fl3 + ((r + 1) & 1) * BM_CAP;
-            int* cn = &sh.cnt[(r + 1) % 3];
-            // 32 S threads per frontier vertex (S = 4, 2, 1 as the frontier grows): thread t
-            // takes bits [(t / 32) 32 / S, (t / 32 + 1) 32 / S) of word t % 32 of the row, so
-            // that a small frontier spreads its decrements over more lanes
-            const int S = nL <= 8 ? 4 : nL <= 16 ? 2 : 1;
-            const int per = 32 * S, bits = 32 / S;
-            const int sub = tid % per, wd = sub & 31;
-            const unsigned slice = S == 1 ? 0xffffffffu : (((1u << bits) - 1u) << ((sub >> 5) * bits));
-            for (int i = tid / per; i < nL; i += SOLO_THREADS / per) {
-                const int v = fl[i];
-                if (wd < BM_W) {
-                    unsigned w = sh.u.bm[v * BM_W + wd] & slice;
-                    while (w) {
-                        const int u = wd * 32 + __ffs(w) - 1;
-                        w &= w - 1;
-                        if (atomicSub(&deg3[u], 1) == k + 1) solo_push(u, fn, cn, BM_CAP);
-                    }
-                }
-                if (sub == 0) {
-                    a.rnd[gid3[v]] = r;
-                    a.core[gid3[v]] = k;
-                }
-            }
-            r++;
-            rounds++;
-        }
-    }
-}
-
-// The same peeling once more (levels, rounds, k + 1 -> k crossings), continuing the level
-// k and round r where the cluster stopped. A round lays the frontier's rows out flat (a
-// prefix of their lengths) and deals the entries to all threads alike. A frontier of at
-// most 32 vertices (most rounds) is laid out by every warp in its own registers, so such
-// a round costs one barrier, one adjacency load and one shared-memory decrement per
-// entry; a larger one goes through shared memory in passes of SOLO_PASS vertices. At a
-// level start each thread checks the vertices it owns (tid + j SOLO_THREADS) that were
-// still alive at the previous one.
-__global__ void __launch_bounds__(SOLO_THREADS, 1) k_peel_solo(SoloArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    SoloShared& sh = *reinterpret_cast<SoloShared*>(smem);
-    if (a.ctl[C_SOLO] != 1 || a.ctl[C_ERR] != 0) return;
-    const int ns = *a.ns;
-    if (ns > SOLO_CAP) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint64_t keep = l2_keep_policy();
-    int miscount = 0;
-    for (int i = tid; i <= ns; i += SOLO_THREADS) {
-        if (i < ns) {
-            sh.u.deg[i] = a.sdeg[i];
-            miscount |= a.fc[i] != a.sdeg[i];
-        }
-        sh.rs[i] = a.srow[i];
-    }
-    unsigned mine = 0;  // owned slots alive at the last level start
-    for (int j = 0; j < SOLO_SLOTS; j++)
-        if (tid + j * SOLO_THREADS < ns) mine |= 1u << j;
-    if (tid < 3) sh.cnt[tid] = 0;
-    if (tid < 2) {
-        sh.smin[tid] = INT_MAX;
-        sh.acnt[tid] = 0;
-    }
-    int k = a.ctl[C_SOLO_K], r = a.ctl[C_SOLO_R], rounds = a.ctl[C_ROUNDS], lvl = 0;
-    int n3 = 0;  // vertices handed to the bit-matrix phase
-    // every level and every round removes at least one vertex: more than 2 ns + 2 steps
-    // (or a frontier above SOLO_CAP) can only come from an internal error
-    int steps = 0;
-    bool bad = false;
-    if (__syncthreads_or(miscount)) {
-        if (tid == 0) atomicExch(&a.ctl[C_ERR], 4);
-        return;
-    }
-    while (true) {
-        // ---- level start: vertices of degree k + 1 (or the smallest degree) join round
-        // r + 1 (r is the empty round that ended the last level, or the hand-off round)
-        uint16_t* fs = sh.FL[(r + 1) & 1];
-        int* cs = &sh.cnt[(r + 1) % 3];
-        int kk = k + 1, lmin = INT_MAX, na = 0;
-        for (unsigned m = mine; m; m &= m - 1) {
-            const int j = __ffs(m) - 1, i = tid + j * SOLO_THREADS;
-            const int d = sh.u.deg[i];
-            if (d <= k) {
-                mine &= ~(1u << j);  // left at an earlier level
-                continue;
-            }
-            na++;
-            if (d <= kk) solo_push(i, fs, cs);
-            else lmin = min(lmin, d);
-        }
-        lmin = __reduce_min_sync(0xffffffffu, lmin);
-        na = __reduce_add_sync(0xffffffffu, na);
-        if (lane == 0) {
-            if (lmin != INT_MAX) atomicMin(&sh.smin[lvl & 1], lmin);
-            if (na) atomicAdd(&sh.acnt[lvl & 1], na);
-        }
-        __syncthreads();
-        const int c0 = *cs, m0 = sh.smin[lvl & 1], alive = sh.acnt[lvl & 1];
-        if (tid == 0) {  // both last read at the previous level start
-            sh.smin[(lvl + 1) & 1] = INT_MAX;
-            sh.acnt[(lvl + 1) & 1] = 0;
-        }
-        if (++steps > 2 * ns + 2 || c0 > SOLO_CAP) {
-            bad = true;
-            break;
-        }
-        if (c0 == 0 && m0 == INT_MAX) break;  // nothing left
-        if (alive <= BM_CAP) {  // the rest fits the bit matrix (this level starts again there)
-            n3 = alive;
-            break;
-        }
-        if (c0 == 0) {
-            kk = m0;                   // jump to the smallest remaining degree
-            __syncthreads();           // every thread has read c0 before the jump appends
-            for (unsigned m = mine; m; m &= m - 1) {
-                const int i = tid + (__ffs(m) - 1) * SOLO_THREADS;
-                if (sh.u.deg[i] <= kk) solo_push(i, fs, cs);  // every kept slot has degree > k + 1
-            }
-        }
-        k = kk;
-        r += 1;
-        lvl++;
-        // ---- rounds at level k
-        while (true) {
-            __syncthreads();  // the round's frontier is complete
-            const int nL = sh.cnt[r % 3];
-            if (tid == 0) sh.cnt[(r + 2) % 3] = 0;  // read in round r - 1, appended to in round r + 1
-            if (nL == 0) break;
-            if (++steps > 2 * ns + 2 || nL > SOLO_CAP) {
-                bad = true;
-                break;
-            }
-            const uint16_t* fl = sh.FL[r & 1];
-            uint16_t* fn = sh.FL[(r + 1) & 1];
-            int* cn = &sh.cnt[(r + 1) % 3];
-            if (nL <= 32) {
-                // warp 0 lays the (at most 32) rows out: lane o holds frontier vertex o
-                int gid = -1;
-                if (warp == 0) {
-                    const bool have = lane < nL;
-                    const int q = have ? fl[lane] : 0;
-                    const int rb = have ? sh.rs[q] : 0;
-                    const int len = have ? sh.rs[q + 1] - rb : 0;
-                    if (have) gid = a.sgid[q];
-                    int inc = len;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    sh.sx[lane] = inc - len;
-                    sh.sb[lane] = rb - (inc - len);
-                    if (lane == 31) sh.sW = inc;
-                }
-                __syncthreads();
-                const int W = sh.sW;
-                for (int x0 = 0; x0 < W; x0 += SOLO_THREADS * SOLO_CHUNK_S) {
-                    if (x0 + warp * 32 >= W) break;  // nothing left for this warp (warp-uniform)
-                    const int nch = min(SOLO_CHUNK_S, (W - x0 + SOLO_THREADS - 1) / SOLO_THREADS);  // block-uniform
-                    int vv[SOLO_CHUNK_S];
-#pragma unroll
-                    for (int c = 0; c < SOLO_CHUNK_S; c++) {
-                        const int x = x0 + c * SOLO_THREADS + tid;
-                        vv[c] = -1;
-                        if (c < nch && x < W) {
-                            int lo = 0;  // last row o < nL with sx[o] <= x
-#pragma unroll
-                            for (int st = 16; st > 0; st >>= 1)
-                                if (lo + st < nL && sh.sx[lo + st] <= x) lo += st;
-                            vv[c] = ld_keep_u16(&a.sadj[sh.sb[lo] + x], keep);
-                        }
-                    }
-                    solo_check_rows(vv, ns, a.ctl);
-                    solo_decrement(sh, vv, nch, k, fn, cn, a.sadj);
-                }
-                if (gid >= 0) {
-                    a.rnd[gid] = r;
-                    a.core[gid] = k;
-                }
-            } else {
-                for (int p0 = 0; p0 < nL; p0 += SOLO_PASS) {
-                    const int np = min(SOLO_PASS, nL - p0);
-                    // two frontier vertices per thread: row lengths, global ids
-                    int len[2], rb[2], gid[2];
-#pragma unroll
-                    for (int u = 0; u < 2; u++) {
-                        const int i = 2 * tid + u;
-                        len[u] = 0;
-                        rb[u] = 0;
-                        gid[u] = -1;
-                        if (i < np) {
-                            const int q = fl[p0 + i];
-                            rb[u] = sh.rs[q];
-                            len[u] = sh.rs[q + 1] - rb[u];
-                            gid[u] = a.sgid[q];
-                        }
-                    }
-                    // block-wide exclusive prefix of the thread sums
-                    const int mysum = len[0] + len[1];
-                    int inc = mysum;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    if (lane == 31) sh.wsum[warp] = inc;
-                    __syncthreads();
-                    if (warp == 0) {
-                        int w = sh.wsum[lane], wi = w;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int y = __shfl_up_sync(0xffffffffu, wi, o);
-                            if (lane >= o) wi += y;
-                        }
-                        sh.wsum[lane] = wi - w;  // exclusive warp offsets
-                        if (lane == 31) sh.P[np] = wi;
-                    }
-                    __syncthreads();
-                    const int ex = sh.wsum[warp] + inc - mysum;
-#pragma unroll
-                    for (int u = 0; u < 2; u++) {
-                        const int i = 2 * tid + u;
-                        if (i < np) {
-                            const int off = ex + (u ? len[0] : 0);
-                            sh.P[i] = off;
-                            sh.D[i] = rb[u] - off;
-                        }
-                    }
-                    __syncthreads();
-                    const int W = sh.P[np];
-                    // coarse owners: entry b << cs lies in row coarse[b] (cs keeps W >> cs below
-                    // SOLO_COARSE), so that an entry's row is searched between two of them
-                    const int cs = max(4, 32 - __clz(max(W, 1) >> 10));
-#pragma unroll
-                    for (int u = 0; u < 2; u++) {
-                        const int i = 2 * tid + u;
-                        if (i < np) {
-                            const int b0 = (sh.P[i] + (1 << cs) - 1) >> cs, b1 = (sh.P[i + 1] + (1 << cs) - 1) >> cs;
-                            for (int b = b0; b < b1 && b < SOLO_COARSE; b++) sh.coarse[b] = (uint16_t)i;
-                        }
-                    }
-                    __syncthreads();
-                    for (int x0 = 0; x0 < W; x0 += SOLO_THREADS * SOLO_CHUNK) {
-                        if (x0 + warp * 32 >= W) break;  // nothing left for this warp (warp-uniform)
-                        const int nch = min(SOLO_CHUNK, (W - x0 + SOLO_THREADS - 1) / SOLO_THREADS);
-                        int vv[SOLO_CHUNK];
-#pragma unroll
-                        for (int c = 0; c < SOLO_CHUNK; c++) {
-                            const int x = x0 + c * SOLO_THREADS + tid;
-                            vv[c] = -1;
-                            if (c < nch && x < W) {
-                                const int b = x >> cs;  // last row with P[row] <= x, from coarse[b]
-                                int lo = sh.coarse[b], hi = ((b + 1) << cs) < W ? sh.coarse[b + 1] : np - 1;
-                                while (lo < hi) {
-                                    const int mid = (lo + hi + 1) >> 1;
-                                    if (sh.P[mid] <= x) lo = mid;
-                                    else hi = mid - 1;
-                                }
-                                vv[c] = ld_keep_u16(&a.sadj[sh.D[lo] + x], keep);
-                            }
-                        }
-                        solo_check_rows(vv, ns, a.ctl);
-                        solo_decrement(sh, vv, nch, k, fn, cn, a.sadj);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 2; u++) {
-                        if (gid[u] >= 0) {
-                            a.rnd[gid[u]] = r;
-                            a.core[gid[u]] = k;
-                        }
-                    }
-                    __syncthreads();  // P and D are rewritten by the next pass
-                }
-            }
-            r++;
-            rounds++;
-        }
-        if (bad) break;
-    }
-    if (n3 > 0 && !bad) bm_phase(sh, a, ns, n3, mine, k, r, rounds, lvl, steps, bad);
-    // the rows' lines go back to normal eviction priority
-    for (int x = tid * 64; x < sh.rs[ns]; x += SOLO_THREADS * 64) l2_release_line(a.sadj + x);
-    if (tid == 0) {
-        if (bad) atomicExch(&a.ctl[C_ERR], 2);
-        a.ctl[C_ROUNDS] = rounds;
-        a.ctl[C_ALPHA] = k;
-    }
-}
-
-static void launch_solo(const SoloArgs& sa, cudaStream_t s) {
-    const int smem = (int)sizeof(SoloShared);
-    FOLTY_CUDA(cudaFuncSetAttribute(k_peel_solo, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FOLTY_LAUNCH(k_peel_solo, 1, SOLO_THREADS, smem, s, sa);
-}
-
-__global__ void k_iota(int32_t* __restrict__ a, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = (int32_t)i;
-}
-
 // ================================================================== A4
 
 __device__ __forceinline__ bool rank_less(int32_t u, int32_t v, const int32_t* __restrict__ rnd) {
@@ -2551,6 +995,8 @@ class SideStream {
     bool forked_ = false;
 };
 
+constexpr int64_t STORE_BESIDE = 8;  // temporal edges per static one from which the store runs beside the core numbers
+
 // The sorted values index other arrays: a sort whose look-back ran out must stop here
 // (read_back checks the graph's error word).
 static void sort_check(folty_graph* g, cudaStream_t s) { read_back(g, nullptr, nullptr, 0, nullptr, s); }
@@ -2868,7 +1314,6 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     // triangle passes (which need only its per-pair counts). On an error in between, the
     // side streams are drained before the call's buffers go.
     SideStream side(s, false);
-    SideStream hi(s, true);
     struct EventHolder {
         cudaEvent_t e = nullptr;
         ~EventHolder() {
@@ -2922,120 +1367,25 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         FOLTY_LAUNCH(k_fill_adj, grid_for(S, T), T, 0, s, g->ea, g->eb, S, rowptr, deg_lo, hi_first, lo_first,
                      by_b, adj, adj_eid, adj_src, g->binv);
 
-    // ---------------- A3: peeling
-    int* peel_ctl = nullptr;
+    // ---------------- A3: core numbers and the removal order
     g->core = graph_alloc<int32_t>(g, n, s);
-    int32_t* core = g->core;
     int32_t* rnd = sc.get<int32_t>(n);
-    {
-        PeelArgs pa;
-        pa.rowptr = rowptr;
-        pa.adj = adj;
-        pa.n = n;
-        pa.deg = sc.get<int32_t>(n);
-        FOLTY_CUDA(cudaMemcpyAsync(pa.deg, g->deg, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        FOLTY_CUDA(cudaMemsetAsync(rnd, 0xff, sizeof(int32_t) * (size_t)n, s));
-        pa.rnd = rnd;
-        pa.core = core;
-        pa.alive[0] = sc.get<int32_t>(n);
-        pa.alive[1] = sc.get<int32_t>(n);
-        pa.fr[0] = sc.get<int32_t>(n);
-        pa.fr[1] = sc.get<int32_t>(n);
-        pa.hcap = (int32_t)((int64_t)n + (2 * (int64_t)S) / PEEL_PIECE + 1);
-        pa.hr[0] = sc.get<int64_t>(pa.hcap);
-        pa.hr[1] = sc.get<int64_t>(pa.hcap);
-        pa.ctl = sc.get<int>(C_SLOTS);
-        pa.timeout_ns = 10ll * 1000 * 1000 * 1000;
-        const int tail_c = tail_cluster_size(s);
-        pa.tail_n = TAIL_OWN * tail_c;
-        int init[C_SLOTS] = {0};
-        init[C_MIN] = INT_MAX;
-        init[C_MIN + 1] = INT_MAX;
-        int* init_dev = (int*)(g->host_stage + READBACK_MAX + 16);  // pinned staging
-        std::memcpy(init_dev, init, sizeof(init));
-        g->stage_busy = 1;
-        FOLTY_CUDA(cudaMemcpyAsync(pa.ctl, init_dev, sizeof(init), cudaMemcpyHostToDevice, s));
-        FOLTY_LAUNCH(k_iota, grid_for(n, T), T, 0, s, pa.alive[0], (int64_t)n);
-        int per_sm = 0;
-        FOLTY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel, PEEL_THREADS, 0));
-        if (per_sm < 1) fail(FOLTY_ECUDA, "peeling kernel cannot be resident");
-        if (per_sm > 1) per_sm = 1;
-        dim3 grid(num_sms() * per_sm), block(PEEL_THREADS);
-        void* args[] = {&pa};
-        StageSpan span(ST_PEEL, s, 12 * 2 * (int64_t)S + 16 * (int64_t)n);
-        if (n > 0) {
-            FOLTY_CUDA(cudaLaunchCooperativeKernel((const void*)k_peel, grid, block, args, 0, s));
-            after_launch("k_peel");
-        }
-        // the store and, at the end of its stream, the run-ends table (ready when it is
-        // joined), after the grid peel: the cooperative peel waits for SMs that the store's
-        // blocks hold (it took 0.8 ms instead of 0.3 beside the store's first pass), and
-        // the store still ends before the triangle listing
-        if (ids) {
-            store_s = side.fork();
-            Scratch sc2(g->alloc, store_s, g->dev_err);
-            temporal_store(g, job, sc2, sigma, packed_ev.e);
-            build_run_ends(g, store_s);
-        }
-        if (n > 0) {
-            // the cluster and single-CTA phases: latency-bound chains of small rounds, on
-            // a high-priority side stream so that their blocks go first on SMs that the
-            // temporal store's kernels free
-            const cudaStream_t ts = hi.fork();
-            Scratch sct(g->alloc, ts, g->dev_err);
-            // cluster tail on the induced subgraph of the vertices the grid kernel left;
-            // always enqueued (its kernels do nothing when the grid kernel finished), so
-            // no host round trip separates the two
-            const int tn = pa.tail_n;
-            int32_t* L = sct.get<int32_t>(tn);
-            int32_t* gmap = sct.get<int32_t>(n);
-            int32_t* ld = sct.get<int32_t>(tn + 1);
-            int32_t* d0 = sct.get<int32_t>(tn + 1);
-            int32_t* lrow = sct.get<int32_t>(tn + 1);
-            int32_t* eoff = sct.get<int32_t>(tn + 1);
-            // zeroed together: the local vertex count, then the fill counters
-            int32_t* zblk = sct.get<int32_t>(tn + 1);
-            int* nl = zblk;
-            int32_t* fillc = zblk + 1;
-            uint32_t* ladj = sct.get<uint32_t>(2 * (int64_t)S);
-            FOLTY_CUDA(cudaMemsetAsync(zblk, 0, sizeof(int32_t) * (size_t)(tn + 1), ts));
-            FOLTY_LAUNCH(k_tail_select, grid_for(n, T), T, 0, ts, pa.alive[0], pa.alive[1], pa.ctl, rnd, tn, L, gmap,
-                         nl, pa.ctl + C_ERR);
-            FOLTY_LAUNCH(k_tail_degrees, grid_for(tn, T), T, 0, ts, L, nl, pa.deg, rowptr, tn, ld, d0);
-            exclusive_scan(sct, ld, lrow, tn);
-            exclusive_scan(sct, d0, eoff, tn);
-            FOLTY_LAUNCH(k_tail_fill, grid_for(2 * (int64_t)S, T), T, 0, ts, L, eoff, tn, rowptr, adj, rnd, gmap,
-                         lrow, ld, fillc, ladj, pa.ctl + C_ERR);
-            // single-CTA phase for the last SOLO_CAP vertices (does nothing unless the
-            // cluster hands off)
-            // zeroed together: the exported count, the degrees, the fill counters
-            int32_t* sblk = sct.get<int32_t>(1 + (SOLO_CAP + 1) + SOLO_CAP);
-            int* ns = sblk;
-            int32_t* sdeg = sblk + 1;
-            int32_t* fc = sdeg + (SOLO_CAP + 1);
-            int32_t* slist = sct.get<int32_t>(SOLO_CAP);
-            int32_t* srow = sct.get<int32_t>(SOLO_CAP + 1);
-            int32_t* dl = sct.get<int32_t>(SOLO_CAP + 1);
-            int32_t* eo = sct.get<int32_t>(SOLO_CAP + 1);
-            int32_t* sgid = sct.get<int32_t>(SOLO_CAP);
-            int32_t* map2 = sct.get<int32_t>(tn);
-            uint16_t* sadj = sct.get<uint16_t>(2 * (int64_t)S);
-            FOLTY_CUDA(cudaMemsetAsync(sblk, 0, sizeof(int32_t) * (size_t)(1 + (SOLO_CAP + 1) + SOLO_CAP), ts));
-            FOLTY_CUDA(cudaMemsetAsync(map2, 0xff, sizeof(int32_t) * (size_t)tn, ts));
-            int32_t* tdec = sct.get<int32_t>((int64_t)TAIL_OWN * tail_c);
-            FOLTY_CUDA(cudaMemsetAsync(tdec, 0, sizeof(int32_t) * (size_t)TAIL_OWN * (size_t)tail_c, ts));
-            TailArgs ta{nl, L, ld, lrow, ladj, rnd, core, pa.ctl, SOLO_CAP, ns, slist, sdeg, map2, tdec};
-            if (tail_c == 16) launch_tail<16>(ta, ts);
-            else launch_tail<8>(ta, ts);
-            FOLTY_LAUNCH(k_solo_rows, grid_for(SOLO_CAP, T), T, 0, ts, pa.ctl, ns, slist, lrow, L, dl, sgid);
-            exclusive_scan(sct, sdeg, srow, SOLO_CAP);
-            exclusive_scan(sct, dl, eo, SOLO_CAP);
-            FOLTY_LAUNCH(k_solo_fill, grid_for(2 * (int64_t)S, T), T, 0, ts, pa.ctl, eo, slist, sdeg, srow, lrow, ladj,
-                         map2, fc, sadj, pa.ctl + C_ERR);
-            launch_solo(SoloArgs{ns, sdeg, fc, srow, sadj, sgid, rnd, core, pa.ctl}, ts);
-            hi.join();
-        }
-        peel_ctl = pa.ctl;  // rounds, alpha and the error word are read with the triangle totals
+    // The store and, at the end of its stream, the run-ends table (ready when it is joined).
+    // The core numbers' cooperative kernel waits for SMs that the store's blocks hold, so it is
+    // launched first. Where the store is the longer of the two (many temporal edges per static
+    // one) it takes half the SMs, whose registers it fills, and the store the others: most of
+    // its rounds are bound by latency. Preprocessing of 20M edges, 24 per pair: 1.64 ms
+    // against 1.92 one after the other; of 6M edges, 2 per pair: 3.66 against 3.51.
+    const bool beside = ids && g->m_kept >= STORE_BESIDE * (int64_t)S;
+    if (beside) store_s = side.fork();
+    // rounds, alpha and the error word are read with the triangle totals
+    const int* core_ctl =
+        enqueue_core_numbers(g, rowptr, adj, adj_src, rnd, beside ? std::max(num_sms() / 2, 1) : num_sms(), sc, s);
+    if (ids) {
+        if (!beside) store_s = side.fork();
+        Scratch sc2(g->alloc, store_s, g->dev_err);
+        temporal_store(g, job, sc2, sigma, packed_ev.e);
+        build_run_ends(g, store_s);
     }
 
     // ---------------- A4: orientation
@@ -3111,15 +1461,12 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     int64_t bound = 0;
     {
         const void* ptrs[9] = {bounded ? (const void*)(boff + S) : (const void*)(toff + S), stat + 0, stat + 1,
-                               stat + 2, merged, merged + 1, peel_ctl + C_ERR, peel_ctl + C_ROUNDS, peel_ctl + C_ALPHA};
+                               stat + 2, merged, merged + 1, core_ctl + CORE_ERR, core_ctl + CORE_ROUNDS, core_ctl + CORE_ALPHA};
         int sizes[9] = {8, 4, 4, 4, 8, 8, 4, 4, 4};
         int64_t outv[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-        read_back(g, ptrs, sizes, peel_ctl ? 9 : 6, outv, s);  // no peeling state for n = 0
-        if (outv[6] == 1) fail(FOLTY_ETIMEOUT, "peeling: a grid barrier wait ran out");
-        if (outv[6] != 0)
-            fail(FOLTY_ECUDA, "peeling: internal error " + std::to_string(outv[6]) +
-                                  " (2: a vertex list overflowed, 3/4: a subgraph row count differs, 5: a row entry "
-                                  "is out of range)");
+        read_back(g, ptrs, sizes, 9, outv, s);
+        if (outv[6] == 1) fail(FOLTY_ETIMEOUT, "core numbers: a grid barrier wait ran out");
+        if (outv[6] != 0) fail(FOLTY_ECUDA, "core numbers: a vertex list overflowed");
         g->info.peel_rounds = (int32_t)outv[7];
         g->info.degeneracy = (int32_t)outv[8];
         g->info.max_degree = (int32_t)outv[1];
