@@ -495,47 +495,58 @@ struct EdgeStat {
     }
 };
 
-__global__ void k_validate(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                           const int64_t* __restrict__ t, int64_t m, int32_t n,
-                           unsigned long long* __restrict__ stat) {
-    EdgeStat st;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x)
-        st.edge(i, src[i], dst[i], t[i], i > 0 ? t[i - 1] : 0, n);
-    st.flush(stat);
-}
-
-// The pair table's first try, filled while the load reads the edges (INSERT): the
-// slot word of every edge (PAIR_LOOP for a self-loop or an invalid edge, which fails the
-// load anyway).
-struct LoadPairs {
+// One pass over the edge list: its checks, the low 32 bits of its timestamps (the store's
+// offsets, once the range is known to fit), and with INSERT every edge's pair into the first
+// pair table and its slot word (PAIR_LOOP for a self-loop or an invalid edge, which fails the
+// load anyway). src, dst and t are device memory or pinned host memory (read over the host
+// link, as fast as a copy engine's pull). Nothing else of the input is kept: 16 B read and 8
+// written per edge, where copies of the three arrays took 16 B more; a table that turns out
+// not to serve, or a range of times past 32 bits, has the input copied afterwards.
+//
+// Four edges per thread and step (16-byte accesses when VEC; otherwise, and for the m mod 4
+// last edges, one by one), the previous edge's timestamp from the neighbouring lane; the four
+// edges' first probes in flight together (most find their pair, or an empty slot, there),
+// the rest of a probe sequence one edge at a time (advancing the four sequences together was
+// slower, 0.86 against 0.80 ms for 70M edges).
+struct LoadArgs {
+    const int32_t* src;
+    const int32_t* dst;
+    const int64_t* t;
+    int64_t m;
+    int32_t n;
+    uint32_t* t32;
+    unsigned long long* stat;
     uint64_t* table;
     int lg;
     uint32_t* slotw;
     int* flags;
 };
 
-template <bool INSERT>
-__device__ __forceinline__ uint32_t load_slot_word(const LoadPairs& lp, int32_t x, int32_t y, int32_t n) {
-    if (!INSERT || x < 0 || x >= n || y < 0 || y >= n) return PAIR_LOOP;
-    return pair_slot_word(lp.table, lp.lg, x, y, n, lp.flags);
+template <int E>
+__device__ __forceinline__ void load_slot_words(const LoadArgs& a, const int32_t (&x)[E], const int32_t (&y)[E],
+                                                uint32_t (&w)[E]) {
+    uint64_t key[E], h[E], cur[E];
+    bool ok[E];
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        ok[e] = x[e] >= 0 && x[e] < a.n && y[e] >= 0 && y[e] < a.n && x[e] != y[e];
+        key[e] = ok[e] ? pair_rank_of(x[e], y[e], a.n) + 1 : 0;
+        h[e] = (key[e] * PAIR_HASH_MUL) >> (64 - a.lg);
+        cur[e] = ok[e] ? __ldcg(&a.table[h[e]]) : 0;
+    }
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        if (!ok[e]) w[e] = PAIR_LOOP;
+        else if (cur[e] == key[e]) w[e] = (uint32_t)h[e] | (x[e] > y[e] ? PAIR_DIR : 0u);
+        else w[e] = pair_slot_word(a.table, a.lg, x[e], y[e], a.n, a.flags);
+    }
 }
 
-// The same checks fused with the copy of the input into the graph's own arrays: one
-// read and one write of every input byte. The input is device memory or pinned host
-// memory (read over the host link, as fast as a copy engine's pull); with INSERT the
-// edges' pairs also go into the pair table (work that the host link's pace leaves room
-// for). Four edges per thread and iteration (16-byte accesses; all pointers 16-byte
-// aligned), the previous edge's timestamp from the neighbouring lane, the m mod 4 last
-// edges one by one.
-template <bool INSERT>
-__global__ void k_load_copy(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                            const int64_t* __restrict__ t, int64_t m, int32_t n, int32_t* __restrict__ osrc,
-                            int32_t* __restrict__ odst, int64_t* __restrict__ ot,
-                            unsigned long long* __restrict__ stat, LoadPairs lp) {
+template <bool INSERT, bool VEC>
+__global__ void __launch_bounds__(256) k_load(const LoadArgs a) {
     EdgeStat st;
     const int lane = threadIdx.x & 31;
-    const int64_t m4 = m >> 2;
+    const int64_t m4 = VEC ? a.m >> 2 : 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;  // a multiple of 32
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (int64_t j0 = tid - lane; j0 < m4; j0 += stride) {  // warp-uniform trip count
@@ -543,59 +554,43 @@ __global__ void k_load_copy(const int32_t* __restrict__ src, const int32_t* __re
         const bool act = j < m4;
         int4 x{}, y{};
         longlong2 t01{}, t23{};
-        const bool over = INSERT && pair_table_over(lp.flags);  // the table serves no more
+        const bool over = INSERT && pair_table_over(a.flags);  // the table serves no more
         if (act) {
-            x = __ldcs(reinterpret_cast<const int4*>(src) + j);
-            y = __ldcs(reinterpret_cast<const int4*>(dst) + j);
-            t01 = __ldcs(reinterpret_cast<const longlong2*>(t) + 2 * j);
-            t23 = __ldcs(reinterpret_cast<const longlong2*>(t) + 2 * j + 1);
+            x = __ldcs(reinterpret_cast<const int4*>(a.src) + j);
+            y = __ldcs(reinterpret_cast<const int4*>(a.dst) + j);
+            t01 = __ldcs(reinterpret_cast<const longlong2*>(a.t) + 2 * j);
+            t23 = __ldcs(reinterpret_cast<const longlong2*>(a.t) + 2 * j + 1);
         }
         int64_t tp = __shfl_up_sync(0xffffffffu, (long long)t23.y, 1);
-        if (lane == 0) tp = j > 0 ? t[4 * j - 1] : 0;
+        if (lane == 0) tp = j > 0 ? a.t[4 * j - 1] : 0;
         if (act) {
-            reinterpret_cast<int4*>(osrc)[j] = x;
-            reinterpret_cast<int4*>(odst)[j] = y;
-            reinterpret_cast<longlong2*>(ot)[2 * j] = t01;
-            reinterpret_cast<longlong2*>(ot)[2 * j + 1] = t23;
+            __stcs(reinterpret_cast<uint4*>(a.t32) + j,
+                   make_uint4((uint32_t)t01.x, (uint32_t)t01.y, (uint32_t)t23.x, (uint32_t)t23.y));
             const int64_t i = 4 * j;
-            st.edge(i, x.x, y.x, t01.x, tp, n);
-            st.edge(i + 1, x.y, y.y, t01.y, t01.x, n);
-            st.edge(i + 2, x.z, y.z, t23.x, t01.y, n);
-            st.edge(i + 3, x.w, y.w, t23.y, t23.x, n);
+            st.edge(i, x.x, y.x, t01.x, tp, a.n);
+            st.edge(i + 1, x.y, y.y, t01.y, t01.x, a.n);
+            st.edge(i + 2, x.z, y.z, t23.x, t01.y, a.n);
+            st.edge(i + 3, x.w, y.w, t23.y, t23.x, a.n);
             if (INSERT && !over) {
-                // the four edges' first probes issued together (most find their pair, or
-                // an empty slot, there); the rest of a probe sequence one edge at a time
                 const int32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
                 uint32_t ws[4];
-                uint64_t key[4], h[4], cur[4];
-                bool ok[4];
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    ok[e] = xs[e] >= 0 && xs[e] < n && ys[e] >= 0 && ys[e] < n && xs[e] != ys[e];
-                    key[e] = ok[e] ? pair_rank_of(xs[e], ys[e], n) + 1 : 0;
-                    h[e] = (key[e] * PAIR_HASH_MUL) >> (64 - lp.lg);
-                    cur[e] = ok[e] ? __ldcg(&lp.table[h[e]]) : 0;
-                }
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    if (!ok[e]) ws[e] = PAIR_LOOP;
-                    else if (cur[e] == key[e]) ws[e] = (uint32_t)h[e] | (xs[e] > ys[e] ? PAIR_DIR : 0u);
-                    else ws[e] = load_slot_word<INSERT>(lp, xs[e], ys[e], n);
-                }
-                reinterpret_cast<uint4*>(lp.slotw)[j] = make_uint4(ws[0], ws[1], ws[2], ws[3]);
+                load_slot_words<4>(a, xs, ys, ws);
+                __stcs(reinterpret_cast<uint4*>(a.slotw) + j, make_uint4(ws[0], ws[1], ws[2], ws[3]));
             }
         }
     }
-    for (int64_t i = 4 * m4 + tid; i < m; i += stride) {
-        const int32_t x = src[i], y = dst[i];
-        const int64_t ti = t[i];
-        osrc[i] = x;
-        odst[i] = y;
-        ot[i] = ti;
-        st.edge(i, x, y, ti, i > 0 ? t[i - 1] : 0, n);
-        if (INSERT && !pair_table_over(lp.flags)) lp.slotw[i] = load_slot_word<INSERT>(lp, x, y, n);
+    for (int64_t i = 4 * m4 + tid; i < a.m; i += stride) {
+        const int32_t x[1] = {a.src[i]}, y[1] = {a.dst[i]};
+        const int64_t ti = a.t[i];
+        a.t32[i] = (uint32_t)ti;
+        st.edge(i, x[0], y[0], ti, i > 0 ? a.t[i - 1] : 0, a.n);
+        if (INSERT && !pair_table_over(a.flags)) {
+            uint32_t w[1];
+            load_slot_words<1>(a, x, y, w);
+            a.slotw[i] = w[0];
+        }
     }
-    st.flush(stat);
+    st.flush(a.stat);
 }
 
 // The address under which kernels of the current device read p: p itself for memory
@@ -617,75 +612,126 @@ static const void* kernel_address(const void* p) {
     return nullptr;
 }
 
+void release_input(folty_graph* g, cudaStream_t s) {
+    graph_release(g, g->in_t32, s);
+    graph_release(g, g->in_t, s);
+    graph_release(g, g->in_src, s);
+    graph_release(g, g->in_dst, s);
+    graph_release(g, g->pre_slotw, s);
+    graph_release(g, g->pre_rank, s);
+    graph_release(g, g->pre_slot, s);
+    g->in_t32 = g->pre_slotw = g->pre_slot = nullptr;
+    g->in_t = nullptr;
+    g->in_src = g->in_dst = nullptr;
+    g->pre_rank = nullptr;
+}
+
 static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, const int64_t* t,
                        cudaStream_t s) {
     const int64_t m = g->m;
-    g->in_src = graph_alloc<int32_t>(g, m, s);
-    g->in_dst = graph_alloc<int32_t>(g, m, s);
-    g->in_t = graph_alloc<int64_t>(g, m, s);
     g->dev_err = graph_alloc<int>(g, 1, s);
     FOLTY_CUDA(cudaMemsetAsync(g->dev_err, 0, sizeof(int), s));
-    auto a16 = [](const void* p) { return p && ((uintptr_t)p & 15) == 0; };
-    const void* ksrc = m > 0 ? kernel_address(src) : nullptr;
-    const void* kdst = m > 0 ? kernel_address(dst) : nullptr;
-    const void* kt = m > 0 ? kernel_address(t) : nullptr;
-    const bool fused = a16(ksrc) && a16(kdst) && a16(kt) && a16(g->in_src) && a16(g->in_dst) && a16(g->in_t);
-    if (m > 0 && !fused) {
+    auto a16 = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+    auto copy_edges = [&] {
+        g->in_src = graph_alloc<int32_t>(g, m, s);
+        g->in_dst = graph_alloc<int32_t>(g, m, s);
         FOLTY_CUDA(cudaMemcpyAsync(g->in_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, s));
         FOLTY_CUDA(cudaMemcpyAsync(g->in_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, s));
+    };
+    auto copy_times = [&] {
+        g->in_t = graph_alloc<int64_t>(g, m, s);
         FOLTY_CUDA(cudaMemcpyAsync(g->in_t, t, sizeof(int64_t) * (size_t)m, cudaMemcpyDefault, s));
-    }
+    };
+    g->in_t32 = graph_alloc<uint32_t>(g, m, s);
     Scratch sc(g->alloc, s, g->dev_err);
+    // the checks' results, then the table's flags
     unsigned long long* stat = sc.get<unsigned long long>(5);
     unsigned long long init[5] = {~0ull, ~0ull, 0ull, 0ull, 0ull};
     std::memcpy(g->host_stage + READBACK_MAX, init, sizeof(init));
     g->stage_busy = 1;
     FOLTY_CUDA(cudaMemcpyAsync(stat, g->host_stage + READBACK_MAX, sizeof(init), cudaMemcpyHostToDevice, s));
-    // the pair table's first try rides along with a fused load (the preprocessing uses
-    // it when its first try has the same size)
-    bool insert = fused && g->n >= 2 && !pair_table_forced_off();
-    LoadPairs lp{nullptr, 0, nullptr, nullptr};
-    if (insert) {
-        lp.lg = pair_table_lg_first(m);
-        g->pre_lg = lp.lg;
-        g->pre_table = graph_alloc<uint64_t>(g, 1ll << lp.lg, s);
-        g->pre_slotw = graph_alloc<uint32_t>(g, m, s);
-        g->pre_flags = graph_alloc<int>(g, PAIR_FLAGS, s);
-        if (!a16(g->pre_slotw)) {  // a caller's allocator may not align it for 16-byte stores
-            graph_release(g, g->pre_table, s);
-            graph_release(g, g->pre_slotw, s);
-            graph_release(g, g->pre_flags, s);
-            g->pre_table = nullptr;
-            g->pre_slotw = nullptr;
-            g->pre_flags = nullptr;
-            insert = false;
-        } else {
-            FOLTY_CUDA(cudaMemsetAsync(g->pre_table, 0, sizeof(uint64_t) * ((size_t)1 << lp.lg), s));
-            FOLTY_CUDA(cudaMemsetAsync(g->pre_flags, 0, PAIR_FLAGS * sizeof(int), s));
-            lp = LoadPairs{g->pre_table, lp.lg, g->pre_slotw, g->pre_flags};
+    int* flags = sc.get<int>(PAIR_FLAGS);
+    FOLTY_CUDA(cudaMemsetAsync(flags, 0, PAIR_FLAGS * sizeof(int), s));
+    const bool insert = m > 0 && g->n >= 2 && !pair_table_forced_off();
+    const int lg = insert ? pair_table_lg_first(m) : 0;
+    const int cap = insert ? (1 << lg) / 2 : 0;  // load factor at most 1/2
+    bool staged = false;  // in_src, in_dst and in_t hold the input
+    if (m > 0) {
+        LoadArgs a{(const int32_t*)kernel_address(src), (const int32_t*)kernel_address(dst),
+                   (const int64_t*)kernel_address(t), m, g->n, g->in_t32, stat, nullptr, lg, nullptr, flags};
+        if (!a.src || !a.dst || !a.t) {
+            copy_edges();
+            copy_times();
+            a.src = g->in_src;
+            a.dst = g->in_dst;
+            a.t = g->in_t;
+            staged = true;
+        }
+        if (insert) {
+            g->pre_slotw = graph_alloc<uint32_t>(g, m, s);
+            a.slotw = g->pre_slotw;
+            a.table = sc.get<uint64_t>(1ll << lg);
+            FOLTY_CUDA(cudaMemsetAsync(a.table, 0, sizeof(uint64_t) << lg, s));
+        }
+        const bool vec = a16(a.src) && a16(a.dst) && a16(a.t) && a16(a.t32) && a16(a.slotw);
+        const unsigned grid = grid_for(vec ? m / 4 + 1 : m, 256, 8);
+        if (insert && vec) FOLTY_LAUNCH((k_load<true, true>), grid, 256, 0, s, a);
+        else if (insert) FOLTY_LAUNCH((k_load<true, false>), grid, 256, 0, s, a);
+        else if (vec) FOLTY_LAUNCH((k_load<false, true>), grid, 256, 0, s, a);
+        else FOLTY_LAUNCH((k_load<false, false>), grid, 256, 0, s, a);
+        if (insert) {
+            g->pre_rank = graph_alloc<uint64_t>(g, cap, s);
+            g->pre_slot = graph_alloc<uint32_t>(g, cap, s);
+            enqueue_pair_list(a.table, lg, g->pre_rank, g->pre_slot, flags + 1, cap, s);
         }
     }
-    if (fused && insert)
-        FOLTY_LAUNCH(k_load_copy<true>, grid_for(m / 4 + 1, 256, 8), 256, 0, s, (const int32_t*)ksrc,
-                     (const int32_t*)kdst, (const int64_t*)kt, m, g->n, g->in_src, g->in_dst, g->in_t, stat, lp);
-    else if (fused)
-        FOLTY_LAUNCH(k_load_copy<false>, grid_for(m / 4 + 1, 256, 4), 256, 0, s, (const int32_t*)ksrc,
-                     (const int32_t*)kdst, (const int64_t*)kt, m, g->n, g->in_src, g->in_dst, g->in_t, stat, lp);
-    else if (m > 0)
-        FOLTY_LAUNCH(k_validate, grid_for(m, 256), 256, 0, s, g->in_src, g->in_dst, g->in_t, m, g->n, stat);
-    const void* ptrs[5] = {stat, stat + 1, stat + 2, stat + 3, stat + 4};
-    int sizes[5] = {8, 8, 8, 8, 8};
-    int64_t v[5];
-    read_back(g, ptrs, sizes, 5, v, s);
+    const void* ptrs[7] = {stat, stat + 1, stat + 2, stat + 3, stat + 4, flags, flags + 1};
+    int sizes[7] = {8, 8, 8, 8, 8, 4, 4};
+    int64_t v[7];
+    read_back(g, ptrs, sizes, 7, v, s);
     if ((unsigned long long)v[0] != ~0ull)
         fail(FOLTY_EINVAL, "edge " + std::to_string(v[0]) + ": vertex id outside [0, n) or timestamp outside [0, 2^62)");
     g->tmin = (m > 0) ? v[1] : 0;
     g->tmax = (m > 0) ? v[2] : 0;
+    // 32-bit offsets from tmin when the time range leaves room for the "none" marker
+    g->ts32 = (g->tmax - g->tmin) < (int64_t)0xffffffffll;
     g->info.time_sorted = v[3] ? 0 : 1;
     g->m_kept = m - v[4];
     g->info.n = g->n;
     g->info.m = m;
     g->info.m_kept = g->m_kept;
+    // what the preprocessing needs of the input beside the times' low bits
+    const bool serves = insert && v[5] == 0 && v[6] <= cap && g->m_kept > 0;
+    g->pre_lg = lg;
+    if (serves) {
+        g->pre_pairs = (int32_t)v[6];
+        graph_release(g, g->in_src, s);
+        graph_release(g, g->in_dst, s);
+        g->in_src = g->in_dst = nullptr;
+    } else {
+        graph_release(g, g->pre_slotw, s);
+        graph_release(g, g->pre_rank, s);
+        graph_release(g, g->pre_slot, s);
+        g->pre_slotw = g->pre_slot = nullptr;
+        g->pre_rank = nullptr;
+    }
+    bool copies = false;
+    if (!serves && !staged && m > 0) {
+        copy_edges();
+        copies = true;
+    }
+    if (g->ts32) {
+        graph_release(g, g->in_t, s);
+        g->in_t = nullptr;
+    } else {
+        graph_release(g, g->in_t32, s);
+        g->in_t32 = nullptr;
+        if (!staged && m > 0) {
+            copy_times();
+            copies = true;
+        }
+    }
+    if (copies) FOLTY_CUDA(cudaStreamSynchronize(s));  // the caller's arrays are not read after the call
 }
 
 template <typename F>

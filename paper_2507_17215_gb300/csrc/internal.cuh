@@ -160,16 +160,18 @@ struct folty_graph {
     int state;  // 0 loaded, 1 preprocessed
     int32_t n;
     int64_t m;
-    // ---- loaded input (device copies; released by preprocess)
+    // ---- loaded input (device; released by preprocess)
+    uint32_t* in_t32; // [m] low 32 bits of the timestamps, when their range fits 32 bits
+    int64_t* in_t;    // [m] the timestamps, when it does not
+    // the pair table the load filled (pairs.cuh), when it serves
+    int pre_lg;           // log2 of its slots (also of one that did not serve; 0: none tried)
+    uint32_t* pre_slotw;  // [m] slot word of each edge
+    uint64_t* pre_rank;   // the distinct pairs' ranks and slots, in no particular order
+    uint32_t* pre_slot;
+    int32_t pre_pairs;
+    // the edges themselves, when it does not
     int32_t* in_src;
     int32_t* in_dst;
-    int64_t* in_t;
-    // the first try of the pair table, filled by a load of device or pinned input
-    // (pairs.cuh; released by preprocess): table of 2^pre_lg slots, slot words, flags
-    uint64_t* pre_table;
-    uint32_t* pre_slotw;
-    int* pre_flags;
-    int pre_lg;
     // ---- preprocessed store (device)
     int64_t m_kept;
     int32_t* perm;    // [m_kept] input index of each sorted temporal edge (null while cw
@@ -238,6 +240,8 @@ T* graph_alloc(folty_graph* g, int64_t count, cudaStream_t s) {
     return static_cast<T*>(p);
 }
 void graph_release(folty_graph* g, void* p, cudaStream_t s);
+// Releases what the load kept of the input.
+void release_input(folty_graph* g, cudaStream_t s);
 
 // Reads `count` int64 values from device memory through the graph's pinned staging
 // buffer (synchronises the stream). Also reads the graph's device error word: when a
@@ -275,7 +279,7 @@ bool radix_sort_pairs(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, uint32_t*
 bool radix_sort_keys(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, int64_t n, int lo, int bits);
 
 // The temporal store's sort of a time-ordered edge list: the n edges by sort id cw[j]
-// (< 2^cbits; equal ids keep input order), each carrying its time offset t[j] - tmin;
+// (< 2^cbits; equal ids keep input order), each carrying its time offset t[j] - tmin (modulo 2^32);
 // sorted position i < limit receives T[i] = t[j] - tmin and sd[i] = cw[j] (the positions
 // past limit hold the largest ids and are dropped). hist[p][b]: the number of ids whose
 // 8-bit digit p (bits 8p ...) is b, for the ceil(cbits / 8) passes, counted by the
@@ -285,8 +289,8 @@ constexpr int STORE_DIGIT_BITS = 8;
 constexpr int STORE_MAX_PASSES = 4;
 struct StoreSortArgs {
     const uint32_t* cw;
-    const int64_t* t;
-    int64_t tmin;
+    const uint32_t* t;  // times, modulo 2^32
+    uint32_t tmin;
     int64_t n;
     int cbits;
     const uint32_t* hist;  // [STORE_MAX_PASSES][1 << STORE_DIGIT_BITS]

@@ -1,5 +1,5 @@
-// The dense pair-id table shared by the load (which fills it while it copies device or
-// pinned input) and the preprocessing (which fills it otherwise, and numbers its pairs).
+// The dense pair-id table shared by the load (which fills it while it reads the edges) and
+// the preprocessing (which tries a larger one otherwise, and numbers its pairs).
 // An open-addressed table of 2^lg slots (linear probing from a multiplicative hash of the
 // pair rank); slot value = rank + 1, 0 = empty.
 #pragma once
@@ -32,12 +32,26 @@ __device__ __forceinline__ uint64_t pair_rank_of(int32_t x, int32_t y, int32_t n
 constexpr int PAIR_COUNTED = 64;
 constexpr int PAIR_COUNTED_LG = 20;
 
-// flags: [0] the table is abandoned, [1] distinct pairs (k_pair_table_compact), [2] pairs
-// placed in counted slots.
-constexpr int PAIR_FLAGS = 3;
+// flags: [0] the table is abandoned, [1] distinct pairs (k_pair_table_compact),
+// [PAIR_COUNT_AT] pairs placed in counted slots: additions to the line that every thread
+// reads [0] from made the load of 70M edges take 1.2 ms instead of 0.8.
+constexpr int PAIR_COUNT_AT = 64;
+constexpr int PAIR_FLAGS = PAIR_COUNT_AT + 32;
 
 // Whether the table is abandoned, on any thread: the edges still to come need no slot.
 __device__ __forceinline__ bool pair_table_over(const int* flags) { return *(const volatile int*)flags != 0; }
+
+// Places key in the empty slot h unless another thread was first; returns what the slot
+// then holds.
+__device__ __forceinline__ uint64_t pair_place(uint64_t* table, int lg, uint64_t h, uint64_t key, int* flags) {
+    const unsigned long long old = atomicCAS((unsigned long long*)&table[h], 0ull, (unsigned long long)key);
+    if (old != 0) return old;
+    if ((h & (PAIR_COUNTED - 1)) == 0 && lg >= PAIR_COUNTED_LG) {
+        const int most = (1 << lg) / 2 / PAIR_COUNTED;
+        if (atomicAdd(flags + PAIR_COUNT_AT, 1) >= most + most / 8) atomicExch(flags, 1);
+    }
+    return key;
+}
 
 // Slot holding table value key (rank + 1), placing it in the first empty slot of its probe
 // sequence when absent; -1 after PAIR_MAX_PROBE steps.
@@ -45,17 +59,9 @@ __device__ __forceinline__ int64_t pair_slot(uint64_t* table, int lg, uint64_t k
     const uint64_t mask = (1ull << lg) - 1;
     uint64_t h = (key * PAIR_HASH_MUL) >> (64 - lg);
     for (int pr = 0; pr < PAIR_MAX_PROBE; pr++) {
-        const uint64_t cur = __ldcg(&table[h]);
+        uint64_t cur = __ldcg(&table[h]);
+        if (cur == 0) cur = pair_place(table, lg, h, key, flags);
         if (cur == key) return (int64_t)h;
-        if (cur == 0) {
-            const unsigned long long old =
-                atomicCAS((unsigned long long*)&table[h], 0ull, (unsigned long long)key);
-            if (old == 0 && (h & (PAIR_COUNTED - 1)) == 0 && lg >= PAIR_COUNTED_LG) {
-                const int most = (1 << lg) / 2 / PAIR_COUNTED;
-                if (atomicAdd(flags + 2, 1) >= most + most / 8) atomicExch(flags, 1);
-            }
-            if (old == 0 || old == key) return (int64_t)h;
-        }
         h = (h + 1) & mask;
     }
     return -1;
@@ -92,6 +98,10 @@ inline int pair_table_lg_first(int64_t m) {
     b = b < PAIR_COUNTED_LG ? PAIR_COUNTED_LG : (b > 22 ? 22 : b);
     return pair_table_lg_max(m) < b ? pair_table_lg_max(m) : b;
 }
+
+// The occupied slots of a table as (rank, slot) lists (at most cap entries), their number
+// added to *cnt.
+void enqueue_pair_list(const uint64_t* table, int lg, uint64_t* rank, uint32_t* slot, int* cnt, int cap, cudaStream_t s);
 
 // The dense-id path is off when FOLTY_PAIR_SORT=keys (the full-key sort then runs).
 inline bool pair_table_forced_off() {

@@ -46,11 +46,12 @@ __global__ void k_build_keys(const int32_t* __restrict__ src, const int32_t* __r
     }
 }
 
-__global__ void k_time_keys(const int64_t* __restrict__ t, int64_t m, int64_t tmin,
+// The times as sort keys t - tmin (t32: modulo 2^32).
+__global__ void k_time_keys(const uint32_t* __restrict__ t32, const int64_t* __restrict__ t, int64_t m, int64_t tmin,
                             uint64_t* __restrict__ key, uint32_t* __restrict__ val) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
-        key[i] = (uint64_t)(t[i] - tmin);
+        key[i] = t32 ? (uint64_t)(t32[i] - (uint32_t)tmin) : (uint64_t)(t[i] - tmin);
         val[i] = (uint32_t)i;
     }
 }
@@ -62,28 +63,20 @@ __global__ void k_gather_keys(const uint64_t* __restrict__ key_in, const uint32_
         key_out[i] = key_in[order[i]];
 }
 
-// perm, T (gathered from t: 32-bit offsets from tmin, or the raw int64 timestamps), and
+// perm, T (gathered from t: 32-bit offsets from tbase, or the raw int64 timestamps), and
 // the "new static pair" flag of every kept sorted position.
 template <typename TS>
 __global__ void k_store(const uint64_t* __restrict__ key, const uint32_t* __restrict__ order,
-                        const TS* __restrict__ t, int64_t mk, int32_t* __restrict__ perm,
+                        const TS* __restrict__ t, TS tbase, int64_t mk, int32_t* __restrict__ perm,
                         TS* __restrict__ T, int32_t* __restrict__ newpair) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < mk;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t o = __ldcs(order + i);
         __stcs(perm + i, (int32_t)o);
-        T[i] = t[o];
+        T[i] = t[o] - tbase;
         const uint64_t k = __ldcs(key + i);
         __stcs(newpair + i, (int32_t)((i == 0) || ((k >> 1) != (key[i - 1] >> 1))));
     }
-}
-
-// 32-bit offsets t - tbase of the input timestamps. 4 bytes an edge keep the gather of
-// k_store inside L2 for inputs of up to ~25M edges (the int64 input is twice that).
-__global__ void k_offsets32(const int64_t* __restrict__ t, int64_t m, int64_t tbase, uint32_t* __restrict__ t32) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x)
-        t32[i] = (uint32_t)(__ldcs(t + i) - tbase);
 }
 
 // Static edge ids and segment starts. pscan = exclusive scan of newpair.
@@ -237,7 +230,7 @@ __global__ void k_pair_ids(const uint64_t* __restrict__ urank, const uint32_t* _
 // the temporal edges of pair p, which the triangle passes need before the sort is done.
 __global__ void k_pair_pack(const uint32_t* __restrict__ slotw, const uint32_t* __restrict__ order, int64_t m,
                             const int32_t* __restrict__ sid, int32_t S, int ib, uint64_t* __restrict__ packed,
-                            const int64_t* __restrict__ t, int64_t tmin, uint32_t* __restrict__ tv,
+                            const uint32_t* __restrict__ t, uint32_t tmin, uint32_t* __restrict__ tv,
                             int32_t* __restrict__ sigma) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = order ? (int64_t)order[j] : j;
@@ -249,7 +242,7 @@ __global__ void k_pair_pack(const uint32_t* __restrict__ slotw, const uint32_t* 
             if ((unsigned)p < (unsigned)S) atomicAdd(&sigma[p], 1);
         }
         packed[j] = (c << ib) | (uint64_t)j;
-        if (tv) tv[j] = (uint32_t)((order ? t[o] : __ldcs(t + j)) - tmin);
+        if (tv) tv[j] = (order ? t[o] : __ldcs(t + j)) - tmin;
     }
 }
 
@@ -1024,13 +1017,13 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
     if (!job.order && g->ts32) {
         // time-ordered input with 32-bit offsets: the sort ids and their counts (4 B slot
         // word read and 4 B id written per edge), then the stable sort of the ids, whose
-        // first pass reads the ids and times (12 B per edge, 8 B written) and whose last
+        // first pass reads the ids and times (8 B per edge, 8 B written) and whose last
         // writes T and sd (8 B read and written per edge, as the passes between). perm,
         // the same order of the input indices, is sorted on first use from the ids the
         // graph keeps, except for graphs the allocation-free entry point takes (it needs
         // perm and may not allocate): they get it here.
         const int passes = cbits > STORE_DIGIT_BITS ? (cbits + STORE_DIGIT_BITS - 1) / STORE_DIGIT_BITS : 1;
-        StageSpan span(ST_STORE, s, 8 * m + 16 * m * passes + 4 * m);
+        StageSpan span(ST_STORE, s, 8 * m + 16 * m * passes);
         const bool eager = mk <= FOLTY_NOALLOC_MAX_EDGES;
         uint32_t* cw = eager ? sc.get<uint32_t>(m) : graph_alloc<uint32_t>(g, m, s);
         int32_t* cnt = sc.get<int32_t>(2 * (int64_t)S + 1);
@@ -1047,7 +1040,7 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
         FOLTY_LAUNCH(k_store_sigma, grid_for(S, T), T, 0, s, g->seg, S, sigma);
         FOLTY_CUDA(cudaEventRecord(packed_ev, s));
         FOLTY_LAUNCH(k_store_hist, grid_for(2 * (int64_t)S + 1, T, 2), T, 0, s, cnt, S, passes, hist);
-        const StoreSortArgs sa{cw, g->in_t, g->tmin, m, cbits, hist, (uint32_t*)g->T, g->sd, nullptr, mk};
+        const StoreSortArgs sa{cw, g->in_t32, (uint32_t)g->tmin, m, cbits, hist, (uint32_t*)g->T, g->sd, nullptr, mk};
         store_sort(sc, sa);
         if (eager) {
             g->perm = graph_alloc<int32_t>(g, mk, s);
@@ -1075,7 +1068,7 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
     uint32_t* tv_alt = g->ts32 ? sc.get<uint32_t>(m) : nullptr;
     FOLTY_CUDA(cudaMemsetAsync(sigma, 0, sizeof(int32_t) * (size_t)S, s));
     FOLTY_LAUNCH(k_pair_pack, (unsigned)((m + T - 1) / T), T, 0, s, job.slotw, job.order, m, job.sid, S, ib, packed,
-                 g->in_t, g->tmin, tv, sigma);
+                 g->in_t32, (uint32_t)g->tmin, tv, sigma);
     FOLTY_CUDA(cudaEventRecord(packed_ev, s));
     const bool palt = g->ts32 ? radix_sort_pairs(sc, packed, packed_alt, tv, tv_alt, m, ib, cbits)
                               : radix_sort_keys(sc, packed, packed_alt, m, ib, cbits);
@@ -1090,6 +1083,12 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
     FOLTY_LAUNCH(k_segments_fix, grid_for(S, T), T, 0, s, S, mk, g->seg);
 }
 
+void enqueue_pair_list(const uint64_t* table, int lg, uint64_t* rank, uint32_t* slot, int* cnt, int cap, cudaStream_t s) {
+    const int64_t tb = 1ll << lg;
+    FOLTY_LAUNCH(k_pair_table_compact, grid_for(tb, (int64_t)256 * PAIR_COMPACT_ITEMS), 256, 0, s, table, tb, rank, slot, cnt,
+                 cap);
+}
+
 // A1 with dense pair ids (see k_pair_insert) up to the static edge list (ea, eb) and
 // the job of the temporal store: false, with nothing of the graph written, when the
 // table cannot serve (too many distinct pairs, a probe sequence ran out, or ids and
@@ -1100,46 +1099,39 @@ static bool pair_ids_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
     const int T = 256;
     const int64_t m = g->m, mk = g->m_kept;
     const int32_t n = g->n;
-    if (pair_table_forced_off()) return false;
+    if (!g->pre_slotw && pair_table_forced_off()) return false;  // a load that forced it off kept the edges
     if (mk == 0 || n < 2) return false;
     const int ib = bit_length((uint64_t)(m - 1));
-    const int lg_max = pair_table_lg_max(m);
-    int lg = pair_table_lg_first(m);
-    int64_t tb = 0, S64 = 0;
-    int cap = 0;
-    uint64_t* table = nullptr;
-    uint64_t* urank = nullptr;
-    uint32_t* uslot = nullptr;
-    // the first try's table, slot words and flags may already be filled by the load
-    const bool pre = g->pre_table != nullptr && g->pre_lg == lg;
-    int* flags = pre ? g->pre_flags : sc.get<int>(PAIR_FLAGS);
-    uint32_t* slotw = pre ? g->pre_slotw : sc.get<uint32_t>(m);
-    bool first = true;
-    while (true) {
-        tb = 1ll << lg;
-        cap = (int)(tb / 2);  // load factor at most 1/2
-        if (first && pre) {
-            table = g->pre_table;
-        } else {
-            table = sc.get<uint64_t>(tb);
-            FOLTY_CUDA(cudaMemsetAsync(table, 0, sizeof(uint64_t) * (size_t)tb, s));
-            FOLTY_CUDA(cudaMemsetAsync(flags, 0, PAIR_FLAGS * sizeof(int), s));
-            FOLTY_LAUNCH(k_pair_insert, grid_for(m, T), T, 0, s, g->in_src, g->in_dst, m, n, table, lg, slotw, flags);
-        }
-        first = false;
+    // the distinct pairs: listed by the load when its table served; otherwise a table of the
+    // largest size, unless the load tried that one
+    int lg = g->pre_lg;
+    int64_t S64 = g->pre_pairs;
+    const uint32_t* slotw = g->pre_slotw;
+    uint64_t* urank = g->pre_rank;
+    uint32_t* uslot = g->pre_slot;
+    if (!slotw) {
+        const int lg_max = pair_table_lg_max(m);
+        if (lg == lg_max) return false;
+        lg = lg_max;
+        const int cap = (1 << lg) / 2;  // load factor at most 1/2
+        int* flags = sc.get<int>(PAIR_FLAGS);
+        uint32_t* sw = sc.get<uint32_t>(m);
+        uint64_t* table = sc.get<uint64_t>(1ll << lg);
+        FOLTY_CUDA(cudaMemsetAsync(table, 0, sizeof(uint64_t) << lg, s));
+        FOLTY_CUDA(cudaMemsetAsync(flags, 0, PAIR_FLAGS * sizeof(int), s));
+        FOLTY_LAUNCH(k_pair_insert, grid_for(m, T), T, 0, s, g->in_src, g->in_dst, m, n, table, lg, sw, flags);
         urank = sc.get<uint64_t>(cap);
         uslot = sc.get<uint32_t>(cap);
-        FOLTY_LAUNCH(k_pair_table_compact, grid_for(tb, (int64_t)T * PAIR_COMPACT_ITEMS), T, 0, s, table, tb, urank, uslot,
-                     flags + 1, cap);
+        enqueue_pair_list(table, lg, urank, uslot, flags + 1, cap, s);
         const void* ptrs[2] = {flags, flags + 1};
         int sizes[2] = {4, 4};
         int64_t fv[2];
         read_back(g, ptrs, sizes, 2, fv, s);
         S64 = fv[1];
-        if (fv[0] == 0 && S64 <= cap) break;
-        if (lg == lg_max) return false;
-        lg = lg_max;
+        if (fv[0] != 0 || S64 > cap) return false;
+        slotw = sw;
     }
+    const int64_t tb = 1ll << lg;
     if (bit_length((uint64_t)(2 * S64)) + ib > 64) return false;
     const int32_t S = (int32_t)S64;
     // the distinct pairs in (a, b) order: ids, ends
@@ -1190,17 +1182,13 @@ static void pair_key_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
     sort_check(g, s);
     int32_t* newpair = sc.get<int32_t>(mk + 1);
     int32_t* pscan = sc.get<int32_t>(mk + 1);
-    // 32-bit offsets of the input timestamps, written right before the gather so that
-    // they are still in L2 there
-    uint32_t* t32 = (g->ts32 && mk > 0) ? sc.get<uint32_t>(m) : nullptr;
     if (mk > 0) {
-        if (t32) FOLTY_LAUNCH(k_offsets32, grid_for(m, T), T, 0, s, g->in_t, m, g->tmin, t32);
         if (g->ts32)
-            FOLTY_LAUNCH(k_store<uint32_t>, grid_for(mk, T), T, 0, s, skey, sval, t32, mk, g->perm, (uint32_t*)g->T,
-                         newpair);
+            FOLTY_LAUNCH(k_store<uint32_t>, grid_for(mk, T), T, 0, s, skey, sval, g->in_t32, (uint32_t)g->tmin, mk,
+                         g->perm, (uint32_t*)g->T, newpair);
         else
-            FOLTY_LAUNCH(k_store<int64_t>, grid_for(mk, T), T, 0, s, skey, sval, g->in_t, mk, g->perm, (int64_t*)g->T,
-                         newpair);
+            FOLTY_LAUNCH(k_store<int64_t>, grid_for(mk, T), T, 0, s, skey, sval, g->in_t, (int64_t)0, mk, g->perm,
+                         (int64_t*)g->T, newpair);
     }
     exclusive_scan(sc, newpair, pscan, mk);
     const int32_t S = read_i32(g, pscan + mk, s);
@@ -1299,7 +1287,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         uint64_t* tk_alt = sc.get<uint64_t>(m);
         uint32_t* iv = sc.get<uint32_t>(m);
         uint32_t* iv_alt = sc.get<uint32_t>(m);
-        FOLTY_LAUNCH(k_time_keys, grid_for(m, T), T, 0, s, g->in_t, m, g->tmin, tk, iv);
+        FOLTY_LAUNCH(k_time_keys, grid_for(m, T), T, 0, s, g->ts32 ? g->in_t32 : nullptr, g->in_t, m, g->tmin, tk, iv);
         const bool alt = radix_sort_pairs(sc, tk, tk_alt, iv, iv_alt, m, bit_length((uint64_t)(g->tmax - g->tmin)));
         sort_check(g, s);
         order = alt ? iv_alt : iv;
@@ -1539,19 +1527,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     } else if (ids) {
         sort_check(g, s);  // the store's sort completed before its arrays index anything
     }
-    // the raw input is no longer needed
-    graph_release(g, g->in_src, s);
-    graph_release(g, g->in_dst, s);
-    graph_release(g, g->in_t, s);
-    g->in_src = g->in_dst = nullptr;
-    g->in_t = nullptr;
-    // and neither is the pair table the load filled
-    graph_release(g, g->pre_table, s);
-    graph_release(g, g->pre_slotw, s);
-    graph_release(g, g->pre_flags, s);
-    g->pre_table = nullptr;
-    g->pre_slotw = nullptr;
-    g->pre_flags = nullptr;
+    release_input(g, s);  // the raw input and the pair table's lists are no longer needed
     // the run-ends table (built beside the triangle passes with the store) and every
     // triangle's liveness bytes
     if (!ids) build_run_ends(g, s);

@@ -192,8 +192,8 @@ struct OnesweepArgs {
     // the store's first pass (ST_FIRST): key j = cw[j], value t[j] - tmin (ST_IOTA: j),
     // read from the edge list itself (keys and vals unused)
     const uint32_t* cw;
-    const int64_t* t;
-    int64_t tmin;
+    const uint32_t* t;
+    uint32_t tmin;
     // its last pass (ST_LAST): sorted position i < limit gets T[i] = value and sd[i] =
     // key (ST_IOTA: perm[i] = value); okeys and ovals are unused, and the positions past
     // limit (the self-loops' ids) are dropped
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 
             if (MODE & ST_FIRST) {
                 kr[i] = (idx < tn) ? (K)__ldcs(a.cw + t0 + idx) : (K)0;
                 if (MODE & ST_IOTA) vr[i] = (uint32_t)(t0 + idx);
-                else vr[i] = (idx < tn) ? (uint32_t)(__ldcs(a.t + t0 + idx) - a.tmin) : 0u;
+                else vr[i] = (idx < tn) ? __ldcs(a.t + t0 + idx) - a.tmin : 0u;
             } else {
                 kr[i] = (idx < tn) ? kin[idx] : (K)0;
                 if (V) vr[i] = (idx < tn) ? vin[idx] : 0u;
@@ -514,7 +514,7 @@ static void store_sort_impl(Scratch& sc, const StoreSortArgs& a) {
     }
     constexpr int F = ST_FIRST | (IOTA ? ST_IOTA : 0), L = ST_LAST | (IOTA ? ST_IOTA : 0);
     for (int p = 0; p < passes; p++) {
-        // 8 B read and written per edge (the first pass reads a 4 B id and an 8 B time, or
+        // 8 B read and written per edge (the first pass reads a 4 B id and a 4 B time, or
         // the id alone; the last writes two 4 B entries, or one)
         StageSpan span(ST_SORT, s, 16 * n);
         FOLTY_CUDA(cudaMemsetAsync(lbc, 0, sizeof(unsigned long long) * (size_t)(tiles * RS_BINS + 1), s));
