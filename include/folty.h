@@ -234,15 +234,14 @@ uint64_t folty_kernel_launches(void);
  *             window (k_live_select): 1 B read per triangle; per kept triangle its record
  *             and its edges' run ends read and 13 B written, counted on the device;
  *   TRIANGLES triangle listing: 4 B per merged out-list entry + 8 B per static edge and
- *             16 B written per triangle (graphs past FOLTY_NOALLOC_MAX_EDGES edges: one
- *             pass into a layout bounded per oriented edge); graphs up to that size also
+ *             16 B written per triangle; graphs up to FOLTY_NOALLOC_MAX_EDGES edges also
  *             count first (the same merge bytes again) and write 8 B more per triangle;
+ *             larger ones read 4 B per list entry looked up and write the out motif's
+ *             liveness byte with each triangle;
  *   ROLES     the run-ends table (12 B of run bounds + 4 timestamps read, one record
  *             written per static edge) and the liveness pass of one direction variant (16 B
- *             read and 1 B written per triangle, the run-ends table read once; after a
- *             one-pass listing, preprocessing's pass also moves each triangle into the
- *             dense layout: 16 B more written per triangle, and the per-edge counts and
- *             offsets read);
+ *             read and 1 B written per triangle, the run-ends table read once; the out
+ *             motif's of graphs past FOLTY_NOALLOC_MAX_EDGES edges is part of TRIANGLES);
  *   BATCH     the batched threshold over the plain queries of a direction variant: the
  *             32-edge group bits, and (counted on the device) the bin row and 4 B of pair
  *             key of every edge in a group with a hit;
@@ -326,8 +325,9 @@ void folty_server_destroy(folty_server *sv);
  * of the triangle passes between one thread and one whole warp per oriented edge (by
  * the total length of the edge's two out-lists), and the probe tile (the granularity in
  * which the flat probe space of the kept roles is partitioned over thread blocks) with
- * the probe kernel's blocks per SM. The split is timed during folty_preprocess, the
- * probe shape on the graph's first query; both are cached for the process under the
+ * the probe kernel's blocks per SM. The split is timed during folty_preprocess (of graphs
+ * up to FOLTY_NOALLOC_MAX_EDGES edges: larger ones are listed in one pass, which has no such
+ * split), the probe shape on the graph's first query; both are cached for the process under the
  * graph's statistics (sizes, triangles, probes), so later graphs of the same statistics
  * skip the trials. Every shape gives the same results. */
 typedef struct {

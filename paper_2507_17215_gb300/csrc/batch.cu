@@ -405,7 +405,7 @@ int64_t batch_footprint(const folty_graph* g, const folty_query_params* qs, int 
     // per role through the two sorts (44 B each), on top of its own counters
     bool triples = false;
     for (int i = 0; i < nq; i++) triples = triples || qs[i].want_triples;
-    const int64_t tri_part = triples ? 53 * 6 * g->ntri + 4 * g->m_kept + per_q : 0;
+    const int64_t tri_part = triples ? 53 * 6 * g->tri_cap + 4 * g->m_kept + per_q : 0;
     if (bins_part) *bins_part = bins;
     return std::max(bins + marks + fused + group * per_q, tri_part);
 }

@@ -197,7 +197,8 @@ struct folty_graph {
     int32_t* binv;    // [S] place of each static edge in by_b
     int32_t* prank;   // [2S] rank of directed pair 2s + d in (u, v) order (batched queries; made on first use)
     int64_t ntri;
-    int4* tri;        // [ntri] {s_uv, s_uw, s_vw, id-order bits}, u < v < w in degeneracy rank
+    int64_t tri_cap;  // entries of tri: ntri, or a few more (a one-pass listing leaves some empty)
+    int4* tri;        // [tri_cap] {s_uv, s_uw, s_vw, id-order bits (-1: empty)}, u < v < w in degeneracy rank
     int64_t* tri_off; // [ntri + 1] prefix of per-triangle probe counts (null past FOLTY_NOALLOC_MAX_EDGES edges)
     int64_t* tile_tri;  // [probe tiles + 1] triangle holding each tile's first probe (null with tri_off)
     unsigned long long* prof_bytes;  // [PROF_SLOTS] device counters of probe-stage model bytes
@@ -373,19 +374,12 @@ bool tune_forced(TuneParams* p, bool probe);
 // unless forced or cached (live.cu); the triangle split is picked in preprocess.cu.
 void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s);
 
-// The run-ends table (live.cu; needs the sorted store), the rows of per-triangle
-// liveness bytes with their padding; triangle_liveness then fills the out motif's row
-// from the listed triangles. With from, the triangles still lie in the bounded layout
-// of a one-pass listing, and the same pass moves them into g->tri.
-struct TriLayout {
-    const int32_t* cnt;   // [S] triangles of each oriented edge
-    const int64_t* toff;  // [S + 1] prefix of cnt
-    const int64_t* boff;  // [S + 1] prefix of the per-edge bounds: edge j's triangles at tri_b[boff[j] ...]
-    const int4* tri_b;
-};
+// The run-ends table (live.cu; needs the sorted store); the rows of liveness bytes of the
+// triangle array's entries with their padding; and the mark that the out motif's row is
+// written by what was enqueued on s so far (a one-pass listing writes it itself).
 void build_run_ends(folty_graph* g, cudaStream_t s);
-void prepare_liveness(folty_graph* g, cudaStream_t s);
-void triangle_liveness(folty_graph* g, cudaStream_t s, const TriLayout* from = nullptr);
+void prepare_liveness(folty_graph* g, int64_t entries, cudaStream_t s);
+void listed_liveness(folty_graph* g, cudaStream_t s);
 // Makes the liveness row of direction variant dir ready for work enqueued on s after the
 // call: computes it on s the first time (thread-safe), else makes s wait for the
 // computation. Not while s is capturing.

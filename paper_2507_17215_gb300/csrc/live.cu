@@ -46,66 +46,14 @@ __global__ void k_run_ends(const int32_t* __restrict__ seg, int64_t S, const TS*
 }
 
 // The liveness byte of every listed triangle for direction variant DIR (liveness_byte),
-// one thread per triangle: consecutive triangles share their first edge, so its record
-// mostly comes from L1.
+// one thread per entry of the triangle array (an empty one gets "never"): consecutive
+// triangles share their first edge, so its record mostly comes from L1.
 template <typename TS, int DIR>
-__global__ void k_tri_live(const int4* __restrict__ tri, int64_t ntri, const RunEnds<TS>* __restrict__ ends,
+__global__ void k_tri_live(const int4* __restrict__ tri, int64_t cap, const RunEnds<TS>* __restrict__ ends,
                            uint8_t* __restrict__ row) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ntri; t += (int64_t)gridDim.x * blockDim.x)
-        row[t] = liveness_byte<TS, DIR>(__ldcs(tri + t), ends);
-}
-
-// The same while the triangles move from the bounded layout of a one-pass listing into
-// the dense one: the cnt[j] triangles of oriented edge j from tri_b[boff[j] ...] to
-// tri[toff[j] ...] (toff: prefix of cnt). A warp takes 32 consecutive edges, whose
-// triangles are contiguous in tri; its lanes stride over them, two triangles a lane per
-// step (both loads in flight before either is used), and find each one's edge by a
-// binary search of the lanes' running counts. One warp per 32 edges and short blocks:
-// the dense communities' edges hold far more triangles than the rest.
-template <typename TS, int DIR>
-__global__ void k_tri_live_copy(const int32_t* __restrict__ cnt, const int64_t* __restrict__ toff,
-                                const int64_t* __restrict__ boff, int32_t S, const int4* __restrict__ tri_b,
-                                int4* __restrict__ tri, const RunEnds<TS>* __restrict__ ends,
-                                uint8_t* __restrict__ row) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wstride = ((int64_t)gridDim.x * blockDim.x) & ~31ll;
-    for (int64_t j0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); j0 < S; j0 += wstride) {
-        const int64_t j = j0 + lane;
-        const int32_t c = j < S ? cnt[j] : 0;
-        const int64_t src0 = j < S ? boff[j] : 0;
-        int32_t inc = c;  // inclusive running count over the warp's edges
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const int32_t total = __shfl_sync(0xffffffffu, inc, 31);
-        if (total == 0) continue;
-        const int64_t dst0 = toff[j0];
-        for (int32_t t0 = 0; t0 < total; t0 += 64) {
-            int4 tr[2];
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int32_t t = t0 + 32 * h + lane;
-                int e = 0;  // the first lane whose running count exceeds t
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int32_t v = __shfl_sync(0xffffffffu, inc, e + step - 1);
-                    if (v <= t) e += step;
-                }
-                const int32_t before = __shfl_sync(0xffffffffu, inc - c, e);
-                const int64_t from = __shfl_sync(0xffffffffu, src0, e);
-                tr[h] = t < total ? __ldcs(tri_b + from + (t - before)) : make_int4(0, 0, 0, 0);
-            }
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int32_t t = t0 + 32 * h + lane;
-                if (t < total) {
-                    tri[dst0 + t] = tr[h];
-                    row[dst0 + t] = liveness_byte<TS, DIR>(tr[h], ends);
-                }
-            }
-        }
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cap; t += (int64_t)gridDim.x * blockDim.x) {
+        const int4 tr = __ldcs(tri + t);
+        row[t] = tr.w < 0 ? DMIN_NEVER : liveness_byte<TS, DIR>(tr, ends);
     }
 }
 
@@ -521,31 +469,30 @@ void build_run_ends(folty_graph* g, cudaStream_t s) {
     else run_ends_t<int64_t>(g, s);
 }
 
-void prepare_liveness(folty_graph* g, cudaStream_t s) {
-    const int64_t ntri = g->ntri;
+void prepare_liveness(folty_graph* g, int64_t entries, cudaStream_t s) {
     // three rows of liveness bytes, each padded with DMIN_NEVER to whole 16-byte chunks
-    // (triangle_liveness writes the first ntri bytes of each)
-    g->tlive_stride = (ntri + 15) & ~int64_t(15);
+    // (every pass writes the bytes of all entries of the triangle array)
+    g->tlive_stride = (entries + 15) & ~int64_t(15);
     g->tlive = graph_alloc<uint8_t>(g, 3 * g->tlive_stride, s);
     for (int d = 0; d < 3; d++)
-        if (g->tlive_stride > ntri)
-            FOLTY_CUDA(cudaMemsetAsync(g->tlive + d * g->tlive_stride + ntri, DMIN_NEVER,
-                                       (size_t)(g->tlive_stride - ntri), s));
+        if (g->tlive_stride > entries)
+            FOLTY_CUDA(cudaMemsetAsync(g->tlive + d * g->tlive_stride + entries, DMIN_NEVER,
+                                       (size_t)(g->tlive_stride - entries), s));
 }
 
 template <typename TS>
 static void liveness_row_t(folty_graph* g, int dir, cudaStream_t s) {
-    const int64_t ntri = g->ntri;
-    // per triangle: its record read and one byte written; the run-ends table (shared by
+    const int64_t cap = g->tri_cap;
+    // per entry: its record read and one byte written; the run-ends table (shared by
     // the triangles of an edge, and small) read once
-    StageSpan span(ST_ROLES, s, ntri * (16 + 1) + g->S * (int64_t)sizeof(RunEnds<TS>));
-    if (ntri == 0) return;
+    StageSpan span(ST_ROLES, s, cap * (16 + 1) + g->S * (int64_t)sizeof(RunEnds<TS>));
+    if (g->ntri == 0) return;
     const RunEnds<TS>* ends = (const RunEnds<TS>*)g->run_ends;
     uint8_t* row = g->tlive + (int64_t)dir * g->tlive_stride;
-    const unsigned grid = grid_for(ntri, 256);
-    if (dir == FOLTY_DIR_OUT) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_OUT>), grid, 256, 0, s, g->tri, ntri, ends, row);
-    else if (dir == FOLTY_DIR_IN) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_IN>), grid, 256, 0, s, g->tri, ntri, ends, row);
-    else FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_EITHER>), grid, 256, 0, s, g->tri, ntri, ends, row);
+    const unsigned grid = grid_for(cap, 256);
+    if (dir == FOLTY_DIR_OUT) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_OUT>), grid, 256, 0, s, g->tri, cap, ends, row);
+    else if (dir == FOLTY_DIR_IN) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_IN>), grid, 256, 0, s, g->tri, cap, ends, row);
+    else FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_EITHER>), grid, 256, 0, s, g->tri, cap, ends, row);
 }
 
 // Each direction variant's liveness row is computed by the first call that needs it
@@ -564,26 +511,8 @@ void ensure_liveness(folty_graph* g, int dir, cudaStream_t s) {
     }
 }
 
-template <typename TS>
-static void liveness_copy_t(folty_graph* g, const TriLayout& from, cudaStream_t s) {
-    const int64_t ntri = g->ntri;
-    // per triangle: its record read in the bounded layout and written in the dense one,
-    // and one byte written; the per-edge counts, offsets and run ends read once
-    StageSpan span(ST_ROLES, s, ntri * (16 + 16 + 1) + g->S * (int64_t)(4 + 8 + 8 + sizeof(RunEnds<TS>)));
-    if (ntri == 0) return;
-    FOLTY_LAUNCH((k_tri_live_copy<TS, FOLTY_DIR_OUT>), (unsigned)((g->S + 255) / 256), 256, 0, s, from.cnt, from.toff,
-                 from.boff, g->S, from.tri_b, g->tri, (const RunEnds<TS>*)g->run_ends,
-                 g->tlive + (int64_t)FOLTY_DIR_OUT * g->tlive_stride);
-}
-
-void triangle_liveness(folty_graph* g, cudaStream_t s, const TriLayout* from) {
-    if (!from) {
-        ensure_liveness(g, FOLTY_DIR_OUT, s);
-        return;
-    }
+void listed_liveness(folty_graph* g, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(g->live_mu);
-    if (g->ts32) liveness_copy_t<uint32_t>(g, *from, s);
-    else liveness_copy_t<int64_t>(g, *from, s);
     if (!g->live_ev[FOLTY_DIR_OUT]) FOLTY_CUDA(cudaEventCreateWithFlags(&g->live_ev[FOLTY_DIR_OUT], cudaEventDisableTiming));
     FOLTY_CUDA(cudaEventRecord(g->live_ev[FOLTY_DIR_OUT], s));
     g->live_ready[FOLTY_DIR_OUT] = 1;
@@ -622,8 +551,8 @@ static void launch_select_t(const folty_graph* g, int dir, const uint8_t* tl, in
     SelectCtl* ctl = reinterpret_cast<SelectCtl*>(ls.ctl);
     const SelectArgs a{g->tri,  ls.cand, delta,    qp,           ls.ush,   ctl,       ls.L,
                        ls.loff, ls.lmask, ls.ltile, ls.max_tiles, PB_GROUP, ls.totals, prof};
-    FOLTY_LAUNCH(k_live_candidates<LS_ITEMS>, grid_for((g->ntri + LS_ITEMS - 1) / LS_ITEMS, LS_THREADS, LS_PER_SM), LS_THREADS,
-                 0, s, tl, g->ntri, delta, qp, ctl, ls.cand);
+    FOLTY_LAUNCH(k_live_candidates<LS_ITEMS>, grid_for((g->tri_cap + LS_ITEMS - 1) / LS_ITEMS, LS_THREADS, LS_PER_SM),
+                 LS_THREADS, 0, s, tl, g->tri_cap, delta, qp, ctl, ls.cand);
     const unsigned grid = grid_for(g->ntri, LS_THREADS, LS_PER_SM);
     if (dir == FOLTY_DIR_OUT) FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_OUT>), grid, LS_THREADS, 0, s, a, ends);
     else if (dir == FOLTY_DIR_IN) FOLTY_LAUNCH((k_live_select<TS, FOLTY_DIR_IN>), grid, LS_THREADS, 0, s, a, ends);
@@ -671,7 +600,7 @@ unsigned long long* prof_counter(folty_graph* g, cudaStream_t s) {
 // receives the selection's model bytes beyond its one byte per triangle.
 static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& ls,
                            unsigned long long* prof_sel, const int64_t* qp, cudaStream_t s) {
-    StageSpan span(ST_SELECT, s, g->ntri, prof_sel);
+    StageSpan span(ST_SELECT, s, g->tri_cap, prof_sel);
     const uint8_t* tl = g->tlive + (int64_t)dir * g->tlive_stride;
     if (g->ts32) launch_select_t<uint32_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
     else launch_select_t<int64_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
@@ -887,7 +816,7 @@ void probe_stats(folty_graph* g, int64_t delta, int dir, folty_probe_stats* out,
     out->triangles = g->ntri;
     out->all_roles = 6 * g->ntri;
     out->all_probes = g->info.probes;  // every (temporal edge, witness) pair
-    out->select_bytes = g->ntri;
+    out->select_bytes = g->tri_cap;
     if (g->ntri == 0 || g->info.probes == 0) return;
     Scratch sc(g->alloc, s, g->dev_err);
     const ProbeBuffers ls = select_live(g, delta, dir, sc, s, nullptr);

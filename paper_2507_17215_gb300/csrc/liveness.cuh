@@ -134,4 +134,32 @@ __device__ __forceinline__ uint8_t liveness_byte(const int4 tr, const RunEnds<TS
     return dmin_bucket<TS>(m);
 }
 
+// The runs of one static edge as the listing reads them, at its place in the out-lists:
+// direction 0 is the oriented edge's own (tail to head), whatever the ids' order, and no
+// sizes: half a run-ends record.
+template <typename TS>
+struct __align__(16) OutEnds {
+    TS f0, l0, f1, l1;
+};
+
+// The out motif's liveness byte of the triangle of the oriented edges (u, v), (u, w) and
+// (v, w). The six roles are the same for every labelling of its vertices, so u, v, w in
+// their own order serve as the frame and nothing is permuted.
+template <typename TS>
+__device__ __forceinline__ uint8_t out_liveness(const OutEnds<TS>& uv, const OutEnds<TS>& uw, const OutEnds<TS>& vw) {
+    FrameRuns<TS> fr;
+    const OutEnds<TS> e[3] = {uv, uw, vw};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        fr.f[2 * k] = e[k].f0;
+        fr.l[2 * k] = e[k].l0;
+        fr.f[2 * k + 1] = e[k].f1;
+        fr.l[2 * k + 1] = e[k].l1;
+    }
+    TS m = frame_dmin<FOLTY_DIR_OUT, TS>(fr, 0);
+#pragma unroll
+    for (int r = 1; r < 6; r++) m = min(m, frame_dmin<FOLTY_DIR_OUT, TS>(fr, r));
+    return dmin_bucket<TS>(m);
+}
+
 }  // namespace folty

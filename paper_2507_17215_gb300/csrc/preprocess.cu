@@ -15,6 +15,7 @@
 
 #include "core.cuh"
 #include "internal.cuh"
+#include "liveness.cuh"
 #include "pairs.cuh"
 #include "probe.cuh"
 
@@ -599,11 +600,15 @@ __global__ void k_outptr(const int32_t* __restrict__ rowptr, const int32_t* __re
 // lanes look up their share of out(v), the loads of the next share issued before the
 // lookups. Both passes find the same set, so the counts match the writes.
 constexpr int TRI_THREADS = 256;
-constexpr int TRI_HEAVY = 48;
 constexpr int TRI_HCAP = 256;    // out(u) entries a warp's table holds (longer lists: one lane merges)
 constexpr int TRI_HSLOTS = 512;  // table slots (load at most one half)
-// the largest bounded layout of a one-pass listing (the scratch copy and the graph's
-// array each hold that many bytes); a larger bound takes the counting pass
+// entries of a warp's chunk of the one-pass listing's array: fewer when the bound is small,
+// so that the empty ends of the chunks stay below a sixteenth of the bound or 32 a warp
+constexpr int TRI_BUCKETS = 128; // of four slots, of the one-pass listing (load at most one half)
+constexpr int TRI_LIST_THREADS = 128;
+constexpr int TRI_PER_SM = 8;    // resident blocks (what their tables leave room for)
+constexpr int TRI_CHUNK_MIN = 32, TRI_CHUNK_MAX = 512;
+// the largest array of a one-pass listing; a larger bound takes the counting pass
 constexpr int64_t TRI_BOUND_MAX_BYTES = int64_t(16) << 30;
 
 // FOLTY_TRI_LAYOUT=counted: every graph takes the counting pass before the listing.
@@ -650,9 +655,9 @@ __device__ __forceinline__ void warp_hash_out(const int32_t* __restrict__ nbr, c
 }
 
 // Looks up out(v) = [i2, e2) of the out-lists (nbr, osig and, when EID, eid by position)
-// in the warp's table of out(u). Calls hit(found, w, sig_u, eid_u, sig_v, eid_v) once per
-// lane and step (w = -1 for an idle lane): the counts and (EID) ids of the static edges
-// (u, w) and (v, w) of a common neighbour w. The whole warp must call it.
+// in the warp's table of out(u). Calls hit(pos_u, w, sig_v, eid_v) once per lane and step
+// (w = -1 for an idle lane): the position in out(u) of a common neighbour w (-1: none), and the
+// count and (EID) id of the static edge (v, w). The whole warp must call it.
 template <bool EID, typename F>
 __device__ __forceinline__ void warp_probe_out(const int32_t* __restrict__ nbr, const int32_t* __restrict__ osig,
                                                const int32_t* __restrict__ eid, int32_t i2, int32_t e2,
@@ -686,7 +691,7 @@ __device__ __forceinline__ void warp_probe_out(const int32_t* __restrict__ nbr, 
                 h = (h + 1) & (TRI_HSLOTS - 1);
             }
         }
-        hit(pu >= 0, w, pu >= 0 ? H.sig[pu] : 0, (EID && pu >= 0) ? H.eid[pu] : 0, sv, ev);
+        hit(pu, w, sv, ev);
         w = wn;
         sv = sn;
         ev = en;
@@ -756,10 +761,10 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_count(const int32_t* __rest
             int32_t c = 0;
             unsigned long long hp = 0;
             warp_probe_out<false>(out_nbr, osig, nullptr, b2, f2, table[warp],
-                                  [&](bool found, int32_t, int32_t su, int32_t, int32_t sv, int32_t) {
-                                      if (found) {
+                                  [&](int pu, int32_t, int32_t sv, int32_t) {
+                                      if (pu >= 0) {
                                           c++;
-                                          hp += (unsigned long long)(su + sv);
+                                          hp += (unsigned long long)(table[warp].sig[pu] + sv);
                                       }
                                   });
 #pragma unroll
@@ -803,10 +808,7 @@ __global__ void k_tile_starts(const int64_t* __restrict__ tri_off, int64_t ntri,
 // Writes every triangle, with OFF its probe offset (the running sum of the probe slots of
 // the triangles before it, from the counting pass's prefix per oriented edge), and counts
 // the triangles on every static edge. The triangles of oriented edge j start at toff[j].
-// BOUND (no counting pass before it): toff[j] is the prefix of the per-edge bounds
-// min(|N+(u)|, |N+(v)|), the pass writes each edge's triangle count to cnt[j], and adds
-// the list lengths merged to merged[0] and the triangles' probe slots to merged[1].
-template <bool OFF, bool BOUND = false>
+template <bool OFF>
 __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __restrict__ outptr,
                                                            const int32_t* __restrict__ out_nbr,
                                                            const int32_t* __restrict__ out_eid,
@@ -815,13 +817,10 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
                                                            const int64_t* __restrict__ toff,
                                                            const int64_t* __restrict__ poff, int4* __restrict__ tri,
                                                            int64_t* __restrict__ tri_off, int32_t* __restrict__ common,
-                                                           int heavy_min, int32_t* __restrict__ cnt = nullptr,
-                                                           unsigned long long* __restrict__ merged = nullptr) {
-    static_assert(!(OFF && BOUND), "probe offsets need the counting pass");
+                                                           int heavy_min) {
     __shared__ TriHashW table[TRI_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long acc = 0, pacc = 0;  // BOUND: list lengths merged, probe slots
     int32_t hashed = -1;  // the vertex whose out-list is in this warp's table
     for (int64_t j0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); j0 < S; j0 += stride) {
         const int64_t j = j0 + lane;
@@ -835,13 +834,11 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
             e1 = outptr[u + 1];
             i2 = outptr[v];
             e2 = outptr[v + 1];
-            if (BOUND) acc += (unsigned long long)((e1 - i1) + (e2 - i2));
         }
         const bool heavy = j < S && (e1 - i1) + (e2 - i2) > heavy_min && e1 - i1 <= TRI_HCAP;
         if (j < S && !heavy) {
             int64_t p = toff[j], q = OFF ? poff[j] : 0;
             int32_t n_here = 0;
-            unsigned long long ps = 0;
             int32_t a1 = i1, a2 = i2;
             while (a1 < e1 && a2 < e2) {
                 const int32_t x = out_nbr[a1], y = out_nbr[a2];
@@ -853,7 +850,6 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
                         tri_off[p] = q;
                         q += (int64_t)sig_uv + osig[a1] + osig[a2];
                     }
-                    if (BOUND) ps += (unsigned long long)(sig_uv + osig[a1] + osig[a2]);
                     atomicAdd(&common[s_uw], 1);
                     atomicAdd(&common[s_vw], 1);
                     p++;
@@ -863,10 +859,6 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
                 a2 += (y <= x);
             }
             if (n_here) atomicAdd(&common[s_uv], n_here);
-            if (BOUND) {
-                cnt[j] = n_here;
-                pacc += ps;
-            }
         }
         unsigned hm = __ballot_sync(0xffffffffu, heavy);
         while (hm) {
@@ -886,10 +878,11 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
             }
             warp_probe_out<true>(
                 out_nbr, osig, out_eid, b2, f2, table[warp],
-                [&](bool found, int32_t w, int32_t su, int32_t s_uw, int32_t sv, int32_t s_vw) {
+                [&](int pu, int32_t w, int32_t sv, int32_t s_vw) {
+                    const bool found = pu >= 0;
                     const unsigned m = __ballot_sync(0xffffffffu, found);
                     // the hits' probe offsets: a warp prefix of their costs, in lane order
-                    const int64_t c = found ? (int64_t)hsig + su + sv : 0;
+                    const int64_t c = OFF && found ? (int64_t)hsig + table[warp].sig[pu] + sv : 0;
                     int64_t inc = c;
                     if (OFF) {
 #pragma unroll
@@ -899,6 +892,7 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
                         }
                     }
                     if (found) {
+                        const int32_t s_uw = table[warp].eid[pu];
                         const int64_t at = p + __popc(m & ((1u << lane) - 1u));
                         const int flags = (hu < hv ? 1 : 0) | (hu < w ? 2 : 0) | (hv < w ? 4 : 0);
                         tri[at] = make_int4(hs, s_uw, s_vw, flags);
@@ -906,34 +900,313 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
                         atomicAdd(&common[s_uw], 1);
                         atomicAdd(&common[s_vw], 1);
                     }
-                    if (BOUND) pacc += (unsigned long long)c;
                     p += __popc(m);
                     if (OFF) q += __shfl_sync(0xffffffffu, inc, 31);
                     n_here += __popc(m);
                 });
             if (lane == 0 && n_here) atomicAdd(&common[hs], n_here);
-            if (BOUND && lane == 0) cnt[j0 + src] = n_here;
         }
-    }
-    if (BOUND) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            pacc += __shfl_xor_sync(0xffffffffu, pacc, o);
-        }
-        if (lane == 0 && acc) atomicAdd(merged, acc);
-        if (lane == 0 && pacc) atomicAdd(merged + 1, pacc);
     }
 }
 
-// bnd[j] = min(|N+(u)|, |N+(v)|) for oriented edge j = (u, v): at most that many common
-// out-neighbours, so an upper bound of the triangles the listing finds on j.
+// The triangles of graphs past the allocation-free counts' limit, in one pass without a
+// counting pass before it. A warp takes 32 consecutive oriented edges (u, v) off a common
+// counter (the dense communities' edges hold far more triangles than the rest). Their out(u)
+// are one stretch of the out-lists: it goes into a hash table in the warp's shared memory, and
+// the lanes look up all their out(v), laid end to end so that short lists leave no lane idle,
+// the loads of the next 32 entries issued before this step's lookups. (A tail with more than
+// TRI_HCAP out-neighbours has each of its edges merged by one lane.) The triangles found, few
+// or many a step, go through a queue that the whole warp empties 32 at a time: only then are
+// their records made, from the entries at their places in the out-lists, and with each the out
+// motif's liveness byte from the runs of its three edges. A warp writes into chunks of `chunk`
+// entries taken off a second counter; the rest of its last chunk stays empty (w = -1, never
+// live), so the array holds at most chunk - 1 empty entries a warp and no pass has to move it.
+// The triangles of the stretch's edges, as (u, v) and as (u, w), are counted in shared memory
+// and added to common once; merged[0] receives the list entries looked up, merged[1] the
+// triangles.
+// Bound by instruction issue (80% of the slots; 4 blocks more or less an SM: 5% slower). At full
+// size, 77M triangles from 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M
+// lookups: 400. A lane or a warp per edge, into a layout by upper bounds with three additions to
+// common a triangle, and a second pass that gathered the three edges' runs and moved the
+// triangles took 1110 + 750 and 584 + 75; the same without the queue, the records made by the
+// lanes that found them, 1400 and 690. Looking up the shorter of the two lists (111M and 29M
+// lookups) needs a table per row and edge direction: 1220 and 400.
+struct TriListArgs {
+    const int32_t *outptr, *out_nbr, *out_src;
+    const uint32_t* out_eup;  // static edge at a place of the out-lists; bit 31: the tail has the smaller id
+    int32_t S;
+    int chunk;  // a multiple of 32
+    int4* tri;
+    uint8_t* row;
+    int32_t* common;
+    unsigned long long *merged, *next, *used;  // next: edges taken; used: entries taken
+};
+
+// One warp's table of a stretch of the out-lists, in buckets of four filled from the first slot
+// on: head (-1: empty) and position in the stretch; by position, the triangles found so far.
+// The queue: the places of a triangle's edges (u, v), (u, w), (v, w) in the out-lists.
+struct TriStretch {
+    int4 key[TRI_BUCKETS];
+    uint8_t pos[4 * TRI_BUCKETS];
+    int32_t cnt[TRI_HCAP];
+    int4 queue[64];
+    uint8_t lane_of[32];
+};
+
+template <typename TS>
+__global__ void __launch_bounds__(TRI_LIST_THREADS, TRI_PER_SM) k_tri_list(const TriListArgs a,
+                                                                      const OutEnds<TS>* __restrict__ oe) {
+    __shared__ TriStretch table[TRI_LIST_THREADS / 32];
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr uint32_t ID = 0x7fffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1;
+    TriStretch& H = table[threadIdx.x >> 5];
+    unsigned long long acc = 0, found = 0;  // found: the same in every lane
+    int64_t at = 0, end = 0;                // free entries of the warp's chunk
+    int queued = 0;
+    auto take = [&](unsigned long long* counter, int n) {
+        unsigned long long x = 0;
+        if (lane == 0) x = atomicAdd(counter, (unsigned long long)n);
+        return (int64_t)__shfl_sync(FULL, x, 0);
+    };
+    // writes the first n <= 32 queued triangles, and empty entries up to 32
+    auto write = [&](int n) {
+        if (at == end) {
+            at = take(a.used, a.chunk);
+            end = at + a.chunk;
+        }
+        __syncwarp();
+        int4 tr = make_int4(0, 0, 0, -1);
+        uint8_t live = DMIN_NEVER;
+        if (lane < n) {
+            const int4 q = H.queue[lane];
+            const int32_t uv = q.x, uw = q.y, vw = q.z;
+            const uint32_t x = a.out_eup[uv], y = a.out_eup[uw], z = a.out_eup[vw];
+            live = out_liveness<TS>(oe[uv], oe[uw], oe[vw]);
+            tr = make_int4((int)(x & ID), (int)(y & ID), (int)(z & ID),
+                           (int)(x >> 31) | (int)((y >> 31) << 1) | (int)((z >> 31) << 2));
+            atomicAdd(&a.common[tr.z], 1);
+        }
+        __stcs(a.tri + at + lane, tr);
+        a.row[at + lane] = live;
+        at += 32;
+        found += n;
+    };
+    // queues the triangles of the lanes of m
+    auto push = [&](unsigned m, int32_t uv, int32_t uw, int32_t vw) {
+        if ((m >> lane) & 1) H.queue[queued + __popc(m & below)] = make_int4(uv, uw, vw, 0);
+        queued += __popc(m);
+        if (queued < 32) return;
+        write(32);
+        queued -= 32;
+        __syncwarp();
+        if (lane < queued) H.queue[lane] = H.queue[32 + lane];
+        __syncwarp();
+    };
+    // bucket of head w in the list at position lo of the stretch
+    auto bucket = [](int lo, int32_t w) { return (int)(((uint32_t)(w + 31 * lo) * 0x9E3779B1u) >> 25); };
+    static_assert(TRI_BUCKETS == 128 && TRI_HCAP <= 256, "7 bits of hash; positions are bytes");
+    int64_t j0 = take(a.next, 32);
+    while (j0 < a.S) {
+        const int64_t j_next = take(a.next, 32);
+        const int64_t j = j0 + lane;
+        int32_t u = -1, i1 = 0, e1 = 0, i2 = 0, e2 = 0;
+        if (j < a.S) {
+            u = a.out_src[j];
+            const int32_t v = a.out_nbr[j];
+            i1 = a.outptr[u];
+            e1 = a.outptr[u + 1];
+            i2 = a.outptr[v];
+            e2 = a.outptr[v + 1];
+            acc += (unsigned long long)(e2 - i2);
+        }
+        unsigned left = __ballot_sync(FULL, j < a.S);
+        while (left) {
+            // the edges whose tails' lists fit the table together, from the first one left on
+            const int first = __ffs(left) - 1;
+            const int32_t b = __shfl_sync(FULL, i1, first);
+            const bool here = (left >> lane) & 1;
+            const bool mine = here && e1 - b <= TRI_HCAP;
+            const unsigned batch = __ballot_sync(FULL, mine);
+            if (batch == 0) {  // not even the first one's
+                const bool merge = here && i1 == b;
+                left &= ~__ballot_sync(FULL, merge);
+                int32_t a1 = merge ? i1 : e1, a2 = i2, n_here = 0;
+                while (__any_sync(FULL, a1 < e1 && a2 < e2)) {
+                    const int32_t p1 = a1, p2 = a2;
+                    bool hit = false;
+                    if (a1 < e1 && a2 < e2) {
+                        const int32_t x = a.out_nbr[a1], y = a.out_nbr[a2];
+                        hit = x == y;
+                        a1 += (x <= y);
+                        a2 += (y <= x);
+                    }
+                    if (hit) {
+                        n_here++;
+                        atomicAdd(&a.common[a.out_eup[p1] & ID], 1);
+                    }
+                    const unsigned m = __ballot_sync(FULL, hit);
+                    if (m) push(m, (int32_t)j, p1, p2);
+                }
+                if (n_here) atomicAdd(&a.common[a.out_eup[j] & ID], n_here);
+                continue;
+            }
+            left &= ~batch;
+            const int n_e = __shfl_sync(FULL, e1, 31 - __clz(batch)) - b;
+            __syncwarp();  // the previous table's counts are added up
+            for (int t = lane; t < TRI_BUCKETS; t += 32) H.key[t] = make_int4(-1, -1, -1, -1);
+            __syncwarp();
+            int32_t* keys = reinterpret_cast<int32_t*>(H.key);
+            for (int t = lane; t < n_e; t += 32) {
+                const int32_t w = a.out_nbr[b + t];
+                int h = 4 * bucket(a.outptr[a.out_src[b + t]] - b, w);
+                H.cnt[t] = 0;
+                for (int p = 0; p < 4 * TRI_BUCKETS; p++) {  // ends: at most half of the slots are taken
+                    if (atomicCAS(&keys[h], -1, w) == -1) {
+                        H.pos[h] = (uint8_t)t;
+                        break;
+                    }
+                    h = (h + 1) & (4 * TRI_BUCKETS - 1);
+                }
+            }
+            // the batch's edges with a list to look up, one a lane, and the lists laid end to end
+            const int32_t len = mine ? e2 - i2 : 0;
+            int32_t inc = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const int32_t total = __shfl_sync(FULL, inc, 31);
+            const unsigned some = __ballot_sync(FULL, len > 0);
+            if (len > 0) H.lane_of[__popc(some & below)] = (uint8_t)lane;
+            __syncwarp();
+            const bool on = lane < __popc(some);
+            const int src = on ? H.lane_of[lane] : 0;
+            const int32_t c_start = __shfl_sync(FULL, inc - len, src);
+            const int32_t start = on ? c_start : INT_MAX;
+            const int32_t shift = __shfl_sync(FULL, i2, src) - c_start;
+            // the list's edge and its tail's list as positions in the stretch
+            const int32_t where = __shfl_sync(FULL, ((i1 - b) << 20) | ((e1 - i1) << 10), src) | (int)(j0 + src - b);
+            int before = 0;  // lists begun before the step
+            int e_n = 0;
+            int32_t at_n = 0, w_n = -1;
+            auto fetch = [&](int32_t t0) {  // the step's list, entry and head of this lane
+                const unsigned begun =
+                    __reduce_or_sync(FULL, start >= t0 && start < t0 + 32 ? 1u << (start - t0) : 0u);
+                e_n = before + __popc(begun & (below | (1u << lane))) - 1;
+                before += __popc(begun);
+                at_n = t0 + lane + __shfl_sync(FULL, shift, e_n);
+                w_n = t0 + lane < total ? a.out_nbr[at_n] : -1;
+            };
+            if (total > 0) fetch(0);
+            for (int32_t t0 = 0; t0 < total; t0 += 32) {
+                const int e = e_n;
+                const int32_t at_v = at_n, w = w_n;
+                if (t0 + 32 < total) fetch(t0 + 32);
+                const int32_t wh = __shfl_sync(FULL, where, e);
+                const int lo = wh >> 20, puv = wh & 0x3ff;
+                int pu = -1;
+                if (w >= 0) {
+                    int h = bucket(lo, w);
+                    for (int p = 0; p < TRI_BUCKETS; p++) {
+                        const int4 k = H.key[h];
+                        const int s4 = k.x == w ? 0 : k.y == w ? 1 : k.z == w ? 2 : k.w == w ? 3 : -1;
+                        if (s4 >= 0) {
+                            const int at_first = 4 * h + s4;
+                            pu = H.pos[at_first];
+                            // another tail's entry of that head: on through the slots
+                            for (int q = at_first; (unsigned)(pu - lo) >= (unsigned)((wh >> 10) & 0x3ff);) {
+                                q = (q + 1) & (4 * TRI_BUCKETS - 1);
+                                const int32_t kq = keys[q];
+                                pu = kq == w ? H.pos[q] : -1;
+                                if (kq < 0 || q == at_first) break;
+                            }
+                            break;
+                        }
+                        if (k.w < 0) break;
+                        h = (h + 1) & (TRI_BUCKETS - 1);
+                    }
+                    if (pu >= 0) {
+                        atomicAdd(&H.cnt[puv], 1);
+                        atomicAdd(&H.cnt[pu], 1);
+                    }
+                }
+                const unsigned m = __ballot_sync(FULL, pu >= 0);
+                if (m) push(m, b + puv, b + pu, at_v);
+            }
+            __syncwarp();
+            for (int t = lane; t < n_e; t += 32)
+                if (H.cnt[t]) atomicAdd(&a.common[a.out_eup[b + t] & ID], H.cnt[t]);
+        }
+        j0 = j_next;
+    }
+    if (queued) write(queued);
+    for (; at < end; at += 32) {
+        a.tri[at + lane] = make_int4(0, 0, 0, -1);
+        a.row[at + lane] = DMIN_NEVER;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if (lane == 0 && acc) atomicAdd(a.merged, acc);
+    if (lane == 0 && found) atomicAdd(a.merged + 1, found);
+}
+
+// The out-lists' static edges as the listing reads them: oe[j] = the run ends of the one at
+// place j in its orientation, eup[j] = its id and whether its tail has the smaller id.
+template <typename TS>
+__global__ void k_out_ends(const int32_t* __restrict__ out_src, const int32_t* __restrict__ out_nbr,
+                           const int32_t* __restrict__ out_eid, int32_t S, const RunEnds<TS>* __restrict__ ends,
+                           OutEnds<TS>* __restrict__ oe, uint32_t* __restrict__ eup) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < S; j += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = out_eid[j];
+        const RunEnds<TS> r = ends[e];
+        const bool up = out_src[j] < out_nbr[j];
+        OutEnds<TS> o;
+        o.f0 = up ? r.f0 : r.f1;
+        o.l0 = up ? r.l0 : r.l1;
+        o.f1 = up ? r.f1 : r.f0;
+        o.l1 = up ? r.l1 : r.l0;
+        oe[j] = o;
+        eup[j] = (uint32_t)e | (up ? 0x80000000u : 0u);
+    }
+}
+
+// Probe slots of all triangles (every temporal edge of a triangle's three static edges: the
+// sum over the static edges of their temporal edges times their triangles) and the largest
+// number of temporal edges of a static edge.
+__global__ void k_probe_total(const int32_t* __restrict__ seg, const int32_t* __restrict__ common, int32_t S,
+                              unsigned long long* __restrict__ probes, int* __restrict__ sigma_max) {
+    unsigned long long acc = 0;
+    int best = 0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < S; e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t c = seg[2 * e + 2] - seg[2 * e];
+        acc += (unsigned long long)c * (unsigned long long)common[e];
+        best = max(best, c);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (acc) atomicAdd(probes, acc);
+        atomicMax(sigma_max, best);
+    }
+}
+
+// Sum over the oriented edges (u, v) of min(|N+(u)|, |N+(v)|), at least the triangles.
 __global__ void k_tri_bound(const int32_t* __restrict__ outptr, const int32_t* __restrict__ out_src,
-                            const int32_t* __restrict__ out_nbr, int32_t S, int64_t* __restrict__ bnd) {
+                            const int32_t* __restrict__ out_nbr, int32_t S, unsigned long long* __restrict__ bound) {
+    unsigned long long acc = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < S; j += (int64_t)gridDim.x * blockDim.x) {
         const int32_t u = out_src[j], v = out_nbr[j];
-        bnd[j] = min(outptr[u + 1] - outptr[u], outptr[v + 1] - outptr[v]);
+        acc += (unsigned long long)min(outptr[u + 1] - outptr[u], outptr[v + 1] - outptr[v]);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(bound, acc);
 }
 
 // ================================================================== driver
@@ -1214,12 +1487,11 @@ static void pair_key_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
 // is neither forced nor cached) and nothing else, for a listing without counting pass.
 static void tune_triangles(folty_graph* g, const int32_t* outptr, const int32_t* out_nbr, const int32_t* out_src,
                            const int32_t* osig, int32_t* tcnt, int64_t* pcnt, unsigned long long* merged,
-                           cudaStream_t s, bool trials_only) {
+                           cudaStream_t s) {
     const int32_t S = g->S;
     const unsigned grid = grid_for(S, TRI_THREADS);
     const std::vector<int64_t> key{g->n, g->m_kept, S};
     bool trials = !(tune_forced(&g->tune, false) || tune_lookup(key, &g->tune, false)) && !profiling_on();
-    if (!trials && trials_only) return;
     if (!trials) {
         FOLTY_CUDA(cudaMemsetAsync(merged, 0, 2 * sizeof(unsigned long long), s));
         FOLTY_LAUNCH(k_tri_count, grid, TRI_THREADS, 0, s, outptr, out_nbr, out_src, osig, S, tcnt, pcnt, merged,
@@ -1248,6 +1520,14 @@ static void tune_triangles(folty_graph* g, const int32_t* outptr, const int32_t*
     g->tune.tri_heavy = TRI_HEAVY_CAND[best];
     g->tune.tri_source = 1;
     tune_store(key, g->tune, false);
+}
+
+template <typename TS>
+static void list_triangles(folty_graph* g, const TriListArgs& a, const int32_t* out_eid, OutEnds<TS>* oe, uint32_t* eup,
+                           int grid, cudaStream_t s) {
+    FOLTY_LAUNCH(k_out_ends<TS>, grid_for(a.S, 256), 256, 0, s, a.out_src, a.out_nbr, out_eid, a.S,
+                 (const RunEnds<TS>*)g->run_ends, oe, eup);
+    FOLTY_LAUNCH(k_tri_list<TS>, grid, TRI_LIST_THREADS, 0, s, a, oe);
 }
 
 void ensure_perm(folty_graph* g, cudaStream_t s) {
@@ -1393,48 +1673,44 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
                      out_eid, out_src);
 
     // ---------------- A5: triangles
-    // the triangle listing needs the static graph and every static edge's temporal edge
-    // count, not the store itself: it runs beside the store's sort (joined before the
-    // run-ends table)
-    if (ids) FOLTY_CUDA(cudaStreamWaitEvent(s, packed_ev.e, 0));
     g->common = graph_alloc<int32_t>(g, S, s);
     FOLTY_CUDA(cudaMemsetAsync(g->common, 0, sizeof(int32_t) * ((size_t)S > 0 ? (size_t)S : 1), s));
-    int32_t* tcnt = sc.get<int32_t>((int64_t)S + 1);
-    int64_t* toff = sc.get<int64_t>((int64_t)S + 1);
-    unsigned long long* merged = sc.get<unsigned long long>(2);  // list lengths merged, probe slots
-    FOLTY_CUDA(cudaMemsetAsync(merged, 0, 2 * sizeof(unsigned long long), s));
-    int32_t* osig = sc.get<int32_t>(S);
-    if (S > 0) FOLTY_LAUNCH(k_out_sigma, grid_for(S, T), T, 0, s, sigma, g->seg, out_eid, S, osig, stat + 2);
+    // [0] list lengths merged, [1] probe slots (of the counting pass) or triangles (of the
+    // one-pass listing); of the latter: [2] the bound, [3] the probe slots, [4] edges taken,
+    // [5] entries taken
+    unsigned long long* merged = sc.get<unsigned long long>(6);
+    FOLTY_CUDA(cudaMemsetAsync(merged, 0, 6 * sizeof(unsigned long long), s));
     FOLTY_LAUNCH(k_max_i32, grid_for(n, T), T, 0, s, g->deg, (int64_t)n, stat + 0);
     // the all-roles probe map (each triangle's first slot in the flat space of every
     // role's probes, and the tile starts) serves only the allocation-free per-edge counts,
     // which take graphs of at most FOLTY_NOALLOC_MAX_EDGES edges; the queries lay out the
     // kept roles of their own selection
     const bool probe_map = g->m_kept <= FOLTY_NOALLOC_MAX_EDGES;
-    int64_t* pcnt = probe_map ? sc.get<int64_t>((int64_t)S + 1) : nullptr;  // slots per oriented edge, then prefix
-    // Larger graphs list their triangles in one pass into a bounded layout (the triangles
-    // of oriented edge (u, v) from the prefix of the bounds min(|N+(u)|, |N+(v)|) on)
-    // that the liveness pass makes dense while it computes the out motif's bytes: no
-    // counting pass before the listing, and no wait for its total. The probe map needs
-    // the counting pass's slots per edge, and a bound past TRI_BOUND_MAX_BYTES takes the
-    // counting pass too.
+    // Larger graphs list their triangles and the out motif's liveness bytes in one pass, into
+    // an array of the upper bound's size: no counting pass before it and no wait for its total.
+    // The pass reads the store's run ends, so it follows the store's sort; the counting pass
+    // needs the static edges' temporal edge counts only and the listing after it neither, so
+    // both run beside that sort. The probe map needs the counting pass's slots per edge, and a
+    // bound past TRI_BOUND_MAX_BYTES takes it too.
     bool bounded = !probe_map && S > 0 && !tri_layout_counted();
-    int64_t* boff = nullptr;
-    std::optional<StageSpan> tri_span;
-    int4* tri_b = nullptr;  // the bounded layout, moved into g->tri by the liveness pass
-    TriLayout layout{};
-    if (bounded) {
-        boff = sc.get<int64_t>((int64_t)S + 1);
-        FOLTY_LAUNCH(k_tri_bound, grid_for(S, T), T, 0, s, outptr, out_src, out_nbr, S, boff);
-        exclusive_scan(sc, boff, boff, S);
-    }
+    int32_t* tcnt = nullptr;
+    int64_t *toff = nullptr, *pcnt = nullptr;  // pcnt: slots per oriented edge, then their prefix
+    int32_t* osig = nullptr;
+    if (bounded)
+        FOLTY_LAUNCH(k_tri_bound, grid_for(S, T), T, 0, s, outptr, out_src, out_nbr, S, merged + 2);
     // the counting pass merges the two out-lists of every oriented edge: 4 B per merged
     // entry (known after its read-back) + 8 B per static edge
     std::optional<StageSpan> count_span;
     auto count_pass = [&]() {
+        if (ids) FOLTY_CUDA(cudaStreamWaitEvent(s, packed_ev.e, 0));
+        tcnt = sc.get<int32_t>((int64_t)S + 1);
+        toff = sc.get<int64_t>((int64_t)S + 1);
+        if (probe_map) pcnt = sc.get<int64_t>((int64_t)S + 1);
+        osig = sc.get<int32_t>(S);
+        if (S > 0) FOLTY_LAUNCH(k_out_sigma, grid_for(S, T), T, 0, s, sigma, g->seg, out_eid, S, osig, stat + 2);
         count_span.emplace(ST_TRIANGLES, s, 8 * (int64_t)S);
         FOLTY_CUDA(cudaMemsetAsync(merged, 0, 2 * sizeof(unsigned long long), s));
-        if (S > 0) tune_triangles(g, outptr, out_nbr, out_src, osig, tcnt, pcnt, merged, s, false);
+        if (S > 0) tune_triangles(g, outptr, out_nbr, out_src, osig, tcnt, pcnt, merged, s);
         exclusive_scan(sc, tcnt, toff, S);
         if (probe_map) exclusive_scan(sc, pcnt, pcnt, S);
         count_span->end();
@@ -1448,7 +1724,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     if (!bounded) count_pass();
     int64_t bound = 0;
     {
-        const void* ptrs[9] = {bounded ? (const void*)(boff + S) : (const void*)(toff + S), stat + 0, stat + 1,
+        const void* ptrs[9] = {bounded ? (const void*)(merged + 2) : (const void*)(toff + S), stat + 0, stat + 1,
                                stat + 2, merged, merged + 1, core_ctl + CORE_ERR, core_ctl + CORE_ROUNDS, core_ctl + CORE_ALPHA};
         int sizes[9] = {8, 4, 4, 4, 8, 8, 4, 4, 4};
         int64_t outv[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -1466,36 +1742,50 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     if (bounded && bound > TRI_BOUND_MAX_BYTES / (int64_t)sizeof(int4)) {
         bounded = false;
         count_pass();
-        const void* ptrs[3] = {toff + S, merged, merged + 1};
-        int sizes[3] = {8, 8, 8};
-        int64_t outv[3] = {0, 0, 0};
-        read_back(g, ptrs, sizes, 3, outv, s);
+        const void* ptrs[4] = {toff + S, merged, merged + 1, stat + 2};
+        int sizes[4] = {8, 8, 8, 4};
+        int64_t outv[4] = {0, 0, 0, 0};
+        read_back(g, ptrs, sizes, 4, outv, s);
         counted(outv[0], outv[1], outv[2]);
+        g->info.sigma_max = (int32_t)outv[3];
     }
     if (bounded) {
-        // the autotuner's trials (the first graph of its size only) time the counting pass
-        tune_triangles(g, outptr, out_nbr, out_src, osig, tcnt, pcnt, merged, s, true);
-        tri_b = sc.get<int4>(bound);
-        // the graph's array holds bound entries, the first ntri of them the triangles
-        // (moved there by the liveness pass): an array of ntri would wait for the
-        // listing's total, a host round trip
-        g->tri = graph_alloc<int4>(g, bound, s);
+        tune_forced(&g->tune, false);  // recorded; the listing has no split to choose
+        const int warps = TRI_LIST_THREADS / 32;
+        const int grid = (int)std::min<int64_t>((S + TRI_LIST_THREADS - 1) / TRI_LIST_THREADS, (int64_t)num_sms() * TRI_PER_SM);
+        int chunk = TRI_CHUNK_MAX;
+        while (chunk > TRI_CHUNK_MIN && (int64_t)chunk * grid * warps * 16 > bound) chunk >>= 1;
+        const int64_t cap = bound + (int64_t)chunk * grid * warps;
+        g->tri = graph_alloc<int4>(g, cap, s);
         g->tri_off = nullptr;
+        prepare_liveness(g, cap, s);
         FOLTY_CUDA(cudaMemsetAsync(merged, 0, 2 * sizeof(unsigned long long), s));
-        // the listing (8 B per static edge + 4 B per merged entry + 16 B per triangle):
-        // the totals come with the read-back after the store's join
-        tri_span.emplace(ST_TRIANGLES, s, 8 * (int64_t)S);
-        // one warp per 32 oriented edges, in short blocks: the dense communities' edges
-        // take far longer than the rest
-        FOLTY_LAUNCH((k_tri_write<false, true>), (unsigned)((S + TRI_THREADS - 1) / TRI_THREADS), TRI_THREADS, 0, s,
-                     outptr, out_nbr,
-                     out_eid, out_src, osig, S, boff, nullptr, tri_b, nullptr, g->common, g->tune.tri_heavy, tcnt,
-                     merged);
-        exclusive_scan(sc, tcnt, toff, S);
-        tri_span->end();
-        layout = TriLayout{tcnt, toff, boff, tri_b};
+        if (ids) side.join();
+        if (!ids) build_run_ends(g, s);
+        // the listing: 8 B per static edge + 4 B per merged entry + 17 B per triangle; the
+        // totals come with the last read-back
+        StageSpan span(ST_TRIANGLES, s, 8 * (int64_t)S);
+        uint32_t* eup = sc.get<uint32_t>(S);
+        const TriListArgs a{outptr, out_nbr, out_src, eup, S, chunk, g->tri,
+                            g->tlive + (int64_t)FOLTY_DIR_OUT * g->tlive_stride, g->common, merged, merged + 4, merged + 5};
+        if (g->ts32) list_triangles<uint32_t>(g, a, out_eid, sc.get<OutEnds<uint32_t>>(S), eup, grid, s);
+        else list_triangles<int64_t>(g, a, out_eid, sc.get<OutEnds<int64_t>>(S), eup, grid, s);
+        FOLTY_LAUNCH(k_probe_total, grid_for(S, T), T, 0, s, g->seg, g->common, S, merged + 3, stat + 2);
+        span.end();
+        listed_liveness(g, s);
+        const void* ptrs[5] = {merged, merged + 1, merged + 3, merged + 5, stat + 2};
+        int sizes[5] = {8, 8, 8, 8, 4};
+        int64_t outv[5] = {0, 0, 0, 0, 0};
+        read_back(g, ptrs, sizes, 5, outv, s);  // it also checks that the store's sort completed
+        g->ntri = outv[1];
+        g->tri_cap = outv[3];
+        g->info.probes = outv[2];
+        g->info.sigma_max = (int32_t)outv[4];
+        g->enum_bytes = 4 * outv[0] + 8 * (int64_t)S;
+        span.add_bytes(4 * outv[0] + 17 * g->ntri);
     } else {
         const int64_t ntri = g->ntri;
+        g->tri_cap = ntri;
         g->tri = graph_alloc<int4>(g, ntri, s);
         g->tri_off = probe_map ? graph_alloc<int64_t>(g, ntri + 1, s) : nullptr;
         if (S > 0) {
@@ -1511,28 +1801,16 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         // the probe offsets of the triangles come from the writing pass; the last entry is the total
         if (probe_map)
             FOLTY_CUDA(cudaMemcpyAsync(g->tri_off + ntri, pcnt + S, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    }
-    if (ids) side.join();
-    if (bounded) {
-        // the listing's totals; the same read-back checks the store's sort, which completed
-        // before its arrays index anything
-        const void* ptrs[3] = {toff + S, merged, merged + 1};
-        int sizes[3] = {8, 8, 8};
-        int64_t outv[3] = {0, 0, 0};
-        read_back(g, ptrs, sizes, 3, outv, s);
-        g->ntri = outv[0];
-        g->info.probes = outv[2];
-        g->enum_bytes = 4 * outv[1] + 8 * (int64_t)S;
-        tri_span->add_bytes(g->enum_bytes - 8 * (int64_t)S + 16 * g->ntri);
-    } else if (ids) {
-        sort_check(g, s);  // the store's sort completed before its arrays index anything
+        if (ids) {
+            side.join();
+            sort_check(g, s);  // the store's sort completed before its arrays index anything
+        } else {
+            build_run_ends(g, s);
+        }
+        prepare_liveness(g, ntri, s);
+        ensure_liveness(g, FOLTY_DIR_OUT, s);
     }
     release_input(g, s);  // the raw input and the pair table's lists are no longer needed
-    // the run-ends table (built beside the triangle passes with the store) and every
-    // triangle's liveness bytes
-    if (!ids) build_run_ends(g, s);
-    prepare_liveness(g, s);
-    triangle_liveness(g, s, bounded ? &layout : nullptr);
     g->info.triangles = g->ntri;
     // tile -> first triangle map of the all-roles probe kernel (query independent)
     g->n_tiles = probe_map ? (g->info.probes + PB_TILE - 1) / PB_TILE : 0;

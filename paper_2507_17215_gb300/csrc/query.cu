@@ -794,7 +794,7 @@ void finish_queries(folty_graph* g, const folty_query_params* const* qs, const C
 
 // ------------------------------------------------------------------ all-existential triples
 
-// Flag i of the 6 * ntri roles as an int32 (input of the scan).
+// Flag i of the 6 * cap roles as an int32 (input of the scan).
 __global__ void k_triple_flags(const uint8_t* __restrict__ rflag, int64_t n6, int32_t* __restrict__ flag) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n6; i += (int64_t)gridDim.x * blockDim.x)
         flag[i] = rflag[i];
@@ -805,9 +805,9 @@ __global__ void k_triple_flags(const uint8_t* __restrict__ rflag, int64_t n6, in
 // witness goes to key_w (the first sort key), x and y to xs and ys.
 __global__ void k_triple_write(const int4* __restrict__ tri, const int32_t* __restrict__ ea,
                                const int32_t* __restrict__ eb, const uint8_t* __restrict__ rflag,
-                               const int32_t* __restrict__ pos, int64_t ntri, uint64_t* __restrict__ key_w,
+                               const int32_t* __restrict__ pos, int64_t cap, uint64_t* __restrict__ key_w,
                                uint32_t* __restrict__ idx, int32_t* __restrict__ xs, int32_t* __restrict__ ys) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 6 * ntri;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 6 * cap;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (!rflag[i]) continue;
         const int64_t t = i / 6;
@@ -852,7 +852,7 @@ __global__ void k_triple_out(const uint32_t* __restrict__ order, const int32_t* 
 // radix sorts (by w, then by (x, y)), into the result's host arrays. Synchronises.
 static void triples_result(folty_graph* g, const uint8_t* rflag, folty_result* out, cudaStream_t s) {
     const int T = 256;
-    const int64_t n6 = 6 * g->ntri;
+    const int64_t n6 = 6 * g->tri_cap;
     Scratch sc(g->alloc, s, g->dev_err);
     int32_t* flag = sc.get<int32_t>(n6 + 1);
     int32_t* pos = sc.get<int32_t>(n6 + 1);
@@ -867,7 +867,7 @@ static void triples_result(folty_graph* g, const uint8_t* rflag, folty_result* o
     uint32_t* ix_alt = sc.get<uint32_t>(nt);
     int32_t* xs = sc.get<int32_t>(nt);
     int32_t* ys = sc.get<int32_t>(nt);
-    FOLTY_LAUNCH(k_triple_write, grid_for(n6, T), T, 0, s, g->tri, g->ea, g->eb, rflag, pos, g->ntri, kw, ix, xs, ys);
+    FOLTY_LAUNCH(k_triple_write, grid_for(n6, T), T, 0, s, g->tri, g->ea, g->eb, rflag, pos, g->tri_cap, kw, ix, xs, ys);
     const int nb = bit_length((uint64_t)(g->n > 1 ? g->n - 1 : 1));
     // the witness value of written triple j stays in kw_src[j] (kept before sorting)
     uint64_t* kw_src = sc.get<uint64_t>(nt);
@@ -1098,8 +1098,8 @@ void run_query(folty_graph* g, const folty_query_params& q, folty_result* out, c
     if (mk > 0 && !c16) FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)mk, s));
     uint8_t* rflag = nullptr;
     if (q.want_triples) {
-        rflag = sc.get<uint8_t>(6 * g->ntri + 1);
-        FOLTY_CUDA(cudaMemsetAsync(rflag, 0, (size_t)(6 * g->ntri + 1), s));
+        rflag = sc.get<uint8_t>(6 * g->tri_cap + 1);
+        FOLTY_CUDA(cudaMemsetAsync(rflag, 0, (size_t)(6 * g->tri_cap + 1), s));
     }
     launch_probe_live(g, q.delta, q.dir, cnt, cnt16, rflag, s);
     const folty_query_params* qp = &q;
@@ -1121,12 +1121,13 @@ void run_query(folty_graph* g, const folty_query_params& q, folty_result* out, c
 // for the direction variant, w = bytes per stored timestamp. Bytes = w sigma1 (read L1)
 // + w min(sigma2, sigma1 * ceil(log2(sigma2 + 1))) + the same for L3 + 8 sigma1
 // (counter read-modify-write).
-__global__ void k_traffic(const int4* __restrict__ tri, int64_t ntri, const int32_t* __restrict__ seg, int dir,
+__global__ void k_traffic(const int4* __restrict__ tri, int64_t cap, const int32_t* __restrict__ seg, int dir,
                           int64_t w, unsigned long long* __restrict__ out) {
     unsigned long long acc = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ntri;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < cap;
          i += (int64_t)gridDim.x * blockDim.x) {
         int4 tr = tri[i];
+        if (tr.w < 0) continue;
         int32_t off[9];
         const int32_t se[3] = {tr.x, tr.y, tr.z};
 #pragma unroll
@@ -1162,7 +1163,7 @@ void traffic_model(folty_graph* g, int dir, folty_traffic_model* out, cudaStream
     unsigned long long* acc = sc.get<unsigned long long>(1);
     FOLTY_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long), s));
     if (g->ntri > 0)
-        FOLTY_LAUNCH(k_traffic, grid_for(g->ntri, 256), 256, 0, s, g->tri, g->ntri, g->seg, dir,
+        FOLTY_LAUNCH(k_traffic, grid_for(g->tri_cap, 256), 256, 0, s, g->tri, g->tri_cap, g->seg, dir,
                      (int64_t)(g->ts32 ? 4 : 8), acc);
     out->probe_bytes = read_i64(g, (const int64_t*)acc, s);
     out->enum_bytes = g->enum_bytes;

@@ -133,3 +133,69 @@ def test_probes_from_every_list(F, sizes, t_max, scale):
     with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G, oracle.OracleGraph.of(g) as og:
         for q, r in zip(batch, G.query_batch(batch)):
             assert pairs_of(r) == pairs_of(og.query(q)), str(q)
+
+
+def _cliques_and_hubs(cliques, hubs, spread, seed, scale=1):
+    """Cliques of the given sizes; per hub size one vertex pair joined to that many others (its
+    triangles share one edge); a sparse remainder. Every edge repeated until the graph is past
+    the allocation-free counts' limit, so that its triangles are listed in one pass."""
+    rng = np.random.default_rng(seed)
+    pairs, n = [], 0
+    for k in cliques:
+        i, j = np.triu_indices(k, 1)
+        pairs.append(np.stack([i + n, j + n], 1))
+        n += k
+    for k in hubs:
+        leaf = np.arange(k) + n + 2
+        pairs += [np.stack([np.full(k, n + h), leaf], 1) for h in (0, 1)] + [np.array([[n, n + 1]])]
+        n += k + 2
+    a = rng.integers(0, n + spread, (spread, 2))
+    pairs.append(a[a[:, 0] != a[:, 1]])
+    n += spread
+    pairs = np.concatenate(pairs)
+    pairs = np.concatenate([pairs] * (1_100_000 // len(pairs) + 1))
+    order = rng.permutation(n).astype(np.int32)  # degeneracy order and id order differ
+    flip = rng.random(len(pairs)) < 0.4
+    src = order[np.where(flip, pairs[:, 1], pairs[:, 0])]
+    dst = order[np.where(flip, pairs[:, 0], pairs[:, 1])]
+    return W.TemporalGraph(n, src, dst, np.sort(rng.integers(0, 20_000, len(pairs))) * scale)
+
+
+# the one-pass listing: stretches of out-lists up to, at and past the table's 256 entries, lists
+# of a whole step of 32 and around it, a warp's chunk filled exactly and overrun, triangles so few
+# that most of a chunk stays empty, none; 32- and 64-bit stores; against the counting pass
+@pytest.mark.parametrize("cliques,hubs,spread", [((3,), (), 1000), ((31, 32, 33, 34), (31, 33), 0), ((255, 257), (700,), 9),
+                                                 ((300,), (), 50_000), ((), (), 900_000), ((), (40_000,), 0),
+                                                 ((5,) * 4000, (), 0)])
+@pytest.mark.parametrize("scale", [1, 10 ** 6])
+def test_one_pass_listing(F, monkeypatch, cliques, hubs, spread, scale):
+    g = _cliques_and_hubs(cliques, hubs, spread, 17 * len(cliques) + len(hubs) + spread, scale)
+    qs = [W.Query(d * scale, 1, 2, W.Q_EXISTS, dr, W.U_HEAD, True) for d in (0, 40, 20_000)
+          for dr in (W.DIR_IN, W.DIR_OUT, W.DIR_EITHER)]
+    got = []
+    for layout in ("", "counted"):
+        monkeypatch.setenv("FOLTY_TRI_LAYOUT", layout)
+        with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G:
+            assert G.info()["m_kept"] > F.NOALLOC_MAX_EDGES
+            got.append((G.info(), [G.query(q) for q in qs], G.query_batch([W.Query(q.delta, 1, 2, W.Q_EXISTS, q.dir, W.U_HEAD)
+                                                                          for q in qs])))
+    (info, res, batch), (info2, res2, batch2) = got
+    keys = ("triangles", "probes", "sigma_max", "degeneracy", "max_out_degree")
+    assert [info[k] for k in keys] == [info2[k] for k in keys]
+    n_clique = sum(k * (k - 1) * (k - 2) // 6 for k in cliques) + sum(hubs)
+    assert info["triangles"] >= n_clique
+    for x, y in zip(res, res2):
+        np.testing.assert_array_equal(x["edge_count"], y["edge_count"])
+        assert pairs_of(x) == pairs_of(y)
+    for x, y in zip(batch, batch2):
+        assert pairs_of(x) == pairs_of(y)
+
+
+def test_triples_of_a_one_pass_listing(F):
+    """The exists-triples output, which numbers roles by the triangle array's entries."""
+    g = _cliques_and_hubs((9, 4), (20,), 200, 5)
+    q = W.Query(3, 1, 2, W.Q_EXISTS, W.DIR_OUT, W.U_HEAD, False, want_triples=True)
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G, oracle.OracleGraph.of(g) as og:
+        got, want = G.query(q)["triples"], og.triples(q.delta, q.dir)
+    assert len(want) > 0
+    np.testing.assert_array_equal(got, want)
