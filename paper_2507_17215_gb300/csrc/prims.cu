@@ -117,7 +117,7 @@ void exclusive_scan(Scratch& sc, const uint32_t* in, uint32_t* out, int64_t n) {
 // ================================================================== radix sort
 //
 // Stable LSD radix sort, one kernel per 8-bit digit ("onesweep"): the histograms of all
-// digits come from one read of the keys up front; each pass takes tiles of 4096 keys in
+// digits come from one read of the keys up front; each pass takes tiles of 4096 or 8192 keys in
 // the order blocks start (a dynamic tile counter), ranks them by digit within the tile,
 // publishes the tile's digit counts, and adds the counts of all earlier tiles by looking
 // back over their published values (decoupled look-back: a tile's entry holds either its
@@ -127,6 +127,10 @@ void exclusive_scan(Scratch& sc, const uint32_t* in, uint32_t* out, int64_t n) {
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // 4096 keys per tile
+constexpr int RS_AHEAD = 4;  // items whose peer masks are made together
+// look-back entries in flight a thread: two take as long, sixteen (mostly read in vain, 2 KB an
+// entry) 10% longer at 70M keys
+constexpr int RS_LOOK = 4;
 constexpr int RS_BITS = 8;
 constexpr int RS_BINS = 1 << RS_BITS;
 constexpr int RS_MAX_PASSES = 8;
@@ -221,25 +225,30 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d) {
 }
 
 // One pass of one 8-bit digit over a tile of NT * RS_ITEMS keys:
-//  1. every load of the tile is issued before any is used; keys and values are staged
-//     in shared memory in load order;
+//  1. every load of the tile is issued before any is used; keys and values stay in
+//     registers;
 //  2. ranks within the tile: warp w owns keys [w * 32 * ITEMS, ...) in order, ranked by
 //     digit with per-bit ballots and per-warp 16-bit counters (stable);
-//  3. thread d < RS_BINS (one per digit) turns the per-warp counts into offsets,
-//     publishes the tile's count of digit d and looks back over earlier tiles for its
-//     global offset;
-//  4. a 16-bit permutation in shared memory lists the tile in digit order, and the
-//     writes of each digit's run are contiguous. Positions are 32-bit (n < 2^32).
+//  3. thread d < RS_BINS (one per digit) turns the per-warp counts into offsets and
+//     publishes the tile's count of digit d;
+//  4. keys and values go to shared memory in digit order, while earlier tiles publish;
+//  5. thread d looks back over earlier tiles for the global offset of digit d;
+//  6. the tile is written, each digit's run contiguous. Positions are 32-bit (n < 2^32).
+// Bound by instruction issue (60% of the slots: a third of it the peer masks) and the
+// look-back's waits: 70M ids with values take 390 us a pass (1.1 GB, 2.9 TB/s). Staging the tile
+// in load order and listing it through a 16-bit permutation after the look-back moved twice
+// the bytes through shared memory and left the look-back uncovered: 500 us.
 // V: values travel with the keys (a keys-only sort moves 8 bytes a key instead of 12).
-// NT: threads per block. The keys-only sort runs 512-thread blocks: tiles of 8192 keys
-// halve the tiles in flight, and with them the depth of every look-back, and double the
-// length of each digit's written run.
+// NT: threads per block. The keys-only sort and the store's passes run 512-thread blocks:
+// tiles of 8192 keys halve the tiles in flight, and with them the depth of every look-back,
+// and double the length of each digit's written run (the store at 70M edges: 390 us a pass; 256
+// threads 464, 1024 threads 469).
 // K: the key type; 32-bit keys (the store's sorts, key-value only) move 8 bytes a key.
 // MODE (ST_FIRST, ST_LAST, ST_IOTA flags, 32-bit keys only): the store's passes that
 // build their keys from the edge list and write the store's arrays instead of keys and
 // values.
 template <bool V, int NT, int MODE = 0, typename K = uint64_t>
-__global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 ? 2 : 4))
+__global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     k_rs_onesweep(OnesweepArgs a) {
     static_assert(sizeof(K) == 8 || V, "32-bit keys carry values");
     static_assert(MODE == 0 || sizeof(K) == 4, "the store's passes sort 32-bit ids");
@@ -247,9 +256,8 @@ __global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 
     constexpr int TILE = NT * RS_ITEMS;
     static_assert(NT % RS_BINS == 0 && NT >= RS_BINS, "one thread per digit at least");
     extern __shared__ __align__(16) unsigned char rs_smem[];
-    K* skey = (K*)rs_smem;                                  // TILE, load order
-    uint32_t* sval = (uint32_t*)(skey + TILE);              // TILE, load order (V only)
-    uint16_t* sperm = (uint16_t*)(V ? (void*)(sval + TILE) : (void*)sval);  // TILE, digit order -> load order
+    K* skey = (K*)rs_smem;                      // TILE, digit order
+    uint32_t* sval = (uint32_t*)(skey + TILE);  // TILE, digit order (V only)
     __shared__ uint16_t wh[WARPS][RS_BINS];                 // per-warp counts, then offsets
     __shared__ uint32_t bstart[RS_BINS];                    // tile-local start of each digit
     __shared__ uint32_t adj[RS_BINS];                       // final position of digit-order slot j: adj + j
@@ -269,54 +277,53 @@ __global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 
     K* kout = sizeof(K) == 8 ? (K*)a.okeys : (K*)a.okeys32;
     const uint32_t* vin = a.vals + t0;
     const int wbase = warp * 32 * RS_ITEMS;
-    // ---- 1. loads, staging, digits
-    uint32_t info[RS_ITEMS];  // digit | rank within (warp, digit) << 8
-    {
-        K kr[RS_ITEMS];
-        uint32_t vr[RS_ITEMS];
-#pragma unroll
-        for (int i = 0; i < RS_ITEMS; i++) {
-            const int idx = wbase + i * 32 + lane;
-            if (MODE & ST_FIRST) {
-                kr[i] = (idx < tn) ? (K)__ldcs(a.cw + t0 + idx) : (K)0;
-                if (MODE & ST_IOTA) vr[i] = (uint32_t)(t0 + idx);
-                else vr[i] = (idx < tn) ? __ldcs(a.t + t0 + idx) - a.tmin : 0u;
-            } else {
-                kr[i] = (idx < tn) ? kin[idx] : (K)0;
-                if (V) vr[i] = (idx < tn) ? vin[idx] : 0u;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < RS_ITEMS; i++) {
-            const int idx = wbase + i * 32 + lane;
-            if (idx < tn) {
-                skey[idx] = kr[i];
-                if (V) sval[idx] = vr[i];
-            }
-            info[i] = (unsigned)(kr[i] >> a.shift) & (RS_BINS - 1);
-        }
-    }
-    // ---- 2. ranks: every item's peer mask first (independent ballot chains the scheduler
-    // can interleave), then the per-warp counters item by item
-    const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned pm[RS_ITEMS];
-#pragma unroll
-    for (int i = 0; i < RS_ITEMS; i++) pm[i] = digit_peers(info[i]);
+    // ---- 1. loads
+    K kr[RS_ITEMS];
+    uint32_t vr[V ? RS_ITEMS : 1];
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; i++) {
         const int idx = wbase + i * 32 + lane;
-        const bool valid = idx < tn;
-        const unsigned dd = info[i];
-        const unsigned peers = pm[i] & __ballot_sync(0xffffffffu, valid);
-        unsigned before = 0;
-        if (valid) before = wh[warp][dd];
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) wh[warp][dd] = (uint16_t)(before + __popc(peers));
-        __syncwarp();
-        info[i] = dd | ((before + __popc(peers & lt_mask)) << 8);
+        if (MODE & ST_FIRST) {
+            kr[i] = (idx < tn) ? (K)__ldcs(a.cw + t0 + idx) : (K)0;
+        } else {
+            kr[i] = (idx < tn) ? kin[idx] : (K)0;
+        }
+    }
+    if (V) {
+#pragma unroll
+        for (int i = 0; i < RS_ITEMS; i++) {
+            const int idx = wbase + i * 32 + lane;
+            if (MODE & ST_IOTA && MODE & ST_FIRST) vr[i] = (uint32_t)(t0 + idx);
+            else if (MODE & ST_FIRST) vr[i] = (idx < tn) ? __ldcs(a.t + t0 + idx) - a.tmin : 0u;
+            else vr[i] = (idx < tn) ? vin[idx] : 0u;
+        }
+    }
+    // ---- 2. ranks: the peer masks of RS_AHEAD items (independent ballot chains the scheduler
+    // can interleave), then the per-warp counters item by item
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint32_t rank[RS_ITEMS / 2];  // within (warp, digit), two items a word
+#pragma unroll
+    for (int i0 = 0; i0 < RS_ITEMS; i0 += RS_AHEAD) {
+        unsigned pm[RS_AHEAD];
+#pragma unroll
+        for (int i = 0; i < RS_AHEAD; i++) pm[i] = digit_peers((unsigned)(kr[i0 + i] >> a.shift) & (RS_BINS - 1));
+#pragma unroll
+        for (int i = 0; i < RS_AHEAD; i++) {
+            const bool valid = wbase + (i0 + i) * 32 + lane < tn;
+            const unsigned dd = (unsigned)(kr[i0 + i] >> a.shift) & (RS_BINS - 1);
+            const unsigned peers = pm[i] & __ballot_sync(0xffffffffu, valid);
+            unsigned before = 0;
+            if (valid) before = wh[warp][dd];
+            __syncwarp();
+            if (valid && lane == __ffs(peers) - 1) wh[warp][dd] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            const uint32_t r = before + __popc(peers & lt_mask);
+            if (((i0 + i) & 1) == 0) rank[(i0 + i) / 2] = r;
+            else rank[(i0 + i) / 2] |= r << 16;
+        }
     }
     __syncthreads();
-    // ---- 3. per digit (thread d < RS_BINS): warp offsets, tile count, publish, look back
+    // ---- 3. per digit (thread d < RS_BINS): warp offsets, tile count, publish
     const int d = threadIdx.x;
     const bool dig = d < RS_BINS;  // whole warps: RS_BINS is a multiple of 32
     uint32_t cnt = 0;
@@ -346,20 +353,32 @@ __global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 
             bs = off + inc - cnt;
             bstart[d] = bs;
         }
+        __syncthreads();
     }
+    // ---- 4. the tile in digit order
+#pragma unroll
+    for (int i = 0; i < RS_ITEMS; i++) {
+        if (wbase + i * 32 + lane < tn) {
+            const unsigned dd = (unsigned)(kr[i] >> a.shift) & (RS_BINS - 1);
+            const int at = (int)(bstart[dd] + wh[warp][dd] + ((rank[i / 2] >> (16 * (i & 1))) & 0xffffu));
+            skey[at] = kr[i];
+            if (V) sval[at] = vr[i];
+        }
+    }
+    // ---- 5. look back
     unsigned long long excl = 0;
     if (dig && tile > 0) {
-        // four entries in flight per step; an entry not yet published is polled again
+        // RS_LOOK entries in flight per step; an entry not yet published is polled again
         int64_t p = tile - 1;
         long long t_start = 0;
         bool done = false;
         while (!done) {
-            unsigned long long e[4];
+            unsigned long long e[RS_LOOK];
 #pragma unroll
-            for (int j = 0; j < 4; j++) e[j] = (p - j >= 0) ? (unsigned long long)lb[(p - j) * RS_BINS + d] : LB_PREFIX;
+            for (int j = 0; j < RS_LOOK; j++) e[j] = (p - j >= 0) ? (unsigned long long)lb[(p - j) * RS_BINS + d] : LB_PREFIX;
             bool stall = false;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
+            for (int j = 0; j < RS_LOOK; j++) {
                 if (!done && !stall) {
                     if (e[j] == 0) {
                         stall = true;
@@ -387,39 +406,31 @@ __global__ void __launch_bounds__(NT, V ? (sizeof(K) == 4 ? 4 : 3) : (NT == 512 
     if (dig) adj[d] = (uint32_t)((unsigned long long)a.base[d] + excl) - bs;  // mod 2^32
     __syncthreads();
     if (s_fail) return;  // block-uniform: positions are unknown
-    // ---- 4. digit-order permutation, then contiguous runs
-#pragma unroll
-    for (int i = 0; i < RS_ITEMS; i++) {
-        const int idx = wbase + i * 32 + lane;
-        if (idx < tn) {
-            const unsigned dd = info[i] & (RS_BINS - 1);
-            sperm[bstart[dd] + wh[warp][dd] + (info[i] >> 8)] = (uint16_t)idx;
-        }
-    }
-    __syncthreads();
+    // ---- 6. contiguous runs
     for (int j = threadIdx.x; j < tn; j += NT) {
-        const int src = sperm[j];
-        const K kk = skey[src];
+        const K kk = skey[j];
         const uint32_t pos = adj[(unsigned)(kk >> a.shift) & (RS_BINS - 1)] + (uint32_t)j;
         if (MODE & ST_LAST) {
             if ((int64_t)pos < a.limit) {
                 if (MODE & ST_IOTA) {
-                    __stcs(a.perm + pos, (int32_t)sval[src]);
+                    __stcs(a.perm + pos, (int32_t)sval[j]);
                 } else {
-                    __stcs(a.T + pos, sval[src]);
+                    __stcs(a.T + pos, sval[j]);
                     __stcs(a.sd + pos, (int32_t)kk);
                 }
             }
         } else {
             kout[pos] = kk;
-            if (V) a.ovals[pos] = sval[src];
+            if (V) a.ovals[pos] = sval[j];
         }
     }
 }
 
 constexpr int RS_NT_K = 512;  // threads of a keys-only block
-constexpr size_t RS_DYN_SMEM = RS_TILE * (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(uint16_t));
-constexpr size_t RS_DYN_SMEM_K = (size_t)RS_NT_K * RS_ITEMS * (sizeof(uint64_t) + sizeof(uint16_t));
+constexpr int RS_NT_S = 512;  // of a block of the store's passes
+constexpr int RS_TILE_S = RS_NT_S * RS_ITEMS;
+constexpr size_t RS_DYN_SMEM = RS_TILE * (sizeof(uint64_t) + sizeof(uint32_t));
+constexpr size_t RS_DYN_SMEM_K = (size_t)RS_NT_K * RS_ITEMS * sizeof(uint64_t);
 
 // Sorts by the digits of bits [lo, lo + bits); vals may be null (keys only).
 static bool radix_sort_impl(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt,
@@ -449,7 +460,7 @@ static bool radix_sort_impl(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, uin
     } else {
         FOLTY_CUDA(cudaFuncSetAttribute(k_rs_onesweep<false, RS_NT_K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)RS_DYN_SMEM_K));
-        // two blocks of 90 KB each need the largest shared-memory carveout
+        // two blocks of 74 KB each need a large shared-memory carveout
         FOLTY_CUDA(cudaFuncSetAttribute(k_rs_onesweep<false, RS_NT_K>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     }
     bool alt = false;
@@ -484,10 +495,10 @@ static_assert(STORE_DIGIT_BITS == RS_BITS, "the caller's digit histograms match 
 
 template <int MODE>
 static void store_pass(const OnesweepArgs& oa, int64_t tiles, cudaStream_t s) {
-    constexpr size_t smem = RS_TILE * (sizeof(uint32_t) + sizeof(uint32_t) + sizeof(uint16_t));
-    FOLTY_CUDA(cudaFuncSetAttribute(k_rs_onesweep<true, RS_THREADS, MODE, uint32_t>,
+    constexpr size_t smem = RS_TILE_S * (sizeof(uint32_t) + sizeof(uint32_t));
+    FOLTY_CUDA(cudaFuncSetAttribute(k_rs_onesweep<true, RS_NT_S, MODE, uint32_t>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    FOLTY_LAUNCH((k_rs_onesweep<true, RS_THREADS, MODE, uint32_t>), (unsigned)tiles, RS_THREADS, smem, s, oa);
+    FOLTY_LAUNCH((k_rs_onesweep<true, RS_NT_S, MODE, uint32_t>), (unsigned)tiles, RS_NT_S, smem, s, oa);
 }
 
 // The key-value sort of 32-bit sort ids (radix_sort_pairs' passes on 32-bit keys) whose
@@ -501,7 +512,7 @@ static void store_sort_impl(Scratch& sc, const StoreSortArgs& a) {
     const int passes = a.cbits > RS_BITS ? (a.cbits + RS_BITS - 1) / RS_BITS : 1;
     if (passes > STORE_MAX_PASSES) fail(FOLTY_EINVAL, "store sort: sort ids past 32 bits");
     cudaStream_t s = sc.stream();
-    const int64_t tiles = (n + RS_TILE - 1) / RS_TILE;
+    const int64_t tiles = (n + RS_TILE_S - 1) / RS_TILE_S;
     uint32_t* base = sc.get<uint32_t>(STORE_MAX_PASSES * RS_BINS);
     unsigned long long* lbc = sc.get<unsigned long long>(tiles * RS_BINS + 1);
     FOLTY_LAUNCH(k_rs_bases, 1, RS_BINS, 0, s, a.hist, passes, base);

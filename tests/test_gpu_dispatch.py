@@ -199,3 +199,71 @@ def test_triples_of_a_one_pass_listing(F):
         got, want = G.query(q)["triples"], og.triples(q.delta, q.dir)
     assert len(want) > 0
     np.testing.assert_array_equal(got, want)
+
+
+# the sorts at the edges of their tiles (4096 pairs of 64-bit keys, 8192 ids) and with one digit
+# holding every key; in time order (the store's passes) and not (the time sort)
+@pytest.mark.parametrize("m", [4095, 4096, 4097, 8191, 8192, 8193, 16_385, 24_576])
+@pytest.mark.parametrize("n", [2, 700])
+def test_sorts_at_tile_edges(F, m, n):
+    rng = np.random.default_rng(m + n)
+    g = W.random_small_graph(rng, n, m, 10 ** 6)
+    p = rng.permutation(len(g.src))
+    for x in (g, W.TemporalGraph(g.n, g.src[p], g.dst[p], g.t[p])):
+        _check(F, x, [W.Query(d, 1, 2, W.Q_FORALL_T, W.DIR_OUT, W.U_HEAD, True) for d in (1000, 10 ** 6)])
+
+
+def _core_numbers(n, pairs):
+    """Core numbers by the bucket algorithm: remove a vertex of least degree, one at a time."""
+    adj = [[] for _ in range(n)]
+    for a, b in pairs.tolist():
+        adj[a].append(b)
+        adj[b].append(a)
+    deg = [len(x) for x in adj]
+    buckets = [[] for _ in range(max(deg) + 1)]
+    for v in range(n):
+        buckets[deg[v]].append(v)
+    core, level, d = [-1] * n, 0, 0
+    while d < len(buckets):
+        if not buckets[d]:
+            d += 1
+            continue
+        v = buckets[d].pop()
+        if core[v] >= 0 or deg[v] != d:
+            continue
+        level = max(level, d)
+        core[v] = level
+        for w in adj[v]:
+            if core[w] < 0:
+                deg[w] -= 1
+                buckets[deg[w]].append(w)
+                d = min(d, deg[w])
+    return np.array(core)
+
+
+# adjacency rows at the lengths where the work on a row changes hands (a lane, a warp, a block,
+# several), hubs past the longest histogram, cores of every size up to the largest clique
+@pytest.mark.parametrize("rows,cliques", [((8, 9, 64, 65), (5, 9)), ((511, 512, 513), (33,)), ((8192, 8193), (65, 130)),
+                                          ((16_384, 16_385, 40_000), (10,)), ((), (520,))])
+def test_core_numbers_at_row_edges(F, rows, cliques):
+    rng = np.random.default_rng(sum(rows) + len(cliques))
+    n = max((0,) + rows) + len(rows) + sum(cliques) + 50
+    pairs = [rng.integers(0, n, (n, 2))]
+    at = 0
+    for k in cliques:
+        i, j = np.triu_indices(k, 1)
+        pairs.append(np.stack([i + at, j + at], 1))
+        at += k
+    for k in rows:
+        others = rng.choice(np.setdiff1d(np.arange(n), [at]), k, replace=False)
+        pairs.append(np.stack([np.full(k, at), others], 1))
+        at += 1
+    pairs = np.concatenate(pairs)
+    pairs = np.unique(np.sort(pairs[pairs[:, 0] != pairs[:, 1]], axis=1), axis=0)
+    ids = rng.permutation(n)
+    pairs = ids[pairs]
+    want = _core_numbers(n, pairs)
+    with F.TemporalGraph(n, pairs[:, 0].astype(np.int32), pairs[:, 1].astype(np.int32),
+                         np.zeros(len(pairs), np.int64)) as G:
+        np.testing.assert_array_equal(G.core_numbers(), want)
+        assert G.info()["degeneracy"] == want.max()
