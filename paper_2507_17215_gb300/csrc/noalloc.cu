@@ -52,7 +52,8 @@ void edge_counts_noalloc(folty_graph* g, int64_t delta, int dir, int32_t* edge_c
                                std::to_string((long long)FOLTY_NOALLOC_MAX_EDGES));
     if (mk > 0 && !g->perm) fail(FOLTY_EINVAL, "graph has no input order of its store");  // made by preprocessing
     int32_t* cnt = noalloc_counts_on_current_device();
-    if (g->m > 0) FOLTY_CUDA(cudaMemsetAsync(edge_count, 0, sizeof(int32_t) * (size_t)g->m, s));
+    // the scatter writes the count of every edge that is no self-loop
+    if (g->m > mk) FOLTY_CUDA(cudaMemsetAsync(edge_count, 0, sizeof(int32_t) * (size_t)g->m, s));
     if (mk == 0) return;
     FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)mk, s));  // previous call's counts
     launch_probe(g, delta, dir, cnt, s);
