@@ -63,18 +63,19 @@ WORKLOADS = {
 
 STAGE_KERNELS = {
     "probe": "k_probe_live (persistent window probes over the kept roles)",
-    "select": "k_live_sums + k_live_offsets + k_live_write (selection of the kept triangles by their liveness bytes)",
+    "select": "k_live_candidates + k_live_select (the kept triangles by their liveness bytes)",
     "sort": "radix sort spans: k_rs_hist_all + k_rs_bases (all digit histograms), or one k_rs_onesweep digit pass",
-    "peel": "k_peel (cooperative) + k_tail_* + k_peel_tail + k_solo_* + k_peel_solo",
-    "threshold": "k_threshold",
-    "triangles": "k_tri_bound + k_tri_write (one pass into the bounded layout; k_tri_count first on small graphs)",
-    "roles": "k_run_ends + k_tri_live_copy (liveness bytes while the triangles move to the dense layout)",
-    "batch": "k_batch_threshold",
-    "store": "temporal store beside the peel: k_store_ids, k_store_hist, the id sort's k_rs_onesweep passes "
+    "peel": "k_core (cooperative: h-index rounds, then removal rounds of all levels)",
+    "threshold": "k_threshold_hits (plain queries), k_threshold (optional outputs)",
+    "triangles": "k_out_ends + k_tri_list + k_probe_total (one pass with the out motif's liveness bytes; "
+                 "k_tri_count + k_tri_write on small graphs)",
+    "roles": "k_run_ends, and k_tri_live for a motif's liveness bytes on first use",
+    "batch": "k_word_counts + k_row_edges + k_batch_threshold",
+    "store": "temporal store beside the core numbers: k_store_ids, k_store_hist, the id sort's k_rs_onesweep passes "
              "(contains sort spans)",
 }
 STAGE_SOURCES = {"probe": ("live.cu", "probe.cuh"), "select": ("live.cu", "scan.cuh"), "sort": ("prims.cu",),
-                 "peel": ("preprocess.cu",), "threshold": ("query.cu",), "triangles": ("preprocess.cu",),
+                 "peel": ("core.cu",), "threshold": ("query.cu",), "triangles": ("preprocess.cu", "liveness.cuh"),
                  "roles": ("live.cu", "liveness.cuh"), "batch": ("batch.cu",), "store": ("preprocess.cu", "prims.cu")}
 QUERY_STAGES = ("select", "probe", "threshold")
 

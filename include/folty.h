@@ -117,7 +117,7 @@ typedef struct {
     int32_t max_degree;     /* max |N(u)|                                      */
     int32_t degeneracy;     /* alpha = max core number (Definition 2.1)        */
     int32_t max_out_degree; /* max |N+(u)| in the oriented graph (<= alpha)    */
-    int32_t peel_rounds;    /* rounds of the parallel peeling                  */
+    int32_t peel_rounds;    /* removal rounds, over all levels                 */
     int64_t triangles;      /* triangles of G_S                                */
     int64_t probes;         /* sum over triangles of the sizes of its 3 edges' */
                             /* temporal lists (= (edge, witness) pairs)        */
@@ -134,12 +134,12 @@ typedef struct {
     int64_t threshold_bytes;
 } folty_traffic_model;
 
-/* Section 1.2 / Section 2 input. Copies the m edges (src[i] -> dst[i] at t[i]) into
- * device memory owned by the new graph and validates them. The three arrays may be
- * host or device pointers (detected per pointer); they stay owned by the caller and
- * are not referenced after the call returns. Memory of the current device and pinned
- * host memory, all three 16-byte aligned, are copied and checked by one kernel pass;
- * other input is copied first, then checked. alloc may be NULL. On success *out
+/* Section 1.2 / Section 2 input. Reads the m edges (src[i] -> dst[i] at t[i]),
+ * validates them, and keeps what preprocessing needs of them in device memory owned by
+ * the new graph. The three arrays may be host or device pointers (detected per
+ * pointer); they stay owned by the caller and are not referenced after the call
+ * returns. Memory of the current device and pinned host memory are read in place by one
+ * kernel pass; other input is copied to the device first. alloc may be NULL. On success *out
  * receives a graph in the "loaded" state. Errors: FOLTY_EINVAL (n, m out of range, an
  * id outside [0, n), t outside [0, 2^62)), FOLTY_ENOMEM, FOLTY_ECUDA. */
 folty_status folty_load_temporal_graph(int32_t n, int64_t m, const int32_t *src,
@@ -148,10 +148,10 @@ folty_status folty_load_temporal_graph(int32_t n, int64_t m, const int32_t *src,
                                        folty_graph **out);
 
 /* Section 2 preprocessing: drops self-loops, sorts edges into E_{x,y} lists, builds
- * G_S, its degeneracy order (Definition 2.1, by parallel peeling) and orientation,
+ * G_S, its degeneracy order (Definition 2.1, by its core numbers and removal rounds) and orientation,
  * and lists every triangle of G_S once. Moves the graph to the "preprocessed" state.
  * Errors: FOLTY_ESTATE (already preprocessed), FOLTY_ENOMEM, FOLTY_ECUDA,
- * FOLTY_ETIMEOUT (a device-side barrier of the peeling kernel gave up). */
+ * FOLTY_ETIMEOUT (a device-side barrier of the core number kernel gave up). */
 folty_status folty_preprocess(folty_graph *g, void *stream);
 
 /* One query (Algorithm 6 semantics): window probes for every (edge, witness) pair,
@@ -192,7 +192,7 @@ folty_status folty_graph_traffic_model(folty_graph *g, int32_t dir,
 typedef struct {
     int64_t triangles, all_roles, all_probes;  /* 6 roles per triangle; every (edge, witness) */
     int64_t kept_triangles, kept_roles, kept_probes;
-    int64_t select_bytes;  /* liveness pass: 30 B per triangle + 13 B per kept triangle */
+    int64_t select_bytes;  /* selection: 1 B per triangle entry + per kept triangle its record, run ends and 21 B */
     int64_t probe_bytes;   /* probe pass: 61 B per kept triangle + the per-role bytes    */
 } folty_probe_stats;
 
@@ -227,12 +227,13 @@ uint64_t folty_kernel_launches(void);
  *             timestamp), counted on the device;
  *   SORT      one radix pass: 8 B read for the histogram, 12 B read + 12 B written per key
  *             (8 B + 8 B for the temporal store's 32-bit sort ids with their values);
- *   PEEL      the degeneracy peeling: 12 B per adjacency entry + 16 B per vertex;
+ *   PEEL      core numbers and removal rounds: 12 B per adjacency entry + 16 B per vertex;
  *   THRESHOLD certificate test and per-pair reduction: 8 B per temporal edge (4 with 16-bit
  *             counters) + 20 B per directed pair;
  *   SELECT    the per-query selection of the triangles whose liveness byte admits the
- *             window (k_live_select): 1 B read per triangle; per kept triangle its record
- *             and its edges' run ends read and 13 B written, counted on the device;
+ *             window (k_live_candidates, k_live_select): 1 B read per triangle; per kept
+ *             triangle its record and its edges' run ends read, 13 B written, and its place
+ *             in the list of candidates written and read, counted on the device;
  *   TRIANGLES triangle listing: 4 B per merged out-list entry + 8 B per static edge and
  *             16 B written per triangle; graphs up to FOLTY_NOALLOC_MAX_EDGES edges also
  *             count first (the same merge bytes again) and write 8 B more per triangle;
@@ -245,7 +246,7 @@ uint64_t folty_kernel_launches(void);
  *   BATCH     the batched threshold over the plain queries of a direction variant: the
  *             32-edge group bits, and (counted on the device) the bin row and 4 B of pair
  *             key of every edge in a group with a hit;
- *   STORE     the temporal store built beside the peeling: its span contains SORT spans.
+ *   STORE     the temporal store built beside the core numbers: its span contains SORT spans.
  *             Time-ordered input with 32-bit offsets: 8 B per input edge for the sort ids
  *             and 16 B per edge and radix pass (the first pass reads 4 B more: the ids and
  *             the input times); other inputs: 24 B per input edge for the pair words and

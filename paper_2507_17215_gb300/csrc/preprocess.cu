@@ -924,8 +924,8 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
 // The triangles of the stretch's edges, as (u, v) and as (u, w), are counted in shared memory
 // and added to common once; merged[0] receives the list entries looked up, merged[1] the
 // triangles.
-// Bound by instruction issue (80% of the slots; 4 blocks more or less an SM: 5% slower). At full
-// size, 77M triangles from 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M
+// Bound by issue slots and by gathers from L2 (46% of the slots, 33% of the warps at 20M edges;
+// seven or nine blocks an SM are 3 to 5% slower at full size). At full size, 77M triangles from 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M
 // lookups: 400. A lane or a warp per edge, into a layout by upper bounds with three additions to
 // common a triangle, and a second pass that gathered the three edges' runs and moved the
 // triangles took 1110 + 750 and 584 + 75; the same without the queue, the records made by the

@@ -235,13 +235,13 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d) {
 //  5. thread d looks back over earlier tiles for the global offset of digit d;
 //  6. the tile is written, each digit's run contiguous. Positions are 32-bit (n < 2^32).
 // Bound by instruction issue (60% of the slots: a third of it the peer masks) and the
-// look-back's waits: 70M ids with values take 390 us a pass (1.1 GB, 2.9 TB/s). Staging the tile
+// look-back's waits: 70M ids with values take 390 to 435 us a pass (1.1 GB, 2.7 TB/s). Staging the tile
 // in load order and listing it through a 16-bit permutation after the look-back moved twice
 // the bytes through shared memory and left the look-back uncovered: 500 us.
 // V: values travel with the keys (a keys-only sort moves 8 bytes a key instead of 12).
 // NT: threads per block. The keys-only sort and the store's passes run 512-thread blocks:
 // tiles of 8192 keys halve the tiles in flight, and with them the depth of every look-back,
-// and double the length of each digit's written run (the store at 70M edges: 390 us a pass; 256
+// and double the length of each digit's written run (the store at 70M edges: 410 us a pass; 256
 // threads 464, 1024 threads 469).
 // K: the key type; 32-bit keys (the store's sorts, key-value only) move 8 bytes a key.
 // MODE (ST_FIRST, ST_LAST, ST_IOTA flags, 32-bit keys only): the store's passes that
