@@ -247,13 +247,13 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d) {
 // MODE (ST_FIRST, ST_LAST, ST_IOTA flags, 32-bit keys only): the store's passes that
 // build their keys from the edge list and write the store's arrays instead of keys and
 // values.
-template <bool V, int NT, int MODE = 0, typename K = uint64_t>
+template <bool V, int NT, int MODE = 0, typename K = uint64_t, int ITEMS = RS_ITEMS>
 __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     k_rs_onesweep(OnesweepArgs a) {
     static_assert(sizeof(K) == 8 || V, "32-bit keys carry values");
     static_assert(MODE == 0 || sizeof(K) == 4, "the store's passes sort 32-bit ids");
     constexpr int WARPS = NT / 32;
-    constexpr int TILE = NT * RS_ITEMS;
+    constexpr int TILE = NT * ITEMS;
     static_assert(NT % RS_BINS == 0 && NT >= RS_BINS, "one thread per digit at least");
     extern __shared__ __align__(16) unsigned char rs_smem[];
     K* skey = (K*)rs_smem;                      // TILE, digit order
@@ -276,12 +276,12 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     const K* kin = (sizeof(K) == 8 ? (const K*)a.keys : (const K*)a.keys32) + t0;
     K* kout = sizeof(K) == 8 ? (K*)a.okeys : (K*)a.okeys32;
     const uint32_t* vin = a.vals + t0;
-    const int wbase = warp * 32 * RS_ITEMS;
+    const int wbase = warp * 32 * ITEMS;
     // ---- 1. loads
-    K kr[RS_ITEMS];
-    uint32_t vr[V ? RS_ITEMS : 1];
+    K kr[ITEMS];
+    uint32_t vr[V ? ITEMS : 1];
 #pragma unroll
-    for (int i = 0; i < RS_ITEMS; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         const int idx = wbase + i * 32 + lane;
         if (MODE & ST_FIRST) {
             kr[i] = (idx < tn) ? (K)__ldcs(a.cw + t0 + idx) : (K)0;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     }
     if (V) {
 #pragma unroll
-        for (int i = 0; i < RS_ITEMS; i++) {
+        for (int i = 0; i < ITEMS; i++) {
             const int idx = wbase + i * 32 + lane;
             if (MODE & ST_IOTA && MODE & ST_FIRST) vr[i] = (uint32_t)(t0 + idx);
             else if (MODE & ST_FIRST) vr[i] = (idx < tn) ? __ldcs(a.t + t0 + idx) - a.tmin : 0u;
@@ -301,9 +301,9 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     // ---- 2. ranks: the peer masks of RS_AHEAD items (independent ballot chains the scheduler
     // can interleave), then the per-warp counters item by item
     const unsigned lt_mask = (1u << lane) - 1u;
-    uint32_t rank[RS_ITEMS / 2];  // within (warp, digit), two items a word
+    uint32_t rank[ITEMS / 2];  // within (warp, digit), two items a word
 #pragma unroll
-    for (int i0 = 0; i0 < RS_ITEMS; i0 += RS_AHEAD) {
+    for (int i0 = 0; i0 < ITEMS; i0 += RS_AHEAD) {
         unsigned pm[RS_AHEAD];
 #pragma unroll
         for (int i = 0; i < RS_AHEAD; i++) pm[i] = digit_peers((unsigned)(kr[i0 + i] >> a.shift) & (RS_BINS - 1));
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     }
     // ---- 4. the tile in digit order
 #pragma unroll
-    for (int i = 0; i < RS_ITEMS; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         if (wbase + i * 32 + lane < tn) {
             const unsigned dd = (unsigned)(kr[i] >> a.shift) & (RS_BINS - 1);
             const int at = (int)(bstart[dd] + wh[warp][dd] + ((rank[i / 2] >> (16 * (i & 1))) & 0xffffu));
@@ -426,6 +426,13 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 3)
     }
 }
 
+// Sorts of at most RS_SMALL 64-bit keys are bound by the latency of one tile's chain, with SMs
+// left over: tiles of 1024 keys spread them out. 20K edges: preprocessing 550 -> 519 us; a
+// query with every output on 2M edges: its sorts 108 -> 82. From about 2^18 keys on the deeper
+// look-backs cost more (800K keys: 1.40 -> 1.45 ms for a preprocessing with two sorts of them).
+constexpr int RS_ITEMS_SMALL = 4;
+constexpr int RS_TILE_SMALL = RS_THREADS * RS_ITEMS_SMALL;
+constexpr int64_t RS_SMALL = 1 << 18;
 constexpr int RS_NT_K = 512;  // threads of a keys-only block
 constexpr int RS_NT_S = 512;  // of a block of the store's passes
 constexpr int RS_TILE_S = RS_NT_S * RS_ITEMS;
@@ -440,7 +447,8 @@ static bool radix_sort_impl(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, uin
     cudaStream_t s = sc.stream();
     const bool kv = vals != nullptr;
     const int passes = (bits + RS_BITS - 1) / RS_BITS;
-    const int64_t tile = kv ? RS_TILE : (int64_t)RS_NT_K * RS_ITEMS;
+    const bool few = n <= RS_SMALL;
+    const int64_t tile = few ? RS_TILE_SMALL : kv ? RS_TILE : (int64_t)RS_NT_K * RS_ITEMS;
     const int64_t tiles = (n + tile - 1) / tile;
     uint32_t* hist = sc.get<uint32_t>(2 * RS_MAX_PASSES * RS_BINS);
     uint32_t* base = hist + RS_MAX_PASSES * RS_BINS;
@@ -470,7 +478,13 @@ static bool radix_sort_impl(Scratch& sc, uint64_t* keys, uint64_t* keys_alt, uin
         OnesweepArgs oa{alt ? keys_alt : keys, kv ? (alt ? vals_alt : vals) : nullptr, alt ? keys : keys_alt,
                         kv ? (alt ? vals : vals_alt) : nullptr, n, lo + RS_BITS * p, base + p * RS_BINS, lb, counter,
                         sc.err(), LOOKBACK_TIMEOUT_NS};
-        if (kv) FOLTY_LAUNCH((k_rs_onesweep<true, RS_THREADS>), (unsigned)tiles, RS_THREADS, RS_DYN_SMEM, s, oa);
+        if (few && kv)
+            FOLTY_LAUNCH((k_rs_onesweep<true, RS_THREADS, 0, uint64_t, RS_ITEMS_SMALL>), (unsigned)tiles, RS_THREADS,
+                         RS_TILE_SMALL * (sizeof(uint64_t) + sizeof(uint32_t)), s, oa);
+        else if (few)
+            FOLTY_LAUNCH((k_rs_onesweep<false, RS_THREADS, 0, uint64_t, RS_ITEMS_SMALL>), (unsigned)tiles, RS_THREADS,
+                         RS_TILE_SMALL * sizeof(uint64_t), s, oa);
+        else if (kv) FOLTY_LAUNCH((k_rs_onesweep<true, RS_THREADS>), (unsigned)tiles, RS_THREADS, RS_DYN_SMEM, s, oa);
         else FOLTY_LAUNCH((k_rs_onesweep<false, RS_NT_K>), (unsigned)tiles, RS_NT_K, RS_DYN_SMEM_K, s, oa);
         alt = !alt;
     }

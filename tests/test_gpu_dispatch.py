@@ -267,3 +267,14 @@ def test_core_numbers_at_row_edges(F, rows, cliques):
                          np.zeros(len(pairs), np.int64)) as G:
         np.testing.assert_array_equal(G.core_numbers(), want)
         assert G.info()["degeneracy"] == want.max()
+
+
+# the tile of the small sorts and the size at which the larger tiles take over
+@pytest.mark.parametrize("m", [1023, 1024, 1025, 3072, (1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+def test_small_sorts(F, m):
+    rng = np.random.default_rng(m)
+    n = 60 if m < 5000 else 60_000
+    src, dst = rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32)
+    dst = np.where(src == dst, (dst + 1) % n, dst).astype(np.int32)
+    _check(F, W.TemporalGraph(n, src, dst, rng.integers(0, 10 ** 6, m)),
+           [W.Query(10 ** 5, 1, 2, W.Q_FORALL_T, W.DIR_EITHER, W.U_HEAD, True)])
