@@ -25,8 +25,11 @@
 // A hub of 35,000 neighbours on the medium graph ends at 71, and changes in most rounds: its
 // row would be read again and again for the hundred neighbours that matter. When its value
 // falls, a vertex of more than CORE_ROW8 neighbours keeps the ones whose value is at least
-// a part (CORE_KEEP) of its new one; values only fall, so the others cannot count while it
-// stays at or above that. Below, the whole row is read again, and shortened anew.
+// a part (CORE_KEEP) of its new one. A shortened row holds every neighbour whose value is at
+// least slo, the highest of the bounds it has been cut at (a later cut's may be lower, but
+// what an earlier one dropped does not come back); values only fall, so the others cannot
+// count while the vertex stays at or above slo. Below, the whole row is read again, and
+// shortened anew.
 //
 // The last rounds of both halves hold a few vertices each: one block runs them alone, with
 // block barriers.
@@ -100,7 +103,7 @@ struct CoreArgs {
     int32_t bcap;  // entries of big, bfr
     int32_t* srow;  // shortened rows, at the places of the whole ones in adj
     int32_t* slen;  // their lengths, -1: the whole row stands
-    int32_t* slo;   // and the least value kept
+    int32_t* slo;   // a shortened row holds every neighbour of at least this value
     int32_t* lev;  // [hcap + 2] rounds of each level (zeroed)
     int* ctl;      // zeroed
     long long timeout_ns;
@@ -457,7 +460,7 @@ __device__ int long_h(const CoreArgs& a, const int32_t* row, int d, int top, int
 }
 
 // Step A over a list of vertices (rows of more than CORE_MID entries skipped). A shortened
-// row answers for values from its least kept one on. Below, the whole row stands again: read
+// row answers for values from its bound (slo) on. Below, the whole row stands again: read
 // at once when a warp holds it, else by a block in the next round (nx; the vertex keeps its
 // value until then).
 __device__ void h_pass(const CoreArgs& a, Team t, const int32_t* list, int count, Next nx) {
@@ -735,7 +738,7 @@ __device__ void tell_pass_big(const CoreArgs& a, Team t, const int32_t* list, in
         __syncthreads();
         if (!REMOVE && threadIdx.x == 0) {
             a.val[v] = to;
-            a.slo[v] = (to + keep_part - 1) / keep_part;
+            a.slo[v] = max(r.cut ? __ldcg(&a.slo[v]) : 0, (to + keep_part - 1) / keep_part);
             a.slen[v] = s_kept;
         }
         __syncthreads();  // s_kept is read before the next vertex clears it
