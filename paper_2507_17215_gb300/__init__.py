@@ -286,12 +286,14 @@ class _Held:
 # per-edge counts stay in the library's memory (8 MB at 2M edges took 0.48 ms to copy); the
 # other lists are short, and copied in one piece
 _RESULT_WORDS = ctypes.sizeof(folty_result) // 8
+_start_of = (ctypes.c_char * 0).from_buffer
 
 
 def _block(addr: int, count: int, dtype) -> np.ndarray:
-    if count == 0:
-        return np.zeros(0, dtype)
-    return np.frombuffer(bytearray(ctypes.string_at(addr, count * np.dtype(dtype).itemsize)), dtype)
+    b = np.empty(count, dtype)
+    if count:
+        ctypes.memmove(_start_of(b), addr, b.nbytes)  # its size is a size_t: lists may pass 2^31 bytes
+    return b
 
 
 def _take_results(rs, n: int) -> List[Dict[str, object]]:

@@ -1,0 +1,58 @@
+"""How the binding takes results over from the library's memory: lists past 2^31 bytes.
+Results are made here as the library makes them (host memory of malloc, released by
+folty_free)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+RESULT_TAG, FREED_TAG = 0x464F4C5459525354, 0x464F4C5459465245
+
+
+@pytest.fixture(scope="module")
+def F():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2507_17215_gb300 as F
+    return F
+
+
+@pytest.fixture(scope="module")
+def libc():
+    libc = ctypes.CDLL(None)
+    libc.calloc.restype = ctypes.c_void_p
+    libc.calloc.argtypes = [ctypes.c_size_t, ctypes.c_size_t]
+    return libc
+
+
+def _set_pairs(F, libc, r, k, m=0):
+    """k pairs (0 so far) in one block, and with m > 0 that many per-edge counts."""
+    r.tag, r.n_pairs = RESULT_TAG, k
+    block = libc.calloc(4 * k, 4)
+    for i, name in enumerate(("u", "v", "count", "ncert")):
+        setattr(r, name, ctypes.cast(block + 4 * k * i, ctypes.POINTER(ctypes.c_int32)))
+    if m:
+        r.m = m
+        r.edge_count = ctypes.cast(libc.calloc(m, 4), ctypes.POINTER(ctypes.c_int32))
+
+
+@pytest.mark.parametrize("count", [(1 << 28) + 2])
+def test_certificates_past_two_gigabytes(F, libc, count):
+    r = F.folty_result()
+    r.tag, r.n_cert_edges = RESULT_TAG, count
+    r.certificate = ctypes.cast(libc.calloc(count, 8), ctypes.POINTER(ctypes.c_int64))
+    r.certificate[count - 1] = 7
+    got = F._take_results(r, 1)[0]["certificates"]
+    assert got.shape == (count,) and got.dtype == np.int64 and got[-1] == 7 and got[0] == 0
+    assert r.tag == FREED_TAG
+
+
+@pytest.mark.parametrize("k", [(1 << 27) + 1])
+def test_pairs_past_two_gigabytes(F, libc, k):
+    r = F.folty_result()
+    _set_pairs(F, libc, r, k)
+    r.u[k - 1], r.ncert[k - 1] = 5, 9
+    got = F._take_results(r, 1)[0]
+    assert [got[x].shape for x in ("u", "v", "count", "ncert")] == [(k,)] * 4
+    assert got["u"][-1] == 5 and got["v"][0] == 0 and got["ncert"][-1] == 9
+    assert r.tag == FREED_TAG
