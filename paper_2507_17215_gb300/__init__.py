@@ -285,7 +285,7 @@ class _Held:
 
 # per-edge counts stay in the library's memory (8 MB at 2M edges took 0.48 ms to copy); the
 # other lists are short, and copied in one piece
-_RESULT_WORDS = ctypes.sizeof(folty_result) // 8
+_RESULT_BYTES = ctypes.sizeof(folty_result)
 _start_of = (ctypes.c_char * 0).from_buffer
 
 
@@ -296,12 +296,23 @@ def _block(addr: int, count: int, dtype) -> np.ndarray:
     return b
 
 
+def _take_edge_counts(rs, i: int, m: int, addr: int) -> np.ndarray:
+    """The per-edge counts of result i as an array that owns them; the result keeps the rest."""
+    if m == 0:
+        return np.zeros(0, np.int32)
+    r = folty_result.from_buffer(rs, i * _RESULT_BYTES)
+    memory = (c_int32 * m).from_address(addr)
+    memory.held = _Held(folty_result(tag=r.tag, edge_count=r.edge_count))
+    r.edge_count = None
+    return np.frombuffer(memory, np.int32)
+
+
 def _take_results(rs, n: int) -> List[Dict[str, object]]:
     """The n results of a ctypes array, whose memory is released or handed over."""
     out: List[Dict[str, object]] = []
     if n == 0:
         return out
-    for i, row in enumerate(np.frombuffer(rs, np.int64, n * _RESULT_WORDS).reshape(n, _RESULT_WORDS).tolist()):
+    for i, row in enumerate(np.frombuffer(rs, np.int64, n * _RESULT_BYTES // 8).reshape(n, -1).tolist()):
         (_, k, u, v, count, ncert, certs, m, edges, nv, vertex, vertex_count, certificate, nt, tx, ty, tw) = row
         if k == 0:
             r = {name: np.zeros(0, np.int32) for name in ("u", "v", "count", "ncert")}
@@ -312,16 +323,7 @@ def _take_results(rs, n: int) -> List[Dict[str, object]]:
             r = {"u": _block(u, k, np.int32), "v": _block(v, k, np.int32), "count": _block(count, k, np.int32),
                  "ncert": _block(ncert, k, np.int32)}
         r["n_cert_edges"] = certs
-        r["edge_count"] = None
-        held = None
-        if edges:
-            if m > 0:
-                held = _Held(folty_result.from_buffer_copy(rs, i * ctypes.sizeof(folty_result)))
-                memory = (c_int32 * m).from_address(edges)
-                memory.held = held
-                r["edge_count"] = np.frombuffer(memory, np.int32)
-            else:
-                r["edge_count"] = np.zeros(0, np.int32)
+        r["edge_count"] = _take_edge_counts(rs, i, m, edges) if edges else None
         if vertex:
             r["vertex"] = _block(vertex, nv, np.int32)
             r["vertex_count"] = _block(vertex_count, nv, np.int32)
@@ -329,8 +331,8 @@ def _take_results(rs, n: int) -> List[Dict[str, object]]:
             r["certificates"] = _block(certificate, certs, np.int64)
         if tx:
             r["triples"] = np.stack([_block(p, nt, np.int32) for p in (tx, ty, tw)], axis=1)
-        if held is None and (u or edges or vertex or certificate or tx):
-            lib.folty_free(ctypes.byref(rs, i * ctypes.sizeof(folty_result)))
+        if u or edges or vertex or certificate or tx:
+            lib.folty_free(ctypes.byref(rs, i * _RESULT_BYTES))
         out.append(r)
     return out
 

@@ -1,6 +1,6 @@
-"""How the binding takes results over from the library's memory: lists past 2^31 bytes.
-Results are made here as the library makes them (host memory of malloc, released by
-folty_free)."""
+"""How the binding takes results over from the library's memory: lists past 2^31 bytes,
+and what an array of per-edge counts keeps alive. Results are made here as
+the library makes them (host memory of malloc, released by folty_free)."""
 import ctypes
 
 import numpy as np
@@ -56,3 +56,18 @@ def test_pairs_past_two_gigabytes(F, libc, k):
     assert [got[x].shape for x in ("u", "v", "count", "ncert")] == [(k,)] * 4
     assert got["u"][-1] == 5 and got["v"][0] == 0 and got["ncert"][-1] == 9
     assert r.tag == FREED_TAG
+
+
+def test_edge_counts_keep_their_own_memory_only(F, libc):
+    rs = (F.folty_result * 2)()
+    for i, r in enumerate(rs):
+        _set_pairs(F, libc, r, 3, 5 + i)
+        r.edge_count[4] = 11 + i
+    got = F._take_results(rs, 2)
+    # the lists have been released, the counts live on with their arrays
+    assert [r.tag for r in rs] == [FREED_TAG] * 2
+    assert [bool(r.u) for r in rs] == [False] * 2
+    counts = [x["edge_count"] for x in got]
+    del got
+    assert [c.tolist() for c in counts] == [[0, 0, 0, 0, 11], [0, 0, 0, 0, 12, 0]]
+    assert all(c.flags["WRITEABLE"] for c in counts)
