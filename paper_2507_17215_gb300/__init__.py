@@ -308,32 +308,37 @@ def _take_edge_counts(rs, i: int, m: int, addr: int) -> np.ndarray:
 
 
 def _take_results(rs, n: int) -> List[Dict[str, object]]:
-    """The n results of a ctypes array, whose memory is released or handed over."""
+    """The n results of a ctypes array, whose memory is released or handed over, also when
+    taking one of them fails."""
     out: List[Dict[str, object]] = []
     if n == 0:
         return out
-    for i, row in enumerate(np.frombuffer(rs, np.int64, n * _RESULT_BYTES // 8).reshape(n, -1).tolist()):
-        (_, k, u, v, count, ncert, certs, m, edges, nv, vertex, vertex_count, certificate, nt, tx, ty, tw) = row
-        if k == 0:
-            r = {name: np.zeros(0, np.int32) for name in ("u", "v", "count", "ncert")}
-        elif v - u == count - v == ncert - count == 4 * k:  # one allocation
-            b = _block(u, 4 * k, np.int32)
-            r = {"u": b[:k], "v": b[k:2 * k], "count": b[2 * k:3 * k], "ncert": b[3 * k:]}
-        else:
-            r = {"u": _block(u, k, np.int32), "v": _block(v, k, np.int32), "count": _block(count, k, np.int32),
-                 "ncert": _block(ncert, k, np.int32)}
-        r["n_cert_edges"] = certs
-        r["edge_count"] = _take_edge_counts(rs, i, m, edges) if edges else None
-        if vertex:
-            r["vertex"] = _block(vertex, nv, np.int32)
-            r["vertex_count"] = _block(vertex_count, nv, np.int32)
-        if certificate:
-            r["certificates"] = _block(certificate, certs, np.int64)
-        if tx:
-            r["triples"] = np.stack([_block(p, nt, np.int32) for p in (tx, ty, tw)], axis=1)
-        if u or edges or vertex or certificate or tx:
+    try:
+        for i, row in enumerate(np.frombuffer(rs, np.int64, n * _RESULT_BYTES // 8).reshape(n, -1).tolist()):
+            (_, k, u, v, count, ncert, certs, m, edges, nv, vertex, vertex_count, certificate, nt, tx, ty, tw) = row
+            if k == 0:
+                r = {name: np.zeros(0, np.int32) for name in ("u", "v", "count", "ncert")}
+            elif v - u == count - v == ncert - count == 4 * k:  # one allocation
+                b = _block(u, 4 * k, np.int32)
+                r = {"u": b[:k], "v": b[k:2 * k], "count": b[2 * k:3 * k], "ncert": b[3 * k:]}
+            else:
+                r = {"u": _block(u, k, np.int32), "v": _block(v, k, np.int32), "count": _block(count, k, np.int32),
+                     "ncert": _block(ncert, k, np.int32)}
+            r["n_cert_edges"] = certs
+            r["edge_count"] = _take_edge_counts(rs, i, m, edges) if edges else None
+            if vertex:
+                r["vertex"] = _block(vertex, nv, np.int32)
+                r["vertex_count"] = _block(vertex_count, nv, np.int32)
+            if certificate:
+                r["certificates"] = _block(certificate, certs, np.int64)
+            if tx:
+                r["triples"] = np.stack([_block(p, nt, np.int32) for p in (tx, ty, tw)], axis=1)
+            if u or edges or vertex or certificate or tx:
+                lib.folty_free(ctypes.byref(rs, i * _RESULT_BYTES))
+            out.append(r)
+    finally:
+        for i in range(len(out), n):
             lib.folty_free(ctypes.byref(rs, i * _RESULT_BYTES))
-        out.append(r)
     return out
 
 

@@ -1,5 +1,5 @@
-"""How the binding takes results over from the library's memory: lists past 2^31 bytes,
-and what an array of per-edge counts keeps alive. Results are made here as
+"""How the binding takes results over from the library's memory: lists past 2^31 bytes, an
+error on the way, and what an array of per-edge counts keeps alive. Results are made here as
 the library makes them (host memory of malloc, released by folty_free)."""
 import ctypes
 
@@ -71,3 +71,21 @@ def test_edge_counts_keep_their_own_memory_only(F, libc):
     del got
     assert [c.tolist() for c in counts] == [[0, 0, 0, 0, 11], [0, 0, 0, 0, 12, 0]]
     assert all(c.flags["WRITEABLE"] for c in counts)
+
+
+def test_an_error_releases_every_result(F, libc, monkeypatch):
+    rs = (F.folty_result * 4)()
+    for r in rs:
+        _set_pairs(F, libc, r, 3, 5)
+    real, calls = F._block, []
+
+    def failing(*args):
+        calls.append(args)
+        if len(calls) == 2:
+            raise MemoryError
+        return real(*args)
+
+    monkeypatch.setattr(F, "_block", failing)
+    with pytest.raises(MemoryError):
+        F._take_results(rs, 4)
+    assert [r.tag for r in rs] == [FREED_TAG] * 4
