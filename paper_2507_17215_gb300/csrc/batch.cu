@@ -10,7 +10,7 @@
 // rho and universe only enter the threshold (Definition 1.1; Algorithm 5), so one pass over
 // the rows answers every query of the variant (k_batch_threshold); the solution pairs of
 // all queries are appended as (query, rank of the pair in (u, v) order) keys and sorted
-// once. Queries that also want per-edge counts, certificates or vertex solutions take the
+// once, or whenever their buffer is full (BatchSolutions). Queries that also want per-edge counts, certificates or vertex solutions take the
 // single-query threshold path on the prefix-summed rows instead. When the rows of all
 // deltas do not fit in the memory budget, the deltas are cut into chunks, one binning pass
 // per chunk (bin 0 of a chunk also holds every smaller gap).
@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <optional>
 
 #include "internal.cuh"
 #include "probe.cuh"
@@ -514,11 +515,12 @@ static void fused_threshold(folty_graph* g, const C* bins, const BatchRows& br, 
     FOLTY_LAUNCH(k_batch_threshold<C>, (unsigned)blocks, BT_THREADS, smem, s, a);
 }
 
-// The results of the plain queries from their n solutions: sorted by (query, pair rank),
-// gathered into per-query (u, v, count, ncert), copied out. slot i is the query plain[i].
-static void batch_results(folty_graph* g, const BatchOutput& out, int64_t n, const std::vector<int>& plain,
-                          folty_result* outs, Scratch& so, cudaStream_t s) {
+// The results of the queries of `slots` from their n < 2^31 solutions: sorted by (query, pair
+// rank), gathered into per-query (u, v, count, ncert), copied out. slot i is the query plain[i].
+static void batch_results(folty_graph* g, const BatchOutput& out, int64_t n, const std::vector<int>& slots,
+                          const std::vector<int>& plain, folty_result* outs, cudaStream_t s) {
     const int nq = (int)plain.size();
+    Scratch so(g->alloc, s, g->dev_err);
     std::vector<int32_t> qstart((size_t)nq + 1, -1);
     std::vector<int32_t> host;
     const int32_t* packed_h = nullptr;
@@ -557,7 +559,7 @@ static void batch_results(folty_graph* g, const BatchOutput& out, int64_t n, con
     for (int i = nq - 1; i >= 0; i--) {
         if (qstart[(size_t)i] < 0) qstart[(size_t)i] = qstart[(size_t)i + 1];
     }
-    for (int i = 0; i < nq; i++) {
+    for (int i : slots) {
         const int64_t b = qstart[(size_t)i], e = qstart[(size_t)i + 1], np = e - b;
         folty_result* r = &outs[plain[(size_t)i]];
         fill_result_host(r, np, g->m, false, 0, false, 0, false);
@@ -573,6 +575,92 @@ static void batch_results(folty_graph* g, const BatchOutput& out, int64_t n, con
     }
 }
 
+// The solutions of a batch's plain queries. Fused passes append theirs to one buffer, so that
+// an ordinary batch is sorted and copied out once; when the buffer cannot take a pass's, the
+// queries before it get their results first, and that pass's threshold runs again with room
+// for all of them. So the memory is that of one pass (at most BT_MAXQ queries), not of the
+// batch, and fewer than 2^31 solutions are in the buffer at a time.
+constexpr int64_t BT_MAX_SOLUTIONS = 0x7fffffff;
+
+class BatchSolutions {
+  public:
+    BatchSolutions(folty_graph* g, const std::vector<int>& plain, folty_result* outs, int64_t cap, cudaStream_t s)
+        : g_(g), plain_(plain), outs_(outs), s_(s) {
+        out_.rb = bit_length((uint64_t)(g->S > 0 ? 2 * (int64_t)g->S - 1 : 1));
+        if (!plain.empty()) reserve(cap);
+    }
+
+    // The buffer's solution count on the device, for a read-back the caller makes anyway, and
+    // its value. Null without plain queries.
+    const unsigned long long* counter() const { return out_.n_out; }
+    void counted(int64_t n) {
+        n_ = n;
+        exact_ = true;
+    }
+
+    // The queries of one fused pass, which has at most `most` solutions: launch(out) appends.
+    template <typename Launch>
+    void pass(const std::vector<BatchQuery>& hq, int64_t most, Launch&& launch) {
+        if (n_ + most > out_.cap) count();
+        const int64_t before = n_;
+        launch(out_);
+        n_ += most;
+        exact_ = most == 0 && exact_;
+        if (n_ > out_.cap) {
+            count();
+            if (n_ > out_.cap) {
+                const int64_t mine = n_ - before;
+                results(before);
+                if (mine > out_.cap) reserve(mine);
+                launch(out_);
+                counted(mine);
+            }
+        }
+        for (const BatchQuery& q : hq) slots_.push_back(q.slot);
+    }
+
+    void finish() {
+        if (plain_.empty()) return;
+        count();
+        results(n_);
+    }
+
+  private:
+    void clear() {
+        FOLTY_CUDA(cudaMemsetAsync(out_.n_out, 0, sizeof(unsigned long long), s_));
+        counted(0);
+    }
+    void count() {
+        if (!exact_) counted(read_i64(g_, (const int64_t*)out_.n_out, s_));
+    }
+    void reserve(int64_t cap) {
+        buf_.reset();
+        buf_.emplace(g_->alloc, s_, g_->dev_err);
+        out_.cap = cap;
+        out_.n_out = buf_->get<unsigned long long>(1);
+        out_.key = buf_->get<uint64_t>(cap);
+        out_.run = buf_->get<int32_t>(cap);
+        out_.cnt = buf_->get<int32_t>(cap);
+        out_.nc = buf_->get<int32_t>(cap);
+        clear();
+    }
+    void results(int64_t n) {
+        if (!slots_.empty()) batch_results(g_, out_, n, slots_, plain_, outs_, s_);
+        slots_.clear();
+        clear();
+    }
+
+    folty_graph* g_;
+    const std::vector<int>& plain_;
+    folty_result* outs_;
+    cudaStream_t s_;
+    std::optional<Scratch> buf_;
+    BatchOutput out_;
+    std::vector<int> slots_;  // queries whose solutions are in the buffer
+    int64_t n_ = 0;           // the buffer's solutions, or a bound on them
+    bool exact_ = false;
+};
+
 // Queries of one direction variant and their sorted distinct windows.
 struct BatchPass {
     int dir;
@@ -585,9 +673,9 @@ constexpr int64_t BT_SMALL_ROWS = int64_t(256) << 20;
 
 // One direction variant: selection, marks, rows and, per chunk of windows, the bins, the
 // plain queries' solutions (slot[i] = their index among the plain queries, -1 for others)
-// and, with others, the results of the queries with per-edge outputs.
+// and the results of the queries with per-edge outputs.
 static void run_batch_pass(folty_graph* g, const folty_query_params* qs, const BatchPass& ps, const std::vector<int>& slot,
-                           const BatchOutput& out, bool others, folty_result* outs, cudaStream_t s, int64_t bin_budget) {
+                           BatchSolutions& sol, folty_result* outs, cudaStream_t s, int64_t bin_budget) {
     const int64_t mk = g->m_kept;
     // 16-bit bins while no count can reach 2^16 (a count is at most the number of common
     // neighbours of an edge's ends, at most the largest degree): half the memory traffic
@@ -607,7 +695,12 @@ static void run_batch_pass(folty_graph* g, const folty_query_params* qs, const B
         launch_marks(g, ps.D.back(), ps.dir, pb, br.ebits, s);
         FOLTY_LAUNCH(k_word_counts, grid_for(nw, 256), 256, 0, s, br.ebits, nw, br.wpref);
         exclusive_scan(sc, br.wpref, br.wpref, nw);
-        br.rows = read_i32(g, br.wpref + nw, s);
+        const void* ptrs[2] = {br.wpref + nw, sol.counter()};
+        const int sizes[2] = {4, 8};
+        int64_t v[2];
+        read_back(g, ptrs, sizes, sol.counter() ? 2 : 1, v, s);
+        br.rows = v[0];
+        if (sol.counter()) sol.counted(v[1]);
     }
     if (br.rows > 0) {
         br.cpos = sc.get<int32_t>(br.rows);
@@ -662,7 +755,6 @@ static void run_batch_pass(folty_graph* g, const folty_query_params* qs, const B
                                         (int64_t)q.rho_den});
                 continue;
             }
-            if (!others) continue;
             fq.push_back(&q);
             // the query's counts c_e(D_j), gathered from the rows
             void* col = b16 ? (void*)sk.get<uint16_t>(mk + 2) : (void*)sk.get<int32_t>(mk);
@@ -676,11 +768,14 @@ static void run_batch_pass(folty_graph* g, const folty_query_params* qs, const B
             fc.push_back(b16 ? CountView{nullptr, (const uint16_t*)col} : CountView{(const int32_t*)col, nullptr});
             fo.push_back(&outs[i]);
         }
-        for (size_t q0 = 0; q0 < pq.size(); q0 += BT_MAXQ) {
-            const std::vector<BatchQuery> gq(pq.begin() + (long)q0,
-                                             pq.begin() + (long)std::min(pq.size(), q0 + (size_t)BT_MAXQ));
-            if (b16) fused_threshold<uint16_t>(g, bins16, br, k, kstride, gq, out, sk, up, s);
-            else fused_threshold<int32_t>(g, bins, br, k, kstride, gq, out, sk, up, s);
+        // a query has at most one solution per row, so this many queries have fewer than 2^31
+        const size_t group = (size_t)std::min<int64_t>(BT_MAXQ, BT_MAX_SOLUTIONS / std::max<int64_t>(br.rows, 1));
+        for (size_t q0 = 0; q0 < pq.size(); q0 += group) {
+            const std::vector<BatchQuery> gq(pq.begin() + (long)q0, pq.begin() + (long)std::min(pq.size(), q0 + group));
+            sol.pass(gq, (int64_t)gq.size() * br.rows, [&](const BatchOutput& out) {
+                if (b16) fused_threshold<uint16_t>(g, bins16, br, k, kstride, gq, out, sk, up, s);
+                else fused_threshold<int32_t>(g, bins, br, k, kstride, gq, out, sk, up, s);
+            });
         }
         if (!fq.empty()) {
             finish_queries(g, fq.data(), fc.data(), (int)fq.size(), fo.data(), s);  // synchronises
@@ -720,35 +815,13 @@ void run_query_batch(folty_graph* g, const folty_query_params* qs, int nq, folty
         ps.D.erase(std::unique(ps.D.begin(), ps.D.end()), ps.D.end());
         passes.push_back(std::move(ps));
     }
-    // the solutions of all passes' plain queries in one buffer, each (query, directed pair)
-    // at most once; when it was too small, the passes run again with room for all.
-    // FOLTY_BATCH_SOLUTION_CAP sets a smaller first buffer (the tests use it to run them twice)
-    const int64_t S = g->S;
-    BatchOutput out;
-    out.rb = bit_length((uint64_t)(2 * S > 1 ? 2 * S - 1 : 1));
-    out.cap = BT_DEFAULT_CAP;
-    if (const char* env = std::getenv("FOLTY_BATCH_SOLUTION_CAP")) out.cap = std::max<int64_t>(1, std::atoll(env));
-    out.cap = std::min<int64_t>(out.cap, std::max<int64_t>(1, (int64_t)plain.size() * 2 * S));
-    for (int attempt = 0; attempt < 2; attempt++) {
-        Scratch so(g->alloc, s, g->dev_err);
-        if (!plain.empty()) {
-            out.n_out = so.get<unsigned long long>(1);
-            out.key = so.get<uint64_t>(out.cap);
-            out.run = so.get<int32_t>(out.cap);
-            out.cnt = so.get<int32_t>(out.cap);
-            out.nc = so.get<int32_t>(out.cap);
-            FOLTY_CUDA(cudaMemsetAsync(out.n_out, 0, sizeof(unsigned long long), s));
-        }
-        for (const BatchPass& ps : passes) run_batch_pass(g, qs, ps, slot, out, attempt == 0, outs, s, bin_budget);
-        if (plain.empty()) return;
-        const int64_t n = read_i64(g, (const int64_t*)out.n_out, s);
-        if (n <= out.cap) {
-            batch_results(g, out, n, plain, outs, so, s);
-            return;
-        }
-        out.cap = n;
-    }
-    fail(FOLTY_ECUDA, "batched threshold: the solution count grew between two passes over the same bins");
+    // FOLTY_BATCH_SOLUTION_CAP sets a smaller solution buffer (the tests fill it with it)
+    int64_t cap = BT_DEFAULT_CAP;
+    if (const char* env = std::getenv("FOLTY_BATCH_SOLUTION_CAP")) cap = std::max<int64_t>(1, std::atoll(env));
+    cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)plain.size() * 2 * g->S));
+    BatchSolutions sol(g, plain, outs, cap, s);
+    for (const BatchPass& ps : passes) run_batch_pass(g, qs, ps, slot, sol, outs, s, bin_budget);
+    sol.finish();
 }
 
 }  // namespace folty
