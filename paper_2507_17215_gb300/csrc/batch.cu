@@ -668,8 +668,23 @@ struct BatchPass {
     std::vector<int64_t> D;
 };
 
-// Rows of up to this size are allocated without asking how much memory is free.
+// Without a budget of the caller's, rows of up to this size are allocated without asking how
+// much memory is free.
 constexpr int64_t BT_SMALL_ROWS = int64_t(256) << 20;
+
+// Bins of a row of k windows: whole 16-byte chunks of csize-byte counts.
+static int64_t row_stride(int64_t k, int64_t csize) {
+    const int64_t unit = 16 / csize;
+    return (k + unit - 1) / unit * unit;
+}
+
+// Windows per chunk, at most `most`: as many as fit the budget with their padding, a 16-byte
+// chunk at least.
+static int64_t chunk_windows(int64_t most, int64_t rows, int64_t csize, int64_t budget) {
+    if (rows == 0 || (budget <= 0 && rows * csize * row_stride(most, csize) <= BT_SMALL_ROWS)) return most;
+    if (budget <= 0) budget = batch_bin_budget_bytes();
+    return std::min<int64_t>(most, std::max<int64_t>(1, budget / (16 * rows)) * (16 / csize));
+}
 
 // One direction variant: selection, marks, rows and, per chunk of windows, the bins, the
 // plain queries' solutions (slot[i] = their index among the plain queries, -1 for others)
@@ -710,19 +725,14 @@ static void run_batch_pass(folty_graph* g, const folty_query_params* qs, const B
     StageUpload up(g, s);  // the read-back above was the stream's last synchronisation
     // windows per chunk: as many bins as the budget holds and, when plain queries are
     // present, as the fused pass's shared memory does
-    const int64_t per_bin = br.rows * csize;
     int64_t chunk = std::min<int64_t>((int64_t)ps.D.size(), BATCH_MAX_BINS);
     bool plain = false;
     for (int i : ps.members) plain = plain || slot[(size_t)i] >= 0;
     if (plain) chunk = std::min<int64_t>(chunk, b16 ? BT_KMAX : BT_KMAX / 2);
-    if (per_bin * (chunk + 8) > BT_SMALL_ROWS) {
-        const int64_t budget = bin_budget > 0 ? bin_budget : batch_bin_budget_bytes();
-        chunk = std::max<int64_t>(1, std::min<int64_t>(chunk, budget / per_bin));
-    }
+    chunk = chunk_windows(chunk, br.rows, csize, bin_budget);
     for (size_t c0 = 0; c0 < ps.D.size(); c0 += (size_t)chunk) {
         const int k = (int)std::min<int64_t>(chunk, (int64_t)ps.D.size() - (int64_t)c0);
-        // rows of whole 16-byte chunks
-        const int kstride = b16 ? (k + 7) & ~7 : (k + 3) & ~3;
+        const int kstride = (int)row_stride(k, csize);
         Scratch sk(g->alloc, s, g->dev_err);
         const std::vector<int64_t> hd(ps.D.begin() + (long)c0, ps.D.begin() + (long)c0 + k);
         int32_t* bins = nullptr;
@@ -819,6 +829,8 @@ void run_query_batch(folty_graph* g, const folty_query_params* qs, int nq, folty
     int64_t cap = BT_DEFAULT_CAP;
     if (const char* env = std::getenv("FOLTY_BATCH_SOLUTION_CAP")) cap = std::max<int64_t>(1, std::atoll(env));
     cap = std::min<int64_t>(cap, std::max<int64_t>(1, (int64_t)plain.size() * 2 * g->S));
+    // and FOLTY_BATCH_BIN_BUDGET a budget for the bin rows (bytes) where the caller has none
+    if (const char* env = std::getenv("FOLTY_BATCH_BIN_BUDGET"); env && bin_budget <= 0) bin_budget = std::max<int64_t>(1, std::atoll(env));
     BatchSolutions sol(g, plain, outs, cap, s);
     for (const BatchPass& ps : passes) run_batch_pass(g, qs, ps, slot, sol, outs, s, bin_budget);
     sol.finish();
