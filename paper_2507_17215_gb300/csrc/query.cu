@@ -14,6 +14,7 @@
 #include <climits>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 
 #include "internal.cuh"
 #include "scan.cuh"
@@ -937,10 +938,7 @@ void destroy_plans(folty_graph* g) {
     g->plans = nullptr;
 }
 
-static QueryPlans* plans_of(folty_graph* g, cudaStream_t s) {
-    if (g->plans) return g->plans;
-    QueryPlans* p = new QueryPlans();
-    g->plans = p;  // the buffers below are graph-owned; destroy_plans releases the rest
+static void make_plan_buffers(folty_graph* g, QueryPlans* p, cudaStream_t s) {
     const int64_t mk = g->m_kept, S = g->S, n2 = 2 * S;
     if (g->info.max_degree < 65535) p->cnt16 = graph_alloc<uint16_t>(g, mk + 2, s);
     else p->cnt32 = graph_alloc<int32_t>(g, mk, s);
@@ -961,7 +959,22 @@ static QueryPlans* plans_of(folty_graph* g, cudaStream_t s) {
     p->n_cert = (unsigned long long*)(p->tot + 2);
     p->qp = graph_alloc<int64_t>(g, 4, s);
     FOLTY_CUDA(cudaStreamCreateWithFlags(&p->cs, cudaStreamNonBlocking));
-    return p;
+}
+
+// The graph's plans, made on first use: in whole or, when a buffer cannot be had, not at all
+// (the next query makes them anew). The buffers are graph-owned; destroy_plans releases the rest.
+static QueryPlans* plans_of(folty_graph* g, cudaStream_t s) {
+    if (g->plans) return g->plans;
+    auto p = std::make_unique<QueryPlans>();
+    const size_t had = g->owned->size();
+    try {
+        make_plan_buffers(g, p.get(), s);
+    } catch (...) {
+        while (g->owned->size() > had) graph_release(g, g->owned->back().first, s);
+        throw;
+    }
+    g->plans = p.release();
+    return g->plans;
 }
 
 // Everything a plain query expects to be zero.

@@ -1,0 +1,95 @@
+"""Calls whose allocator runs out once, at every allocation in turn: the call says so, and the
+same call on the same graph succeeds afterwards with the results of an undisturbed one."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import workloads as W
+
+from _support import pairs_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2507_17215_gb300 as F
+    return F
+
+
+class _Failing:
+    """A graph on PyTorch's memory whose allocator refuses its `fail`-th request from now on."""
+
+    def __init__(self, F, g):
+        import torch
+        self.F, self.left = F, -1
+
+        @F.ALLOC_FN
+        def alloc(nbytes, stream, ctx):
+            if self.left == 0:
+                self.left = -1
+                return None
+            self.left -= self.left > 0
+            return torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
+
+        @F.FREE_FN
+        def free(ptr, stream, ctx):
+            torch.cuda.caching_allocator_delete(int(ptr))
+
+        self.allocator, h = F.folty_allocator(alloc, free, None), ctypes.c_void_p()
+        st = F.lib.folty_load_temporal_graph(g.n, g.m, g.src.ctypes.data, g.dst.ctypes.data, g.t.ctypes.data,
+                                             ctypes.byref(self.allocator), F.current_stream(), ctypes.byref(h))
+        assert st == F.FOLTY_OK, F.folty_last_error()
+        self.handle = h.value
+
+    def refused(self, fail, call):
+        """Whether call ran out at its fail-th request (else it made fewer)."""
+        self.left = fail
+        try:
+            call()
+        except self.F.FoltyError as e:
+            assert e.status == self.F.FOLTY_ENOMEM, e
+            assert self.left == -1
+            return True
+        finally:
+            self.left, reached = -1, self.left == -1
+        assert not reached, "a refused request went unnoticed"
+        return False
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        self.F.folty_free(self.handle)
+
+
+def _graph(kind):
+    if kind == "small":  # within the allocation-free counts' limit
+        return W.config_graph(2, scale=0.01)
+    return W.config_graph(2, scale=0.06)
+
+
+QUERIES = [W.Query(86400, 1, 10, W.Q_FORALL_T, W.DIR_EITHER, W.U_COMMON, False),
+           W.Query(3600, 1, 2, W.Q_EXISTS, W.DIR_OUT, W.U_HEAD, False)]
+
+
+@pytest.mark.parametrize("kind", ["small", "large"])
+def test_first_query_after_one_that_ran_out_of_memory(F, kind):
+    g = _graph(kind)
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G:
+        want = [pairs_of(G.query(q)) for q in QUERIES]
+    fail = 0
+    while True:
+        with _Failing(F, g) as G:
+            F.folty_preprocess(G.handle)
+            refused = G.refused(fail, lambda: F.folty_query(G.handle, QUERIES[0]))
+            for q, w in zip(QUERIES + QUERIES, want + want):
+                assert pairs_of(F.folty_query(G.handle, q)) == w, (fail, str(q))
+        if not refused:
+            break
+        fail += 1
+    assert fail > 8  # the plan's buffers, at least
