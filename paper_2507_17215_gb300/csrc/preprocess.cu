@@ -1810,7 +1810,6 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         prepare_liveness(g, ntri, s);
         ensure_liveness(g, FOLTY_DIR_OUT, s);
     }
-    release_input(g, s);  // the raw input and the pair table's lists are no longer needed
     g->info.triangles = g->ntri;
     // tile -> first triangle map of the all-roles probe kernel (query independent)
     g->n_tiles = probe_map ? (g->info.probes + PB_TILE - 1) / PB_TILE : 0;
@@ -1819,6 +1818,8 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         FOLTY_LAUNCH(k_tile_starts, grid_for(g->n_tiles + 1, T), T, 0, s, g->tri_off, g->ntri, g->info.probes,
                      g->n_tiles, PB_TILE, g->tile_tri);
     g->prof_bytes = graph_alloc<unsigned long long>(g, PROF_SLOTS, s);
+    // after the last step that can fail: a call that ran out of memory may be repeated
+    release_input(g, s);
     g->info.static_edges = S;
     g->state = 1;
     FOLTY_CUDA(cudaStreamSynchronize(s));

@@ -93,3 +93,28 @@ def test_first_query_after_one_that_ran_out_of_memory(F, kind):
             break
         fail += 1
     assert fail > 8  # the plan's buffers, at least
+
+
+@pytest.mark.parametrize("kind", ["small", "large", "shuffled"])
+def test_preprocessing_repeated_after_it_ran_out_of_memory(F, kind):
+    g = _graph(kind)
+    if kind == "shuffled":
+        p = np.random.default_rng(1).permutation(g.m)
+        g = W.TemporalGraph(g.n, g.src[p], g.dst[p], g.t[p])
+    counts = W.Query(86400, 1, 10, W.Q_EXISTS, W.DIR_IN, W.U_HEAD, True)
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G:
+        want, edges, info = [pairs_of(G.query(q)) for q in QUERIES], G.query(counts)["edge_count"], G.info()
+    fail = 0
+    while True:
+        with _Failing(F, g) as G:
+            refused = G.refused(fail, lambda: F.folty_preprocess(G.handle))
+            if refused:
+                F.folty_preprocess(G.handle)
+            assert [pairs_of(F.folty_query(G.handle, q)) for q in QUERIES] == want, fail
+            np.testing.assert_array_equal(F.folty_query(G.handle, counts)["edge_count"], edges)
+            got = F.folty_graph_get_info(G.handle)
+            assert {k: v for k, v in got.items() if k != "device_bytes"} == {k: v for k, v in info.items() if k != "device_bytes"}
+        if not refused:
+            break
+        fail += 1
+    assert fail > 10
