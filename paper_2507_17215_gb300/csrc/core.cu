@@ -44,6 +44,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 
 #include "core.cuh"
@@ -65,6 +66,7 @@ enum {
     K_BFR = 12,    // 3 slots: above
     K_FR2 = 15,    // the same for the second half
     K_BFR2 = 18,
+    K_BEAT = 21,   // rounds that one block has run alone
     K_SLOTS = 24
 };
 
@@ -116,7 +118,8 @@ __device__ __forceinline__ long long global_ns() {
 }
 
 // Grid-wide barrier for a cooperative launch (all blocks co-resident). The wait is
-// bounded: after timeout_ns the block records an error and every block returns. Also the
+// bounded: after timeout_ns without a round by the block that runs alone (a path of n vertices
+// takes it n / 2 rounds) the block records an error and every block returns. Also the
 // values of two control words after it, read together with the error word by one thread.
 // Its fences order every plain access before it against every one after it (the first
 // level caches hold nothing from before), so values that a pass only reads are read
@@ -139,12 +142,16 @@ __device__ Sizes grid_barrier(int* ctl, long long timeout_ns, int wa = K_BAR, in
             vctl[K_GEN] = gen + 1;
         } else {
             long long t0 = 0;
+            int beat = 0;
             for (int spin = 0; vctl[K_GEN] == gen; spin++) {
                 if ((spin & 63) != 63) continue;
                 if (vctl[CORE_ERR]) break;
                 const long long t = global_ns();
-                if (t0 == 0) t0 = t;
-                else if (t - t0 > timeout_ns) {
+                const int now = vctl[K_BEAT];
+                if (t0 == 0 || now != beat) {
+                    t0 = t;
+                    beat = now;
+                } else if (t - t0 > timeout_ns) {
                     atomicExch(&ctl[CORE_ERR], 1);
                     break;
                 }
@@ -900,6 +907,7 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core(const CoreArgs a) {
             while (z.ok && z.a > 0 && z.a <= 2 * CORE_SOLO && z.b == 0) {
                 z = value_round(a, solo, z.a, 0, r, core_smem, block_wait);
                 r++;
+                if (threadIdx.x == 0) vctl[K_BEAT] = vctl[K_BEAT] + 1;
             }
             if (threadIdx.x == 0) vctl[K_ROUND] = r;
         }
@@ -946,6 +954,7 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core(const CoreArgs a) {
             while (z.ok && z.a > 0 && z.a <= 2 * CORE_SOLO && z.b == 0) {
                 z = removal_round(a, solo, z.a, 0, r, block_wait);
                 r++;
+                if (threadIdx.x == 0) vctl[K_BEAT] = vctl[K_BEAT] + 1;
             }
             if (threadIdx.x == 0) vctl[K_ROUND] = r;
         }
@@ -1020,7 +1029,9 @@ const int* enqueue_core_numbers(folty_graph* g, const int32_t* rowptr, const int
     // the control words and the levels' rounds, zeroed together
     a.ctl = sc.get<int>(K_SLOTS + (int64_t)a.hcap + 2);
     a.lev = a.ctl + K_SLOTS;
+    // FOLTY_CORE_TIMEOUT_MS sets a shorter bound (the tests pass it with long stretches of rounds)
     a.timeout_ns = 10ll * 1000 * 1000 * 1000;
+    if (const char* env = std::getenv("FOLTY_CORE_TIMEOUT_MS")) a.timeout_ns = std::max(1ll, std::atoll(env)) * 1000 * 1000;
     FOLTY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(int) * (K_SLOTS + (size_t)a.hcap + 2), s));
     if (n == 0) return a.ctl;
     const int smem = CORE_BINS * (int)sizeof(int) + (int)sizeof(Stage);

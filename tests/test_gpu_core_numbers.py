@@ -101,3 +101,14 @@ def test_core_numbers_with_rows_shortened_twice(F, groups, cliques, hubs):
         info = G.info()
     assert info["degeneracy"] == want.max()
     assert info["max_out_degree"] <= info["degeneracy"]
+
+
+def test_long_stretches_of_rounds_are_no_timeout(F, monkeypatch):
+    """A path of 60,000 vertices: 30,000 rounds by one block, while the others wait for longer
+    than their bound."""
+    monkeypatch.setenv("FOLTY_CORE_TIMEOUT_MS", "5")
+    n = 60_000
+    a = np.arange(n - 1, dtype=np.int32)
+    with F.TemporalGraph(n, a, a + 1, np.zeros(n - 1, np.int64)) as G:
+        assert (G.core_numbers() == 1).all()
+        assert G.info()["peel_rounds"] == n // 2
