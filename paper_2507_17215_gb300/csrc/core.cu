@@ -32,7 +32,7 @@
 // shortened anew.
 //
 // The last rounds of both halves hold a few vertices each: one block runs them alone, with
-// block barriers.
+// block barriers, and one warp those of up to 32 vertices with short rows.
 //
 // Both halves together, against the phases of one chain: 0.56 against 1.26 ms on the medium
 // graph (20M edges), 0.63 against 1.94 on the paper-scale one (beside nothing else), 1.18
@@ -275,11 +275,12 @@ __device__ __forceinline__ int octet_source(unsigned& m) {
 
 // The largest h <= top such that h entries of a row have val >= h, and that number of
 // entries (0 and any when not even one has, as a shortened row may). One thread, rows of up
-// to 8 entries: 8 counters of 8 bits in a word.
-__device__ __forceinline__ int thread_h(const CoreArgs& a, const int32_t* row, int d, int top, int& cnt) {
-    int32_t x[CORE_SMALL];
+// to 8 entries x (-1: none): 8 counters of 8 bits in a word.
+__device__ __forceinline__ void thread_row(int32_t (&x)[CORE_SMALL], const int32_t* row, int d) {
 #pragma unroll
     for (int i = 0; i < CORE_SMALL; i++) x[i] = i < d ? row[i] : -1;
+}
+__device__ __forceinline__ int thread_h(const CoreArgs& a, const int32_t (&x)[CORE_SMALL], int top, int& cnt) {
     uint64_t bins = 0;  // byte h - 1: entries of value h (or more, for h = top)
 #pragma unroll
     for (int i = 0; i < CORE_SMALL; i++)
@@ -481,8 +482,10 @@ __device__ void h_pass(const CoreArgs& a, Team t, const int32_t* list, int count
         const Row row = on ? row_at(a, v) : Row{nullptr, 0, false};
         const int top = on ? min(min(__ldcg(&a.val[v]), row.cut ? a.deg[v] : row.n), a.hcap) : 0;
         if (on && !row.cut && row.n <= CORE_SMALL) {
+            int32_t x[CORE_SMALL];
+            thread_row(x, row.p, row.n);
             int c;
-            a.nv[v] = thread_h(a, row.p, row.n, top, c);
+            a.nv[v] = thread_h(a, x, top, c);
             a.cnt[v] = c;
         }
         unsigned eight = __ballot_sync(0xffffffffu, on && !row.cut && row.n > CORE_SMALL && row.n <= CORE_ROW8);
@@ -561,18 +564,21 @@ __device__ __forceinline__ void note_round(const CoreArgs& a, int k, int n) {
 // off next when it is the first below its value. REMOVE (c from val): the owner left level
 // `from`; a neighbour of the level loses one, and leaves in round `to` when it is the first
 // at the level.
+// told returns whether x is worked off next.
 template <bool REMOVE>
-__device__ __forceinline__ void tell(const CoreArgs& a, int32_t x, int c, int from, int to, Next nx) {
+__device__ __forceinline__ bool told(const CoreArgs& a, int32_t x, int c, int from, int to) {
     if (REMOVE) {
-        if (c != from) return;
-        if (atomicSub(&a.cnt[x], 1) != from + 1) return;
+        if (c != from) return false;
+        if (atomicSub(&a.cnt[x], 1) != from + 1) return false;
         a.rnd[x] = to;
         note_round(a, from, to + 1);
-        append_next(a, x, nx);
-    } else {
-        if (c <= to || c > from) return;
-        if (atomicSub(&a.cnt[x], 1) == c) append_next(a, x, nx);
+        return true;
     }
+    return c > to && c <= from && atomicSub(&a.cnt[x], 1) == c;
+}
+template <bool REMOVE>
+__device__ __forceinline__ void tell(const CoreArgs& a, int32_t x, int c, int from, int to, Next nx) {
+    if (told<REMOVE>(a, x, c, from, to)) append_next(a, x, nx);
 }
 
 template <bool REMOVE>
@@ -652,8 +658,7 @@ __device__ void tell_pass(const CoreArgs& a, Team t, const int32_t* list, int co
         const bool act = on && row.n <= CORE_MID && (REMOVE || to < from);
         if (act && row.n <= CORE_SMALL) {
             int32_t x[CORE_SMALL], c[CORE_SMALL];
-#pragma unroll
-            for (int i = 0; i < CORE_SMALL; i++) x[i] = i < row.n ? row.p[i] : -1;
+            thread_row(x, row.p, row.n);
 #pragma unroll
             for (int i = 0; i < CORE_SMALL; i++) c[i] = x[i] >= 0 ? told_value<REMOVE>(a, x[i]) : 0;
 #pragma unroll
@@ -807,6 +812,114 @@ __device__ __forceinline__ Sizes removal_round(const CoreArgs& a, Team t, int co
     return barrier(K_FR2 + (r + 1) % 3, K_BFR2 + (r + 1) % 3);
 }
 
+// ------------------------------------------------------------------ rounds of a few vertices
+
+// Rounds of 1 to 32 vertices whose rows are whole and no longer than CORE_SMALL, from round r
+// on, by one warp with a vertex a lane and the lists in shared memory; returns the first round
+// it has not run, with that round's lists and control words as the rounds of a block leave
+// them. Both steps of a round share the row, and there is no barrier: bound by the chain of five
+// dependent accesses to L2. A path of 20,000 vertices (10,000 rounds in either half) takes 42
+// ms, between block barriers 73. Tried at once, not after CORE_LONG rounds, it cost the small
+// graphs, whose rows are longer, 1 to 3% of their preprocessing.
+constexpr int CORE_FEW = 32;
+constexpr int CORE_LONG = 16;  // rounds of a block alone before one warp tries
+static_assert(2 * CORE_FEW * CORE_SMALL <= CORE_STAGE, "both lists lie in the stage");
+
+template <bool REMOVE>
+__device__ __noinline__ int few_rounds(const CoreArgs& a, int count, int r) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    volatile int* vctl = a.ctl;
+    int32_t* cur = stage().v;
+    int32_t* next = cur + CORE_FEW * CORE_SMALL;
+    // round r works off the lists of this parity, counted in this slot
+    auto at = [](int round) { return REMOVE ? round : round - 1; };
+    int beat = vctl[K_BEAT];
+    if (lane < count) cur[lane] = __ldcg(&a.fr[at(r) & 1][lane]);
+    __syncwarp();
+    while (count > 0 && count <= CORE_FEW) {
+        const bool on = lane < count;
+        const int32_t v = on ? cur[lane] : 0;
+        const Row row = on ? row_at(a, v) : Row{nullptr, 0, false};
+        if (__any_sync(FULL, row.cut || row.n > CORE_SMALL)) break;
+        const int from = on ? __ldcg(&a.val[v]) : 0;
+        int32_t x[CORE_SMALL];
+        thread_row(x, row.p, row.n);
+        int to = r + 1;
+        if (!REMOVE) {
+            int c = 0;
+            to = on ? thread_h(a, x, min(min(from, row.n), a.hcap), c) : 0;
+            if (on) {
+                a.nv[v] = to;
+                a.cnt[v] = c;
+            }
+            __syncwarp();
+        }
+        const bool act = on && (REMOVE || to < from);
+        int32_t c[CORE_SMALL];
+#pragma unroll
+        for (int i = 0; i < CORE_SMALL; i++) c[i] = act && x[i] >= 0 ? told_value<REMOVE>(a, x[i]) : 0;
+        unsigned joins = 0;
+#pragma unroll
+        for (int i = 0; i < CORE_SMALL; i++)
+            if (act && x[i] >= 0 && told<REMOVE>(a, x[i], c[i], from, to)) joins |= 1u << i;
+        count = 0;
+#pragma unroll
+        for (int i = 0; i < CORE_SMALL; i++) {
+            const bool j = (joins >> i) & 1u;
+            const unsigned m = __ballot_sync(FULL, j);
+            if (j) next[count + __popc(m & below)] = x[i];
+            count += __popc(m);
+        }
+        if (!REMOVE && act) a.val[v] = to;  // read by no lane since the last __syncwarp
+        if (lane == 0) vctl[K_BEAT] = ++beat;
+        r++;
+        int32_t* t = cur;
+        cur = next;
+        next = t;
+        __syncwarp();
+    }
+    const int slot = at(r) % 3, fr = REMOVE ? K_FR2 : K_FR, bfr = REMOVE ? K_BFR2 : K_BFR;
+    if (lane == 0) {
+        vctl[fr + slot] = vctl[bfr + slot] = 0;
+        vctl[fr + (at(r) + 1) % 3] = vctl[bfr + (at(r) + 1) % 3] = 0;
+    }
+    __syncwarp();
+    for (int i = lane; i < count; i += 32) {
+        const int32_t v = cur[i], sl = __ldcg(&a.slen[v]);
+        if ((sl >= 0 ? sl : a.deg[v]) > CORE_MID) append(v, a.bfr[at(r) & 1], &a.ctl[bfr + slot], a.bcap, a.ctl);
+        else append(v, a.fr[at(r) & 1], &a.ctl[fr + slot], a.n, a.ctl);
+    }
+    return r;
+}
+
+// The rounds of one block alone, from round r with z.a vertices on: while they are few.
+template <bool REMOVE, typename Round, typename Barrier>
+__device__ __forceinline__ void solo_rounds(const CoreArgs& a, Sizes z, int r, Round&& round, Barrier&& barrier) {
+    __shared__ int s_r;
+    volatile int* vctl = a.ctl;
+    int again = r + CORE_LONG;  // most stretches end before; and after rows too long for one warp
+    while (z.ok && z.a > 0 && z.a <= 2 * CORE_SOLO && z.b == 0) {
+        if (z.a <= CORE_FEW && r >= again) {
+            if (threadIdx.x < 32) {
+                const int done = few_rounds<REMOVE>(a, z.a, r);
+                if (threadIdx.x == 0) s_r = done;
+            }
+            __syncthreads();
+            again = s_r == r ? r + CORE_LONG : s_r;
+            r = s_r;
+            const int slot = (REMOVE ? r : r - 1) % 3;
+            z = barrier((REMOVE ? K_FR2 : K_FR) + slot, (REMOVE ? K_BFR2 : K_BFR) + slot);
+            continue;
+        }
+        z = round(z.a, r);
+        r++;
+        if (threadIdx.x == 0) vctl[K_BEAT] = vctl[K_BEAT] + 1;
+    }
+    if (threadIdx.x == 0) vctl[K_ROUND] = r;
+}
+
 // ------------------------------------------------------------------ the kernel
 
 __global__ void __launch_bounds__(CORE_THREADS, 1) k_core(const CoreArgs a) {
@@ -903,14 +1016,8 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core(const CoreArgs a) {
             continue;
         }
         if (!wait()) return;  // every block has read the sizes before one block moves on
-        if (blockIdx.x == 0) {
-            while (z.ok && z.a > 0 && z.a <= 2 * CORE_SOLO && z.b == 0) {
-                z = value_round(a, solo, z.a, 0, r, core_smem, block_wait);
-                r++;
-                if (threadIdx.x == 0) vctl[K_BEAT] = vctl[K_BEAT] + 1;
-            }
-            if (threadIdx.x == 0) vctl[K_ROUND] = r;
-        }
+        if (blockIdx.x == 0)
+            solo_rounds<false>(a, z, r, [&](int n, int k) { return value_round(a, solo, n, 0, k, core_smem, block_wait); }, block_wait);
         z = grid_wait(K_ROUND, K_BAR);
         if (!z.ok) return;
         r = z.a;
@@ -950,14 +1057,8 @@ __global__ void __launch_bounds__(CORE_THREADS, 1) k_core(const CoreArgs a) {
             continue;
         }
         if (!wait()) return;
-        if (blockIdx.x == 0) {
-            while (z.ok && z.a > 0 && z.a <= 2 * CORE_SOLO && z.b == 0) {
-                z = removal_round(a, solo, z.a, 0, r, block_wait);
-                r++;
-                if (threadIdx.x == 0) vctl[K_BEAT] = vctl[K_BEAT] + 1;
-            }
-            if (threadIdx.x == 0) vctl[K_ROUND] = r;
-        }
+        if (blockIdx.x == 0)
+            solo_rounds<true>(a, z, r, [&](int n, int k) { return removal_round(a, solo, n, 0, k, block_wait); }, block_wait);
         z = grid_wait(K_ROUND, K_BAR);
         if (!z.ok) return;
         r = z.a;
