@@ -1,8 +1,10 @@
 // The C ABI of folty.h: argument checks, object lifetime, error reporting, and the
 // load step (copy + validation of the input edge list).
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
+#include <optional>
 #include <unordered_map>
 
 #include "internal.cuh"
@@ -496,12 +498,15 @@ struct EdgeStat {
 };
 
 // One pass over the edge list: its checks, the low 32 bits of its timestamps (the store's
-// offsets, once the range is known to fit), and with INSERT every edge's pair into the first
-// pair table and its slot word (PAIR_LOOP for a self-loop or an invalid edge, which fails the
-// load anyway). src, dst and t are device memory or pinned host memory (read over the host
-// link, as fast as a copy engine's pull). Nothing else of the input is kept: 16 B read and 8
-// written per edge, where copies of the three arrays took 16 B more; a table that turns out
-// not to serve, or a range of times past 32 bits, has the input copied afterwards.
+// offsets, once the range is known to fit) or, where a few of them already span more, all of
+// them, and with INSERT every edge's pair into the first pair table and its
+// slot word (PAIR_LOOP for a self-loop or an invalid edge, which fails the load anyway). src,
+// dst and t are device memory or pinned host memory (read over the host link, as fast as a copy
+// engine's pull, and once: the list is kept meanwhile, at no cost beside the link's pace).
+// Of device memory nothing else is kept: 16 B read and 8 written per edge, where copies of
+// the three arrays took 16 B more; a table that turns out not to serve, or a range of times
+// past 32 bits that the few did not show, has them copied afterwards. 40M edges of 64-bit times:
+// 0.44 ms from the device, 3.18 from pinned memory; with the times read again 0.53 and 4.70.
 //
 // Four edges per thread and step (16-byte accesses when VEC; otherwise, and for the m mod 4
 // last edges, one by one), the previous edge's timestamp from the neighbouring lane; the four
@@ -514,7 +519,10 @@ struct LoadArgs {
     const int64_t* t;
     int64_t m;
     int32_t n;
-    uint32_t* t32;
+    uint32_t* t32;  // the low words; each of these may be null
+    int64_t* kt;    // the list as it is
+    int32_t* ksrc;
+    int32_t* kdst;
     unsigned long long* stat;
     uint64_t* table;
     int lg;
@@ -564,8 +572,17 @@ __global__ void __launch_bounds__(256) k_load(const LoadArgs a) {
         int64_t tp = __shfl_up_sync(0xffffffffu, (long long)t23.y, 1);
         if (lane == 0) tp = j > 0 ? a.t[4 * j - 1] : 0;
         if (act) {
-            __stcs(reinterpret_cast<uint4*>(a.t32) + j,
-                   make_uint4((uint32_t)t01.x, (uint32_t)t01.y, (uint32_t)t23.x, (uint32_t)t23.y));
+            if (a.t32)
+                __stcs(reinterpret_cast<uint4*>(a.t32) + j,
+                       make_uint4((uint32_t)t01.x, (uint32_t)t01.y, (uint32_t)t23.x, (uint32_t)t23.y));
+            if (a.kt) {
+                __stcs(reinterpret_cast<longlong2*>(a.kt) + 2 * j, t01);
+                __stcs(reinterpret_cast<longlong2*>(a.kt) + 2 * j + 1, t23);
+            }
+            if (a.ksrc) {
+                __stcs(reinterpret_cast<int4*>(a.ksrc) + j, x);
+                __stcs(reinterpret_cast<int4*>(a.kdst) + j, y);
+            }
             const int64_t i = 4 * j;
             st.edge(i, x.x, y.x, t01.x, tp, a.n);
             st.edge(i + 1, x.y, y.y, t01.y, t01.x, a.n);
@@ -582,7 +599,12 @@ __global__ void __launch_bounds__(256) k_load(const LoadArgs a) {
     for (int64_t i = 4 * m4 + tid; i < a.m; i += stride) {
         const int32_t x[1] = {a.src[i]}, y[1] = {a.dst[i]};
         const int64_t ti = a.t[i];
-        a.t32[i] = (uint32_t)ti;
+        if (a.t32) a.t32[i] = (uint32_t)ti;
+        if (a.kt) a.kt[i] = ti;
+        if (a.ksrc) {
+            a.ksrc[i] = x[0];
+            a.kdst[i] = y[0];
+        }
         st.edge(i, x[0], y[0], ti, i > 0 ? a.t[i - 1] : 0, a.n);
         if (INSERT && !pair_table_over(a.flags)) {
             uint32_t w[1];
@@ -594,10 +616,12 @@ __global__ void __launch_bounds__(256) k_load(const LoadArgs a) {
 }
 
 // The address under which kernels of the current device read p: p itself for memory
-// of this device, the mapped address for pinned host memory; NULL otherwise (pageable
-// host memory, another device's memory).
-static const void* kernel_address(const void* p) {
+// of this device, the mapped address for pinned host memory (*host set); NULL otherwise
+// (pageable host memory, another device's memory).
+template <typename T>
+static const T* kernel_address(const T* p, bool* host) {
     cudaPointerAttributes a{};
+    *host = false;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
@@ -608,15 +632,14 @@ static const void* kernel_address(const void* p) {
         return nullptr;
     }
     if (a.type == cudaMemoryTypeDevice && a.device == dev) return p;
-    if (a.type == cudaMemoryTypeHost) return a.devicePointer;
-    return nullptr;
+    *host = a.type == cudaMemoryTypeHost;
+    return *host ? static_cast<const T*>(a.devicePointer) : nullptr;
 }
 
 void release_input(folty_graph* g, cudaStream_t s) {
     graph_release(g, g->in_t32, s);
     graph_release(g, g->in_t, s);
-    graph_release(g, g->in_src, s);
-    graph_release(g, g->in_dst, s);
+    graph_release(g, g->in_src, s);  // and in_dst
     graph_release(g, g->pre_slotw, s);
     graph_release(g, g->pre_rank, s);
     graph_release(g, g->pre_slot, s);
@@ -626,23 +649,63 @@ void release_input(folty_graph* g, cudaStream_t s) {
     g->pre_rank = nullptr;
 }
 
+// A look at a few timestamps in device memory before the list is read: whether they already
+// span more than the 32-bit offsets do. It is enqueued first, and what the load allocates and
+// clears meanwhile hides most of it: 6 us of 120 (6M edges) are left; a second read of 64-bit
+// times and its wait cost 27. Lists of fewer than LOAD_LOOK_EDGES edges are read again instead.
+constexpr int64_t LOAD_LOOK_EDGES = int64_t(1) << 22;
+constexpr int LOAD_LOOK = 16;
+// Pinned lists are kept from this many edges on: below, the allocations (10 us) cost more than
+// a second read of what turns out to be needed (at 210 GB/s, 8 B an edge for the times or for
+// the edges of a table that does not serve).
+constexpr int64_t LOAD_KEEP_EDGES = int64_t(1) << 20;
+
+class TimesLook {
+  public:
+    // t: an address of the device
+    TimesLook(folty_graph* g, const int64_t* t, cudaStream_t s) : g_(g) {
+        const void* ptrs[LOAD_LOOK];
+        int sizes[LOAD_LOOK];
+        for (int i = 0; i < LOAD_LOOK; i++) {
+            ptrs[i] = t + (g->m - 1) * i / (LOAD_LOOK - 1);
+            sizes[i] = 8;
+        }
+        FOLTY_CUDA(cudaEventCreateWithFlags(&ev_, cudaEventDisableTiming));
+        enqueue_read_back(g, ptrs, sizes, LOAD_LOOK, s);
+        FOLTY_CUDA(cudaEventRecord(ev_, s));
+    }
+    ~TimesLook() {
+        if (ev_) cudaEventDestroy(ev_);
+    }
+    TimesLook(const TimesLook&) = delete;
+    TimesLook& operator=(const TimesLook&) = delete;
+
+    bool past_32_bits() {
+        FOLTY_CUDA(cudaEventSynchronize(ev_));
+        const int64_t* v = g_->host_stage;
+        const auto r = std::minmax_element(v, v + LOAD_LOOK);
+        return *r.first >= 0 && *r.second - *r.first >= (int64_t)0xffffffffll;
+    }
+
+  private:
+    folty_graph* g_;
+    cudaEvent_t ev_ = nullptr;
+};
+
 static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, const int64_t* t,
                        cudaStream_t s) {
     const int64_t m = g->m;
     g->dev_err = graph_alloc<int>(g, 1, s);
     FOLTY_CUDA(cudaMemsetAsync(g->dev_err, 0, sizeof(int), s));
     auto a16 = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
-    auto copy_edges = [&] {
-        g->in_src = graph_alloc<int32_t>(g, m, s);
-        g->in_dst = graph_alloc<int32_t>(g, m, s);
-        FOLTY_CUDA(cudaMemcpyAsync(g->in_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, s));
-        FOLTY_CUDA(cudaMemcpyAsync(g->in_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, s));
+    auto copy = [&](auto* to, const auto* from) {
+        FOLTY_CUDA(cudaMemcpyAsync(to, from, sizeof(*to) * (size_t)m, cudaMemcpyDefault, s));
     };
-    auto copy_times = [&] {
-        g->in_t = graph_alloc<int64_t>(g, m, s);
-        FOLTY_CUDA(cudaMemcpyAsync(g->in_t, t, sizeof(int64_t) * (size_t)m, cudaMemcpyDefault, s));
+    auto keep_edges = [&] {
+        const int64_t line = (m + 3) & ~int64_t(3);
+        g->in_src = graph_alloc<int32_t>(g, 2 * line, s);
+        g->in_dst = g->in_src + line;
     };
-    g->in_t32 = graph_alloc<uint32_t>(g, m, s);
     Scratch sc(g->alloc, s, g->dev_err);
     // the checks' results, then the table's flags
     unsigned long long* stat = sc.get<unsigned long long>(5);
@@ -655,25 +718,47 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
     const bool insert = m > 0 && g->n >= 2 && !pair_table_forced_off();
     const int lg = insert ? pair_table_lg_first(m) : 0;
     const int cap = insert ? (1 << lg) / 2 : 0;  // load factor at most 1/2
-    bool staged = false;  // in_src, in_dst and in_t hold the input
     if (m > 0) {
-        LoadArgs a{(const int32_t*)kernel_address(src), (const int32_t*)kernel_address(dst),
-                   (const int64_t*)kernel_address(t), m, g->n, g->in_t32, stat, nullptr, lg, nullptr, flags};
-        if (!a.src || !a.dst || !a.t) {
-            copy_edges();
-            copy_times();
+        LoadArgs a{};
+        bool host[3];
+        a.src = kernel_address(src, &host[0]);
+        a.dst = kernel_address(dst, &host[1]);
+        a.t = kernel_address(t, &host[2]);
+        a.m = m;
+        a.n = g->n;
+        a.stat = stat;
+        a.lg = lg;
+        a.flags = flags;
+        const bool staged = !a.src || !a.dst || !a.t;  // in_src, in_dst and in_t hold the input
+        if (staged) {
+            keep_edges();
+            g->in_t = graph_alloc<int64_t>(g, m, s);
+            copy(g->in_src, src);
+            copy(g->in_dst, dst);
+            copy(g->in_t, t);
             a.src = g->in_src;
             a.dst = g->in_dst;
             a.t = g->in_t;
-            staged = true;
         }
+        const bool keep = !staged && m >= LOAD_KEEP_EDGES;
+        if (keep && (host[0] || host[1])) {
+            keep_edges();
+            a.ksrc = g->in_src;
+            a.kdst = g->in_dst;
+        }
+        if (keep && host[2]) a.kt = g->in_t = graph_alloc<int64_t>(g, m, s);
+        std::optional<TimesLook> look;
+        if (m >= LOAD_LOOK_EDGES && !host[2]) look.emplace(g, a.t, s);
         if (insert) {
             g->pre_slotw = graph_alloc<uint32_t>(g, m, s);
             a.slotw = g->pre_slotw;
             a.table = sc.get<uint64_t>(1ll << lg);
             FOLTY_CUDA(cudaMemsetAsync(a.table, 0, sizeof(uint64_t) << lg, s));
         }
-        const bool vec = a16(a.src) && a16(a.dst) && a16(a.t) && a16(a.t32) && a16(a.slotw);
+        if (!look || !look->past_32_bits()) a.t32 = g->in_t32 = graph_alloc<uint32_t>(g, m, s);
+        else if (!staged) a.kt = g->in_t = graph_alloc<int64_t>(g, m, s);
+        const bool vec = a16(a.src) && a16(a.dst) && a16(a.t) && a16(a.t32) && a16(a.kt) && a16(a.ksrc) && a16(a.kdst) &&
+                         a16(a.slotw);
         const unsigned grid = grid_for(vec ? m / 4 + 1 : m, 256, 8);
         if (insert && vec) FOLTY_LAUNCH((k_load<true, true>), grid, 256, 0, s, a);
         else if (insert) FOLTY_LAUNCH((k_load<true, false>), grid, 256, 0, s, a);
@@ -694,19 +779,19 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
     g->tmin = (m > 0) ? v[1] : 0;
     g->tmax = (m > 0) ? v[2] : 0;
     // 32-bit offsets from tmin when the time range leaves room for the "none" marker
-    g->ts32 = (g->tmax - g->tmin) < (int64_t)0xffffffffll;
+    g->ts32 = (m == 0 || g->in_t32) && (g->tmax - g->tmin) < (int64_t)0xffffffffll;
     g->info.time_sorted = v[3] ? 0 : 1;
     g->m_kept = m - v[4];
     g->info.n = g->n;
     g->info.m = m;
     g->info.m_kept = g->m_kept;
-    // what the preprocessing needs of the input beside the times' low bits
+    // what the preprocessing needs of the input beside the times
     const bool serves = insert && v[5] == 0 && v[6] <= cap && g->m_kept > 0;
     g->pre_lg = lg;
+    bool copies = false;
     if (serves) {
         g->pre_pairs = (int32_t)v[6];
-        graph_release(g, g->in_src, s);
-        graph_release(g, g->in_dst, s);
+        graph_release(g, g->in_src, s);  // and in_dst
         g->in_src = g->in_dst = nullptr;
     } else {
         graph_release(g, g->pre_slotw, s);
@@ -714,11 +799,12 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
         graph_release(g, g->pre_slot, s);
         g->pre_slotw = g->pre_slot = nullptr;
         g->pre_rank = nullptr;
-    }
-    bool copies = false;
-    if (!serves && !staged && m > 0) {
-        copy_edges();
-        copies = true;
+        if (!g->in_src && m > 0) {
+            keep_edges();
+            copy(g->in_src, src);
+            copy(g->in_dst, dst);
+            copies = true;
+        }
     }
     if (g->ts32) {
         graph_release(g, g->in_t, s);
@@ -726,8 +812,9 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
     } else {
         graph_release(g, g->in_t32, s);
         g->in_t32 = nullptr;
-        if (!staged && m > 0) {
-            copy_times();
+        if (!g->in_t && m > 0) {
+            g->in_t = graph_alloc<int64_t>(g, m, s);
+            copy(g->in_t, t);
             copies = true;
         }
     }

@@ -169,7 +169,7 @@ struct folty_graph {
     uint64_t* pre_rank;   // the distinct pairs' ranks and slots, in no particular order
     uint32_t* pre_slot;
     int32_t pre_pairs;
-    // the edges themselves, when it does not
+    // the edges themselves, when it does not (one allocation, in_src)
     int32_t* in_src;
     int32_t* in_dst;
     // ---- preprocessed store (device)

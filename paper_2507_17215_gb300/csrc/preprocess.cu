@@ -1555,8 +1555,6 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     // ---------------- A1: canonical order
     const int nb = bit_length((uint64_t)(n > 1 ? n - 1 : 1));
     const int64_t mk = g->m_kept;
-    // 32-bit offsets from tmin when the time range leaves room for the "none" marker
-    g->ts32 = (g->tmax - g->tmin) < (int64_t)0xffffffffll;
     if (g->ts32) g->T = graph_alloc<uint32_t>(g, mk, s);
     else g->T = graph_alloc<int64_t>(g, mk, s);
     g->sd = graph_alloc<int32_t>(g, mk, s);
