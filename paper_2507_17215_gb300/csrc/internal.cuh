@@ -204,8 +204,7 @@ struct folty_graph {
     unsigned long long* prof_bytes;  // [PROF_SLOTS] device counters of probe-stage model bytes
     int prof_next;                   // next slot
     void* run_ends;     // [S] first and last timestamp and size of both runs of every static edge
-    uint8_t* tlive;     // [3][tlive_stride] per direction variant, the smallest window bucket of a triangle's roles
-    int64_t tlive_stride;
+    uint8_t* tlive[3];  // [tri_cap, padded] per direction variant, the smallest window bucket of a triangle's roles
     // a direction variant's row of tlive is written by the first call that needs it
     // (ensure_liveness): the row is ready once live_ev[dir] (recorded on that call's
     // stream) has completed
@@ -375,11 +374,13 @@ bool tune_forced(TuneParams* p, bool probe);
 void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s);
 
 // The run-ends table (live.cu; needs the sorted store); the rows of liveness bytes of the
-// triangle array's entries with their padding; and the mark that the out motif's row is
-// written by what was enqueued on s so far (a one-pass listing writes it itself).
+// triangle array's g->tri_cap entries with their padding; the same after a one-pass listing
+// wrote the out motif's row into `out`, an allocation of the graph's for `room` entries, of
+// which at most `entries` are in use; and such an allocation, of rows one after another.
 void build_run_ends(folty_graph* g, cudaStream_t s);
-void prepare_liveness(folty_graph* g, int64_t entries, cudaStream_t s);
-void listed_liveness(folty_graph* g, cudaStream_t s);
+void prepare_liveness(folty_graph* g, cudaStream_t s);
+void listed_liveness(folty_graph* g, uint8_t* out, int64_t room, int64_t entries, cudaStream_t s);
+uint8_t* liveness_rows(folty_graph* g, int rows, int64_t entries, cudaStream_t s);
 // Makes the liveness row of direction variant dir ready for work enqueued on s after the
 // call: computes it on s the first time (thread-safe), else makes s wait for the
 // computation. Not while s is capturing.

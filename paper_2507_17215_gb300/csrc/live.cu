@@ -469,15 +469,21 @@ void build_run_ends(folty_graph* g, cudaStream_t s) {
     else run_ends_t<int64_t>(g, s);
 }
 
-void prepare_liveness(folty_graph* g, int64_t entries, cudaStream_t s) {
-    // three rows of liveness bytes, each padded with DMIN_NEVER to whole 16-byte chunks
-    // (every pass writes the bytes of all entries of the triangle array)
-    g->tlive_stride = (entries + 15) & ~int64_t(15);
-    g->tlive = graph_alloc<uint8_t>(g, 3 * g->tlive_stride, s);
-    for (int d = 0; d < 3; d++)
-        if (g->tlive_stride > entries)
-            FOLTY_CUDA(cudaMemsetAsync(g->tlive + d * g->tlive_stride + entries, DMIN_NEVER,
-                                       (size_t)(g->tlive_stride - entries), s));
+int64_t liveness_stride(int64_t entries) { return (entries + 15) & ~int64_t(15); }
+
+uint8_t* liveness_rows(folty_graph* g, int rows, int64_t entries, cudaStream_t s) {
+    // each padded with DMIN_NEVER to whole 16-byte chunks (every pass writes the bytes of all
+    // entries of the triangle array)
+    const int64_t stride = liveness_stride(entries);
+    uint8_t* base = graph_alloc<uint8_t>(g, rows * stride, s);
+    for (int d = 0; d < rows && stride > entries; d++)
+        FOLTY_CUDA(cudaMemsetAsync(base + d * stride + entries, DMIN_NEVER, (size_t)(stride - entries), s));
+    return base;
+}
+
+void prepare_liveness(folty_graph* g, cudaStream_t s) {
+    uint8_t* base = liveness_rows(g, 3, g->tri_cap, s);
+    for (int d = 0; d < 3; d++) g->tlive[d] = base + d * liveness_stride(g->tri_cap);
 }
 
 template <typename TS>
@@ -488,7 +494,7 @@ static void liveness_row_t(folty_graph* g, int dir, cudaStream_t s) {
     StageSpan span(ST_ROLES, s, cap * (16 + 1) + g->S * (int64_t)sizeof(RunEnds<TS>));
     if (g->ntri == 0) return;
     const RunEnds<TS>* ends = (const RunEnds<TS>*)g->run_ends;
-    uint8_t* row = g->tlive + (int64_t)dir * g->tlive_stride;
+    uint8_t* row = g->tlive[dir];
     const unsigned grid = grid_for(cap, 256);
     if (dir == FOLTY_DIR_OUT) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_OUT>), grid, 256, 0, s, g->tri, cap, ends, row);
     else if (dir == FOLTY_DIR_IN) FOLTY_LAUNCH((k_tri_live<TS, FOLTY_DIR_IN>), grid, 256, 0, s, g->tri, cap, ends, row);
@@ -511,7 +517,20 @@ void ensure_liveness(folty_graph* g, int dir, cudaStream_t s) {
     }
 }
 
-void listed_liveness(folty_graph* g, cudaStream_t s) {
+// The other variants' rows have the size of the array's part in use, and the out motif's, which the listing
+// wrote with room for its bound, moves into one where it takes less than half of that (6M
+// edges of 2 per pair: 2.9M of 29M bytes; at 70M edges 77M of 111M stay where they are).
+void listed_liveness(folty_graph* g, uint8_t* out, int64_t room, int64_t entries, cudaStream_t s) {
+    const bool move = 2 * entries < room;
+    uint8_t* base = liveness_rows(g, move ? 3 : 2, entries, s);
+    const int64_t stride = liveness_stride(entries);
+    g->tlive[FOLTY_DIR_IN] = base;
+    g->tlive[FOLTY_DIR_EITHER] = base + stride;
+    g->tlive[FOLTY_DIR_OUT] = move ? base + 2 * stride : out;
+    if (move) {
+        FOLTY_CUDA(cudaMemcpyAsync(base + 2 * stride, out, (size_t)g->tri_cap, cudaMemcpyDeviceToDevice, s));
+        graph_release(g, out, s);
+    }
     std::lock_guard<std::mutex> lock(g->live_mu);
     if (!g->live_ev[FOLTY_DIR_OUT]) FOLTY_CUDA(cudaEventCreateWithFlags(&g->live_ev[FOLTY_DIR_OUT], cudaEventDisableTiming));
     FOLTY_CUDA(cudaEventRecord(g->live_ev[FOLTY_DIR_OUT], s));
@@ -601,7 +620,7 @@ unsigned long long* prof_counter(folty_graph* g, cudaStream_t s) {
 static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBuffers& ls,
                            unsigned long long* prof_sel, const int64_t* qp, cudaStream_t s) {
     StageSpan span(ST_SELECT, s, g->tri_cap, prof_sel);
-    const uint8_t* tl = g->tlive + (int64_t)dir * g->tlive_stride;
+    const uint8_t* tl = g->tlive[dir];
     if (g->ts32) launch_select_t<uint32_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
     else launch_select_t<int64_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
 }

@@ -1753,10 +1753,11 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         const int grid = (int)std::min<int64_t>((S + TRI_LIST_THREADS - 1) / TRI_LIST_THREADS, (int64_t)num_sms() * TRI_PER_SM);
         int chunk = TRI_CHUNK_MAX;
         while (chunk > TRI_CHUNK_MIN && (int64_t)chunk * grid * warps * 16 > bound) chunk >>= 1;
-        const int64_t cap = bound + (int64_t)chunk * grid * warps;
+        const int64_t ends = (int64_t)chunk * grid * warps;  // entries in no warp's use at the chunks' ends
+        const int64_t cap = bound + ends;
         g->tri = graph_alloc<int4>(g, cap, s);
         g->tri_off = nullptr;
-        prepare_liveness(g, cap, s);
+        uint8_t* live = liveness_rows(g, 1, cap, s);
         FOLTY_CUDA(cudaMemsetAsync(merged, 0, 2 * sizeof(unsigned long long), s));
         if (ids) side.join();
         if (!ids) build_run_ends(g, s);
@@ -1764,13 +1765,12 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         // totals come with the last read-back
         StageSpan span(ST_TRIANGLES, s, 8 * (int64_t)S);
         uint32_t* eup = sc.get<uint32_t>(S);
-        const TriListArgs a{outptr, out_nbr, out_src, eup, S, chunk, g->tri,
-                            g->tlive + (int64_t)FOLTY_DIR_OUT * g->tlive_stride, g->common, merged, merged + 4, merged + 5};
+        const TriListArgs a{outptr,      out_nbr, out_src, eup,       S,         chunk,
+                            g->tri, live,    g->common, merged, merged + 4, merged + 5};
         if (g->ts32) list_triangles<uint32_t>(g, a, out_eid, sc.get<OutEnds<uint32_t>>(S), eup, grid, s);
         else list_triangles<int64_t>(g, a, out_eid, sc.get<OutEnds<int64_t>>(S), eup, grid, s);
         FOLTY_LAUNCH(k_probe_total, grid_for(S, T), T, 0, s, g->seg, g->common, S, merged + 3, stat + 2);
         span.end();
-        listed_liveness(g, s);
         const void* ptrs[5] = {merged, merged + 1, merged + 3, merged + 5, stat + 2};
         int sizes[5] = {8, 8, 8, 8, 4};
         int64_t outv[5] = {0, 0, 0, 0, 0};
@@ -1781,6 +1781,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         g->info.sigma_max = (int32_t)outv[4];
         g->enum_bytes = 4 * outv[0] + 8 * (int64_t)S;
         span.add_bytes(4 * outv[0] + 17 * g->ntri);
+        listed_liveness(g, live, cap, g->ntri + ends, s);  // (tri_cap itself differs from run to run)
     } else {
         const int64_t ntri = g->ntri;
         g->tri_cap = ntri;
@@ -1805,7 +1806,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         } else {
             build_run_ends(g, s);
         }
-        prepare_liveness(g, ntri, s);
+        prepare_liveness(g, s);
         ensure_liveness(g, FOLTY_DIR_OUT, s);
     }
     g->info.triangles = g->ntri;

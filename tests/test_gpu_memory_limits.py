@@ -26,7 +26,7 @@ class _Failing:
 
     def __init__(self, F, g):
         import torch
-        self.F, self.left = F, -1
+        self.F, self.left, self.live = F, -1, {}
 
         @F.ALLOC_FN
         def alloc(nbytes, stream, ctx):
@@ -34,10 +34,13 @@ class _Failing:
                 self.left = -1
                 return None
             self.left -= self.left > 0
-            return torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
+            p = torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
+            self.live[p] = int(nbytes)
+            return p
 
         @F.FREE_FN
         def free(ptr, stream, ctx):
+            del self.live[int(ptr)]
             torch.cuda.caching_allocator_delete(int(ptr))
 
         self.allocator, h = F.folty_allocator(alloc, free, None), ctypes.c_void_p()
@@ -118,3 +121,30 @@ def test_preprocessing_repeated_after_it_ran_out_of_memory(F, kind):
             break
         fail += 1
     assert fail > 10
+
+
+def _sparse_bounds_graph():
+    """1.2M static edges between two sides of 20,000 vertices, without a triangle: the listing's
+    bound (the sum of the shorter out-lists) has tens of millions of entries, all empty."""
+    rng = np.random.default_rng(4)
+    n, m = 20_000, 1_200_000
+    src, dst = rng.integers(0, n, m), rng.integers(n, 2 * n, m)
+    return W.TemporalGraph(2 * n, src.astype(np.int32), dst.astype(np.int32), np.sort(rng.integers(0, 1000, m)))
+
+
+def test_liveness_rows_have_the_triangles_size(F, monkeypatch):
+    """The array of a one-pass listing has room for its bound, 16 B an entry; the rows of
+    liveness bytes (3 B an entry) have that of the triangles."""
+    g = _sparse_bounds_graph()
+    held, largest = [], []
+    for layout in ("", "counted"):
+        monkeypatch.setenv("FOLTY_TRI_LAYOUT", layout)
+        with _Failing(F, g) as G:
+            F.folty_preprocess(G.handle)
+            info = F.folty_graph_get_info(G.handle)
+            assert info["triangles"] == 0 and info["m_kept"] > F.NOALLOC_MAX_EDGES
+            held.append(sum(G.live.values()))
+            largest.append(max(G.live.values()))
+    entries = largest[0] // 16
+    assert entries > 5_000_000 and largest[0] > 2 * largest[1]
+    assert held[0] - largest[0] - held[1] < entries // 2
