@@ -625,11 +625,13 @@ static void enqueue_select(folty_graph* g, int64_t delta, int dir, const ProbeBu
     else launch_select_t<int64_t>(g, dir, tl, delta, ls, prof_sel, qp, s);
 }
 
+static ProbeBuffers scratch_buffers(folty_graph* g, Scratch& sc, cudaStream_t s) {
+    return make_probe_buffers(g, s, [&](auto* tag, int64_t n) { return sc.get<std::remove_pointer_t<decltype(tag)>>(n); });
+}
+
 static ProbeBuffers select_live(folty_graph* g, int64_t delta, int dir, Scratch& sc, cudaStream_t s,
                                 unsigned long long* prof_sel) {
-    const ProbeBuffers ls = make_probe_buffers(g, s, [&](auto* tag, int64_t n) {
-        return sc.get<std::remove_pointer_t<decltype(tag)>>(n);
-    });
+    const ProbeBuffers ls = scratch_buffers(g, sc, s);
     ensure_liveness(g, dir, s);
     enqueue_select(g, delta, dir, ls, prof_sel, nullptr, s);
     return ls;
@@ -731,6 +733,8 @@ void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s) {
     const bool c16 = g->info.max_degree < 65535;
     int32_t* cnt = c16 ? nullptr : sc.get<int32_t>(mk);
     uint16_t* cnt16 = c16 ? sc.get<uint16_t>(mk + 2) : nullptr;
+    const ProbeBuffers ls = scratch_buffers(g, sc, s);
+    ensure_liveness(g, dir, s);
     cudaEvent_t ev[TUNE_TRIALS + 1];
     for (auto& e : ev) FOLTY_CUDA(cudaEventCreate(&e));
     float best = 0.f;
@@ -740,8 +744,8 @@ void tune_probe(folty_graph* g, int64_t delta, int dir, cudaStream_t s) {
         for (int c = 0; c < TUNE_TRIALS; c++) {
             g->tune.probe_items = PROBE_CAND[c][0];
             g->tune.probe_blocks = PROBE_CAND[c][1];
-            // each trial selects anew (outside its timed span)
-            const ProbeBuffers ls = select_live(g, delta, dir, sc, s, nullptr);
+            // each trial selects anew (outside its timed span), in the same buffers
+            enqueue_select(g, delta, dir, ls, nullptr, nullptr, s);
             if (cnt16) FOLTY_CUDA(cudaMemsetAsync(cnt16, 0, sizeof(uint16_t) * (size_t)(mk + 2), s));
             else FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)mk, s));
             LiveArgs la = live_args(g, ls);

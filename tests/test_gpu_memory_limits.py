@@ -26,7 +26,7 @@ class _Failing:
 
     def __init__(self, F, g):
         import torch
-        self.F, self.left, self.live = F, -1, {}
+        self.F, self.left, self.live, self.peak = F, -1, {}, 0
 
         @F.ALLOC_FN
         def alloc(nbytes, stream, ctx):
@@ -36,6 +36,7 @@ class _Failing:
             self.left -= self.left > 0
             p = torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
             self.live[p] = int(nbytes)
+            self.peak = max(self.peak, sum(self.live.values()))
             return p
 
         @F.FREE_FN
@@ -148,3 +149,24 @@ def test_liveness_rows_have_the_triangles_size(F, monkeypatch):
     entries = largest[0] // 16
     assert entries > 5_000_000 and largest[0] > 2 * largest[1]
     assert held[0] - largest[0] - held[1] < entries // 2
+
+
+def test_tuning_takes_one_set_of_selection_buffers(F):
+    """The first query of a graph with 16M triangles times its probe shapes before it allocates
+    its plan, which holds one set of selection buffers (17 B a triangle) and little else: the
+    trials must not need more."""
+    k, size = 100, 100
+    i, j = np.triu_indices(size, 1)
+    base = np.repeat(np.arange(k) * size, len(i))
+    src, dst = np.tile(i, k) + base, np.tile(j, k) + base
+    src, dst = np.tile(src, 3).astype(np.int32), np.tile(dst, 3).astype(np.int32)
+    g = W.TemporalGraph(k * size, src, dst, np.sort(np.random.default_rng(2).integers(0, 1000, len(src))))
+    F.folty_tuning_clear_cache()
+    with _Failing(F, g) as G:
+        F.folty_preprocess(G.handle)
+        assert F.folty_graph_get_info(G.handle)["triangles"] == k * size * (size - 1) * (size - 2) // 6
+        before = G.peak = sum(G.live.values())
+        F.folty_query(G.handle, QUERIES[1])
+        assert F.folty_graph_tuning(G.handle)["probe_source"] == "timed trials"
+        kept, peak = sum(G.live.values()) - before, G.peak - before
+    assert kept > 17 * 16_000_000 and peak < 1.2 * kept, (kept, peak)
