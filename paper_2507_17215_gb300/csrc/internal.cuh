@@ -451,20 +451,4 @@ __device__ __forceinline__ int32_t row_of(const uint32_t* __restrict__ ebits, co
     return wpref[x >> 5] + __popc(ebits[x >> 5] & ((1u << (x & 31)) - 1u));
 }
 
-// First index in [lo, hi) with a[i] >= key (hi if none).
-__device__ __forceinline__ int lower_bound_i64(const int64_t* __restrict__ a, int lo, int hi,
-                                               int64_t key) {
-    int len = hi - lo;
-    while (len > 0) {
-        int half = len >> 1;
-        if (a[lo + half] < key) {
-            lo += half + 1;
-            len -= half + 1;
-        } else {
-            len = half;
-        }
-    }
-    return lo;
-}
-
 }  // namespace folty

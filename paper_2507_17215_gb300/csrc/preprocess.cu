@@ -351,10 +351,9 @@ __device__ __forceinline__ void pair_run_starts(uint64_t pk, uint64_t prev, int 
 }
 
 // perm, T, sd and the run starts from the sorted words: position i holds time rank
-// j = word mod 2^ib (input index order[j], or j) of pair id and direction word >> ib.
-// SORTED: t holds the timestamps in sorted order already (the sort's values); otherwise
-// they are gathered from the input order.
-template <typename TS, bool SORTED>
+// j = word mod 2^ib (input index order[j], or j) of pair id and direction word >> ib. T is
+// gathered from the timestamps in input order (64-bit stores).
+template <typename TS>
 __global__ void k_pair_store(const uint64_t* __restrict__ packed, const uint32_t* __restrict__ order, int64_t mk,
                              int32_t S, int ib, const TS* __restrict__ t, int32_t* __restrict__ perm,
                              TS* __restrict__ T, int32_t* __restrict__ sd, int32_t* __restrict__ seg) {
@@ -364,7 +363,7 @@ __global__ void k_pair_store(const uint64_t* __restrict__ packed, const uint32_t
         const int64_t j = (int64_t)(pk & jm);
         const uint32_t o = order ? order[j] : (uint32_t)j;
         __stcs(perm + i, (int32_t)o);
-        T[i] = SORTED ? __ldcs(t + i) : t[o];
+        T[i] = t[o];
         __stcs(sd + i, (int32_t)(pk >> ib));
         pair_run_starts(pk, i > 0 ? packed[i - 1] : ~0ull, ib, S, i, seg);
     }
@@ -1351,7 +1350,7 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
         FOLTY_LAUNCH(k_pair_store4, (unsigned)(((mk + 3) / 4 + T - 1) / T), T, 0, s, sp, job.order, mk, S, ib,
                      palt ? tv_alt : tv, g->perm, (uint32_t*)g->T, g->sd, g->seg);
     else
-        FOLTY_LAUNCH((k_pair_store<int64_t, false>), grid_for(mk, T), T, 0, s, sp, job.order, mk, S, ib, g->in_t,
+        FOLTY_LAUNCH((k_pair_store<int64_t>), grid_for(mk, T), T, 0, s, sp, job.order, mk, S, ib, g->in_t,
                      g->perm, (int64_t*)g->T, g->sd, g->seg);
     FOLTY_LAUNCH(k_segments_fix, grid_for(S, T), T, 0, s, S, mk, g->seg);
 }
