@@ -9,8 +9,8 @@ query exists u exists v forall_{3/10} w in N(u) with delta = 3600 s ("out" motif
 "--workload medium" runs the medium graph (1,000,000 vertices, 20,000,000 edges) and its
 three queries (delta in {600, 3600, 86400} s, rho = 1/2) instead.
 
-One step = the whole path on one batch of input: load (copy + validation),
-preprocessing (sort, static graph, peeling, orientation, triangle listing, role summary)
+One step = the whole path on one batch of input: load (checks, pair table),
+preprocessing (sort, static graph, core numbers, orientation, triangle listing, run ends)
 and the workload's queries (selection, probes, counts, threshold, solution pairs back on
 the host).
 
@@ -612,13 +612,13 @@ def main():
     stages = stage_table(prof, prof_steps, peak)
     roofline = query_roofline = None
     if stages:
-        # the store span contains sort spans and runs beside the peel: not a stage of its own
+        # the store span contains sort spans and runs beside the core numbers: not a stage of its own
         dom = max((k for k in stages if k != "store"), key=lambda k: stages[k]["ms_per_step"])
         roofline = roofline_of(prof, dom, peak, peak_kind, args.workload)
         if dom == "peel":
-            roofline["note"] = (f"the peel is bound by the latency of its dependent rounds ({info['peel_rounds']} "
-                                "on this graph: grid, cluster and single-CTA phases), not by bandwidth; its model "
-                                "bytes are tiny, so the fraction is near zero by construction")
+            roofline["note"] = ("the core numbers are bound by the latency of their dependent rounds and by random "
+                                "accesses, not by bandwidth; their model bytes are tiny, so the fraction is near "
+                                "zero by construction")
         qs_ = [k for k in QUERY_STAGES if k in stages]
         if qs_:
             qdom = max(qs_, key=lambda k: stages[k]["ms_per_step"])

@@ -243,9 +243,8 @@ uint64_t folty_kernel_launches(void);
  *             written per static edge) and the liveness pass of one direction variant (16 B
  *             read and 1 B written per triangle, the run-ends table read once; the out
  *             motif's of graphs past FOLTY_NOALLOC_MAX_EDGES edges is part of TRIANGLES);
- *   BATCH     the batched threshold over the plain queries of a direction variant: the
- *             32-edge group bits, and (counted on the device) the bin row and 4 B of pair
- *             key of every edge in a group with a hit;
+ *   BATCH     the batched threshold over the plain queries of a direction variant: the bin
+ *             row (whole 16-byte chunks) and 4 B of pair key of every edge with a hit;
  *   STORE     the temporal store built beside the core numbers: its span contains SORT spans.
  *             Time-ordered input with 32-bit offsets: 8 B per input edge for the sort ids
  *             and 16 B per edge and radix pass (the first pass reads 4 B more: the ids and

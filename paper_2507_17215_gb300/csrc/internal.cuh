@@ -127,7 +127,7 @@ constexpr int PROF_SLOTS = 64;       // probe-stage byte counters per graph
 constexpr int HOST_STAGE = 512;      // pinned int64 slots per graph
 constexpr int64_t PAIR_STAGE = 1 << 16;  // solution pairs staged in pinned memory per read-back
 constexpr int READBACK_MAX = 384;    // slots [0, READBACK_MAX) serve read_back
-constexpr int ERR_SLOT = READBACK_MAX + 8;  // the device error word's copy (load uses +0..+4, peeling +16..+27)
+constexpr int ERR_SLOT = READBACK_MAX + 8;  // the device error word's copy (load uses +0..+4)
 constexpr uint64_t GRAPH_TAG = 0x464f4c5459475248ull;   // "FOLTYGRH"
 constexpr uint64_t RESULT_TAG = 0x464f4c5459525354ull;  // "FOLTYRST"
 constexpr uint64_t FREED_TAG = 0x464f4c5459465245ull;   // "FOLTYFRE"

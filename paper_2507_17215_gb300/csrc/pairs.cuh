@@ -11,7 +11,9 @@
 namespace folty {
 
 // A longer probe sequence abandons the table: at the largest load that serves (1/2) a
-// sequence of linear probing is this long with a probability below 1e-20.
+// sequence of linear probing among random slots is this long with a probability below 1e-20.
+// The slots of a multiplicative hash are not random: ranks in a bad progression only lose the
+// table, not a result.
 constexpr int PAIR_MAX_PROBE = 256;
 constexpr uint64_t PAIR_HASH_MUL = 0x9E3779B97F4A7C15ull;  // 2^64 / golden ratio (Fibonacci hashing)
 constexpr uint32_t PAIR_LOOP = 0x7fffffffu;  // slot word of a self-loop
@@ -24,7 +26,7 @@ __device__ __forceinline__ uint64_t pair_rank_of(int32_t x, int32_t y, int32_t n
 
 // A table with more pairs than half its slots does not serve, and the insert stops as soon
 // as that shows: the pairs placed in every 64th slot are counted, and 9/8 of the number they
-// may reach (of slots from PAIR_COUNTED_LG on: 8192, a hundred standard deviations of 90
+// may reach (of slots from PAIR_COUNTED_LG on: 8192, eleven standard deviations of 90
 // below it) abandons the table at a load of 0.56, where probe sequences are still short.
 // Smaller tables hold 2 slots per edge and always serve. Against a first try of 2^19 slots,
 // 6M edges of 3M pairs took 66.5 ms when every edge still walked 4096 steps of the full

@@ -601,11 +601,11 @@ __global__ void k_outptr(const int32_t* __restrict__ rowptr, const int32_t* __re
 constexpr int TRI_THREADS = 256;
 constexpr int TRI_HCAP = 256;    // out(u) entries a warp's table holds (longer lists: one lane merges)
 constexpr int TRI_HSLOTS = 512;  // table slots (load at most one half)
-// entries of a warp's chunk of the one-pass listing's array: fewer when the bound is small,
-// so that the empty ends of the chunks stay below a sixteenth of the bound or 32 a warp
 constexpr int TRI_BUCKETS = 128; // of four slots, of the one-pass listing (load at most one half)
 constexpr int TRI_LIST_THREADS = 128;
 constexpr int TRI_PER_SM = 8;    // resident blocks (what their tables leave room for)
+// entries of a warp's chunk of the one-pass listing's array: fewer when the bound is small,
+// so that the empty ends of the chunks stay below a sixteenth of the bound or 32 a warp
 constexpr int TRI_CHUNK_MIN = 32, TRI_CHUNK_MAX = 512;
 // the largest array of a one-pass listing; a larger bound takes the counting pass
 constexpr int64_t TRI_BOUND_MAX_BYTES = int64_t(16) << 30;
@@ -1268,8 +1268,8 @@ static void sort_check(folty_graph* g, cudaStream_t s) { read_back(g, nullptr, n
 
 // The second half of A1 with dense pair ids: the temporal edges sorted by (pair id,
 // direction, time rank) into the store (perm, T, sd, seg). It needs nothing of the
-// static graph's later steps, and they nothing of it before the triangle pass, so it
-// runs on a second stream beside the peeling.
+// static graph's later steps, and they nothing of it before the triangles, so it
+// runs on a second stream beside or after the core numbers.
 struct StoreJob {
     const uint32_t* slotw;  // [m] pair table slot and direction of each input edge
     const uint32_t* order;  // time order of an unsorted input, or null
@@ -1303,8 +1303,8 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
                                : graph_alloc<uint32_t>(g, STORE_MAX_PASSES << STORE_DIGIT_BITS, s);
         FOLTY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (2 * (size_t)S + 1), s));
         FOLTY_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (STORE_MAX_PASSES << STORE_DIGIT_BITS), s));
-        // one block per 2048 edges: short blocks, so that the peel's kernels on the
-        // high-priority streams get SMs as soon as any block ends
+        // one block per 2048 edges: short blocks, so that the kernels on the high-priority
+        // stream get SMs as soon as any block ends
         FOLTY_LAUNCH(k_store_ids, (unsigned)(((m + STORE_IDS_EDGES - 1) / STORE_IDS_EDGES + T - 1) / T), T, 0, s,
                      job.slotw, m, job.sid, S, cw, cnt);
         // the runs: seg[c] = first sorted position of id c, seg[2S] = mk
@@ -1327,7 +1327,7 @@ static void temporal_store(folty_graph* g, const StoreJob& job, Scratch& sc, int
         return;
     }
     g->perm = graph_alloc<int32_t>(g, mk, s);
-    // the whole store, beside the peeling: its pair words and time offsets (4 B slot and
+    // the whole store: its pair words and time offsets (4 B slot and
     // 8 B time read, 12 B written per input edge) and the sorted arrays (the word and the
     // time read, perm, T and sd written: 24 B per kept edge); the sort passes inside are
     // also SORT spans
@@ -1482,8 +1482,7 @@ static void pair_key_sort(folty_graph* g, Scratch& sc, const uint32_t* order, cu
 // and probe slots into merged[0], merged[1], zeroed here) under the graph's split between
 // one thread and one warp per oriented edge: forced, cached under the graph's statistics,
 // or picked by timing the pass under each candidate split. All candidates count the same
-// triangles, so the last trial's outputs stand. trials_only: the trials (when the split
-// is neither forced nor cached) and nothing else, for a listing without counting pass.
+// triangles, so the last trial's outputs stand.
 static void tune_triangles(folty_graph* g, const int32_t* outptr, const int32_t* out_nbr, const int32_t* out_src,
                            const int32_t* osig, int32_t* tcnt, int64_t* pcnt, unsigned long long* merged,
                            cudaStream_t s) {
@@ -1573,11 +1572,12 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     const bool ids = pair_ids_sort(g, sc, order, s, &job);
     if (!ids) pair_key_sort(g, sc, order, s);
     const int32_t S = g->S;
-    // the temporal store of the dense-id path: on a side stream of default priority from
-    // the end of the grid peel on (beside the rest of the peel and the triangle passes,
-    // which run on streams of the highest priority and take SMs first), joined after the
-    // triangle passes (which need only its per-pair counts). On an error in between, the
-    // side streams are drained before the call's buffers go.
+    // the temporal store of the dense-id path: on a side stream of default priority, beside
+    // the core numbers or after them beside the orientation (A3 below), whose kernels run on a
+    // stream of the highest priority and take SMs first. It is joined before a one-pass listing,
+    // which reads its run ends, and after the counting pass and the listing of small graphs,
+    // which need its per-pair counts only. On an error in between, the side streams are drained
+    // before the call's buffers go.
     SideStream side(s, false);
     struct EventHolder {
         cudaEvent_t e = nullptr;
@@ -1824,12 +1824,11 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
 }
 
 // Preprocessing runs on a stream of the device's highest priority, forked from the
-// caller's stream and joined back at the end. The temporal store runs beside the peel
-// and the triangle passes on a stream of default priority (its kernels take one block
-// per chunk of work, so their blocks retire quickly), and the chain that decides the
-// preprocessing's length takes SMs first whenever blocks retire: measured with events on
-// the paper-scale graph, the peel's set-up kernels and the orientation otherwise waited
-// behind the store's kernels for ≈ 1 ms each.
+// caller's stream and joined back at the end. The temporal store runs beside it on a stream
+// of default priority (its kernels take one block per chunk of work, so their blocks retire
+// quickly), and the chain that decides the preprocessing's length takes SMs first whenever
+// blocks retire: measured with events on the paper-scale graph, the orientation otherwise
+// waited behind the store's kernels for ≈ 1 ms.
 void preprocess_graph(folty_graph* g, cudaStream_t s) {
     SideStream pri(s, true);
     preprocess_on(g, pri.fork());

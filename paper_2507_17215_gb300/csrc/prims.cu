@@ -1,7 +1,7 @@
 // Device-wide primitives: exclusive prefix sum and a stable LSD radix sort.
 //
-// Both are bandwidth-bound streaming passes over tiles of 4096 elements (2048 for 8-byte
-// scans) per 256-thread block, with coalesced loads and stores; a tile's offset comes
+// Both are streaming passes with coalesced loads and stores, over tiles of 4096 elements (2048
+// for 8-byte scans; 1024 to 8192 keys of a sort, by its size and type); a tile's offset comes
 // from a decoupled look-back over the totals that earlier tiles publish, so each pass is
 // a single kernel. Every look-back wait is bounded in time and reports through the
 // scratch error word.
@@ -117,16 +117,16 @@ void exclusive_scan(Scratch& sc, const uint32_t* in, uint32_t* out, int64_t n) {
 // ================================================================== radix sort
 //
 // Stable LSD radix sort, one kernel per 8-bit digit ("onesweep"): the histograms of all
-// digits come from one read of the keys up front; each pass takes tiles of 4096 or 8192 keys in
+// digits come from one read of the keys up front; each pass takes tiles of 1024, 4096 or 8192 keys in
 // the order blocks start (a dynamic tile counter), ranks them by digit within the tile,
 // publishes the tile's digit counts, and adds the counts of all earlier tiles by looking
 // back over their published values (decoupled look-back: a tile's entry holds either its
-// own count or its inclusive prefix). The tile is then listed in digit order through
-// shared memory, so that the global writes of each digit's run are contiguous.
+// own count or its inclusive prefix). The tile lies in digit order in shared memory by then,
+// so that the global writes of each digit's run are contiguous.
 
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // 4096 keys per tile
+constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // 4096 keys per tile of 64-bit keys with values
 constexpr int RS_AHEAD = 4;  // items whose peer masks are made together
 // look-back entries in flight a thread: two take as long, sixteen (mostly read in vain, 2 KB an
 // entry) 10% longer at 70M keys

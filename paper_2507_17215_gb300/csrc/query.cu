@@ -324,7 +324,7 @@ static void launch_hits(HitArgs a, int quant, int universe, cudaStream_t s) {
 // then one thread per pair. Clears the bits and the pairs' entries for the next query.
 // tot[0] = pairs x < y, tot[1] = all pairs.
 struct EmitArgs {
-    uint32_t* pbits;  // [wa + wb] words, both halves whole 16-word lines
+    uint32_t* pbits;  // [wt] words: wa for the pairs x < y, as many for x > y
     int64_t wa, wt;
     const int32_t* ea;
     const int32_t* eb;
@@ -910,7 +910,7 @@ struct QueryPlans {
     ProbeBuffers pb{};
     int32_t* seg_max = nullptr;    // [2S], then seg_ncert [2S]
     int32_t* seg_ncert = nullptr;
-    uint32_t* pbits = nullptr;     // [wa + wb] solution pair bits
+    uint32_t* pbits = nullptr;     // [wt = 2 wa] solution pair bits
     int64_t wa = 0, wt = 0;
     unsigned long long* ctl = nullptr;  // look-back of k_pair_emit
     int64_t nctl = 0;
