@@ -901,9 +901,15 @@ folty_status folty_query(folty_graph* g, const folty_query_params* q, folty_resu
         if (!q || !out) fail(FOLTY_EINVAL, "query or result is NULL");
         if (g->state != 1) fail(FOLTY_ESTATE, "graph not preprocessed");
         validate_query(*q);
-        ProfileScope prof;
-        run_query(g, *q, out, (cudaStream_t)stream);  // ends with a stream synchronisation
-        prof.commit();
+        std::memset(out, 0, sizeof(*out));
+        try {
+            ProfileScope prof;
+            run_query(g, *q, out, (cudaStream_t)stream);  // ends with a stream synchronisation
+            prof.commit();
+        } catch (...) {
+            if (out->tag == RESULT_TAG) release_result(out);
+            throw;
+        }
     });
 }
 

@@ -170,3 +170,26 @@ def test_tuning_takes_one_set_of_selection_buffers(F):
         assert F.folty_graph_tuning(G.handle)["probe_source"] == "timed trials"
         kept, peak = sum(G.live.values()) - before, G.peak - before
     assert kept > 17 * 16_000_000 and peak < 1.2 * kept, (kept, peak)
+
+
+def test_a_query_that_ran_out_of_memory_holds_no_result(F):
+    """A query with every optional output, whose host arrays exist before its last device
+    buffers: the call that fails leaves nothing for the caller to release."""
+    g = _graph("large")  # its per-edge counts are allocated after the result
+    q = F._params(W.Query(86400, 1, 10, W.Q_EXISTS, W.DIR_EITHER, W.U_COMMON, True, outer=W.OUTER_FORALL_T,
+                          want_certificates=True, want_triples=True))
+    with _Failing(F, g) as G:
+        F.folty_preprocess(G.handle)
+        fail = 0
+        while True:
+            r = F.folty_result()
+            G.left = fail
+            st = F.lib.folty_query(G.handle, ctypes.byref(q), ctypes.byref(r), F.current_stream())
+            G.left, reached = -1, G.left == -1
+            if st == F.FOLTY_OK:
+                F._take_results(r, 1)
+                break
+            assert st == F.FOLTY_ENOMEM and reached, F.folty_last_error()
+            assert r.tag != 0x464F4C5459525354 and not r.u and not r.certificate and not r.edge_count and not r.triple_x, fail
+            fail += 1
+        assert fail > 2
