@@ -1829,10 +1829,24 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
 // quickly), and the chain that decides the preprocessing's length takes SMs first whenever
 // blocks retire: measured with events on the paper-scale graph, the orientation otherwise
 // waited behind the store's kernels for ≈ 1 ms.
+//
+// A call that fails leaves the graph as the load did, so that it may be repeated: what the
+// call had allocated goes (its side streams are drained by then), and no mark of it stays.
 void preprocess_graph(folty_graph* g, cudaStream_t s) {
-    SideStream pri(s, true);
-    preprocess_on(g, pri.fork());
-    pri.join();
+    const size_t had = g->owned->size();
+    try {
+        SideStream pri(s, true);
+        preprocess_on(g, pri.fork());
+        pri.join();
+    } catch (...) {
+        if (g->state == 0) {
+            while (g->owned->size() > had) graph_release(g, g->owned->back().first, s);
+            g->perm = nullptr;
+            g->cw = nullptr;
+            for (auto& ready : g->live_ready) ready = 0;
+        }
+        throw;
+    }
 }
 
 }  // namespace folty

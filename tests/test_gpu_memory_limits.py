@@ -26,7 +26,7 @@ class _Failing:
 
     def __init__(self, F, g):
         import torch
-        self.F, self.left, self.live, self.peak = F, -1, {}, 0
+        self.F, self.left, self.live, self.peak, self.fill = F, -1, {}, 0, None
 
         @F.ALLOC_FN
         def alloc(nbytes, stream, ctx):
@@ -37,6 +37,12 @@ class _Failing:
             p = torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
             self.live[p] = int(nbytes)
             self.peak = max(self.peak, sum(self.live.values()))
+            if self.fill is not None:  # what the memory holds before its first use, on its own stream
+                view = type("Bytes", (), {"__cuda_array_interface__": {"shape": (int(nbytes),), "typestr": "|u1",
+                                                                       "data": (p, False), "version": 3}})()
+                own = torch.cuda.ExternalStream(int(stream)) if stream else torch.cuda.default_stream()
+                with torch.cuda.stream(own):
+                    torch.as_tensor(view, device="cuda").fill_(self.fill)
             return p
 
         @F.FREE_FN
@@ -120,6 +126,28 @@ def test_preprocessing_repeated_after_it_ran_out_of_memory(F, kind):
             assert {k: v for k, v in got.items() if k != "device_bytes"} == {k: v for k, v in info.items() if k != "device_bytes"}
         if not refused:
             break
+        fail += 1
+    assert fail > 10
+
+
+@pytest.mark.parametrize("kind", ["small", "large"])
+def test_preprocessing_that_ran_out_of_memory_leaves_nothing(F, kind):
+    """A refused call gives back what it had taken, and the repeated one computes everything
+    anew, whatever the memory it is given held (255: a triangle of no window)."""
+    g = _graph(kind)
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G:
+        want = [pairs_of(G.query(q)) for q in QUERIES]
+    fail, refused = 0, True
+    while refused:
+        with _Failing(F, g) as G:
+            loaded = dict(G.live)
+            refused = G.refused(fail, lambda: F.folty_preprocess(G.handle))
+            if refused:
+                assert G.live == loaded, fail
+                G.fill = 255
+                F.folty_preprocess(G.handle)
+                G.fill = None
+            assert [pairs_of(F.folty_query(G.handle, q)) for q in QUERIES] == want, fail
         fail += 1
     assert fail > 10
 
