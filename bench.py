@@ -74,34 +74,7 @@ STAGE_KERNELS = {
     "store": "temporal store beside the core numbers: k_store_ids, k_store_hist, the id sort's k_rs_onesweep passes "
              "(contains sort spans)",
 }
-STAGE_SOURCES = {"probe": ("live.cu", "probe.cuh"), "select": ("live.cu", "scan.cuh"), "sort": ("prims.cu",),
-                 "peel": ("core.cu",), "threshold": ("query.cu",), "triangles": ("preprocess.cu", "liveness.cuh"),
-                 "roles": ("live.cu", "liveness.cuh"), "batch": ("batch.cu",), "store": ("preprocess.cu", "prims.cu")}
 QUERY_STAGES = ("select", "probe", "threshold")
-
-
-def stage_traffic(stage, workload):
-    """DRAM bytes per span of a stage from the committed ncu summary of the workload, when
-    it was taken on the current sources (profiles/traffic_<workload>_workload.md lists
-    'traffic <stage> <bytes> <sha256 of the stage's sources>'); None otherwise."""
-    import hashlib
-    import re
-    path = os.path.join(ROOT, "profiles", f"traffic_{workload}_workload.md")
-    if not os.path.exists(path):
-        return None
-    for m in re.finditer(r"^traffic (\w+) (\d+) ([0-9a-f]{64})$", open(path).read(), re.M):
-        if m.group(1) != stage:
-            continue
-        return int(m.group(2)) if source_hash(stage) == m.group(3) else None
-    return None
-
-
-def source_hash(stage):
-    import hashlib
-    h = hashlib.sha256()
-    for f in STAGE_SOURCES.get(stage, ()):
-        h.update(open(os.path.join(ROOT, "paper_2507_17215_gb300", "csrc", f), "rb").read())
-    return h.hexdigest()
 
 
 def _peaks():
@@ -391,11 +364,11 @@ def stage_table(prof, steps, peak):
     return out
 
 
-def roofline_of(prof, stage, peak, peak_kind, workload):
+def roofline_of(prof, stage, peak, peak_kind):
     d = prof[stage]
     achieved = d["bytes"] / (d["ms"] / 1e3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": stage_traffic(stage, workload), "stage": stage, "kernel": STAGE_KERNELS[stage],
+            "traffic": None, "stage": stage, "kernel": STAGE_KERNELS[stage],
             "peak_kind": f"{peak_kind} hbm_gbs (of {peak_kind})",
             "model_bytes_per_launch": d["bytes"] / d["launches"], "launch_ms": d["ms"] / d["launches"]}
 
@@ -614,7 +587,7 @@ def main():
     if stages:
         # the store span contains sort spans and runs beside the core numbers: not a stage of its own
         dom = max((k for k in stages if k != "store"), key=lambda k: stages[k]["ms_per_step"])
-        roofline = roofline_of(prof, dom, peak, peak_kind, args.workload)
+        roofline = roofline_of(prof, dom, peak, peak_kind)
         if dom == "peel":
             roofline["note"] = ("the core numbers are bound by the latency of their dependent rounds and by random "
                                 "accesses, not by bandwidth; their model bytes are tiny, so the fraction is near "
@@ -622,7 +595,7 @@ def main():
         qs_ = [k for k in QUERY_STAGES if k in stages]
         if qs_:
             qdom = max(qs_, key=lambda k: stages[k]["ms_per_step"])
-            query_roofline = roofline_of(prof, qdom, peak, peak_kind, args.workload)
+            query_roofline = roofline_of(prof, qdom, peak, peak_kind)
     q_ms = qt["query_ms"]
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
