@@ -924,12 +924,15 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
 // and added to common once; merged[0] receives the list entries looked up, merged[1] the
 // triangles.
 // Bound by issue slots and by gathers from L2 (46% of the slots, 33% of the warps at 20M edges;
-// seven or nine blocks an SM are 3 to 5% slower at full size). At full size, 77M triangles from 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M
-// lookups: 400. A lane or a warp per edge, into a layout by upper bounds with three additions to
+// seven or nine blocks an SM are 3 to 5% slower at full size). At full size, 77M triangles from
+// 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M lookups: 400. A lane or a warp per edge, into a layout by upper bounds with three additions to
 // common a triangle, and a second pass that gathered the three edges' runs and moved the
 // triangles took 1110 + 750 and 584 + 75; the same without the queue, the records made by the
 // lanes that found them, 1400 and 690. Looking up the shorter of the two lists (111M and 29M
 // lookups) needs a table per row and edge direction: 1220 and 400.
+// Tails with more than TRI_HCAP out-neighbours, merged by single lanes, cost about twice as much a
+// triangle: preprocessing of 20 cliques of 300 vertices (89M triangles) takes 2.1 ms, of 4 of 600
+// (143M) 4.3, of 30 of 240 (68M, all by tables) 1.5; with the two passes above 3.7, 7.6 and 2.1.
 struct TriListArgs {
     const int32_t *outptr, *out_nbr, *out_src;
     const uint32_t* out_eup;  // static edge at a place of the out-lists; bit 31: the tail has the smaller id
@@ -1639,8 +1642,11 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
     // The core numbers' cooperative kernel waits for SMs that the store's blocks hold, so it is
     // launched first. Where the store is the longer of the two (many temporal edges per static
     // one) it takes half the SMs, whose registers it fills, and the store the others: most of
-    // its rounds are bound by latency. Preprocessing of 20M edges, 24 per pair: 1.64 ms
-    // against 1.92 one after the other; of 6M edges, 2 per pair: 3.66 against 3.51.
+    // its rounds are bound by latency. Preprocessing of 20M edges beside against one after the
+    // other, by edges per static edge: 7.28 against 7.26 ms at 2.3, 5.12 against 5.14 at 4.1, 3.06
+    // against 3.27 at 8, 1.50 against 1.79 at 24; of 6M edges 2.78 against 2.69, 1.97 against
+    // 2.03, 1.39 against 1.48, 0.80 against 0.98. From 4 on it is no slower; the line stays on
+    // the side where it gains clearly.
     const bool beside = ids && g->m_kept >= STORE_BESIDE * (int64_t)S;
     if (beside) store_s = side.fork();
     // rounds, alpha and the error word are read with the triangle totals
