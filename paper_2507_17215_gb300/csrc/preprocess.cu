@@ -925,11 +925,12 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tri_write(const int32_t* __rest
 // triangles.
 // Bound by issue slots and by gathers from L2 (46% of the slots, 33% of the warps at 20M edges;
 // seven or nine blocks an SM are 3 to 5% slower at full size). At full size, 77M triangles from
-// 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M lookups: 400. A lane or a warp per edge, into a layout by upper bounds with three additions to
-// common a triangle, and a second pass that gathered the three edges' runs and moved the
-// triangles took 1110 + 750 and 584 + 75; the same without the queue, the records made by the
-// lanes that found them, 1400 and 690. Looking up the shorter of the two lists (111M and 29M
-// lookups) needs a table per row and edge direction: 1220 and 400.
+// 115M lookups: 1150 us; 3M static edges, 2.8M triangles from 90M lookups: 400. A lane or a warp
+// per edge, into a layout by upper bounds with three additions to common a triangle, and a second
+// pass that gathered the three edges' runs and moved the triangles took 1110 + 750 and 584 + 75;
+// the same without the queue, the records made by the lanes that found them, 1400 and 690.
+// Looking up the shorter of the two lists (111M and 29M lookups) needs a table per row and edge
+// direction: 1220 and 400.
 // Tails with more than TRI_HCAP out-neighbours, merged by single lanes, cost about twice as much a
 // triangle: preprocessing of 20 cliques of 300 vertices (89M triangles) takes 2.1 ms, of 4 of 600
 // (143M) 4.3, of 30 of 240 (68M, all by tables) 1.5; with the two passes above 3.7, 7.6 and 2.1.
