@@ -56,6 +56,23 @@ def test_solution_buffers_of_several_passes(F, monkeypatch, cap, windows):
     assert sum(len(r["u"]) for r in got) > 150_000
 
 
+# most probes hit, the others none; lists below and above the length from which they have a plan
+@pytest.mark.parametrize("n, mult", [(64, 1), (40, 20), (24, 150)])
+def test_marked_edges_where_most_probes_hit(F, n, mult):
+    one = _dense_graph(n, mult)
+    g = W.TemporalGraph(n, np.repeat(one.src, mult), np.repeat(one.dst, mult),
+                        np.sort(np.random.default_rng(n).integers(0, 1000, mult * one.m)))
+    p = np.random.default_rng(mult).permutation(g.m)
+    g = W.TemporalGraph(n, g.src[p], g.dst[p], g.t)
+    qs = [W.Query(d, k, 10, quant, dr, W.U_COMMON, True) for d in (0, 30, 1000) for dr in range(3)
+          for quant, k in ((W.Q_EXISTS, 0), (W.Q_FORALL_T, 9))]
+    with F.TemporalGraph(g.n, g.src, g.dst, g.t) as G:
+        for q, r in zip(qs, G.query_batch(qs)):
+            want = G.query(q)
+            np.testing.assert_array_equal(r["edge_count"], want["edge_count"], err_msg=str(q))
+            assert pairs_of(r) == pairs_of(want), str(q)
+
+
 class _Watched:
     """A graph whose device memory is PyTorch's, with the largest amount held at a time."""
 
