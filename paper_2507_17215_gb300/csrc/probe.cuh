@@ -226,6 +226,7 @@ struct RolePlan {
 __host__ __device__ __forceinline__ RolePlan long_role_plan(int32_t n1, int32_t n2, int32_t n3) {
     RolePlan p{n1, 1};
     const int32_t nd = n2 <= n3 ? n2 : n3;
+    if (nd > n1 / 2) return p;  // as below, without the 64-bit arithmetic
     const int64_t chunks = ((int64_t)n1 + (1 << ROLE_CHUNK_LG) - 1) >> ROLE_CHUNK_LG;
     const int64_t spread = ((int64_t)n1 + (1 << ROLE_SPREAD_LG) - 1) >> ROLE_SPREAD_LG;
     const int64_t real = (int64_t)nd * chunks;
