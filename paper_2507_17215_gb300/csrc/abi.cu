@@ -502,7 +502,8 @@ struct EdgeStat {
 // them, and with INSERT every edge's pair into the first pair table and its
 // slot word (PAIR_LOOP for a self-loop or an invalid edge, which fails the load anyway). src,
 // dst and t are device memory or pinned host memory (read over the host link, as fast as a copy
-// engine's pull, and once: the list is kept meanwhile, at no cost beside the link's pace).
+// engine's pull, and once: the edges of a long list are kept meanwhile, and its times as the
+// look says).
 // Of device memory nothing else is kept: 16 B read and 8 written per edge, where copies of
 // the three arrays took 16 B more; a table that turns out not to serve, or a range of times
 // past 32 bits that the few did not show, has them copied afterwards. 40M edges of 64-bit times:
@@ -616,12 +617,12 @@ __global__ void __launch_bounds__(256) k_load(const LoadArgs a) {
 }
 
 // The address under which kernels of the current device read p: p itself for memory
-// of this device, the mapped address for pinned host memory (*host set); NULL otherwise
-// (pageable host memory, another device's memory).
+// of this device, the mapped address for pinned host memory (*host: its address on the host);
+// NULL otherwise (pageable host memory, another device's memory).
 template <typename T>
-static const T* kernel_address(const T* p, bool* host) {
+static const T* kernel_address(const T* p, const T** host) {
     cudaPointerAttributes a{};
-    *host = false;
+    *host = nullptr;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
@@ -632,8 +633,9 @@ static const T* kernel_address(const T* p, bool* host) {
         return nullptr;
     }
     if (a.type == cudaMemoryTypeDevice && a.device == dev) return p;
-    *host = a.type == cudaMemoryTypeHost;
-    return *host ? static_cast<const T*>(a.devicePointer) : nullptr;
+    if (a.type != cudaMemoryTypeHost) return nullptr;
+    *host = static_cast<const T*>(a.hostPointer);
+    return static_cast<const T*>(a.devicePointer);
 }
 
 void release_input(folty_graph* g, cudaStream_t s) {
@@ -649,13 +651,29 @@ void release_input(folty_graph* g, cudaStream_t s) {
     g->pre_rank = nullptr;
 }
 
-// A look at a few timestamps in device memory before the list is read: whether they already
-// span more than the 32-bit offsets do. It is enqueued first, and what the load allocates and
+// A look at a few timestamps before the list is read: whether they already span more than the
+// 32-bit offsets do. Those of pinned memory are read by the host: when work on the stream is
+// still to write them, the look may tell a wrong thing, which costs a second read or a store of
+// 64-bit times and no result. For device memory it is enqueued first, and what the load allocates and
 // clears meanwhile hides most of it: 6 us of 120 (6M edges) are left; a second read of 64-bit
 // times and its wait cost 27. Lists of fewer than LOAD_LOOK_EDGES edges are read again instead.
 constexpr int64_t LOAD_LOOK_EDGES = int64_t(1) << 22;
 constexpr int LOAD_LOOK = 16;
-// Pinned lists are kept from this many edges on: below, the allocations (10 us) cost more than
+
+static bool past_32_bits(const int64_t* v) {
+    const auto r = std::minmax_element(v, v + LOAD_LOOK);
+    return *r.first >= 0 && *r.second - *r.first >= (int64_t)0xffffffffll;
+}
+
+static int64_t look_at(int64_t m, int i) { return (m - 1) * i / (LOAD_LOOK - 1); }
+
+static bool pinned_past_32_bits(const int64_t* t, int64_t m) {
+    int64_t v[LOAD_LOOK];
+    for (int i = 0; i < LOAD_LOOK; i++) v[i] = ((const volatile int64_t*)t)[look_at(m, i)];
+    return past_32_bits(v);
+}
+
+// The edges of pinned lists are kept, and their times looked at, from this many on: below, the allocations (10 us) cost more than
 // a second read of what turns out to be needed (at 210 GB/s, 8 B an edge for the times or for
 // the edges of a table that does not serve).
 constexpr int64_t LOAD_KEEP_EDGES = int64_t(1) << 20;
@@ -667,7 +685,7 @@ class TimesLook {
         const void* ptrs[LOAD_LOOK];
         int sizes[LOAD_LOOK];
         for (int i = 0; i < LOAD_LOOK; i++) {
-            ptrs[i] = t + (g->m - 1) * i / (LOAD_LOOK - 1);
+            ptrs[i] = t + look_at(g->m, i);
             sizes[i] = 8;
         }
         FOLTY_CUDA(cudaEventCreateWithFlags(&ev_, cudaEventDisableTiming));
@@ -682,9 +700,7 @@ class TimesLook {
 
     bool past_32_bits() {
         FOLTY_CUDA(cudaEventSynchronize(ev_));
-        const int64_t* v = g_->host_stage;
-        const auto r = std::minmax_element(v, v + LOAD_LOOK);
-        return *r.first >= 0 && *r.second - *r.first >= (int64_t)0xffffffffll;
+        return folty::past_32_bits(g_->host_stage);
     }
 
   private:
@@ -720,10 +736,11 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
     const int cap = insert ? (1 << lg) / 2 : 0;  // load factor at most 1/2
     if (m > 0) {
         LoadArgs a{};
-        bool host[3];
-        a.src = kernel_address(src, &host[0]);
-        a.dst = kernel_address(dst, &host[1]);
-        a.t = kernel_address(t, &host[2]);
+        const int32_t *host_src, *host_dst;
+        const int64_t* host_t;
+        a.src = kernel_address(src, &host_src);
+        a.dst = kernel_address(dst, &host_dst);
+        a.t = kernel_address(t, &host_t);
         a.m = m;
         a.n = g->n;
         a.stat = stat;
@@ -741,21 +758,22 @@ static void load_graph(folty_graph* g, const int32_t* src, const int32_t* dst, c
             a.t = g->in_t;
         }
         const bool keep = !staged && m >= LOAD_KEEP_EDGES;
-        if (keep && (host[0] || host[1])) {
+        if (keep && (host_src || host_dst)) {
             keep_edges();
             a.ksrc = g->in_src;
             a.kdst = g->in_dst;
         }
-        if (keep && host[2]) a.kt = g->in_t = graph_alloc<int64_t>(g, m, s);
+        bool wide = keep && host_t && pinned_past_32_bits(host_t, m);
         std::optional<TimesLook> look;
-        if (m >= LOAD_LOOK_EDGES && !host[2]) look.emplace(g, a.t, s);
+        if (m >= LOAD_LOOK_EDGES && !host_t) look.emplace(g, a.t, s);
         if (insert) {
             g->pre_slotw = graph_alloc<uint32_t>(g, m, s);
             a.slotw = g->pre_slotw;
             a.table = sc.get<uint64_t>(1ll << lg);
             FOLTY_CUDA(cudaMemsetAsync(a.table, 0, sizeof(uint64_t) << lg, s));
         }
-        if (!look || !look->past_32_bits()) a.t32 = g->in_t32 = graph_alloc<uint32_t>(g, m, s);
+        if (look) wide = look->past_32_bits();
+        if (!wide) a.t32 = g->in_t32 = graph_alloc<uint32_t>(g, m, s);
         else if (!staged) a.kt = g->in_t = graph_alloc<int64_t>(g, m, s);
         const bool vec = a16(a.src) && a16(a.dst) && a16(a.t) && a16(a.t32) && a16(a.kt) && a16(a.ksrc) && a16(a.kdst) &&
                          a16(a.slotw);

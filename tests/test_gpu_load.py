@@ -89,6 +89,24 @@ def test_long_lists_in_device_memory(F, m, times):
     assert results[0] == results[1] and len(results[0][1]) > 0
 
 
+# pinned lists whose times the load looks at first (2^20 edges and up), and just too few; a look
+# that misses the one late edge
+@pytest.mark.parametrize("m", [(1 << 20) - 1, 1 << 20, (1 << 20) + 3])
+@pytest.mark.parametrize("times", ["narrow", "wide", "one outlier", "largest offsets", "outlier unseen"])
+def test_long_lists_in_pinned_memory(F, m, times):
+    g = _graph(30_000, m, times.replace("outlier unseen", "one outlier"))
+    if times == "outlier unseen":
+        g.t[[-1, m // 2 + 5]] = g.t[[m // 2 + 5, -1]]
+    scale = 10 ** 5 if times == "wide" else 1
+    queries = [W.Query(d * scale, 1, 10, W.Q_EXISTS, W.DIR_OUT, W.U_HEAD, False) for d in (1, 50)]
+    results = []
+    for xs in ([_place(a, "pinned") for a in (g.src, g.dst, g.t)], (g.src, g.dst, g.t)):
+        with F.TemporalGraph(g.n, *xs) as G:
+            results.append([pairs_of(G.query(q)) for q in queries])
+            assert G.info()["time_sorted"] == (times != "outlier unseen")
+    assert results[0] == results[1] and len(results[0][1]) > 0
+
+
 def test_pinned_lists_cross_the_link_once(F):
     """4M edges of 64-bit times whose pair table does not serve: read once, the 64 MB take about a
     third of a millisecond; read twice, as much again. The load must stay within 1.6 times
