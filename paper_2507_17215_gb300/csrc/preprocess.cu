@@ -1760,7 +1760,7 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         int chunk = TRI_CHUNK_MAX;
         while (chunk > TRI_CHUNK_MIN && (int64_t)chunk * grid * warps * 16 > bound) chunk >>= 1;
         const int64_t ends = (int64_t)chunk * grid * warps;  // entries in no warp's use at the chunks' ends
-        const int64_t cap = bound + ends;
+        const int64_t cap = (bound + ends + 31) & ~int64_t(31);  // whole chunks are in use: no padding to clear
         g->tri = graph_alloc<int4>(g, cap, s);
         g->tri_off = nullptr;
         uint8_t* live = liveness_rows(g, 1, cap, s);
@@ -1787,7 +1787,8 @@ static void preprocess_on(folty_graph* g, cudaStream_t s) {
         g->info.sigma_max = (int32_t)outv[4];
         g->enum_bytes = 4 * outv[0] + 8 * (int64_t)S;
         span.add_bytes(4 * outv[0] + 17 * g->ntri);
-        listed_liveness(g, live, cap, g->ntri + ends, s);  // (tri_cap itself differs from run to run)
+        // (tri_cap itself, whole chunks, differs from run to run)
+        listed_liveness(g, live, cap, (g->ntri + ends + 31) & ~int64_t(31), s);
     } else {
         const int64_t ntri = g->ntri;
         g->tri_cap = ntri;
